@@ -125,8 +125,8 @@ typedef struct {
     int atoms_per_thread; /* atoms per thread group: 0 or 1 (2, two atoms sharing
                            a union list, is no longer provided:
                            PTA_EUNSUPPORTED)                                  */
-    double prune_margin;  /* mixed precision: the pair passes read an inner list
-                           of the pairs within rc + prune_margin, pruned from the
+    double prune_margin;  /* the pair passes read an inner list of the pairs within
+                           rc + prune_margin, pruned from the
                            Verlet list whenever an atom has moved more than
                            prune_margin / 2 since the last pruning; it holds every
                            pair within rc in the same order, so results do not
@@ -163,7 +163,7 @@ typedef struct {
     int64_t nsteps;
     int32_t rebuilds;
     int32_t status;    /* pta_status of this burst */
-    int32_t prunes;    /* inner-list prunings during the burst (mixed precision) */
+    int32_t prunes;    /* inner-list prunings during the burst */
     int32_t converged; /* adaptive length: bit m set when variable m converged */
     int64_t nsamples[3];
 } pta_averages;

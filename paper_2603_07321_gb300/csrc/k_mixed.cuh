@@ -3,9 +3,9 @@
 // and the per-atom velocity-Verlet update of Eqs. (vv_algo_*) fused behind
 // the force pass.
 //
-// Precision: pair terms in FP32 on relative coordinates; positions are an
-// exact FP32 pair x = hi + lo (hi on a 2^-12 A grid, |lo| <= 2^-13 A);
-// velocities an exact FP32 pair v = vh + vl (|vl| <= ulp(vh) / 2) updated by
+// Precision: pair terms in FP32 on exact differences of fixed-point records;
+// positions are an exact FP32 pair x = hi + lo (hi on a 2^-12 A grid, |lo| <=
+// 2^-13 A); velocities an exact FP32 pair v = vh + vl (|vl| <= ulp(vh) / 2) updated by
 // error-free addition, so that half-kicks lose nothing to rounding over long
 // bursts; K, U and R are converted to FP64 per atom and reduced in FP64.
 #pragma once
@@ -14,95 +14,110 @@
 
 namespace pta {
 
-template <bool SC76>
-struct PowF {
-    // s^m and s^n for the Sutton-Chen exponents
-    __device__ __forceinline__ static void pw(float s, int n, int m, float &sn, float &sm) {
-        if (SC76) {
-            const float s2 = s * s, s3 = s2 * s;
-            sm = s3 * s3;
-            sn = sm * s;
-        } else {
-            float p = 1.f, q = 1.f;
-            for (int i = 0; i < m; ++i) p *= s;
-            for (int i = 0; i < n; ++i) q *= s;
-            sm = p;
-            sn = q;
-        }
-    }
-    __device__ __forceinline__ static float pm(float s, int m) {
-        if (SC76) {
-            const float s2 = s * s, s3 = s2 * s;
-            return s3 * s3;
-        }
-        float p = 1.f;
-        for (int i = 0; i < m; ++i) p *= s;
-        return p;
-    }
+// hardware estimates without the subnormal handling of rsqrtf / division
+// (three instructions of each pair's terms): relative errors at most 2^-22.9
+// and 2^-23; an infinite argument gives 0
+__device__ __forceinline__ float rsq_approx(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+__device__ __forceinline__ float powi(float s, int k) {
+    float p = 1.f;
+    for (int i = 0; i < k; ++i) p *= s;
+    return p;
+}
+
+// Squared distance (A^2) of a neighbour's record from the atom's, and the
+// displacement in quanta (q2: square of the quantum).
+__device__ __forceinline__ float pair_r2(float q2, const int4 &a, const int4 &b, float &dx,
+                                         float &dy, float &dz) {
+    dx = (float)(b.x - a.x);
+    dy = (float)(b.y - a.y);
+    dz = (float)(b.z - a.z);
+    return fmaf(dz, dz, fmaf(dy, dy, dx * dx)) * q2;
+}
+
+// A pair beyond rc gets y = 1/r = 0 (the force pass) or r^2 = infinity, whose
+// estimates are 0 (the density pass), which makes every term exactly zero: no
+// branch, and no trace of such pairs in the sums.
+//
+// Bound: instruction dispatch (an FP32 multiply-add of three registers takes
+// 1.5 cycles of it; packed FP32 instructions take 2-3 and gave nothing), ~25
+// and ~34 instructions per entry.  How the powers of 1/r are formed decides
+// the accuracy.  Velocities after 300 steps of the 32,000-atom cube are off by
+// 4.6e-7 of their norm in this form; by 6.1e-7 with both passes' powers
+// raised from a Newton-refined 1/r (as many instructions in the force pass,
+// four more in the density pass), and by 6.9e-7 with plain estimates in the
+// force pass as well: an estimate's error changes slowly with r, so it acts
+// on a pair in the same direction for many steps.
+
+// density pass, one pair: sums of (1/r)^n, r and the pair count, from which
+// phi_n = a^n (1/r)^n - A_n + B_n (r - rc) is assembled once per atom, and of
+// (1/r)^m, assembled likewise for the Sutton-Chen exponents (m = 6: the sum is
+// far larger than what is taken off it), or of phi_m itself
+struct RhoSums {
+    float sm = 0.f, sn = 0.f, sr = 0.f;
+    int cnt = 0;
 };
-
-// 1 / sqrt(r2): the hardware estimate refined by one Newton-Raphson step
-// y' = y + y (1 - r2 y^2) / 2 (the residual formed with a fused multiply-add),
-// which brings it to about one unit in the last place; the pair terms raise
-// s = a / r to the 6th and 7th power, which multiplies its relative error
-__device__ __forceinline__ float rsqrt_nr(float r2) {
-    const float y = rsqrtf(r2);
-    const float e = fmaf(-(r2 * y), y, 1.0f);
-    return fmaf(0.5f * y, e, y);
-}
-
-// packed FP32 (two lanes of one instruction), round to nearest
-__device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
-__device__ __forceinline__ float2 rsqrt2_nr(float2 r2) {
-    // rsqrt_nr on both halves: y' = y + (-y/2) (r2 y y - 1), the same
-    // operations and roundings as the scalar form
-    const float2 y = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
-    const float2 e = __ffma2_rn(__fmul2_rn(r2, y), y, f2(-1.0f));
-    return __ffma2_rn(__fmul2_rn(y, f2(-0.5f)), e, y);
-}
-
-// phi_m of two pairs at once (squared distances r2), for the density sum:
-// with y = 1/r, phi_m = (a^m y^m - Am) + Bm (r - rc); the caller adds the
-// halves whose r2 is below rc^2, in order
-__device__ __forceinline__ float2 phi_m2_sc76(const PotF &P, float2 r2) {
-    const float2 y = rsqrt2_nr(r2);
-    const float2 y2 = __fmul2_rn(y, y);
-    const float2 y3 = __fmul2_rn(y2, y);
-    const float2 y6 = __fmul2_rn(y3, y3);
-    const float2 u = __ffma2_rn(r2, y, f2(-P.rc));
-    return __ffma2_rn(f2(P.Bm), u, __ffma2_rn(f2(P.am), y6, f2(-P.Am)));
-}
-
-// phi_m of one pair (r2 < rc^2)
 template <bool SC76>
-__device__ __forceinline__ float phi_m1(const PotF &P, float r2) {
-    const float ir = rsqrt_nr(r2);
-    const float s = P.a * ir;
-    return PowF<SC76>::pm(s, P.m) - P.Am + P.Bm * (r2 * ir - P.rc);
+__device__ __forceinline__ void rho_pair(const PotF &P, float q2, const int4 &a, const int4 &b,
+                                         RhoSums &s) {
+    float dx, dy, dz;
+    const float r2 = pair_r2(q2, a, b, dx, dy, dz);
+    const bool in = r2 < P.rc2;
+    if (SC76) {
+        const float rm = in ? r2 : __int_as_float(0x7f800000);
+        const float u = rcp_approx(rm), y = rsq_approx(rm);
+        const float u3 = (u * u) * u;
+        s.sm += u3;
+        s.sn = fmaf(u3, y, s.sn);
+        s.sr = fmaf(r2, y, s.sr);
+    } else {
+        float y = rsq_approx(r2);
+        y = in ? y : 0.f;
+        y = fmaf(0.5f * y, fmaf(-r2, y * y, 1.f), y);
+        s.sm += in ? powi(P.a * y, P.m) - P.Am + P.Bm * fmaf(r2, y, -P.rc) : 0.f;
+        s.sn += powi(y, P.n);
+        s.sr = fmaf(r2, y, s.sr);
+    }
+    s.cnt += in;
 }
 
-// one pair's contribution to the force on the atom and to its pair-energy
-// sums: displacement (ex, ey, ez) = r_j - r_i, r2 = |r_j - r_i|^2 < rc^2,
-// q = w_i + w_j where each record carries w = m a^m B'(rho).  With y = 1/r,
+// force pass, one pair: with q = w_i + w_j where each record carries
+// w = m a^m B'(rho),
 //   [eps phi_n'(r) + (B'_i + B'_j) phi_m'(r)] / r
-//       = y (eps Bn + q Bm / (m a^m)) - y^2 (eps n a^n y^n + q y^m),
-// and phi_n(r) = a^n y^n + Bn (r + c1) with c1 = -(An / Bn + rc): the pass
-// sums y^n into e7 and r + c1 into er (the constants applied once per atom)
+//       = y (eps Bn + q Bm / (m a^m)) - y^(m+2) (q + eps n a^n y^(n-m))
+// (n = 7, m = 6: y^8 = u^4)
 template <bool SC76>
-__device__ __forceinline__ void force_pair(const PotF &P, float ex, float ey, float ez, float r2,
-                                           float q, float &fx, float &fy, float &fz, float &e7,
-                                           float &er) {
-    const float y = rsqrt_nr(r2);
-    float yn, ym;
-    PowF<SC76>::pw(y, P.n, P.m, yn, ym);
-    const float t = fmaf(q, ym, P.kn * yn);
+__device__ __forceinline__ void force_pair(const PotF &P, float q2, const int4 &a, float wa,
+                                           const int4 &b, float &fx, float &fy, float &fz) {
+    float dx, dy, dz;
+    const float r2 = pair_r2(q2, a, b, dx, dy, dz);
+    const float q = wa + __int_as_float(b.w);
     const float c = fmaf(q, P.bmq, P.ebn);
-    const float gg = y * fmaf(-y, t, c);
-    fx += gg * ex;
-    fy += gg * ey;
-    fz += gg * ez;
-    e7 += yn;
-    er += fmaf(r2, y, P.c1);
+    float y = rsq_approx(r2), v;
+    y = r2 < P.rc2 ? y : 0.f;
+    // one Newton-Raphson step on both 1/r^2 and 1/r from the same residual
+    const float y2 = y * y, e = fmaf(-r2, y2, 1.f);
+    y = fmaf(0.5f * y, e, y);
+    if (SC76) {
+        const float u = fmaf(y2, e, y2), u2 = u * u;
+        v = (u2 * u2) * fmaf(P.kn, y, q);
+    } else {
+        const float ym = powi(y, P.m), yn = powi(y, P.n);
+        v = (y * y) * fmaf(q, ym, P.kn * yn);
+    }
+    const float g = fmaf(y, c, -v);
+    fx = fmaf(g, dx, fx);
+    fy = fmaf(g, dy, fy);
+    fz = fmaf(g, dz, fz);
 }
 
 // (h, l) += d exactly up to the final renormalisation: Knuth's two-sum of h
@@ -118,24 +133,21 @@ __device__ __forceinline__ void hl_add(float &h, float &l, float d) {
     h = hh;
 }
 
-// After the force pass of atom a (compact slot; force f, pair-energy sum
-// en = sum_j phi_n(r_aj), record weight fpa = m a^m B'(rho_a)): its energy, its share of the reaction, and the
-// velocity-Verlet update -- the half-kick that finishes the step (phase RUN),
+// After the force pass of atom a (force f, record weight fpa = m a^m
+// B'(rho_a); its pair energy from the density pass): its energy, its share of
+// the reaction, and the velocity-Verlet update -- the half-kick that finishes the step (phase RUN),
 // the sample of K, and unless the burst ends the half-kick and drift of the
 // next step; the new position (hi + lo, whole grid quanta moved from lo to
-// hi), its neighbour record (position relative to the reference point C,
-// written at record index rec), and the displacements since the last list
+// hi), its neighbour record, and the displacements since the last list
 // build (and, with `pruned`, since the last pruning).  Grip
 // atoms keep v = 0.  MODE_EVAL stores F and the energy instead.
 __device__ __forceinline__ void atom_update_mixed(const SpecDev &S, SpecCtl *ctl, int par, int a,
-                                                  long long rec, float3 C, bool pruned, float fpa,
-                                                  float fx, float fy, float fz, float en, int mode,
-                                                  int phase, long long done, long long nsteps,
-                                                  double &ke, double &pe, double &rr, float &d2,
-                                                  float &dp2) {
+                                                  bool pruned, float fpa, float fx, float fy,
+                                                  float fz, int mode, int phase, long long done,
+                                                  long long nsteps, double &ke, double &pe,
+                                                  double &rr, float &d2, float &dp2) {
     chk_force(S, fx, fy, fz);
-    const float eps = S.pot.f_eps;
-    const float pe_a = 0.5f * eps * en + (fpa != 0.f ? S.pot.f_ec2hq / fpa : 0.f);
+    const float pe_a = S.pen[a] + (fpa != 0.f ? S.pot.f_ec2hq / fpa : 0.f);
     pe += (double)pe_a;
     const uint8_t flag = S.flags[a];
     if (flag == FLAG_RIGHT) rr -= (double)(S.axis == 0 ? fx : (S.axis == 1 ? fy : fz));
@@ -204,8 +216,7 @@ __device__ __forceinline__ void atom_update_mixed(const SpecDev &S, SpecCtl *ctl
     }
     ((float4 *)S.pos[par ^ 1])[a] = make_float4(hh[0], hh[1], hh[2], 0.f);
     S.lo[par ^ 1][a] = make_float4(qq[0], qq[1], qq[2], 0.f);
-    S.rel[par ^ 1][rec] = make_float4((hh[0] - C.x) + qq[0], (hh[1] - C.y) + qq[1],
-                                      (hh[2] - C.z) + qq[2], 0.f);
+    S.rec[par ^ 1][a] = rec_mixed(S, hh[0], hh[1], hh[2], qq[0], qq[1], qq[2]);
     *vp = v;
     const float4 rf = S.ref[a];
     const float ex = (hh[0] - rf.x) + qq[0], ey = (hh[1] - rf.y) + qq[1],

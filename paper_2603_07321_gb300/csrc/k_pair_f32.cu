@@ -1,221 +1,119 @@
 // Mixed-precision pair kernels on Verlet lists: Sutton-Chen EAM density and
-// forces in FP32 on relative coordinates.  What a neighbour reads is one
-// 16-byte record, its position relative to the centre C of its half-cell
-// (one of the 8 octants of its cell, fixed at the list build),
-// rel = (hi - C) + lo with |rel| <= h / 4 + skin / 2, so that with the
-// half-cell offset d coded in the list entry
-//     r_j - r_i = (rel_j - rel_i) + (h / 2) d
-// (C and h on exact grids).  The one-lane loops take two entries per
-// iteration (four in the density pass) and decode both offsets with packed
-// FP32 instructions (two lanes of one instruction, sm_100 family); the
-// density pass also forms both pair terms packed, then adds them to its sum
-// in entry order.
+// forces in FP32.  What a neighbour reads is one 16-byte record, its position
+// in fixed point (see the record format), so that r_j - r_i is an exact
+// integer difference converted once.
 //
 // Pass 1 (density): rho_i = sum_j phi_m(r_ij), then B'(rho_i) =
 // -eps c / (2 sqrt(rho_i)), stored beside the record scaled by m a^m (the
-// force pass's pair terms are arranged around that weight).  Eq. (pe).
+// force pass's pair terms are arranged around that weight), and the atom's
+// pair energy.  Eq. (pe).
 // Pass 2 (force):   F_i = sum_j [eps phi_n'(r) + (B'_i + B'_j) phi_m'(r)] (r_j - r_i)/r,
-// Eq. (f_int), the per-atom energy 1/2 eps sum_j phi_n + B(rho_i), and the
-// velocity-Verlet update fused behind it (atom_update_mixed).  Grip atoms
-// keep v = 0 and F = 0 in the update; their internal force still enters the
-// reaction R = -sum_{right grip} F . e of Eq. (state_variables).
+// Eq. (f_int), and the velocity-Verlet update fused behind it
+// (atom_update_mixed).  Grip atoms keep v = 0 and F = 0 in the update; their
+// internal force still enters the reaction R = -sum_{right grip} F . e of
+// Eq. (state_variables).
 #include "k_mixed.cuh"
 
 namespace pta {
 
-// Every lane's list ends with sentinel entries that bring its count to a
-// multiple of four (they name a record far from every atom, so their pairs
-// fail the cutoff test like any distant neighbour): the loops take four
-// entries per iteration (two with several lanes per atom) without per-entry
-// bounds tests, and read the next group's list words before evaluating the
-// current one; those reads go past the count into the sixteen spare rows
-// every list keeps and are never gathered.
-
-// the entries lane l of atom u reads (the inner list when pruning is on, else
-// the Verlet list), as a pointer to its first word (stride 32) and a count,
-// rounded up to a multiple of four over the sentinel rows
-__device__ __forceinline__ const unsigned *lane_list(const SpecDev &S, int u, int l, int L, int &cl) {
-    const long long off = nl_base(u, L, S.cap) + l;
-    if (S.prune_on) {
-        cl = chk_count(S, S.pnn[(long long)u * L + l], S.cap_use / L + 4);
-        return (const unsigned *)S.plist + off;
-    }
-    const int nn = S.nn[u];
-    cl = chk_count(S, (nn > l ? (nn - l + L - 1) / L : 0), S.cap_use / L);
-    cl = (cl + 3) & ~3;
-    return (const unsigned *)S.nlist + off;
-}
-
-// one list word: read once per pass, so it skips L1 (the neighbour records
-// keep the space) and asks L2 to fetch the 256-byte block around it, which
-// holds the warp's next row as well
-__device__ __forceinline__ unsigned ld_list(const unsigned *p) {
-    unsigned v;
-    asm("ld.global.nc.L1::no_allocate.L2::256B.u32 %0, [%1];" : "=r"(v) : "l"(p));
+// four list entries: read once per pass, so they skip L1 (the neighbour
+// records keep the space) and ask L2 to fetch the 256-byte block around them
+__device__ __forceinline__ uint4 ld_quad(const uint4 *p) {
+    uint4 v;
+    asm("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];"
+        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+        : "l"(p));
     return v;
 }
-
-// displacements of two entries from the atom, packed by axis
-__device__ __forceinline__ void entry_disp2(unsigned ea, unsigned eb, float4 xa, float4 xb, float4 r0,
-                                            float h, float h8, float h64, float2 &dx, float2 &dy,
-                                            float2 &dz) {
-    const float2 ox = __fadd2_rn(make_float2(__int_as_float(0x4B400000 | (int)(ea & 0x7u)),
-                                             __int_as_float(0x4B400000 | (int)(eb & 0x7u))),
-                                 f2(-12582915.0f));
-    const float2 oy = __fadd2_rn(make_float2(__int_as_float(0x4B400000 | (int)(ea & 0x38u)),
-                                             __int_as_float(0x4B400000 | (int)(eb & 0x38u))),
-                                 f2(-12582936.0f));
-    const float2 oz = __fadd2_rn(make_float2(__int_as_float(0x4B400000 | (int)(ea & 0x1C0u)),
-                                             __int_as_float(0x4B400000 | (int)(eb & 0x1C0u))),
-                                 f2(-12583104.0f));
-    dx = __ffma2_rn(ox, f2(h), __fadd2_rn(make_float2(xa.x, xb.x), f2(-r0.x)));
-    dy = __ffma2_rn(oy, f2(h8), __fadd2_rn(make_float2(xa.y, xb.y), f2(-r0.y)));
-    dz = __ffma2_rn(oz, f2(h64), __fadd2_rn(make_float2(xa.z, xb.z), f2(-r0.z)));
+__device__ __forceinline__ int4 ld_rec(const SpecDev &S, const void *rec, unsigned e) {
+    return __ldg((const int4 *)((const char *)rec + nl_off(S, e)));
 }
 
-// density terms of two entries, added in entry order
-template <bool SC76>
-__device__ __forceinline__ void rho_add2(const PotF &P, float2 dx, float2 dy, float2 dz,
-                                         float &rho) {
-    float2 r2 = __fmul2_rn(dx, dx);
-    r2 = __ffma2_rn(dy, dy, r2);
-    r2 = __ffma2_rn(dz, dz, r2);
-    const float rc2 = P.rc2;
-    if (SC76) {
-        const float2 phi = phi_m2_sc76(P, r2);
-        if (r2.x < rc2) rho += phi.x;
-        if (r2.y < rc2) rho += phi.y;
-    } else {
-        if (r2.x < rc2) rho += phi_m1<false>(P, r2.x);
-        if (r2.y < rc2) rho += phi_m1<false>(P, r2.y);
+// f(record) for the entries lane l of atom u reads, in list order: a quad per
+// iteration (four gathers in flight), the next quad read ahead, then what is
+// left of the last one
+template <class F>
+__device__ __forceinline__ void for_entries(const SpecDev &S, const void *rec, int u, int l, int L,
+                                            F f) {
+    const uint4 *p = S.plist + nl_col(u, l, L, S.capq);
+    const int cnt = chk_count(S, S.pnn[u * L + l], 4 * (S.capq - 1));
+    uint4 e = ld_quad(p);
+    for (int t = cnt >> 2; t > 0; --t) {
+        p += 32;
+        const uint4 nx = ld_quad(p);
+        const int4 x0 = ld_rec(S, rec, e.x), x1 = ld_rec(S, rec, e.y);
+        const int4 x2 = ld_rec(S, rec, e.z), x3 = ld_rec(S, rec, e.w);
+        f(x0);
+        f(x1);
+        f(x2);
+        f(x3);
+        e = nx;
+    }
+    const int left = cnt & 3;
+    if (left) {
+        int4 x0 = ld_rec(S, rec, e.x), x1 = x0, x2 = x0;
+        if (left > 1) x1 = ld_rec(S, rec, e.y);
+        if (left > 2) x2 = ld_rec(S, rec, e.z);
+        f(x0);
+        if (left > 1) f(x1);
+        if (left > 2) f(x2);
     }
 }
 
 template <int L, bool SC76>
-__global__ void __launch_bounds__(TPB, 8) k_density_f32(const SpecDev *__restrict__ specs,
-                                                        const int *__restrict__ b2s, int force,
-                                                        const PotF P) {
-    const SpecDev &S = specs[b2s[blockIdx.x]];
-    const SpecCtl *ctl = S.ctl;
-    if (!force && ctl->phase == PH_IDLE) return;
-    const int par = ctl->parity;
+__device__ __forceinline__ void density_block(const SpecDev &S, int lb, int par, const PotF &P) {
     constexpr int UPB = TPB / L;
-    const int u = (blockIdx.x - S.blk_pair0) * UPB + threadIdx.x / L;
-    const int l = threadIdx.x % L;
-    const bool valid = u < S.n;
-    const float4 *__restrict__ rel = S.rel[par];
-    const float h = S.f_q, h8 = S.f_q8, h64 = S.f_q64;
-    float rho = 0.f;
-    float4 ra = make_float4(0, 0, 0, 0);
-    if (valid) {
-        ra = rel[u];
-        int cl;
-        const unsigned *__restrict__ lst = lane_list(S, u, l, L, cl);
-        if constexpr (L == 1) {
-            unsigned e0 = ld_list(lst), e1 = ld_list(lst + 32), e2 = ld_list(lst + 64), e3 = ld_list(lst + 96);
-            for (int q = 0; q < cl; q += 4) {
-                const unsigned n0 = ld_list(lst + (q + 4) * 32), n1 = ld_list(lst + (q + 5) * 32);
-                const unsigned n2 = ld_list(lst + (q + 6) * 32), n3 = ld_list(lst + (q + 7) * 32);
-                const float4 x0 = __ldg(rel + nl_atom(S, e0)), x1 = __ldg(rel + nl_atom(S, e1));
-                const float4 x2 = __ldg(rel + nl_atom(S, e2)), x3 = __ldg(rel + nl_atom(S, e3));
-                float2 dx, dy, dz;
-                entry_disp2(e0, e1, x0, x1, ra, h, h8, h64, dx, dy, dz);
-                rho_add2<SC76>(P, dx, dy, dz, rho);
-                entry_disp2(e2, e3, x2, x3, ra, h, h8, h64, dx, dy, dz);
-                rho_add2<SC76>(P, dx, dy, dz, rho);
-                e0 = n0; e1 = n1; e2 = n2; e3 = n3;
-            }
-        } else {
-            unsigned ea = ld_list(lst), eb = ld_list(lst + 32);
-            for (int q = 0; q < cl; q += 2) {
-                const unsigned na = ld_list(lst + (q + 2) * 32), nb = ld_list(lst + (q + 3) * 32);
-                const float4 xa = __ldg(rel + nl_atom(S, ea));
-                const float4 xb = __ldg(rel + nl_atom(S, eb));
-                float2 dx, dy, dz;
-                entry_disp2(ea, eb, xa, xb, ra, h, h8, h64, dx, dy, dz);
-                rho_add2<SC76>(P, dx, dy, dz, rho);
-                ea = na;
-                eb = nb;
-            }
-        }
-    }
-    rho = lane_sum<L>(rho);
-    if (valid && l == 0) {
-        // w = m a^m B'(rho), B'(rho) = -eps c / (2 sqrt(rho))
-        const float fp = rho > 0.f ? P.fpsc * rsqrtf(rho) : 0.f;
-        ((float4 *)S.posfp)[u] = make_float4(ra.x, ra.y, ra.z, fp);
-    }
-}
-
-template <int L, bool SC76>
-__global__ void __launch_bounds__(TPB, 8) k_force_f32(const SpecDev *__restrict__ specs,
-                                                      const int *__restrict__ b2s, int mode,
-                                                      const PotF P) {
-    const SpecDev &S = specs[b2s[blockIdx.x]];
-    SpecCtl *ctl = S.ctl;
-    const int phase = ctl->phase;
-    if (mode == MODE_STEP && phase == PH_IDLE) return;
-    const int par = ctl->parity;
-    const long long done = ctl->done, nsteps = ctl->nsteps;
-    constexpr int UPB = TPB / L;
-    const int lb = blockIdx.x - S.blk_pair0;
     const int u = lb * UPB + threadIdx.x / L;
     const int l = threadIdx.x % L;
     const bool valid = u < S.n;
-    const float4 *__restrict__ lf = (const float4 *)S.posfp;
-    const float h = S.f_q, h8 = S.f_q8, h64 = S.f_q64;
-    const float rc2 = P.rc2;
-    float fx = 0.f, fy = 0.f, fz = 0.f, e7 = 0.f, er = 0.f;
-    float4 ra = make_float4(0, 0, 0, 0);
+    RhoSums s;
+    int4 ra = make_int4(0, 0, 0, 0);
     if (valid) {
-        ra = lf[u];
-        int cl;
-        const unsigned *__restrict__ lst = lane_list(S, u, l, L, cl);
-        // the offsets of two entries decoded in packed instructions; the pair
-        // terms stay scalar (packed, they measured slower here)
-        auto two = [&](unsigned ea, unsigned eb, float4 xa, float4 xb) {
-            float2 dx, dy, dz;
-            entry_disp2(ea, eb, xa, xb, ra, h, h8, h64, dx, dy, dz);
-            const float r2a = dx.x * dx.x + dy.x * dy.x + dz.x * dz.x;
-            if (r2a < rc2)
-                force_pair<SC76>(P, dx.x, dy.x, dz.x, r2a, ra.w + xa.w, fx, fy, fz, e7, er);
-            const float r2b = dx.y * dx.y + dy.y * dy.y + dz.y * dz.y;
-            if (r2b < rc2)
-                force_pair<SC76>(P, dx.y, dy.y, dz.y, r2b, ra.w + xb.w, fx, fy, fz, e7, er);
-        };
-        if constexpr (L == 1) {
-            unsigned e0 = ld_list(lst), e1 = ld_list(lst + 32), e2 = ld_list(lst + 64),
-                     e3 = ld_list(lst + 96);
-            for (int q = 0; q < cl; q += 4) {
-                const unsigned n0 = ld_list(lst + (q + 4) * 32), n1 = ld_list(lst + (q + 5) * 32);
-                const unsigned n2 = ld_list(lst + (q + 6) * 32), n3 = ld_list(lst + (q + 7) * 32);
-                const float4 x0 = __ldg(lf + nl_atom(S, e0)), x1 = __ldg(lf + nl_atom(S, e1));
-                const float4 x2 = __ldg(lf + nl_atom(S, e2)), x3 = __ldg(lf + nl_atom(S, e3));
-                two(e0, e1, x0, x1);
-                two(e2, e3, x2, x3);
-                e0 = n0; e1 = n1; e2 = n2; e3 = n3;
-            }
-        } else {
-            unsigned ea = ld_list(lst), eb = ld_list(lst + 32);
-            for (int q = 0; q < cl; q += 2) {
-                const unsigned na = ld_list(lst + (q + 2) * 32), nb = ld_list(lst + (q + 3) * 32);
-                const float4 xa = __ldg(lf + nl_atom(S, ea));
-                const float4 xb = __ldg(lf + nl_atom(S, eb));
-                two(ea, eb, xa, xb);
-                ea = na;
-                eb = nb;
-            }
-        }
+        ra = S.rec[par][u];
+        const float q2 = S.f_q2;
+        for_entries(S, S.rec[par], u, l, L,
+                    [&](const int4 &x) { rho_pair<SC76>(P, q2, ra, x, s); });
     }
-    fx = lane_sum<L>(fx);
-    fy = lane_sum<L>(fy);
-    fz = lane_sum<L>(fz);
-    const float en = lane_sum<L>(P.an * e7 + P.Bn * er);
+    s.sm = lane_sum<L>(s.sm);
+    s.sn = lane_sum<L>(s.sn);
+    s.sr = lane_sum<L>(s.sr);
+    const float cnt = (float)lane_sum<L>(s.cnt);
+    if (valid && l == 0) {
+        const float dr = fmaf(-cnt, P.rc, s.sr);  // sum of r - rc
+        const float rho = SC76 ? fmaf(P.am, s.sm, fmaf(P.Bm, dr, -cnt * P.Am)) : s.sm;
+        const float phn = fmaf(P.an, s.sn, fmaf(P.Bn, dr, -cnt * P.An));
+        // w = m a^m B'(rho), B'(rho) = -eps c / (2 sqrt(rho))
+        const float w = rho > 0.f ? P.fpsc * rsqrtf(rho) : 0.f;
+        S.pen[u] = 0.5f * P.eps * phn;
+        ((int4 *)S.posfp)[u] = make_int4(ra.x, ra.y, ra.z, __float_as_int(w));
+    }
+}
+
+template <int L, bool SC76>
+__device__ __forceinline__ void force_block(const SpecDev &S, int lb, int par, const PotF &P,
+                                            int mode, int phase, long long done,
+                                            long long nsteps) {
+    constexpr int UPB = TPB / L;
+    const int u = lb * UPB + threadIdx.x / L;
+    const int l = threadIdx.x % L;
+    const bool valid = u < S.n;
+    float fx = 0.f, fy = 0.f, fz = 0.f, wa = 0.f;
+    if (valid) {
+        const int4 ra = ((const int4 *)S.posfp)[u];
+        wa = __int_as_float(ra.w);
+        const float q2 = S.f_q2;
+        for_entries(S, S.posfp, u, l, L,
+                    [&](const int4 &x) { force_pair<SC76>(P, q2, ra, wa, x, fx, fy, fz); });
+    }
+    // sums of (eV/A^2) x quanta
+    fx = lane_sum<L>(fx) * S.f_q;
+    fy = lane_sum<L>(fy) * S.f_q;
+    fz = lane_sum<L>(fz) * S.f_q;
     double ke = 0.0, pe = 0.0, rr = 0.0;
     float d2 = 0.f, dp2 = 0.f;
     if (valid && l == 0)
-        atom_update_mixed(S, ctl, par, u, u, half_centre(S, S.atom_cell[u], S.hsub[u]), S.prune_on != 0,
-                          ra.w, fx, fy, fz, en, mode, phase, done, nsteps, ke, pe, rr, d2, dp2);
+        atom_update_mixed(S, S.ctl, par, u, S.prune_on != 0, wa, fx, fy, fz, mode, phase, done,
+                          nsteps, ke, pe, rr, d2, dp2);
     ke = warp_sum(ke);
     pe = warp_sum(pe);
     rr = warp_sum(rr);
@@ -225,63 +123,82 @@ __global__ void __launch_bounds__(TPB, 8) k_force_f32(const SpecDev *__restrict_
                    nsteps);
 }
 
-// Inner list: every lane keeps, in order, the entries of its own column of
-// the Verlet list that lie within the pruning radius of the atom (FP32
-// distances tested against (rc + margin)^2 widened by 1e-5).  Pairs within
-// rc are therefore all kept, in the order the lane sums them.  Sentinel
-// entries then bring the lane's count to a multiple of four.
-template <int L>
-__global__ void __launch_bounds__(TPB, 7) k_prune_f32(const SpecDev *__restrict__ specs,
-                                                      const int *__restrict__ b2s, int force) {
+template <int L, bool SC76>
+__global__ void __launch_bounds__(TPB, 8) k_density_f32(const SpecDev *__restrict__ specs,
+                                                        const int *__restrict__ b2s, int force,
+                                                        const PotF P) {
     const SpecDev &S = specs[b2s[blockIdx.x]];
-    if (S.prec == PTA_PREC_FP64 || !prune_active(S, force)) return;
+    if (!force && S.ctl->phase == PH_IDLE) return;
+    density_block<L, SC76>(S, blockIdx.x - S.blk_pair0, S.ctl->parity, P);
+}
+
+template <int L, bool SC76>
+__global__ void __launch_bounds__(TPB, 8) k_force_f32(const SpecDev *__restrict__ specs,
+                                                      const int *__restrict__ b2s, int mode,
+                                                      const PotF P) {
+    const SpecDev &S = specs[b2s[blockIdx.x]];
     const SpecCtl *ctl = S.ctl;
-    const int par = ctl->parity;
+    const int phase = ctl->phase;
+    if (mode == MODE_STEP && phase == PH_IDLE) return;
+    force_block<L, SC76>(S, blockIdx.x - S.blk_pair0, ctl->parity, P, mode, phase, ctl->done,
+                         ctl->nsteps);
+}
+
+// Pruning (both precisions): every lane appends to the near part of its
+// column, in order, the entries of its far part within the pruning radius
+// (FP32 distances of the records against (rc + margin)^2 with slack).  Pairs
+// within rc are therefore all kept, in the order the lane sums them.
+//
+// Bound: the gathers of the far part's records (~118 of the ~252 entries of a
+// bulk atom at the default 2 A skin).
+template <int L>
+__global__ void __launch_bounds__(TPB, 8) k_prune(const SpecDev *__restrict__ specs,
+                                                  const int *__restrict__ b2s, int force) {
+    const SpecDev &S = specs[b2s[blockIdx.x]];
+    if (!prune_active(S, force)) return;
+    const int par = S.ctl->parity;
     constexpr int UPB = TPB / L;
     const int u = (blockIdx.x - S.blk_pair0) * UPB + threadIdx.x / L;
     const int l = threadIdx.x % L;
     if (u >= S.n) return;
-    const float4 *__restrict__ rel = S.rel[par];
-    const float h = S.f_q, h8 = S.f_q8, h64 = S.f_q64, rp2 = S.f_rp2;
-    const float4 ra = rel[u];
-    const long long off = nl_base(u, L, S.cap) + l;
-    const unsigned *__restrict__ src = (const unsigned *)S.nlist + off;
-    unsigned *__restrict__ dst = (unsigned *)S.plist + off;
-    const int nn = S.nn[u];
-    const int cl = chk_count(S, nn > l ? (nn - l + L - 1) / L : 0, S.cap_use / L);
-    int kept = 0;
-    // eight entries per iteration (eight gathers in flight), the next eight
-    // words read ahead: rows up to cl + 14, within the spare iterations
-    unsigned e[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) e[k] = ld_list(src + k * 32);
-    for (int q = 0; q < cl; q += 8) {
-        unsigned nx[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) nx[k] = ld_list(src + (q + 8 + k) * 32);
-        float4 x[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) x[k] = __ldg(rel + nl_atom(S, e[k]));
-#pragma unroll
-        for (int k = 0; k < 8; k += 2) {
-            float2 dx, dy, dz;
-            entry_disp2(e[k], e[k + 1], x[k], x[k + 1], ra, h, h8, h64, dx, dy, dz);
-            const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
-            if (q + k < cl && r2.x < rp2) dst[(kept++) * 32] = e[k];
-            if (q + k + 1 < cl && r2.y < rp2) dst[(kept++) * 32] = e[k + 1];
+    const int4 *rec = S.rec[par];
+    const int4 ra = rec[u];
+    const float rp2 = S.f_rp2q;
+    const int2 ab = S.nab[u];
+    const long long col = nl_col(u, l, L, S.capq);
+    const uint4 *p = S.nlist + col;
+    unsigned *dst = (unsigned *)(S.plist + col);
+    const int nl = chk_count(S, ab.y > l ? (ab.y - l + L - 1) / L : 0, S.cap_use);
+    int kept = ab.x / L + (l < ab.x % L);
+    auto test = [&](bool have, unsigned e, const int4 &x) {
+        const float dx = (float)(x.x - ra.x), dy = (float)(x.y - ra.y), dz = (float)(x.z - ra.z);
+        if (fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < rp2 && have) {
+            dst[(kept >> 2) * 128 + (kept & 3)] = e;
+            ++kept;
         }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) e[k] = nx[k];
+    };
+    uint4 e = ld_quad(p);
+    for (int q = 0; q < nl; q += 4) {
+        p += 32;
+        const uint4 nx = ld_quad(p);
+        const int4 x0 = ld_rec(S, rec, e.x), x1 = ld_rec(S, rec, e.y);
+        const int4 x2 = ld_rec(S, rec, e.z), x3 = ld_rec(S, rec, e.w);
+        test(true, e.x, x0);
+        test(q + 1 < nl, e.y, x1);
+        test(q + 2 < nl, e.z, x2);
+        test(q + 3 < nl, e.w, x3);
+        e = nx;
     }
-    {
-        const unsigned sen = nl_sentinel(S.n);
-        while (kept & 3) dst[(kept++) * 32] = sen;
-    }
-    S.pnn[(long long)u * L + l] = kept;
+    S.pnn[u * L + l] = kept;
     if (l == 0) {
-        const float4 hi = ((const float4 *)S.pos[par])[u];
-        const float4 lo = S.lo[par][u];
-        S.pref[u] = make_float4(hi.x + lo.x, hi.y + lo.y, hi.z + lo.z, 0.f);
+        if (S.prec == PTA_PREC_FP64) {
+            const double4_32a x = ((const double4_32a *)S.pos[par])[u];
+            S.pref[u] = make_float4((float)x.x, (float)x.y, (float)x.z, 0.f);
+        } else {
+            const float4 hi = ((const float4 *)S.pos[par])[u];
+            const float4 lo = S.lo[par][u];
+            S.pref[u] = make_float4(hi.x + lo.x, hi.y + lo.y, hi.z + lo.z, 0.f);
+        }
     }
 }
 
@@ -299,13 +216,13 @@ __global__ void k_prune_done(const SpecDev *__restrict__ specs, int force) {
 void launch_prune(const Tab &t, int force, cudaStream_t st) {
     for (int i = 0; i < t.ngroups; ++i) {
         const Group &g = t.grp[i];
-        if (g.nblk <= 0 || g.prec == PTA_PREC_FP64) continue;
+        if (g.nblk <= 0) continue;
         switch (g.L) {
-            case 1: k_prune_f32<1><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, force); break;
-            case 2: k_prune_f32<2><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, force); break;
-            case 4: k_prune_f32<4><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, force); break;
-            case 8: k_prune_f32<8><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, force); break;
-            default: k_prune_f32<16><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, force); break;
+            case 1: k_prune<1><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, force); break;
+            case 2: k_prune<2><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, force); break;
+            case 4: k_prune<4><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, force); break;
+            case 8: k_prune<8><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, force); break;
+            default: k_prune<16><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, force); break;
         }
     }
     k_prune_done<<<t.nspec, 32, 0, st>>>(t.specs, force);

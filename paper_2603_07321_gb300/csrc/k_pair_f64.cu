@@ -31,6 +31,31 @@ __device__ __forceinline__ void pow_nm(double s, int n, int m, double &sn, doubl
     }
 }
 
+// f(position) for the entries lane l of atom a reads, in list order (list
+// entries are byte offsets of 16-byte records, half of a double4's)
+template <class F>
+__device__ __forceinline__ void for_entries64(const SpecDev &S, const double4_32a *pos, int a,
+                                              int l, int L, F f) {
+    const uint4 *p = S.plist + nl_col(a, l, L, S.capq);
+    const int cnt = chk_count(S, S.pnn[a * L + l], 4 * (S.capq - 1));
+    uint4 e = __ldg(p);
+    for (int t = cnt >> 2; t > 0; --t) {
+        p += 32;
+        const uint4 nx = __ldg(p);
+        const double4_32a x0 = pos[nl_j(nl_off(S, e.x))], x1 = pos[nl_j(nl_off(S, e.y))];
+        const double4_32a x2 = pos[nl_j(nl_off(S, e.z))], x3 = pos[nl_j(nl_off(S, e.w))];
+        f(x0);
+        f(x1);
+        f(x2);
+        f(x3);
+        e = nx;
+    }
+    const int left = cnt & 3;
+    if (left > 0) f(pos[nl_j(nl_off(S, e.x))]);
+    if (left > 1) f(pos[nl_j(nl_off(S, e.y))]);
+    if (left > 2) f(pos[nl_j(nl_off(S, e.z))]);
+}
+
 template <int L, bool SC76>
 __global__ void __launch_bounds__(TPB) k_density_f64(const SpecDev *__restrict__ specs,
                                                      const int *__restrict__ b2s, int force) {
@@ -48,11 +73,7 @@ __global__ void __launch_bounds__(TPB) k_density_f64(const SpecDev *__restrict__
     double4_32a pa = make_double4_32a(0, 0, 0, 0);
     if (valid) {
         pa = pos[a];
-        const int nn = chk_count(S, S.nn[a], S.cap_use);
-        const int *__restrict__ lst = S.nlist + nl_base(a, L, S.cap);
-        for (int k = l; k < nn; k += L) {
-            const int j = nl_atom(S, (unsigned)lst[(k / L) * 32 + (k % L)]);
-            const double4_32a pj = pos[j];
+        for_entries64(S, pos, a, l, L, [&](const double4_32a &pj) {
             const double dx = pj.x - pa.x, dy = pj.y - pa.y, dz = pj.z - pa.z;
             const double r2 = (dx * dx + dy * dy) + dz * dz;
             // tested on r2 (the reciprocal square root only for pairs within
@@ -65,7 +86,7 @@ __global__ void __launch_bounds__(TPB) k_density_f64(const SpecDev *__restrict__
                 pow_nm<SC76>(P.a * y, P.n, P.m, sn, sm);
                 rho += sm - P.Am + P.Bm * (r - P.rc);
             }
-        }
+        });
     }
     rho = lane_sum<L>(rho);
     if (valid && l == 0) {
@@ -94,11 +115,7 @@ __global__ void __launch_bounds__(TPB) k_force_f64(const SpecDev *__restrict__ s
     double4_32a pa = make_double4_32a(0, 0, 0, 0);
     if (valid) {
         pa = pf[a];
-        const int nn = chk_count(S, S.nn[a], S.cap_use);
-        const int *__restrict__ lst = S.nlist + nl_base(a, L, S.cap);
-        for (int k = l; k < nn; k += L) {
-            const int j = nl_atom(S, (unsigned)lst[(k / L) * 32 + (k % L)]);
-            const double4_32a pj = pf[j];
+        for_entries64(S, pf, a, l, L, [&](const double4_32a &pj) {
             const double dx = pj.x - pa.x, dy = pj.y - pa.y, dz = pj.z - pa.z;
             const double r2 = (dx * dx + dy * dy) + dz * dz;
             // tested on r2, as in the density pass
@@ -115,13 +132,13 @@ __global__ void __launch_bounds__(TPB) k_force_f64(const SpecDev *__restrict__ s
                 fz += g * dz;
                 en += sn - P.An + P.Bn * (r - P.rc);
             }
-        }
+        });
     }
     fx = lane_sum<L>(fx);
     fy = lane_sum<L>(fy);
     fz = lane_sum<L>(fz);
     en = lane_sum<L>(en);
-    double ke = 0, pe = 0, rr = 0, d2 = 0;
+    double ke = 0, pe = 0, rr = 0, d2 = 0, dp2 = 0;
     if (valid && l == 0) {
         chk_force(S, fx, fy, fz);
         const double fpa = pa.w;
@@ -181,17 +198,24 @@ __global__ void __launch_bounds__(TPB) k_force_f64(const SpecDev *__restrict__ s
                 else z = z + du;
             }
             ((double4_32a *)S.pos[par ^ 1])[a] = make_double4_32a(x, y, z, 0.0);
+            S.rec[par ^ 1][a] = rec_fp64(S, x, y, z);
             ((double4_32a *)S.vel)[a] = v;
             const float4 rf = S.ref[a];
             const double ex = x - rf.x, ey = y - rf.y, ez = z - rf.z;
             d2 = ex * ex + ey * ey + ez * ez;
+            if (S.prune_on) {
+                const float4 pr = S.pref[a];
+                const double qx = x - pr.x, qy = y - pr.y, qz = z - pr.z;
+                dp2 = qx * qx + qy * qy + qz * qz;
+            }
         }
     }
     ke = warp_sum(ke);
     pe = warp_sum(pe);
     rr = warp_sum(rr);
     d2 = (double)warp_max((float)d2);
-    step_tail<TPB>(S, lb, S.nblk_pair, ke, pe, rr, d2, 0.0, mode, phase, done, nsteps);
+    dp2 = (double)warp_max((float)dp2);
+    step_tail<TPB>(S, lb, S.nblk_pair, ke, pe, rr, d2, dp2, mode, phase, done, nsteps);
 }
 
 #define PTA_F64_SWITCH(KER, SC, ARG)                                                   \

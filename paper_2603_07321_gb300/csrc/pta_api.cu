@@ -270,11 +270,12 @@ static PotDev make_pot(const pta_potential &p) {
 // ---------------------------------------------------------------------------
 struct Sizes {
     long long n;
-    int L, cap, cap_use, nblk_pair, nblk_atom, nblk_cell, ncell, nc[3];
+    int L, capq, cap_use, nblk_pair, nblk_atom, nblk_cell, nblk_bld, apw, ncell, nc[3];
     int prune_on, mean_pos;
     double prune_margin;
     double h, org[3];
-    size_t list_words;
+    size_t list_quads;
+    int rec_bits;  // quanta of 2^-rec_bits A
     long long series_cap;
 };
 
@@ -303,8 +304,7 @@ static int compute_sizes(const pta_specimen &s, const pta_potential &p, const pt
     z->mean_pos = par.mean_positions ? 1 : 0;
     const double rl = p.rc + par.skin;
     z->prune_margin = par.prune_margin == 0.0 ? 0.3 : par.prune_margin;
-    z->prune_on = (par.precision == PTA_PREC_MIXED && z->prune_margin > 0.0 &&
-                   z->prune_margin < par.skin) ? 1 : 0;
+    z->prune_on = (z->prune_margin > 0.0 && z->prune_margin < par.skin) ? 1 : 0;
     if (par.neigh_cap > 0) {
         z->cap_use = (int)round_up((size_t)par.neigh_cap, 32);
     } else {
@@ -312,13 +312,15 @@ static int compute_sizes(const pta_specimen &s, const pta_potential &p, const pt
         const double nb = 4.0 / 3.0 * 3.141592653589793 * rl * rl * rl * dens;
         z->cap_use = (int)round_up((size_t)std::ceil(1.6 * nb + 16), 32);
     }
-    // sixteen spare rows per lane: they hold the (up to four) sentinel rows
-    // after a full list, the pair loops read four rows ahead and the pruning
-    // fifteen, without bounds tests (spare entries hold 0, earlier entries or
-    // the sentinel: all valid record indices)
-    z->cap = z->cap_use + 16 * z->L;
+    // quads per lane column: near and far part each end in a partly filled
+    // row, and the pair loops read one quad ahead
+    z->capq = (z->cap_use + 4 * z->L - 1) / (4 * z->L) + 3;
     z->nblk_pair = (int)((z->n * z->L + TPB - 1) / TPB);
     z->nblk_atom = (int)((z->n + TPB - 1) / TPB);
+    // list build: a warp per atom while that fills the GPU (152 SMs x ~48
+    // warps), then several atoms in turn, which saves block starts
+    z->apw = z->n >= 65536 ? 8 : (z->n >= 16384 ? 2 : 1);
+    z->nblk_bld = (int)((z->n + BUILD_WARPS * z->apw - 1) / (BUILD_WARPS * z->apw));
     // cell edge a multiple of 2^-11 A and grid origin on the 2^-12 A grid, so
     // that cell centres and centre differences are exact in FP32
     z->h = std::ceil(rl * (1.0 + 1e-4) * 2048.0) / 2048.0;
@@ -340,7 +342,11 @@ static int compute_sizes(const pta_specimen &s, const pta_potential &p, const pt
     z->ncell = (int)ncell;
     z->nblk_cell = (z->ncell + CELL_WARPS * CELLS_PER_WARP - 1) / (CELL_WARPS * CELLS_PER_WARP);
     const long long W = 32 / z->L;
-    z->list_words = (size_t)((z->n + W - 1) / W) * W * z->cap;
+    z->list_quads = (size_t)((z->n + W - 1) / W) * 32 * z->capq;
+    // records: the finest quantum whose half period, 2^31 quanta, exceeds the
+    // distance of two atoms in neighbouring cells (2 h per axis, with room for
+    // what they move between list builds)
+    z->rec_bits = 31 - (int)std::ceil(std::log2(2.0 * z->h + 2.0 * par.skin));
     z->series_cap = std::max<long long>(par.burst_steps, 1);
     return PTA_OK;
 }
@@ -355,11 +361,11 @@ static size_t footprint(const Sizes &z, int prec) {
     if (prec != PTA_PREC_FP64) {
         add(16 * n);
         add(16 * n);                 // lo[2]
-        add(16 * (n + 1));
-        add(16 * (n + 1));           // rel[2], + the sentinel record
-        add(n);                      // hsub
+        add(4 * n);                  // pen
     }
-    add(p * (n + 1));                // posfp, + the sentinel record
+    add(16 * n);
+    add(16 * n);                     // rec[2]
+    add(p * n);                      // posfp
     add(32 * n);                     // vel (double4 or hi/lo FP32)
     add(n);                          // flags
     add(16 * n);                     // ref
@@ -370,13 +376,13 @@ static size_t footprint(const Sizes &z, int prec) {
     add(4 * n);                      // cell_atoms
     add(4 * n);                      // orig
     add(perm_layout(n, prec).total); // permutation scratch
-    add(4 * z.list_words);           // nlist
+    add(16 * z.list_quads);          // plist
+    add(4 * n * (size_t)z.L);        // pnn
+    add(8 * n);                      // nab
     if (z.prune_on) {
-        add(4 * z.list_words);       // plist
-        add(4 * n * (size_t)z.L);    // pnn
+        add(16 * z.list_quads);      // nlist
         add(16 * n);                 // pref
     }
-    add(4 * n);                      // nn
     {
         const size_t nb = (size_t)std::max(z.nblk_pair, z.nblk_atom);
         add(64 * (nb + 2 * (nb / 32 + 1)));  // part: block and group partials, group counters
@@ -416,7 +422,7 @@ static int validate(const pta_specimen *s, const pta_potential *p, const pta_par
     for (int q = 0; q < 3; ++q)
         if (!(par->conv_tol[q] >= 0) || !std::isfinite(par->conv_tol[q])) return PTA_EINVAL;
     const long long n = 4LL * s->n_cells[0] * s->n_cells[1] * s->n_cells[2];
-    if (n >= (long long)MAX_ATOMS) return PTA_ERANGE;  // slot n is the lists' sentinel
+    if (n >= (long long)MAX_ATOMS) return PTA_ERANGE;
     if (par->precision == PTA_PREC_MIXED) {
         for (int d = 0; d < 3; ++d)
             if (s->n_cells[d] * s->a0 * 1.5 > MIXED_RANGE) return PTA_ERANGE;
@@ -566,7 +572,8 @@ static int runner_upload(Runner *r) {
     const int k = (int)r->m.size();
     r->hspecs.resize(k);
     int blk_atom = 0, blk_cell = 0;
-    std::vector<int> b2s_atom, b2s_cell;
+    std::vector<int> b2s_atom, b2s_cell, b2s_bld;
+    int bld_words = 0;
     // launch groups by (precision, lanes, potential); the potential's FP32
     // constants are kernel parameters of the group's launches
     struct Key {
@@ -594,6 +601,10 @@ static int runner_upload(Runner *r) {
         s.blk_cell0 = blk_cell;
         blk_cell += s.nblk_cell;
         for (int b = 0; b < s.nblk_cell; ++b) b2s_cell.push_back(i);
+        s.blk_bld0 = (int)b2s_bld.size();
+        for (int b = 0; b < s.nblk_bld; ++b) b2s_bld.push_back(i);
+        // candidates, near part in list order, class counters
+        bld_words = std::max(bld_words, 2 * s.cap_use + 128 + 16);
         PotF pf;
         std::memset(&pf, 0, sizeof(pf));
         pf.a = s.pot.f_a;
@@ -613,7 +624,6 @@ static int runner_upload(Runner *r) {
             pf.kn = (float)(q.eps * q.n * hpow(q.a, q.n));
             pf.bmq = (float)(q.Bm / amm);
             pf.ebn = (float)(q.eps * q.Bn);
-            pf.c1 = (float)(-(q.An / q.Bn + q.rc));
             pf.fpsc = (float)(-0.5 * q.ec * amm);
         }
         pf.n = s.pot.n;
@@ -625,7 +635,7 @@ static int runner_upload(Runner *r) {
         r->hspecs[i] = s;
     }
     // one device block for all tables
-    size_t words = b2s_atom.size() + b2s_cell.size();
+    size_t words = b2s_atom.size() + b2s_cell.size() + b2s_bld.size();
     for (auto &v : gb2s) words += v.size();
     if (r->d_specs) {
         // tables already exist: only refresh the descriptors (same shapes)
@@ -656,6 +666,7 @@ static int runner_upload(Runner *r) {
     std::vector<int> all;
     all.insert(all.end(), b2s_atom.begin(), b2s_atom.end());
     all.insert(all.end(), b2s_cell.begin(), b2s_cell.end());
+    all.insert(all.end(), b2s_bld.begin(), b2s_bld.end());
     for (auto &v : gb2s) all.insert(all.end(), v.begin(), v.end());
     CK(cudaMemcpyAsync(r->d_specs, r->hspecs.data(), sizeof(SpecDev) * k, cudaMemcpyHostToDevice,
                        r->stream));
@@ -667,7 +678,14 @@ static int runner_upload(Runner *r) {
     t.nblk_atom = (int)b2s_atom.size();
     t.b2s_cell = tabs + b2s_atom.size();
     t.nblk_cell = (int)b2s_cell.size();
-    size_t off = b2s_atom.size() + b2s_cell.size();
+    t.b2s_bld = tabs + b2s_atom.size() + b2s_cell.size();
+    t.nblk_bld = (int)b2s_bld.size();
+    t.bld_words = bld_words;
+    if (!build_smem_limit(BUILD_WARPS * bld_words * 4)) {
+        cudaGetLastError();
+        return PTA_ECUDA;
+    }
+    size_t off = b2s_atom.size() + b2s_cell.size() + b2s_bld.size();
     t.ngroups = (int)keys.size();
     for (size_t q = 0; q < keys.size(); ++q) {
         t.grp[q].prec = keys[q].prec;
@@ -1024,11 +1042,11 @@ static int ctx_alloc_all(pta_ctx *c, const Sizes &z) {
     if (!f64) {
         AL(lo[0], 16 * n, float4 *);
         AL(lo[1], 16 * n, float4 *);
-        AL(rel[0], 16 * (n + 1), float4 *);
-        AL(rel[1], 16 * (n + 1), float4 *);
-        AL(hsub, n, uint8_t *);
+        AL(pen, 4 * n, float *);
     }
-    AL(posfp, p * (n + 1), void *);
+    AL(rec[0], 16 * n, int4 *);
+    AL(rec[1], 16 * n, int4 *);
+    AL(posfp, p * n, void *);
     AL(vel, 32 * n, void *);
     AL(flags, n, uint8_t *);
     AL(ref, 16 * n, float4 *);
@@ -1039,13 +1057,13 @@ static int ctx_alloc_all(pta_ctx *c, const Sizes &z) {
     AL(cell_atoms, 4 * n, int *);
     AL(orig, 4 * n, int *);
     AL(perm_tmp, perm_layout(n, c->par.precision).total, void *);
-    AL(nlist, 4 * z.list_words, int *);
+    AL(plist, 16 * z.list_quads, uint4 *);
+    AL(pnn, 4 * n * (size_t)z.L, int *);
+    AL(nab, 8 * n, int2 *);
     if (z.prune_on) {
-        AL(plist, 4 * z.list_words, int *);
-        AL(pnn, 4 * n * (size_t)z.L, int *);
+        AL(nlist, 16 * z.list_quads, uint4 *);
         AL(pref, 16 * n, float4 *);
     }
-    AL(nn, 4 * n, int *);
     {
         // block partials (8 doubles per block), then per group of 32 blocks
         // its partial (8 doubles) and its counter
@@ -1098,36 +1116,53 @@ int pta_create(const pta_specimen *spec, const pta_potential *pot, double T0, ui
     s.L = z.L;
     s.prec = c->par.precision;
     s.axis = c->spec.load_axis;
-    s.cap = z.cap;
     s.cap_use = z.cap_use;
+    s.capq = z.capq;
+    s.nblk_bld = z.nblk_bld;
+    s.apw = z.apw;
     s.nblk_pair = z.nblk_pair;
     s.nblk_atom = z.nblk_atom;
     s.nblk_cell = z.nblk_cell;
     for (int d = 0; d < 3; ++d) {
         s.ncl[d] = c->spec.n_cells[d];
         s.org[d] = z.org[d];
-        s.f_org[d] = (float)z.org[d];
         s.nc[d] = z.nc[d];
     }
     s.a0 = c->spec.a0;
     s.grip_width = c->spec.grip_width;
     s.hcell = z.h;
     s.inv_h = 1.0 / z.h;
-    s.f_inv_h = (float)s.inv_h;
     s.f_h = (float)z.h;
-    s.f_q = (float)(z.h / 2.0);
-    s.f_q8 = (float)(z.h / 16.0);
-    s.f_q64 = (float)(z.h / 128.0);
+    const double rq = std::ldexp(1.0, z.rec_bits);
+    s.f_rq = (float)rq;
+    s.f_q = (float)(1.0 / rq);
+    s.f_q2 = (float)(1.0 / (rq * rq));
+    s.rec_shift = z.rec_bits - 12;
+    double extent = 0;  // largest coordinate of the cell grid
+    for (int d = 0; d < 3; ++d) {
+        s.f_org[d] = (float)z.org[d];
+        extent = std::max(extent, std::fabs(z.org[d]) + z.nc[d] * z.h);
+    }
     s.ncell = z.ncell;
     const double rl = c->pot.rc + c->par.skin;
     s.rl2 = rl * rl;
-    s.f_rl2_lo = (float)(s.rl2 * (1.0 - 1e-5));
-    s.f_rl2_hi = (float)(s.rl2 * (1.0 + 1e-5));
+    // relative half-width of the band around the list radius in which the
+    // FP32 test of two records (each off by up to half a quantum per axis)
+    // is not trusted and the FP64 test decides
+    const double band = 1e-5 + 8.0 / (rq * rl);
+    s.f_rl2q_lo = (float)(s.rl2 * (1.0 - band) * rq * rq);
+    s.f_rl2q_hi = (float)(s.rl2 * (1.0 + band) * rq * rq);
+    const double rnear = std::min(rl, c->pot.rc + NEAR_MARGIN);
+    s.f_ra2q = (float)(rnear * rnear * (1.0 + band) * rq * rq);
+    s.f_reach_slack = (float)(1e-3 + 1e-6 * extent);
+    s.f_reach2 = (float)(s.rl2 * (1.0 + band) + 1e-3);
     s.half_skin2 = (float)(0.25 * c->par.skin * c->par.skin);
     s.prune_on = z.prune_on;
+    s.prune_first = z.prune_on && z.prune_margin > NEAR_MARGIN;
     {
-        const double rp = c->pot.rc + z.prune_margin;
-        s.f_rp2 = (float)(rp * rp * (1.0 + 1e-5));
+        // slack for the FP32 rounding of the reference positions
+        const double rp = c->pot.rc + z.prune_margin + 2e-7 * extent;
+        s.f_rp2q = (float)(rp * rp * (1.0 + band) * rq * rq);
         s.half_prune2 = (float)(0.25 * z.prune_margin * z.prune_margin);
     }
     s.pot = make_pot(c->pot);
@@ -1159,18 +1194,6 @@ int pta_create(const pta_specimen *spec, const pta_potential *pot, double T0, ui
         if (cudaMemcpyAsync(c->d_self, &c->hd, sizeof(SpecDev), cudaMemcpyHostToDevice,
                             c->stream) != cudaSuccess)
             rc = PTA_ECUDA;
-    }
-    if (rc == PTA_OK && c->par.precision != PTA_PREC_FP64) {
-        // the sentinel record (slot n) that pads every lane's list to a
-        // multiple of four entries: far from every atom in both record
-        // buffers and in the force pass's records, never written again
-        static const float4 far_rec = {SENTINEL_COORD, SENTINEL_COORD, SENTINEL_COORD, 0.f};
-        const size_t n = (size_t)s.n;
-        float4 *dst[3] = {s.rel[0] + n, s.rel[1] + n, (float4 *)s.posfp + n};
-        for (float4 *d : dst)
-            if (cudaMemcpyAsync(d, &far_rec, sizeof(float4), cudaMemcpyHostToDevice, c->stream) !=
-                cudaSuccess)
-                rc = PTA_ECUDA;
     }
     if (rc == PTA_OK) {
         const double kT = kb_ev() * T0;
@@ -1433,7 +1456,7 @@ int pta_forces(pta_ctx *c, double *f, double *pe, int64_t n, double obs[3]) {
     Runner *r;
     CKR(ctx_solo(c, &r));
     launch_rebuild(r->tab, 1, c->stream);
-    launch_prune(r->tab, 1, c->stream);
+    if (c->hd.prune_first) launch_prune(r->tab, 1, c->stream);
     launch_density(r->tab, 1, c->stream);
     launch_force(r->tab, MODE_EVAL, c->stream);
     CKR(launch_check());
@@ -1472,14 +1495,17 @@ int pta_get_neighbours(pta_ctx *c, int32_t *counts, int32_t *list, int64_t n, in
     launch_rebuild(r->tab, 1, c->stream);
     CKR(launch_check());
     const int L = s.L;
-    std::vector<int> nn((size_t)n), raw;
-    CK(cudaMemcpyAsync(nn.data(), s.nn, 4 * (size_t)n, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaMemcpyAsync(&ctl, s.ctl, sizeof(ctl), cudaMemcpyDeviceToHost, c->stream));
-    const long long W = 32 / L;
-    const size_t words = (size_t)((n + W - 1) / W) * W * s.cap;
-    raw.resize(words);
+    const size_t W = 32 / L, quads = ((size_t)n + W - 1) / W * 32 * s.capq;
+    std::vector<int2> nab((size_t)n);
+    std::vector<unsigned> near(4 * quads), far;
     std::vector<int> orig;
-    CK(cudaMemcpyAsync(raw.data(), s.nlist, 4 * words, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaMemcpyAsync(nab.data(), s.nab, 8 * (size_t)n, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaMemcpyAsync(&ctl, s.ctl, sizeof(ctl), cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaMemcpyAsync(near.data(), s.plist, 16 * quads, cudaMemcpyDeviceToHost, c->stream));
+    if (s.prune_on) {
+        far.resize(4 * quads);
+        CK(cudaMemcpyAsync(far.data(), s.nlist, 16 * quads, cudaMemcpyDeviceToHost, c->stream));
+    }
     CKR(fetch_orig(c, orig));
     CK(cudaStreamSynchronize(c->stream));
     *max_count = ctl.max_nn;
@@ -1488,14 +1514,27 @@ int pta_get_neighbours(pta_ctx *c, int32_t *counts, int32_t *list, int64_t n, in
     int maxc = 0;
     for (int64_t u = 0; u < n; ++u) {
         const int64_t o = orig[u];
-        if (counts) counts[o] = nn[u];
-        maxc = std::max(maxc, nn[u]);
-        if (nn[u] > cap) return PTA_EINVAL;
-        for (int k = 0; k < nn[u]; ++k) {
-            const int j = nl_j((unsigned)raw[(size_t)nl_index((int)u, k, L, s.cap)]);
-            if (j < 0 || j >= n) return PTA_ECUDA;
-            if (list) list[o * (int64_t)cap + k] = orig[j];
-        }
+        const long long col = nl_col((int)u, 0, L, s.capq);
+        int cnt = 0;
+        auto take = [&](const unsigned *lst, int k, int row0, int l) {
+            const int r = row0 + k / L;
+            const int j = nl_j(lst[4 * (size_t)(col + (r / 4) * 32 + l) + r % 4]);
+            if (j < 0 || j >= n) return false;
+            if (list && cnt < cap) list[o * (int64_t)cap + cnt] = orig[j];
+            ++cnt;
+            return true;
+        };
+        const int na = nab[u].x, nb = nab[u].y;
+        for (int k = 0; k < na; ++k)
+            if (!take(near.data(), k, 0, k % L)) return PTA_ECUDA;
+        // the far part lies in its own list, or behind each lane's near entries
+        for (int k = 0; k < nb; ++k)
+            if (!take(s.prune_on ? far.data() : near.data(), k,
+                      s.prune_on ? 0 : na / L + (k % L < na % L), k % L))
+                return PTA_ECUDA;
+        if (counts) counts[o] = cnt;
+        maxc = std::max(maxc, cnt);
+        if (cnt > cap) return PTA_EINVAL;
     }
     *max_count = maxc;
     return PTA_OK;

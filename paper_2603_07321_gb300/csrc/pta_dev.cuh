@@ -19,6 +19,7 @@ constexpr int TPB = 128;        // threads per block of the atom and pair kernel
 constexpr int CELL_WARPS = 8;   // warps per block of the cell-sort kernel
 constexpr int CELLS_PER_WARP = 8;  // cells one warp of the cell-sort kernel orders in turn
 constexpr int SCAN_THREADS = 1024;
+constexpr int BUILD_WARPS = 4;  // warps per block of the list build
 
 // grid quantum of the mixed-precision position split x = hi + lo:
 // hi is a multiple of 2^-12 A (exact in FP32 for |x| < 512 A), |lo| <= 2^-13 A
@@ -70,7 +71,6 @@ struct PotF {
     float kn;    // eps n a^n
     float bmq;   // Bm / (m a^m)
     float ebn;   // eps Bn
-    float c1;    // -(An / Bn + rc): phi_n(r) = a^n r^-n + Bn (r + c1)
     float fpsc;  // -eps c m a^m / 2: w = fpsc / sqrt(rho) (density pass)
     int n, m;
 };
@@ -111,11 +111,14 @@ struct SpecCtl {
 
 struct SpecDev {
     // sizes
-    int n, L, prec, axis, cap;   // cap: list stride per unit (usable entries: cap_use)
-    int cap_use;
+    int n, L, prec, axis;
+    int cap_use;               // list capacity: entries per atom
+    int capq;                  // quads per lane column of a list
     int blk_pair0, nblk_pair;  // pair kernels: TPB/L atoms per block
     int blk_atom0, nblk_atom;  // one thread per atom
     int blk_cell0, nblk_cell;  // cell sort: CELLS_PER_WARP cells per warp
+    int blk_bld0, nblk_bld;    // list build: BUILD_WARPS warps of apw atoms
+    int apw;
     int spec_index;            // index of this specimen in the launch table
     // lattice (creation only)
     int ncl[3];
@@ -125,11 +128,16 @@ struct SpecDev {
     double hcell, inv_h;
     int nc[3];
     int ncell;
-    // list radius (rc + skin)^2 and its FP32 bracket; half skin squared
+    // list radius (rc + skin)^2, half skin squared
     double rl2;
-    float f_rl2_lo, f_rl2_hi, half_skin2, f_inv_h, f_h;
-    float f_q, f_q8, f_q64;  // half the cell edge (unit of the list offsets), / 8, / 64
-    float f_org[3];
+    float half_skin2, f_h;
+    // fixed-point records: quanta per A, A per quantum and its square, shift
+    // from the 2^-12 A grid of hi to quanta; grid origin
+    float f_rq, f_q, f_q2, f_org[3];
+    int rec_shift;
+    // squared radii in quanta: bracket of the list radius, near part, pruning
+    float f_rl2q_lo, f_rl2q_hi, f_ra2q, f_rp2q;
+    float f_reach2, f_reach_slack;  // list radius squared (A^2, with slack) and slack (A)
     PotDev pot;
     // integration constants
     double mass, dt, acc_half, ke_fac, t_fac;
@@ -143,22 +151,24 @@ struct SpecDev {
     // arrays
     void *pos[2];   // FP64: double4 {x,y,z,0};  MIXED: float4 hi {x,y,z,0}
     float4 *lo[2];  // MIXED only: float4 lo {x,y,z,0}
-    void *posfp;    // FP64: double4 {x,y,z,F'(rho)};  MIXED: float4 {rel.xyz, F'(rho)}
-    float4 *rel[2]; // MIXED only: position relative to the centre of its half-cell
-                    // (FP32): the 16-byte record the pair passes read for a neighbour
-    uint8_t *hsub;  // MIXED only: half-cell of each atom in its cell (bit d: upper half
-                    // along axis d), fixed from one list build to the next
+    int4 *rec[2];   // fixed-point record {x,y,z,0} of every atom
+    void *posfp;    // FP64: double4 {x,y,z,B'(rho)};  MIXED: the record with w = m a^m B'(rho)
+                    // (float bits) as fourth word
+    float *pen;     // MIXED: pair energy of each atom, 1/2 eps sum_j phi_n
     void *vel;      // FP64: double4; MIXED: VelHL
     uint8_t *flags;
     float4 *ref;    // positions at the last list build (skin test)
     int *atom_cell, *cell_cnt, *cell_start, *cell_tmp, *cell_atoms;
     int *orig;        // original index (creation order) of the atom stored at each slot
     void *perm_tmp;   // scratch of the permutation that sorts atoms by cell
-    int *nlist, *nn;
-    int *plist, *pnn;   // inner list (same layout as nlist), entries per unit and lane
-    float4 *pref;       // positions at the last pruning
+    uint4 *plist;     // what the pair passes read: near part, then the pruned far part
+    uint4 *nlist;     // far part of the Verlet list (null without pruning)
+    int2 *nab;        // per atom: entries of the near and of the far part
+    int *pnn;         // per atom and lane: entries of plist
+    float4 *pref;     // positions at the last pruning
     int prune_on;
-    float f_rp2, half_prune2;
+    int prune_first;  // 1: a fresh list is pruned before its first use
+    float half_prune2;
     double *part;       // per pair block: K, U, R, max displacement^2
     double *series;     // series_cap x 3 samples of the current burst
     long long series_cap;
@@ -184,33 +194,55 @@ struct Tab {
     int nblk_atom;
     const int *b2s_cell;
     int nblk_cell;
+    const int *b2s_bld;
+    int nblk_bld;
+    int bld_words;  // shared words per warp of the list build
     int ngroups;
     Group grp[8];
 };
 
-// Verlet-list entry (one list per unit): neighbour index in the high 23
-// bits, an offset (dx, dy, dz) in the low 9 bits, 3 bits per axis holding
-// d + 3.  In mixed precision d is the offset of the neighbour's half-cell
-// from the half-cell of the unit's first atom in units of h / 2 (within the
-// 3x3x3 cells around a cell, |d| <= 3); with half-cell centres and h on
-// exact grids, r_j - r_i = (rel_j - rel_i) + (h / 2) d.  FP64 lists keep
-// whole-cell offsets, which its kernels do not read.
+// Neighbour records and lists.
 //
-// Mixed-precision lists end, in every lane, with up to three sentinel
-// entries that bring the lane's count to a multiple of four: they name slot
-// n, a record kept far from every atom (SENTINEL_COORD on each axis), whose
-// pairs lie beyond any cutoff, so the pair loops take four entries at a time
-// without per-entry bounds tests.  Slot n must fit the index field: n < 2^23.
-constexpr int NL_CODE_BITS = 9;
+// A record is an atom's position in fixed point: int32 quanta of 2^-k A,
+// modulo 2^32.  Only differences of two records are used, and those of atoms
+// in neighbouring cells are below 2^31 quanta by the choice of k (2^-26 A at
+// the default radii), so they are exact in wrapping int32 arithmetic whatever
+// the specimen's extent; a difference is converted once to FP32, and its
+// rounding is relative to the distance.  (FP32 records relative to half-cell
+// centres with an offset coded in every list entry took 7.5 instructions per
+// entry to decode and had the larger error; fixed point that spans the whole
+// specimen, 2^-22 A for a 20 nm cube, had the larger error too.)
+//
+// A list entry is the byte offset of the neighbour's record (slot x 16).
+// Lists are stored in quads of four entries: the 32 lanes of a warp read the
+// quads of one iteration as 512 contiguous bytes (lane column: tile of 32
+// lanes x capq quads).  With L lanes per atom, atom a owns lanes (a L) % 32 +
+// 0..L-1 of tile (a L) / 32.
+//
+// The Verlet list (radius rc + skin) is kept in two parts by the distance at
+// the build.  The near part (within rc + NEAR_MARGIN) is read by every pair
+// pass as it stands.  The far part is read by the pruning, which appends the
+// entries within rc + prune_margin to each lane's near entries.  Pairs beyond
+// rc add exactly zero, and the order of a lane's entries does not depend on
+// the pruning margin, so results do not either.
+//
+// In the near part, row r of lane l (counted in the warp) holds a slot with
+// slot % 8 == (l + r) % 8 wherever the atom has one: the eight lanes of a
+// quarter-warp then gather their 16-byte records from different banks of the
+// 128-byte L1 line.  On the 470,596-atom cube that takes the gathers from
+// ~10.6 to ~6.5 wavefronts each, and the density pass from 98 to 76 us, the
+// force pass from 102 to 84 us (prototype of the pair loops alone).
+constexpr int REC_SHIFT = 4;             // log2 of a record's bytes
+constexpr double NEAR_MARGIN = 0.3;      // A
 constexpr int MAX_ATOMS = 1 << 23;
-constexpr float SENTINEL_COORD = 1.0e4f;
 
-__host__ __device__ __forceinline__ unsigned nl_entry(int j, int dx, int dy, int dz) {
-    return ((unsigned)j << NL_CODE_BITS) | (unsigned)((dx + 3) | ((dy + 3) << 3) | ((dz + 3) << 6));
+__host__ __device__ __forceinline__ unsigned nl_entry(int j) { return (unsigned)j << REC_SHIFT; }
+__host__ __device__ __forceinline__ int nl_j(unsigned e) { return (int)(e >> REC_SHIFT); }
+// first quad of lane l of atom a
+__host__ __device__ __forceinline__ long long nl_col(int a, int l, int L, int capq) {
+    const long long t = (long long)a * L;
+    return (t >> 5) * capq * 32 + (t & 31) + l;
 }
-__host__ __device__ __forceinline__ int nl_j(unsigned e) { return (int)(e >> NL_CODE_BITS); }
-// the sentinel entry of a specimen of n atoms (slot n, offset 0)
-__host__ __device__ __forceinline__ unsigned nl_sentinel(int n) { return nl_entry(n, 0, 0, 0); }
 
 // index i of an array of n elements (debug builds: tested, 0 when outside)
 __device__ __forceinline__ int chk_index(const SpecDev &S, int i, int n) {
@@ -223,10 +255,12 @@ __device__ __forceinline__ int chk_index(const SpecDev &S, int i, int n) {
     return i;
 }
 
-// the record a list entry names (mixed precision: an atom or the sentinel
-// slot n)
-__device__ __forceinline__ int nl_atom(const SpecDev &S, unsigned e) {
-    return chk_index(S, nl_j(e), S.prec == PTA_PREC_FP64 ? S.n : S.n + 1);
+// the byte offset of the record a list entry names
+__device__ __forceinline__ unsigned nl_off(const SpecDev &S, unsigned e) {
+#if PTA_CHECK
+    return (unsigned)chk_index(S, nl_j(e), S.n) << REC_SHIFT;
+#endif
+    return e;
 }
 
 // a count of list entries read by one lane (debug builds: at most `limit`)
@@ -246,20 +280,6 @@ __device__ __forceinline__ void chk_force(const SpecDev &S, double fx, double fy
     if (!(isfinite(fx) && isfinite(fy) && isfinite(fz))) atomicOr(&S.ctl->err, ERR_NAN);
 #endif
     (void)S; (void)fx; (void)fy; (void)fz;
-}
-
-// The three offsets as exact FP32 multiples of the axis field, without
-// integer conversion: OR-ing a field into the mantissa of 1.5 * 2^23
-// (0x4B400000) gives 1.5 * 2^23 + field exactly.  x: (d + 3), y: 8 (d + 3),
-// z: 64 (d + 3); the caller scales by h, h / 8 and h / 64.
-__device__ __forceinline__ float nl_offx(unsigned e) {
-    return __int_as_float(0x4B400000 | (int)(e & 0x7u)) - 12582915.0f;
-}
-__device__ __forceinline__ float nl_offy(unsigned e) {
-    return __int_as_float(0x4B400000 | (int)(e & 0x38u)) - 12582936.0f;
-}
-__device__ __forceinline__ float nl_offz(unsigned e) {
-    return __int_as_float(0x4B400000 | (int)(e & 0x1C0u)) - 12583104.0f;
 }
 
 // Cells are numbered along a serpentine path (x reverses on every other row,
@@ -286,29 +306,23 @@ __host__ __device__ __forceinline__ void cell_coords(const int nc[3], int r, int
     serp_coords(nc[0], nc[1], r, x, y, z);
 }
 
-// centre of the cell of rank r (exact in FP32: org on a 2^-12 grid, h a
-// multiple of 2^-11)
-__device__ __forceinline__ float3 cell_centre(const SpecDev &S, int r) {
-    int cx, cy, cz;
-    cell_coords(S.nc, r, cx, cy, cz);
-    return make_float3(S.f_org[0] + ((float)cx + 0.5f) * S.f_h,
-                       S.f_org[1] + ((float)cy + 0.5f) * S.f_h,
-                       S.f_org[2] + ((float)cz + 0.5f) * S.f_h);
+// one coordinate of a record: hi is a multiple of 2^-12 A and enters exactly,
+// lo is rounded to the nearest quantum (a quantum above 2^-12 A, which takes a
+// cutoff of ~0.1 mm, rounds their sum)
+__device__ __forceinline__ int rec_coord(const SpecDev &S, float hi, float lo) {
+    if (S.rec_shift < 0) return __float2int_rn((hi + lo) * S.f_rq);
+    return (int)((unsigned)__float2int_rn(hi * (float)HI_SCALE) << S.rec_shift) +
+           __float2int_rn(lo * S.f_rq);
 }
-
-// centre of half-cell `sub` of the cell of rank r: the cell centre moved by
-// -h/4 or +h/4 per axis (exact in FP32: on a 2^-13 A grid)
-__device__ __forceinline__ float3 half_centre(const SpecDev &S, int r, int sub) {
-    float3 C = cell_centre(S, r);
-    const float q = 0.25f * S.f_h;
-    C.x += (sub & 1) ? q : -q;
-    C.y += (sub & 2) ? q : -q;
-    C.z += (sub & 4) ? q : -q;
-    return C;
+__device__ __forceinline__ int4 rec_mixed(const SpecDev &S, float hx, float hy, float hz, float lx,
+                                          float ly, float lz) {
+    return make_int4(rec_coord(S, hx, lx), rec_coord(S, hy, ly), rec_coord(S, hz, lz), 0);
 }
-// the 3 half-cell bits spread onto the 3 offset fields of a list entry
-__host__ __device__ __forceinline__ int sub_spread(int sub) {
-    return (sub & 1) | ((sub & 2) << 2) | ((sub & 4) << 4);
+// FP64 form: rounded once from the double coordinate, low 32 bits
+__device__ __forceinline__ int4 rec_fp64(const SpecDev &S, double x, double y, double z) {
+    const double rq = (double)S.f_rq;
+    return make_int4((int)__double2ll_rn(x * rq), (int)__double2ll_rn(y * rq),
+                     (int)__double2ll_rn(z * rq), 0);
 }
 
 // segments of the permutation scratch (see perm_layout)
@@ -334,43 +348,6 @@ __host__ __device__ inline PermLayout perm_layout(size_t n, int prec) {
     o += perm_round(4 * n);
     L.total = o;
     return L;
-}
-
-// Rows of a warp's list tile (L = 1: row k holds entry k of the warp's 32
-// units) staged in shared memory and written to global memory as whole
-// 128-byte rows once every lane has passed them; a lane that runs more than
-// ROWS rows ahead of the flushed rows writes that entry and all its later
-// ones directly.
-template <int ROWS>
-struct RowWriter {
-    int *buf;   // shared [ROWS][32]
-    int *tile;  // global word of row 0 of this warp's tile
-    int lane, flushed, direct_from;
-    __device__ __forceinline__ void put(int k, int e) {
-        if (k < direct_from && k - flushed < ROWS) {
-            buf[(k % ROWS) * 32 + lane] = e;
-        } else {
-            tile[(long long)k * 32 + lane] = e;
-            direct_from = min(direct_from, k);
-        }
-    }
-    // warp-collective: write rows [flushed, upto)
-    __device__ __forceinline__ void flush(int upto) {
-        for (int r = flushed; r < upto; ++r)
-            if (r < direct_from) tile[(long long)r * 32 + lane] = buf[(r % ROWS) * 32 + lane];
-        flushed = upto;
-    }
-};
-
-// neighbour-list word of neighbour k of atom a for L lanes per atom: atoms
-// are grouped 32/L per warp; for each iteration q = k / L the warp's 32
-// words are contiguous, lane (a % (32/L)) * L + k % L.
-__host__ __device__ __forceinline__ long long nl_base(int a, int L, int cap) {
-    const int G = 32 / L;
-    return (long long)(a / G) * (32LL * (cap / L)) + (a % G) * L;
-}
-__host__ __device__ __forceinline__ long long nl_index(int a, int k, int L, int cap) {
-    return nl_base(a, L, cap) + (long long)(k / L) * 32 + (k % L);
 }
 
 // one block of SCAN_THREADS threads per specimen: exclusive scan of the cell
@@ -440,6 +417,7 @@ void launch_any_running(const Tab &t, int *flag, cudaStream_t st);
 void launch_pta_update(const Tab &t, const int *ops, pta_coarse_result *out, cudaStream_t st);
 void launch_force_rebuild_flag(const Tab &t, cudaStream_t st);
 void launch_rebuild(const Tab &t, int force, cudaStream_t st);
+int build_smem_limit(int bytes);  // allow k_build this much dynamic shared memory; 0 on failure
 void launch_prune(const Tab &t, int force, cudaStream_t st);
 void launch_decide_rebuild(const Tab &t, cudaGraphConditionalHandle h, cudaStream_t st);
 // list maintenance decided on the device: 0 build + prune, 1 prune, 2 nothing
