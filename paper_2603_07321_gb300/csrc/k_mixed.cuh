@@ -133,21 +133,20 @@ __device__ __forceinline__ void hl_add(float &h, float &l, float d) {
     h = hh;
 }
 
-// After the force pass of atom a (force f, record weight fpa = m a^m
-// B'(rho_a); its pair energy from the density pass): its energy, its share of
-// the reaction, and the velocity-Verlet update -- the half-kick that finishes the step (phase RUN),
+// After the force pass of atom a (force f; its energy from the density
+// pass): its share of the reaction, and the velocity-Verlet update -- the half-kick that finishes the step (phase RUN),
 // the sample of K, and unless the burst ends the half-kick and drift of the
 // next step; the new position (hi + lo, whole grid quanta moved from lo to
 // hi), its neighbour record, and the displacements since the last list
 // build (and, with `pruned`, since the last pruning).  Grip
 // atoms keep v = 0.  MODE_EVAL stores F and the energy instead.
 __device__ __forceinline__ void atom_update_mixed(const SpecDev &S, SpecCtl *ctl, int par, int a,
-                                                  bool pruned, float fpa, float fx, float fy,
-                                                  float fz, int mode, int phase, long long done,
+                                                  bool pruned, float fx, float fy, float fz,
+                                                  int mode, int phase, long long done,
                                                   long long nsteps, double &ke, double &pe,
                                                   double &rr, float &d2, float &dp2) {
     chk_force(S, fx, fy, fz);
-    const float pe_a = S.pen[a] + (fpa != 0.f ? S.pot.f_ec2hq / fpa : 0.f);
+    const float pe_a = ((const float *)S.pen)[a];
     pe += (double)pe_a;
     const uint8_t flag = S.flags[a];
     if (flag == FLAG_RIGHT) rr -= (double)(S.axis == 0 ? fx : (S.axis == 1 ? fy : fz));

@@ -83,8 +83,10 @@ __device__ __forceinline__ void density_block(const SpecDev &S, int lb, int par,
         const float rho = SC76 ? fmaf(P.am, s.sm, fmaf(P.Bm, dr, -cnt * P.Am)) : s.sm;
         const float phn = fmaf(P.an, s.sn, fmaf(P.Bn, dr, -cnt * P.An));
         // w = m a^m B'(rho), B'(rho) = -eps c / (2 sqrt(rho))
-        const float w = rho > 0.f ? P.fpsc * rsqrtf(rho) : 0.f;
-        S.pen[u] = 0.5f * P.eps * phn;
+        const float rq = rho > 0.f ? rsqrtf(rho) : 0.f;
+        const float w = P.fpsc * rq;
+        // the atom's energy 1/2 eps sum_j phi_n + B(rho), B = -eps c sqrt(rho)
+        ((float *)S.pen)[u] = fmaf(-P.ec, rho > 0.f ? rho * rq : 0.f, 0.5f * P.eps * phn);
         ((int4 *)S.posfp)[u] = make_int4(ra.x, ra.y, ra.z, __float_as_int(w));
     }
 }
@@ -112,8 +114,8 @@ __device__ __forceinline__ void force_block(const SpecDev &S, int lb, int par, c
     double ke = 0.0, pe = 0.0, rr = 0.0;
     float d2 = 0.f, dp2 = 0.f;
     if (valid && l == 0)
-        atom_update_mixed(S, S.ctl, par, u, S.prune_on != 0, wa, fx, fy, fz, mode, phase, done,
-                          nsteps, ke, pe, rr, d2, dp2);
+        atom_update_mixed(S, S.ctl, par, u, S.prune_on != 0, fx, fy, fz, mode, phase, done, nsteps,
+                          ke, pe, rr, d2, dp2);
     ke = warp_sum(ke);
     pe = warp_sum(pe);
     rr = warp_sum(rr);

@@ -251,6 +251,24 @@ static PotDev make_pot(const pta_potential &p) {
     d.Bn = p.n / p.rc * d.An;
     d.Bm = p.m / p.rc * d.Am;
     d.ec = p.eps * p.c;
+    {
+        // in extended precision, each rounded once: an error of a constant is
+        // the same for every pair and does not average out
+        using ld = long double;
+        auto lpow = [](ld x, int k) {
+            ld r = 1;
+            for (int i = 0; i < k; ++i) r *= x;
+            return r;
+        };
+        const ld a = p.a, rc = p.rc, eps = p.eps, an = lpow(a, p.n), am = lpow(a, p.m);
+        const ld An = lpow(a / rc, p.n), Am = lpow(a / rc, p.m), ec = eps * (ld)p.c;
+        d.an = (double)an;
+        d.am = (double)am;
+        d.kn = (double)(eps * p.n * an);
+        d.bmq = (double)(p.m / rc * Am / (p.m * am));
+        d.ebn = (double)(eps * p.n / rc * An);
+        d.fpsc = (double)(-0.5L * ec * p.m * am);
+    }
     d.f_eps = (float)d.eps;
     d.f_a = (float)d.a;
     d.f_rc = (float)d.rc;
@@ -260,7 +278,6 @@ static PotDev make_pot(const pta_potential &p) {
     d.f_Am = (float)d.Am;
     d.f_Bm = (float)d.Bm;
     d.f_ec = (float)d.ec;
-    d.f_ec2hq = (float)(0.5 * d.ec * d.ec * p.m * hpow(p.a, p.m));
     d.sc76 = (p.n == 7 && p.m == 6) ? 1 : 0;
     return d;
 }
@@ -361,8 +378,8 @@ static size_t footprint(const Sizes &z, int prec) {
     if (prec != PTA_PREC_FP64) {
         add(16 * n);
         add(16 * n);                 // lo[2]
-        add(4 * n);                  // pen
     }
+    add((prec == PTA_PREC_FP64 ? 8 : 4) * n);  // pen
     add(16 * n);
     add(16 * n);                     // rec[2]
     add(p * n);                      // posfp
@@ -1042,8 +1059,8 @@ static int ctx_alloc_all(pta_ctx *c, const Sizes &z) {
     if (!f64) {
         AL(lo[0], 16 * n, float4 *);
         AL(lo[1], 16 * n, float4 *);
-        AL(pen, 4 * n, float *);
     }
+    AL(pen, (f64 ? 8 : 4) * n, void *);
     AL(rec[0], 16 * n, int4 *);
     AL(rec[1], 16 * n, int4 *);
     AL(posfp, p * n, void *);

@@ -54,9 +54,9 @@ enum AtomFlag : uint8_t { FLAG_MOBILE = 0, FLAG_LEFT = 1, FLAG_RIGHT = 2 };
 //   phi_k'(r) = -k s^k / r + B_k
 struct PotDev {
     double eps, c, a, rc, rc2, An, Bn, Am, Bm, ec;
+    double an, am, kn, bmq, ebn, fpsc;  // as in PotF, in FP64
     int n, m;
     float f_eps, f_a, f_rc, f_rc2, f_An, f_Bn, f_Am, f_Bm, f_ec;
-    float f_ec2hq;  // (eps c)^2 m a^m / 2: B(rho) = f_ec2hq / w with w = m a^m B'(rho)
     int sc76;  // 1 when (n, m) == (7, 6): the fast specialised kernels apply
 };
 
@@ -152,9 +152,9 @@ struct SpecDev {
     void *pos[2];   // FP64: double4 {x,y,z,0};  MIXED: float4 hi {x,y,z,0}
     float4 *lo[2];  // MIXED only: float4 lo {x,y,z,0}
     int4 *rec[2];   // fixed-point record {x,y,z,0} of every atom
-    void *posfp;    // FP64: double4 {x,y,z,B'(rho)};  MIXED: the record with w = m a^m B'(rho)
-                    // (float bits) as fourth word
-    float *pen;     // MIXED: pair energy of each atom, 1/2 eps sum_j phi_n
+    void *posfp;    // FP64: double4 {x,y,z,w};  MIXED: the record with w (float bits) as
+                    // fourth word; w = m a^m B'(rho)
+    void *pen;      // energy of each atom, 1/2 eps sum_j phi_n + B(rho) (double; MIXED: float)
     void *vel;      // FP64: double4; MIXED: VelHL
     uint8_t *flags;
     float4 *ref;    // positions at the last list build (skin test)
