@@ -133,100 +133,112 @@ __device__ __forceinline__ void hl_add(float &h, float &l, float d) {
     h = hh;
 }
 
-// After the force pass of atom a (force f; its energy from the density
-// pass): its share of the reaction, and the velocity-Verlet update -- the half-kick that finishes the step (phase RUN),
-// the sample of K, and unless the burst ends the half-kick and drift of the
-// next step; the new position (hi + lo, whole grid quanta moved from lo to
-// hi), its neighbour record, and the displacements since the last list
-// build (and, with `pruned`, since the last pruning).  Grip
-// atoms keep v = 0.  MODE_EVAL stores F and the energy instead.
-__device__ __forceinline__ void atom_update_mixed(const SpecDev &S, SpecCtl *ctl, int par, int a,
-                                                  bool pruned, float fx, float fy, float fz,
-                                                  int mode, int phase, long long done,
-                                                  long long nsteps, double &ke, double &pe,
-                                                  double &rr, float &d2, float &dp2) {
-    chk_force(S, fx, fy, fz);
-    const float pe_a = ((const float *)S.pen)[a];
-    pe += (double)pe_a;
-    const uint8_t flag = S.flags[a];
-    if (flag == FLAG_RIGHT) rr -= (double)(S.axis == 0 ? fx : (S.axis == 1 ? fy : fz));
-    VelHL *vp = (VelHL *)S.vel + a;
-    VelHL v = *vp;
-    if (mode == MODE_EVAL) {
-        const float vx = v.h.x + v.l.x, vy = v.h.y + v.l.y, vz = v.h.z + v.l.z;
-        ke += (double)(S.f_ke_fac * (vx * vx + vy * vy + vz * vz));
-        double4_32a *o = (double4_32a *)S.eval_out;
-        o[S.orig[a]] = make_double4_32a(fx, fy, fz, pe_a);
-        return;
+// An atom's state outside the neighbour records.
+struct AtomMixed {
+    float vh[3], vl[3], hi[3], lo[3];
+    int4 ref, pref;
+    int flag;
+    __device__ __forceinline__ void load(const SpecDev &S, int par, int a) {
+        const VelHL v = ((const VelHL *)S.vel)[a];
+        const float4 h = ((const float4 *)S.pos[par])[a], l = S.lo[par][a];
+        vh[0] = v.h.x; vh[1] = v.h.y; vh[2] = v.h.z;
+        vl[0] = v.l.x; vl[1] = v.l.y; vl[2] = v.l.z;
+        hi[0] = h.x; hi[1] = h.y; hi[2] = h.z;
+        lo[0] = l.x; lo[1] = l.y; lo[2] = l.z;
+        ref = S.ref[a];
+        pref = S.prune_on ? S.pref[a] : ref;
+        flag = S.flags[a];
     }
-    const float kh = S.f_acc_half;
+    __device__ __forceinline__ void store(const SpecDev &S, int par, int a) const {
+        VelHL v;
+        v.h = make_float4(vh[0], vh[1], vh[2], 0.f);
+        v.l = make_float4(vl[0], vl[1], vl[2], 0.f);
+        ((VelHL *)S.vel)[a] = v;
+        ((float4 *)S.pos[par])[a] = make_float4(hi[0], hi[1], hi[2], 0.f);
+        S.lo[par][a] = make_float4(lo[0], lo[1], lo[2], 0.f);
+    }
+};
+
+// After the force pass of atom a (force f; its energy pe from the density
+// pass): its share of the state functions, and the velocity-Verlet update --
+// the half-kick that finishes the step (phase RUN), the sample of K, and
+// unless the burst ends the half-kick and drift of the next step; the new
+// position (hi + lo, whole grid quanta moved from lo to hi), its neighbour
+// record (returned), and the displacements since the last list build and the last
+// pruning.  Grip atoms keep v = 0.  MODE_EVAL stores F and the energy
+// instead.  Sums and products are written as the operations meant, so that
+// every kernel this is compiled into rounds alike.
+__device__ __forceinline__ int4 atom_update_mixed(const SpecDev &S, AtomMixed &A, int par, int a,
+                                                  const float f[3], float pe, int mode, int phase,
+                                                  long long done, long long nsteps,
+                                                  StepVals<FF> &out) {
+    chk_force(S, f[0], f[1], f[2]);
+    SpecCtl *ctl = S.ctl;
+    set(out.s[1], pe);
+    if (A.flag == FLAG_RIGHT) set(out.s[2], -(S.axis == 0 ? f[0] : (S.axis == 1 ? f[1] : f[2])));
+    auto kinetic = [&] {
+        const float x = A.vh[0] + A.vl[0], y = A.vh[1] + A.vl[1], z = A.vh[2] + A.vl[2];
+        set(out.s[0], __fmul_rn(S.f_ke_fac, fmaf(z, z, fmaf(y, y, __fmul_rn(x, x)))));
+    };
+    if (mode == MODE_EVAL) {
+        kinetic();
+        ((double4_32a *)S.eval_out)[S.orig[a]] = make_double4_32a(f[0], f[1], f[2], pe);
+        return make_int4(0, 0, 0, 0);
+    }
     // thermal relaxation: the right grip moves along the load axis only (its
     // other velocity components stay 0, so the drift leaves them in place)
-    const bool rfree = flag == FLAG_RIGHT && ctl->relax;
-    const bool moves = flag == FLAG_MOBILE || rfree;
-    const float kx = (flag == FLAG_MOBILE || (rfree && S.axis == 0)) ? fx * kh : 0.f;
-    const float ky = (flag == FLAG_MOBILE || (rfree && S.axis == 1)) ? fy * kh : 0.f;
-    const float kz = (flag == FLAG_MOBILE || (rfree && S.axis == 2)) ? fz * kh : 0.f;
+    const bool rfree = A.flag == FLAG_RIGHT && ctl->relax;
+    const bool moves = A.flag == FLAG_MOBILE || rfree;
+    float k[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+        k[d] = (A.flag == FLAG_MOBILE || (rfree && S.axis == d)) ? __fmul_rn(f[d], S.f_acc_half)
+                                                                 : 0.f;
     if (phase == PH_RUN) {
         if (moves) {
-            hl_add(v.h.x, v.l.x, kx);
-            hl_add(v.h.y, v.l.y, ky);
-            hl_add(v.h.z, v.l.z, kz);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) hl_add(A.vh[d], A.vl[d], k[d]);
         }
-        const float vx = v.h.x + v.l.x, vy = v.h.y + v.l.y, vz = v.h.z + v.l.z;
-        ke += (double)(S.f_ke_fac * (vx * vx + vy * vy + vz * vz));
+        kinetic();
+        if (S.rsum) {
+            // Eq. (mean_pos): the sampled state's position, hi + lo exactly
+            double *rs = S.rsum + 4LL * S.orig[a];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) rs[d] = rs[d] + ((double)A.hi[d] + (double)A.lo[d]);
+        }
     }
-    const float4 hia = ((const float4 *)S.pos[par])[a];
-    const float4 loa = S.lo[par][a];
-    if (phase == PH_RUN && S.rsum) {
-        // Eq. (mean_pos): the sampled state's position, hi + lo exactly
-        double *rs = S.rsum + 4LL * S.orig[a];
-        rs[0] = rs[0] + ((double)hia.x + (double)loa.x);
-        rs[1] = rs[1] + ((double)hia.y + (double)loa.y);
-        rs[2] = rs[2] + ((double)hia.z + (double)loa.z);
-    }
-    float hh[3] = {hia.x, hia.y, hia.z}, qq[3] = {loa.x, loa.y, loa.z};
     const bool start = (phase == PH_REFRESH) || (done + 1 < nsteps);
     // continuous loading (fine-dynamics verification): a fixed right grip
     // moves by grip_du along the load axis with every step's drift
-    const float gdu = (start && flag == FLAG_RIGHT && !rfree) ? (float)ctl->grip_du : 0.f;
+    const float gdu =
+        (start && A.flag == FLAG_RIGHT && !rfree) ? (float)ctl->grip_du : 0.f;
     if (start && (moves || gdu != 0.f)) {
-        const float dt = S.f_dt;
         if (moves) {
-            hl_add(v.h.x, v.l.x, kx);
-            hl_add(v.h.y, v.l.y, ky);
-            hl_add(v.h.z, v.l.z, kz);
-            qq[0] += (v.h.x + v.l.x) * dt;
-            qq[1] += (v.h.y + v.l.y) * dt;
-            qq[2] += (v.h.z + v.l.z) * dt;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                hl_add(A.vh[d], A.vl[d], k[d]);
+                A.lo[d] = fmaf(A.vh[d] + A.vl[d], S.f_dt, A.lo[d]);
+            }
         } else {
-            qq[S.axis] += gdu;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) A.lo[d] += S.axis == d ? gdu : 0.f;
         }
+        bool far = false;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             // move whole grid quanta from lo to hi (both steps exact)
-            const float sh = rintf(qq[d] * (float)HI_SCALE) * (float)HI_QUANTUM;
-            hh[d] = hh[d] + sh;
-            qq[d] = qq[d] - sh;
+            const float sh = __fmul_rn(rintf(A.lo[d] * (float)HI_SCALE), (float)HI_QUANTUM);
+            A.hi[d] = __fadd_rn(A.hi[d], sh);
+            A.lo[d] = __fsub_rn(A.lo[d], sh);
+            far |= fabsf(A.hi[d]) > (float)MIXED_RANGE;
         }
-        if (fabsf(hh[0]) > (float)MIXED_RANGE || fabsf(hh[1]) > (float)MIXED_RANGE ||
-            fabsf(hh[2]) > (float)MIXED_RANGE)
-            atomicOr(&ctl->err, ERR_RANGE);
+        if (far) atomicOr(&ctl->err, ERR_RANGE);
     }
-    ((float4 *)S.pos[par ^ 1])[a] = make_float4(hh[0], hh[1], hh[2], 0.f);
-    S.lo[par ^ 1][a] = make_float4(qq[0], qq[1], qq[2], 0.f);
-    S.rec[par ^ 1][a] = rec_mixed(S, hh[0], hh[1], hh[2], qq[0], qq[1], qq[2]);
-    *vp = v;
-    const float4 rf = S.ref[a];
-    const float ex = (hh[0] - rf.x) + qq[0], ey = (hh[1] - rf.y) + qq[1],
-                ez = (hh[2] - rf.z) + qq[2];
-    d2 = fmaxf(d2, ex * ex + ey * ey + ez * ez);
-    if (pruned) {
-        const float4 pf = S.pref[a];
-        const float px = (hh[0] - pf.x) + qq[0], py = (hh[1] - pf.y) + qq[1],
-                    pz = (hh[2] - pf.z) + qq[2];
-        dp2 = fmaxf(dp2, px * px + py * py + pz * pz);
-    }
+    const int4 r = rec_mixed(S, A.hi[0], A.hi[1], A.hi[2], A.lo[0], A.lo[1], A.lo[2]);
+    S.rec[par ^ 1][a] = r;
+    out.d2 = moved2(r, A.ref);
+    out.dp2 = moved2(r, A.pref);
+    return r;
 }
 
 }  // namespace pta

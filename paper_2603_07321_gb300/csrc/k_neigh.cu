@@ -337,10 +337,8 @@ __global__ void __launch_bounds__(BUILD_WARPS * 32) k_build(const SpecDev *__res
         }
         if (lane == 0) {
             S.nab[a] = make_int2(na, nb);
-            const float3 x = load_pos32(S, par, a);
-            const float4 p = make_float4(x.x, x.y, x.z, 0.f);
-            S.ref[a] = p;
-            if (S.prune_on) S.pref[a] = p;
+            S.ref[a] = ra;
+            if (S.prune_on) S.pref[a] = ra;
         }
         __syncwarp();
     }
@@ -383,6 +381,23 @@ __global__ void k_decide_rebuild(const SpecDev *__restrict__ specs, int nspec,
     prune = __syncthreads_or(prune);
     if (threadIdx.x == 0)
         cudaGraphSetConditional(handle, build ? LIST_BUILD : (prune ? LIST_PRUNE : LIST_NONE));
+}
+
+// the same for resident runs, which prune by themselves: 1 when any specimen
+// needs a list build; and the run's barrier word starts at 0
+__global__ void k_decide_build(const SpecDev *__restrict__ specs, int nspec, RunCtl *rc,
+                               cudaGraphConditionalHandle handle) {
+    int build = 0;
+    for (int s = threadIdx.x; s < nspec; s += blockDim.x) build |= build_active(specs[s], 0);
+    build = __syncthreads_or(build);
+    if (threadIdx.x == 0) {
+        rc->arrive = 0;
+        cudaGraphSetConditional(handle, build ? 1u : 0u);
+    }
+}
+
+void launch_decide_build(const Tab &t, RunCtl *rc, cudaGraphConditionalHandle h, cudaStream_t st) {
+    k_decide_build<<<1, 128, 0, st>>>(t.specs, t.nspec, rc, h);
 }
 
 void launch_decide_rebuild(const Tab &t, cudaGraphConditionalHandle h, cudaStream_t st) {

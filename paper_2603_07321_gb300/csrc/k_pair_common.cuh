@@ -3,22 +3,11 @@
 // into the state functions K, U, T of Eq. (state_variables) for one step.
 #pragma once
 
+#include <algorithm>
+
 #include "pta_dev.cuh"
 
 namespace pta {
-
-template <typename T>
-__device__ __forceinline__ T warp_sum(T v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-__device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
 
 // sum over the L lanes that share one atom (lanes are contiguous in the warp)
 template <int L, typename T>
@@ -28,183 +17,750 @@ __device__ __forceinline__ T lane_sum(T v) {
     return v;
 }
 
-// Called by every thread of a pair block of NT threads after the warp
-// reductions (values valid in lane 0 of each warp); nblk is the number of
-// the specimen's blocks in this launch.  Block partials go to S.part (8
-// doubles per block).  The reduction is a fixed two-level tree: the last
-// block to finish in each group of 32 consecutive blocks sums the group's
-// partials (one per lane, butterfly shuffles) into a group partial stored
-// after the block partials, and the last group to finish sums the group
-// partials (each thread a strided share, then warp shuffles, then the warps
-// in order).  Each level is one round of parallel loads; a single last
-// block walking every block partial took ~8 us longer per pass on the
-// 470,596-atom cube.  Group counters sit after the group partials, start
-// at 0 and are reset by their group's last block.  The last group then
-// advances the specimen's control block:
+// ---------------------------------------------------------------------------
+// The state functions of a step: sums over the atoms of K, U and the reaction
+// R, and the largest squared displacements since the list build and since the
+// pruning (quanta^2).
+//
+// Sums are double in FP64 contexts and pairs of floats (an unevaluated sum,
+// 48 bits, error-free additions) in mixed precision, whose terms are floats:
+// FP64 additions run two lanes per clock and SM here, and 15 of them per warp
+// (three sums, five shuffle stages) cost the force pass of the 470,596-atom
+// cube ~12 us.
+// ---------------------------------------------------------------------------
+struct FF {
+    float h, l;
+};
+__device__ __forceinline__ FF add(FF a, FF b) {
+    const float s = __fadd_rn(a.h, b.h), t = __fsub_rn(s, a.h);
+    const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
+    const float l = __fadd_rn(__fadd_rn(a.l, b.l), e);
+    FF r;
+    r.h = __fadd_rn(s, l);
+    r.l = __fsub_rn(l, __fsub_rn(r.h, s));
+    return r;
+}
+__device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ FF shfl_xor(FF v, int o) {
+    return {__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
+}
+__device__ __forceinline__ double shfl_xor(double v, int o) {
+    return __shfl_xor_sync(0xffffffffu, v, o);
+}
+__device__ __forceinline__ double to_double(FF v) { return (double)v.h + (double)v.l; }
+__device__ __forceinline__ double to_double(double v) { return v; }
+__device__ __forceinline__ void set(FF &v, float x) { v = {x, 0.f}; }
+__device__ __forceinline__ void set(double &v, double x) { v = x; }
+// non-negative floats order as their bits
+__device__ __forceinline__ float warp_max(float v) {
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+}
+
+template <class T>
+struct StepVals {
+    T s[3];         // K, U, R
+    float d2, dp2;  // displacements
+};
+// sums over the lanes whose values count (every MINO-th), down to offset MINO
+template <int MINO, class T>
+__device__ __forceinline__ void warp_reduce(StepVals<T> &v) {
+#pragma unroll
+    for (int o = 16; o >= MINO; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) v.s[q] = add(v.s[q], shfl_xor(v.s[q], o));
+    v.d2 = warp_max(v.d2);
+    v.dp2 = warp_max(v.dp2);
+}
+// a partial in memory: three sums and the two maxima, 32 bytes
+__device__ __forceinline__ void load_part(const double *p, StepVals<FF> &v) {
+    const float4 a = __ldcg((const float4 *)p), b = __ldcg((const float4 *)p + 1);
+    v.s[0] = {a.x, a.y};
+    v.s[1] = {a.z, a.w};
+    v.s[2] = {b.x, b.y};
+    v.d2 = b.z;
+    v.dp2 = b.w;
+}
+__device__ __forceinline__ void load_part(const double *p, StepVals<double> &v) {
+    const double2 a = __ldcg((const double2 *)p), b = __ldcg((const double2 *)p + 1);
+    v.s[0] = a.x;
+    v.s[1] = a.y;
+    v.s[2] = b.x;
+    v.d2 = __int_as_float(__double2loint(b.y));
+    v.dp2 = __int_as_float(__double2hiint(b.y));
+}
+__device__ __forceinline__ void store_part(double *p, const StepVals<FF> &v) {
+    ((float4 *)p)[0] = make_float4(v.s[0].h, v.s[0].l, v.s[1].h, v.s[1].l);
+    ((float4 *)p)[1] = make_float4(v.s[2].h, v.s[2].l, v.d2, v.dp2);
+}
+__device__ __forceinline__ void store_part(double *p, const StepVals<double> &v) {
+    ((double2 *)p)[0] = make_double2(v.s[0], v.s[1]);
+    ((double2 *)p)[1] = make_double2(
+        v.s[2], __hiloint2double(__float_as_int(v.dp2), __float_as_int(v.d2)));
+}
+// a += b
+template <class T>
+__device__ __forceinline__ void merge(StepVals<T> &a, const StepVals<T> &b) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) a.s[q] = add(a.s[q], b.s[q]);
+    a.d2 = fmaxf(a.d2, b.d2);
+    a.dp2 = fmaxf(a.dp2, b.dp2);
+}
+template <class T>
+__device__ __forceinline__ StepVals<T> zero_vals() {
+    StepVals<T> v;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) set(v.s[q], 0);
+    v.d2 = v.dp2 = 0.f;
+    return v;
+}
+
+// squared displacement of a record from an earlier one, quanta^2
+__device__ __forceinline__ float moved2(const int4 &a, const int4 &b) {
+    const float x = (float)(a.x - b.x), y = (float)(a.y - b.y), z = (float)(a.z - b.z);
+    return fmaf(z, z, fmaf(y, y, __fmul_rn(x, x)));
+}
+
+constexpr int PART = 4;           // doubles per partial
+constexpr int PART_GROUP = 32;    // blocks per group of partials
+
+// the block's partial (warp values valid in lane 0), stored by its first
+// warp; complete for a thread-0 release that follows
+template <int NT, class T>
+__device__ __forceinline__ void block_partial(const SpecDev &S, int lb, const StepVals<T> &v) {
+    constexpr int NW = NT / 32;
+    __shared__ T sh[3][NW];
+    __shared__ float shm[2][NW];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (lane == 0) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) sh[q][w] = v.s[q];
+        shm[0][w] = v.d2;
+        shm[1][w] = v.dp2;
+    }
+    __syncthreads();
+    if (w == 0) {
+        double *P = S.part + (long long)PART * lb;
+        if (lane < 3) {
+            T a = sh[lane][0];
+#pragma unroll
+            for (int k = 1; k < NW; ++k) a = add(a, sh[lane][k]);
+            *(T *)(P + lane) = a;
+        } else if (lane < 5) {
+            float m = shm[lane - 3][0];
+#pragma unroll
+            for (int k = 1; k < NW; ++k) m = fmaxf(m, shm[lane - 3][k]);
+            ((float *)(P + 3))[lane - 3] = m;
+        }
+        __syncwarp();
+    }
+}
+
+// the totals of a step, valid in thread 0, from the group partials: each
+// thread a strided share, then warp shuffles, then the warps in order
+template <int NT, class T, class F>
+__device__ __forceinline__ StepVals<T> total_of_groups(int ngroups, F group) {
+    constexpr int NW = NT / 32;
+    __shared__ T sh[3][NW];
+    __shared__ float shm[2][NW];
+    StepVals<T> v = zero_vals<T>();
+    for (int b = threadIdx.x; b < ngroups; b += NT) {
+        merge(v, group(b));
+    }
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // a single warp holds everything of up to 32 groups: adding the other
+    // warps' zeros changes nothing
+    if (w * 32 < ngroups) warp_reduce<1>(v);
+    if (ngroups <= 32) return v;
+    if (lane == 0) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) sh[q][w] = v.s[q];
+        shm[0][w] = v.d2;
+        shm[1][w] = v.dp2;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int k = 1; k < NW; ++k) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) v.s[q] = add(v.s[q], sh[q][k]);
+            v.d2 = fmaxf(v.d2, shm[0][k]);
+            v.dp2 = fmaxf(v.dp2, shm[1][k]);
+        }
+    return v;
+}
+
+// One thread: the specimen's control block after a step with these totals.
 //   MODE_STEP, phase RUN:     sample (K, U, T) into the series, step count + 1,
 //                             burst over after nsteps samples
 //   MODE_STEP, phase REFRESH: forces refreshed and the first step started
 //   MODE_EVAL:                K, U, T stored in eval_obs
 // and in MODE_STEP the position buffers swap, the skin test sets the
 // rebuild flag and the pruning margin test the prune flag.
-template <int NT>
-__device__ inline void step_tail(const SpecDev &S, int lb, int nblk, double ke_w, double pe_w,
-                                 double rr_w, double d2_w, double dp2_w, int mode, int phase,
-                                 long long done, long long nsteps) {
-    constexpr int NV = 5;  // K, U, R, max displacement^2 since the build and since the pruning
-    constexpr int NW = NT / 32;
-    __shared__ double shw[NV][NW];
-    __shared__ int role;  // 0: done; 1: last block of its group; 2: last group
-    constexpr int GS = 32;  // blocks per group
-    const int ngroups = (nblk + GS - 1) / GS;
-    const int g = lb / GS;
-    const int gsize = min(GS, nblk - g * GS);
-    unsigned *gcnt = (unsigned *)(S.part + 8LL * (nblk + ngroups)) + g;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) {
-        shw[0][w] = ke_w;
-        shw[1][w] = pe_w;
-        shw[2][w] = rr_w;
-        shw[3][w] = d2_w;
-        shw[4][w] = dp2_w;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double k = 0, p = 0, r = 0, d = 0, e = 0;
-        for (int i = 0; i < NW; ++i) {
-            k = k + shw[0][i];
-            p = p + shw[1][i];
-            r = r + shw[2][i];
-            d = fmax(d, shw[3][i]);
-            e = fmax(e, shw[4][i]);
-        }
-        double *P = S.part + 8LL * lb;
-        P[0] = k;
-        P[1] = p;
-        P[2] = r;
-        P[3] = d;
-        P[4] = e;
-        __threadfence();
-        const unsigned prev = atomicAdd(gcnt, 1u);
-        role = (prev == (unsigned)(gsize - 1)) ? 1 : 0;
-    }
-    __syncthreads();
-    if (role == 0) return;
-    __threadfence();
-    if (w == 0) {
-        // the group's partials, one per lane, summed in lane order
-        double a[NV] = {0, 0, 0, 0, 0};
-        if (lane < gsize) {
-            const double *P = S.part + 8LL * (g * GS + lane);
-            a[0] = __ldcg(P);
-            a[1] = __ldcg(P + 1);
-            a[2] = __ldcg(P + 2);
-            a[3] = __ldcg(P + 3);
-            a[4] = __ldcg(P + 4);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            a[0] = a[0] + __shfl_xor_sync(0xffffffffu, a[0], o);
-            a[1] = a[1] + __shfl_xor_sync(0xffffffffu, a[1], o);
-            a[2] = a[2] + __shfl_xor_sync(0xffffffffu, a[2], o);
-            a[3] = fmax(a[3], __shfl_xor_sync(0xffffffffu, a[3], o));
-            a[4] = fmax(a[4], __shfl_xor_sync(0xffffffffu, a[4], o));
-        }
-        if (lane == 0) {
-            double *G = S.part + 8LL * (nblk + g);
-            for (int q = 0; q < NV; ++q) G[q] = a[q];
-            *gcnt = 0u;  // every block of the group has counted: ready for the next launch
-            __threadfence();
-            const unsigned prev = atomicAdd(&S.ctl->blocks_done, 1u);
-            role = (prev == (unsigned)(ngroups - 1)) ? 2 : 0;
-        }
-    }
-    __syncthreads();
-    if (role != 2) return;
-    __threadfence();
-    double v[NV] = {0, 0, 0, 0, 0};
-    for (int b = threadIdx.x; b < ngroups; b += NT) {
-        const double *P = S.part + 8LL * (nblk + b);
-        v[0] = v[0] + __ldcg(P);
-        v[1] = v[1] + __ldcg(P + 1);
-        v[2] = v[2] + __ldcg(P + 2);
-        v[3] = fmax(v[3], __ldcg(P + 3));
-        v[4] = fmax(v[4], __ldcg(P + 4));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        v[0] = v[0] + __shfl_xor_sync(0xffffffffu, v[0], o);
-        v[1] = v[1] + __shfl_xor_sync(0xffffffffu, v[1], o);
-        v[2] = v[2] + __shfl_xor_sync(0xffffffffu, v[2], o);
-        v[3] = fmax(v[3], __shfl_xor_sync(0xffffffffu, v[3], o));
-        v[4] = fmax(v[4], __shfl_xor_sync(0xffffffffu, v[4], o));
-    }
-    __syncthreads();  // every warp has read shw above
-    if (lane == 0)
-        for (int q = 0; q < NV; ++q) shw[q][w] = v[q];
-    __syncthreads();
-    double tot[NV] = {0, 0, 0, 0, 0};
-    if (threadIdx.x == 0)
-        for (int i = 0; i < NW; ++i) {
-            tot[0] = tot[0] + shw[0][i];
-            tot[1] = tot[1] + shw[1][i];
-            tot[2] = tot[2] + shw[2][i];
-            tot[3] = fmax(tot[3], shw[3][i]);
-            tot[4] = fmax(tot[4], shw[4][i]);
-        }
-    if (threadIdx.x != 0) return;
+__device__ inline void advance_ctl(const SpecDev &S, double K, double U, double R, float md2,
+                                   float mp2, int mode, int phase, int par, long long done,
+                                   long long nsteps) {
     SpecCtl *c = S.ctl;
-    const double K = tot[0], U = tot[1], T = tot[2] * S.t_fac, md2 = tot[3], mp2 = tot[4];
+    const double T = R * S.t_fac;
     if (mode == MODE_EVAL) {
         c->eval_obs[0] = K;
         c->eval_obs[1] = U;
         c->eval_obs[2] = T;
         c->rebuild = 0;
-    } else {
-        if (phase == PH_RUN) {
-            if (!isfinite(K) || !isfinite(U) || !isfinite(T)) {
-                c->err |= ERR_NAN;
-                c->phase = PH_IDLE;
-            } else {
-                double *o = S.series + 3 * done;
-                o[0] = K;
-                o[1] = U;
-                o[2] = T;
+        return;
+    }
+    int now = phase;
+    if (phase == PH_RUN) {
+        if (!isfinite(K) || !isfinite(U) || !isfinite(T)) {
+            c->err |= ERR_NAN;
+            now = PH_IDLE;
+        } else {
+            double *o = S.series + 3 * done;
+            o[0] = K;
+            o[1] = U;
+            o[2] = T;
+            if (S.conv_lag > 0) {
                 c->sum[0] = c->sum[0] + K;
                 c->sum[1] = c->sum[1] + U;
                 c->sum[2] = c->sum[2] + T;
-                c->done = done + 1;
-                if (done + 1 >= nsteps) c->phase = PH_IDLE;
-                const long long i = done + 1;
-                if (S.conv_lag > 0 && i % S.conv_lag == 0) {
-                    // appendix, Eq. (R_m_conv): e = |R^(i) - R^(i-k)| / max(|R^(i)|,
-                    // floor), from i = 2k on; each variable converges on its own
-                    if (i >= 2LL * S.conv_lag) {
-                        for (int q = 0; q < 3; ++q) {
-                            if (c->conv_mask & (1 << q)) continue;
-                            const double a = c->sum[q] / (double)i;
-                            const double b = c->sum_chk[q] / (double)(i - S.conv_lag);
-                            const double e = fabs(a - b) / fmax(fabs(a), S.floor_[q]);
-                            if (e < S.conv_tol[q]) {
-                                c->conv_mask |= 1 << q;
-                                c->conv_n[q] = i;
-                                c->conv_val[q] = a;
-                            }
-                        }
-                        if (c->conv_mask == 7) c->phase = PH_IDLE;
-                    }
-                    for (int q = 0; q < 3; ++q) c->sum_chk[q] = c->sum[q];
-                }
             }
-        } else if (phase == PH_REFRESH) {
-            c->phase = PH_RUN;
+            c->done = done + 1;
+            if (done + 1 >= nsteps) now = PH_IDLE;
+            const long long i = done + 1;
+            if (S.conv_lag > 0 && i % S.conv_lag == 0) {
+                // appendix, Eq. (R_m_conv): e = |R^(i) - R^(i-k)| / max(|R^(i)|,
+                // floor), from i = 2k on; each variable converges on its own
+                if (i >= 2LL * S.conv_lag) {
+                    for (int q = 0; q < 3; ++q) {
+                        if (c->conv_mask & (1 << q)) continue;
+                        const double a = c->sum[q] / (double)i;
+                        const double b = c->sum_chk[q] / (double)(i - S.conv_lag);
+                        const double e = fabs(a - b) / fmax(fabs(a), S.floor_[q]);
+                        if (e < S.conv_tol[q]) {
+                            c->conv_mask |= 1 << q;
+                            c->conv_n[q] = i;
+                            c->conv_val[q] = a;
+                        }
+                    }
+                    if (c->conv_mask == 7) now = PH_IDLE;
+                }
+                for (int q = 0; q < 3; ++q) c->sum_chk[q] = c->sum[q];
+            }
         }
-        c->rebuild = (md2 > (double)S.half_skin2) ? 1 : 0;
-        if (S.prune_on && mp2 > (double)S.half_prune2) c->prune = 1;
-        c->parity ^= 1;
+    } else if (phase == PH_REFRESH) {
+        now = PH_RUN;
     }
+    c->phase = now;
+    c->rebuild = md2 > S.half_skin2q;
+    if (S.prune_on && mp2 > S.half_prune2q) c->prune = 1;
+    c->parity = par ^ 1;
+}
+
+// End of a force pass between kernels, called by every thread of a block of
+// NT threads; nblk: the specimen's blocks in this launch.  The block partials
+// are reduced along a fixed two-level tree: the last block to finish in each
+// group of 32 consecutive blocks sums the group's partials (one per lane,
+// butterfly shuffles) into a group partial stored after the block partials,
+// and the last group to finish sums the group partials and advances the
+// control block.  Each level is one round of parallel loads; a single last
+// block walking every block partial took ~8 us longer per pass on the
+// 470,596-atom cube.  Group counters sit beyond the partials (also beyond the
+// per-warp ones of resident runs), start at 0 and are reset by their group's
+// last block.
+template <int NT, class T>
+__device__ inline void step_tail(const SpecDev &S, int lb, int nblk, const StepVals<T> &v, int mode,
+                                 int phase, int par, long long done, long long nsteps) {
+    __shared__ int role;  // 0: done; 1: last block of its group; 2: last group
+    const int ngroups = (nblk + PART_GROUP - 1) / PART_GROUP;
+    const int g = lb / PART_GROUP;
+    const int gsize = min(PART_GROUP, nblk - g * PART_GROUP);
+    double *groups = S.part + (long long)PART * nblk;
+    unsigned *gcnt = (unsigned *)(S.part + (long long)PART * (TPB / 32) * nblk) + g;
+    block_partial<NT>(S, lb, v);
+    if (threadIdx.x == 0) {
+        __threadfence();
+        role = atomicAdd(gcnt, 1u) == (unsigned)(gsize - 1);
+    }
+    __syncthreads();
+    if (role == 0) return;
     __threadfence();
-    c->blocks_done = 0;
+    const int lane = threadIdx.x & 31;
+    StepVals<T> a = zero_vals<T>();
+    if (threadIdx.x < 32) {
+        if (lane < gsize) load_part(S.part + (long long)PART * (g * PART_GROUP + lane), a);
+        warp_reduce<1>(a);
+        if (lane == 0) {
+            *gcnt = 0u;  // every block of the group has counted: ready for the next launch
+            if (ngroups > 1) {
+                store_part(groups + (long long)PART * g, a);
+                __threadfence();
+                role = atomicAdd(&S.ctl->blocks_done, 1u) == (unsigned)(ngroups - 1) ? 2 : 0;
+            } else {
+                role = 2;
+            }
+        }
+    }
+    __syncthreads();
+    if (role != 2) return;
+    if (ngroups > 1) {
+        __threadfence();
+        a = total_of_groups<NT, T>(ngroups, [&](int b) {
+            StepVals<T> v;
+            load_part(groups + (long long)PART * b, v);
+            return v;
+        });
+    }
+    if (threadIdx.x != 0) return;
+    advance_ctl(S, to_double(a.s[0]), to_double(a.s[1]), to_double(a.s[2]), a.d2, a.dp2, mode, phase,
+                par, done, nsteps);
+    S.ctl->blocks_done = 0;
+    __threadfence();
+}
+
+// The same tree in a resident run, whose warps store their partials
+// (part_warp): one warp sums group g from its blocks' warps, in the order of
+// block_partial, and later one warp the groups.
+__device__ __forceinline__ double *part_warp(const SpecDev &S, int tile) {
+    return S.part + (long long)PART * tile;
+}
+__device__ __forceinline__ double *part_group(const SpecDev &S, int g) {
+    return S.gpart + (long long)PART * g;
+}
+template <class T>
+__device__ inline void reduce_group(const SpecDev &S, int g) {
+    constexpr int NW = TPB / 32;
+    const int lane = threadIdx.x & 31, blk = g * PART_GROUP + lane;
+    StepVals<T> a = zero_vals<T>(), b[NW];
+    if (blk < S.nblk_pair) {
+#pragma unroll
+        for (int k = 0; k < NW; ++k) load_part(part_warp(S, blk * NW + k), b[k]);
+        a = b[0];
+#pragma unroll
+        for (int k = 1; k < NW; ++k) merge(a, b[k]);
+    }
+    warp_reduce<1>(a);
+    if (lane == 0) store_part(part_group(S, g), a);
+}
+template <class T>
+__device__ inline StepVals<T> reduce_groups(const SpecDev &S) {
+    const int lane = threadIdx.x & 31;
+    const int ngroups = (S.nblk_pair + PART_GROUP - 1) / PART_GROUP;
+    StepVals<T> t = zero_vals<T>();
+    if (ngroups == 1) {
+        if (lane == 0) load_part(part_group(S, 0), t);
+        return t;
+    }
+    for (int b = 0; b < ngroups; b += 32) {
+        StepVals<T> u = zero_vals<T>();
+        if (b + lane < ngroups) load_part(part_group(S, b + lane), u);
+        warp_reduce<1>(u);
+        if (b == 0) t = u;
+        else merge(t, u);
+    }
+    return t;
+}
+
+// four list entries: read once per pass, so they skip L1 (the neighbour
+// records keep the space).  Between kernels (RES false) they come through the
+// read-only path and ask L2 to fetch the 256-byte block around them; inside a
+// resident run lists and records change between its barriers, so both are
+// read with ordinary (coherent after a barrier) loads.
+template <bool RES>
+__device__ __forceinline__ uint4 ld_quad(const uint4 *p) {
+    if (RES) return __ldcg(p);
+    uint4 v;
+    asm("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];"
+        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+        : "l"(p));
+    return v;
+}
+template <bool RES>
+__device__ __forceinline__ int4 ld_rec(const SpecDev &S, const void *rec, unsigned e) {
+    const int4 *p = (const int4 *)((const char *)rec + nl_off(S, e));
+    return RES ? *p : __ldg(p);
+}
+
+// Pruning (both precisions): every lane appends to its near entries, in
+// order, the entries of its far part within the pruning radius (FP32
+// distances of the records against (rc + margin)^2 with slack).  Pairs
+// within rc are therefore all kept, in the order the lane sums them.
+//
+// Bound: the gathers of the far part's records (~118 of the ~252 entries of a
+// bulk atom at the default 2 A skin).
+template <int L, bool RES>
+__device__ __forceinline__ void prune_lane(const SpecDev &S, int u, int l, int par) {
+    const int4 *rec = S.rec[par];
+    const int4 ra = rec[u];
+    const float rp2 = S.f_rp2q;
+    const int2 ab = S.nab[u];
+    const long long col = nl_col(u, l, L, S.capq);
+    const uint4 *p = S.nlist + col;
+    unsigned *dst = (unsigned *)(S.plist + col);
+    const int nl = chk_count(S, ab.y > l ? (ab.y - l + L - 1) / L : 0, S.cap_use);
+    int kept = ab.x / L + (l < ab.x % L);
+    auto test = [&](bool have, unsigned e, const int4 &x) {
+        const float dx = (float)(x.x - ra.x), dy = (float)(x.y - ra.y), dz = (float)(x.z - ra.z);
+        if (fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < rp2 && have) {
+            dst[(kept >> 2) * 128 + (kept & 3)] = e;
+            ++kept;
+        }
+    };
+    uint4 e = ld_quad<RES>(p);
+    for (int q = 0; q < nl; q += 4) {
+        p += 32;
+        const uint4 nx = ld_quad<RES>(p);
+        const int4 x0 = ld_rec<RES>(S, rec, e.x), x1 = ld_rec<RES>(S, rec, e.y);
+        const int4 x2 = ld_rec<RES>(S, rec, e.z), x3 = ld_rec<RES>(S, rec, e.w);
+        test(true, e.x, x0);
+        test(q + 1 < nl, e.y, x1);
+        test(q + 2 < nl, e.z, x2);
+        test(q + 3 < nl, e.w, x3);
+        e = nx;
+    }
+    S.pnn[u * L + l] = kept;
+    if (l == 0) S.pref[u] = ra;
+}
+
+// ---------------------------------------------------------------------------
+// Resident runs.  A table small enough is advanced by one cooperative kernel
+// of one block per SM that stays on the GPU from one list build to the next:
+// every warp keeps its 32 lanes' atoms, and the passes of a step are separated
+// by grid barriers instead of kernel boundaries.  With one launch each for
+// the decision, the two passes and a conditional node, a step of a small
+// specimen spent ~25 us between kernels.
+//
+// The latency of a step is that of its chain of L2 round trips (~0.5 us
+// each), so whatever can is kept on the SM: the atoms' state, own record and
+// density weight in registers, the lists and the descriptors in shared memory
+// (a barrier empties L1), the step count by every block for itself.  What
+// remains is one round of gathers per pass and two barriers.  The sums of a
+// step do not hold up the next one: a service warp in every block, beside
+// those that hold atoms, sums the groups of partials during the next density
+// pass and the groups during the next force pass.  What the next step must
+// know at once, whether an atom has moved far enough for a list build or a
+// pruning, is counted in the barrier's own word.
+//
+// Every wait is bounded: a barrier not reached by all blocks within
+// BARRIER_POLLS polls (seconds) marks the run as stuck and every block
+// returns; the host reports PTA_ECUDA.
+// ---------------------------------------------------------------------------
+constexpr unsigned BARRIER_POLLS = 1u << 22;
+// fields of RunCtl::arrive: arrivals, and how many of them came with a request
+// for a list build, a stop (a specimen failed), a pruning.  At most
+// RUN_STEPS steps per launch keep every field within its bits.
+constexpr int RUN_STEPS = 4000, RUN_BLOCKS = 512;
+constexpr int BAR_BUILD = 22, BAR_STOP = 32, BAR_PRUNE = 42;
+static_assert((2LL * RUN_STEPS + 8) * RUN_BLOCKS < (1LL << BAR_BUILD) &&
+                  RUN_BLOCKS < (1 << (BAR_STOP - BAR_BUILD)) &&
+                  RUN_BLOCKS < (1 << (BAR_PRUNE - BAR_STOP)) &&
+                  (long long)RUN_STEPS * RUN_BLOCKS < (1LL << (64 - BAR_PRUNE)),
+              "fields of the barrier word");
+
+__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long *p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void fence_gpu() {
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+}
+
+// The grid barriers of one block of a cooperative launch; RunCtl::arrive is 0
+// when the launch begins.
+struct GridBarrier {
+    RunCtl *rc;
+    int *req;                  // shared: requests of this block's warps
+    unsigned target = 0;       // thread 0
+    unsigned long long seen = 0;
+
+    // every block has arrived; returns, at the end of a step, the requests
+    // (RunState) that came with it, and RUN_STUCK when the wait ran out
+    __device__ __forceinline__ int sync(bool step) {
+        __shared__ int sh;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const int r = *req;
+            *req = 0;
+            unsigned long long inc = 1;
+            if (r & RUN_BUILD) inc += 1ULL << BAR_BUILD;
+            if (r & RUN_STOP) inc += 1ULL << BAR_STOP;
+            if (r & RUN_PRUNE) inc += 1ULL << BAR_PRUNE;
+            target += gridDim.x;
+            fence_gpu();
+            atomicAdd(&rc->arrive, inc);
+            unsigned polls = 0;
+            unsigned long long v;
+            do {
+                v = ld_relaxed(&rc->arrive);
+            } while ((unsigned)(v & ((1u << BAR_BUILD) - 1)) < target && ++polls < BARRIER_POLLS);
+            int got = 0;
+            if (polls >= BARRIER_POLLS) {
+                atomicExch(&rc->stuck, 1);
+                got = RUN_STUCK;
+            }
+            // requests come with the end of a step: the fields may grow ahead of
+            // this block in the step's first barrier, and stand still here until
+            // it has arrived at the next step's
+            if (step) {
+                const unsigned long long d = (v >> BAR_BUILD) ^ (seen >> BAR_BUILD);
+                seen = v;
+                if (d & ((1ULL << (BAR_STOP - BAR_BUILD)) - 1)) got |= RUN_BUILD;
+                if ((d >> (BAR_STOP - BAR_BUILD)) & ((1ULL << (BAR_PRUNE - BAR_STOP)) - 1))
+                    got |= RUN_STOP;
+                if (d >> (BAR_PRUNE - BAR_BUILD)) got |= RUN_PRUNE;
+            }
+            fence_gpu();
+            sh = got;
+        }
+        __syncthreads();
+        return sh;
+    }
+};
+
+// A block of a resident run: contiguous warp tiles of the table (tile 4 b + k:
+// warp k of pair block b), one per warp, and the service warp behind them.
+// OPS (one precision and lane count): a warp's part of the passes.  Its atoms'
+// positions and velocities stay in registers from the launch to its end.
+constexpr int RESIDENT_SPECS = 4;  // descriptors kept in shared memory
+template <int L, class T, class OPS>
+__device__ __forceinline__ void run_resident(const SpecDev *specs, int nspec, const int *b2s,
+                                             int nblk, RunCtl *rc,
+                                             cudaGraphConditionalHandle again, OPS &ops) {
+    constexpr int NW = TPB / 32, GT = NW * PART_GROUP;  // tiles per group
+    __shared__ SpecDev sh[RESIDENT_SPECS];
+    __shared__ int requests;
+    const int ntile = nblk * NW, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int t0 = (int)((long long)ntile * blockIdx.x / gridDim.x);
+    const int t1 = (int)((long long)ntile * (blockIdx.x + 1) / gridDim.x);
+    const int s0 = b2s[t0 / NW];  // tiles run through the specimens in order
+    for (int k = 0; k < RESIDENT_SPECS && s0 + k < nspec; ++k) {
+        const int *src = (const int *)(specs + s0 + k);
+        for (int i = threadIdx.x; i < (int)(sizeof(SpecDev) / 4); i += blockDim.x)
+            ((int *)&sh[k])[i] = src[i];
+    }
+    if (threadIdx.x == 0) requests = 0;
+    __syncthreads();
+    auto spec = [&](int s) -> const SpecDev & {
+        return s - s0 < RESIDENT_SPECS ? sh[s - s0] : specs[s];
+    };
+    const int tile = t0 + w;
+    const bool has = tile < t1;
+    const bool service = w == (int)(blockDim.x >> 5) - 1;
+    const SpecDev &S = spec(has ? b2s[tile / NW] : s0);
+    const int local = tile - S.blk_pair0 * NW;  // tile of the specimen
+    SpecCtl *c = S.ctl;
+    // the burst as every warp follows it for its own specimen
+    int phase = has ? __ldcg(&c->phase) : (int)PH_IDLE, par = __ldcg(&c->parity);
+    bool prune = phase != PH_IDLE && S.prune_on && __ldcg(&c->prune);
+    long long done = __ldcg(&c->done);
+    const long long nsteps = __ldcg(&c->nsteps);
+    const bool mine = phase != PH_IDLE;
+    if (mine) ops.load(S, local, par);
+    // passes until the last specimen's burst is over
+    long long passes = 0;
+    for (int s = lane; s < nspec; s += 32) {
+        const SpecCtl *q = specs[s].ctl;
+        const int ph = __ldcg(&q->phase);
+        if (ph != PH_IDLE)
+            passes = max(passes, __ldcg(&q->nsteps) - __ldcg(&q->done) + (ph == PH_REFRESH));
+    }
+    const int limit =
+        (int)__reduce_max_sync(0xffffffffu, (unsigned)min(passes, (long long)RUN_STEPS));
+    // service: the groups that begin in this block's tiles, and of those the
+    // ones that begin a specimen, whose sums this block finishes
+    unsigned starts = 0;
+    if (service) {
+        bool first = false;
+        if (t0 + lane < t1)
+            first = (t0 + lane - specs[b2s[(t0 + lane) / NW]].blk_pair0 * NW) % GT == 0;
+        starts = __ballot_sync(0xffffffffu, first);
+    }
+    auto each_start = [&](auto f) {  // f(specimen, its group)
+        for (unsigned m = starts; m; m &= m - 1) {
+            const int t = t0 + __ffs(m) - 1, s = b2s[t / NW];
+            f(s, (t - spec(s).blk_pair0 * NW) / GT);
+        }
+    };
+    // The phase and step count in a specimen's control block are those of the
+    // sums, one step behind the atoms; the service warp that finishes them
+    // keeps them.
+    auto reduce = [&] {
+        each_start([&](int s, int g) {
+            if (__ldcg(&spec(s).ctl->phase) != PH_IDLE) reduce_group<T>(spec(s), g);
+        });
+    };
+    auto finish = [&] {
+        each_start([&](int s, int g) {
+            const SpecDev &D = spec(s);
+            SpecCtl *q = D.ctl;
+            const int ph = __ldcg(&q->phase);
+            if (g != 0 || ph == PH_IDLE) return;
+            const StepVals<T> t = reduce_groups<T>(D);
+            if (lane != 0) return;
+            if (ph == PH_REFRESH) {
+                q->phase = PH_RUN;
+                return;
+            }
+            const double K = to_double(t.s[0]), U = to_double(t.s[1]),
+                         X = to_double(t.s[2]) * D.t_fac;
+            const long long i = __ldcg(&q->done);
+            if (isfinite(K) && isfinite(U) && isfinite(X)) {
+                double *o = D.series + 3 * i;
+                o[0] = K;
+                o[1] = U;
+                o[2] = X;
+                q->done = i + 1;
+                if (i + 1 >= __ldcg(&q->nsteps)) q->phase = PH_IDLE;
+            } else {
+                q->err |= ERR_NAN;
+                q->phase = PH_IDLE;
+                atomicOr(&requests, RUN_STOP);
+            }
+        });
+        __syncwarp();
+    };
+    if (service)
+        each_start([&](int s, int g) {
+            if (g == 0 && lane == 0) {
+                spec(s).ctl->rebuild = 0;  // asked for the build before this launch
+                spec(s).ctl->prune_at = -1;
+            }
+        });
+    GridBarrier bar{rc, &requests};
+    int state = 0, it = 0;
+    bool sums = false;  // a step's partials are waiting
+    for (; it < limit && !(state & (RUN_BUILD | RUN_STUCK)); ++it) {
+        const bool run = phase != PH_IDLE;
+        if (run && prune) {
+            ops.prune(S, par);
+            if (local == 0 && lane == 0) {
+                c->prunes = __ldcg(&c->prunes) + 1;
+                c->prune = 0;
+            }
+        }
+        if (run) ops.density(S, par);
+        if (service && sums) reduce();
+        state = bar.sync(false);
+        if (state & RUN_STUCK) break;
+        if (run) {
+            const StepVals<T> v = ops.force(S, local, par, phase, done, nsteps);
+            if (lane == 0) {
+                int r = 0;
+                if (v.d2 > S.half_skin2q) {
+                    r = RUN_BUILD;
+                    c->rebuild = 1;
+                }
+                if (S.prune_on && v.dp2 > S.half_prune2q) {
+                    r |= RUN_PRUNE;
+                    c->prune_at = it;
+                }
+                if (r) atomicOr(&requests, r);
+            }
+            par ^= 1;
+            done += phase == PH_RUN;
+            phase = done < nsteps ? PH_RUN : PH_IDLE;
+        }
+        if (service && sums) finish();
+        sums = true;
+        state = bar.sync(true);
+        // of several specimens, which one asked?
+        prune = (state & RUN_PRUNE) && S.prune_on && (nspec == 1 || __ldcg(&c->prune_at) == it);
+        if (state & RUN_STOP) {
+            if (nspec == 1) break;
+            if (__ldcg(&c->phase) == PH_IDLE) phase = PH_IDLE;
+        }
+    }
+    // the last step's sums
+    if (!(state & RUN_STUCK) && it > 0) {
+        if (service) reduce();
+        state |= bar.sync(false) & RUN_STUCK;
+        if (service) finish();
+    }
+    if (mine) {
+        ops.store(S, par);
+        if (local == 0 && lane == 0) {
+            c->parity = par;
+            if (prune) c->prune = 1;
+        }
+    }
+    state |= bar.sync(false) & RUN_STUCK;
+    if (blockIdx.x == 0 && w == 0) {
+        int active = 0;
+        for (int s = lane; s < nspec; s += 32) active |= __ldcg(&specs[s].ctl->phase) != PH_IDLE;
+        active = __any_sync(0xffffffffu, active);
+        if (lane == 0) cudaGraphSetConditional(again, active && !(state & RUN_STUCK) ? 1u : 0u);
+    }
+}
+
+// f(entry) for the entries of a lane's column whose first `cached` quads lie
+// in shared memory
+struct LaneList {
+    const uint4 *p;    // column in memory
+    const uint4 *sh;   // this thread's column in shared memory
+    int cnt, cached;
+    __device__ __forceinline__ void fill(const SpecDev &S, uint4 *cache, int u, int l, int L,
+                                         int quads) {
+        p = S.plist + nl_col(u, l, L, S.capq);
+        cnt = chk_count(S, __ldcg(S.pnn + u * L + l), 4 * (S.capq - 1));
+        cached = min((cnt + 3) >> 2, quads);
+        uint4 *own = cache + (threadIdx.x >> 5) * quads * 32 + (threadIdx.x & 31);
+        sh = own;
+        for (int t = 0; t < cached; ++t) own[t * 32] = __ldcg(p + t * 32);
+    }
+    __device__ __forceinline__ uint4 quad(int t) const {
+        return t < cached ? sh[t * 32] : __ldcg(p + t * 32);
+    }
+};
+
+// The launch shape of a resident run of nblk pair blocks: one block per SM, a
+// warp per tile, as many quads of the lists in shared memory as it holds (up
+// to the ~150 entries of a bulk atom).
+struct RunShape {
+    int blocks = 0, threads = 0, quads = 0;
+    size_t smem = 0;
+};
+inline RunShape run_shape(int nblk, int L, int max_warps) {
+    RunShape r;
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return r;
+    }
+    nsm = std::min(nsm, RUN_BLOCKS);
+    const int tiles = nblk * (TPB / 32);
+    const int warps = (tiles + nsm - 1) / std::max(nsm, 1) + 1;  // and the service warp
+    if (nsm < 1 || warps > max_warps) return r;
+    r.blocks = std::min(nsm, tiles);
+    r.threads = 32 * warps;
+    r.quads = std::min(40 / L + 2, 160 * 1024 / (r.threads * 16));
+    r.smem = (size_t)r.quads * r.threads * 16;
+    return r;
+}
+template <class K>
+bool run_fits(K kernel, const RunShape &r) {
+    int per = 0;
+    if (r.blocks < 1) return false;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, r.threads, r.smem) !=
+            cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return per >= 1;
+}
+template <class K, class... A>
+cudaError_t launch_cooperative(K kernel, const RunShape &r, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.dynamicSmemBytes = r.smem;
+    cfg.gridDim = dim3((unsigned)r.blocks);
+    cfg.blockDim = dim3((unsigned)r.threads);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 }  // namespace pta

@@ -16,19 +16,6 @@
 
 namespace pta {
 
-// four list entries: read once per pass, so they skip L1 (the neighbour
-// records keep the space) and ask L2 to fetch the 256-byte block around them
-__device__ __forceinline__ uint4 ld_quad(const uint4 *p) {
-    uint4 v;
-    asm("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];"
-        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-        : "l"(p));
-    return v;
-}
-__device__ __forceinline__ int4 ld_rec(const SpecDev &S, const void *rec, unsigned e) {
-    return __ldg((const int4 *)((const char *)rec + nl_off(S, e)));
-}
-
 // f(record) for the entries lane l of atom u reads, in list order: a quad per
 // iteration (four gathers in flight), the next quad read ahead, then what is
 // left of the last one
@@ -37,12 +24,12 @@ __device__ __forceinline__ void for_entries(const SpecDev &S, const void *rec, i
                                             F f) {
     const uint4 *p = S.plist + nl_col(u, l, L, S.capq);
     const int cnt = chk_count(S, S.pnn[u * L + l], 4 * (S.capq - 1));
-    uint4 e = ld_quad(p);
+    uint4 e = ld_quad<false>(p);
     for (int t = cnt >> 2; t > 0; --t) {
         p += 32;
-        const uint4 nx = ld_quad(p);
-        const int4 x0 = ld_rec(S, rec, e.x), x1 = ld_rec(S, rec, e.y);
-        const int4 x2 = ld_rec(S, rec, e.z), x3 = ld_rec(S, rec, e.w);
+        const uint4 nx = ld_quad<false>(p);
+        const int4 x0 = ld_rec<false>(S, rec, e.x), x1 = ld_rec<false>(S, rec, e.y);
+        const int4 x2 = ld_rec<false>(S, rec, e.z), x3 = ld_rec<false>(S, rec, e.w);
         f(x0);
         f(x1);
         f(x2);
@@ -51,13 +38,65 @@ __device__ __forceinline__ void for_entries(const SpecDev &S, const void *rec, i
     }
     const int left = cnt & 3;
     if (left) {
-        int4 x0 = ld_rec(S, rec, e.x), x1 = x0, x2 = x0;
-        if (left > 1) x1 = ld_rec(S, rec, e.y);
-        if (left > 2) x2 = ld_rec(S, rec, e.z);
+        int4 x0 = ld_rec<false>(S, rec, e.x), x1 = x0, x2 = x0;
+        if (left > 1) x1 = ld_rec<false>(S, rec, e.y);
+        if (left > 2) x2 = ld_rec<false>(S, rec, e.z);
         f(x0);
         if (left > 1) f(x1);
         if (left > 2) f(x2);
     }
+}
+
+// the same in a resident run, from the list in shared memory: twelve gathers
+// in flight (a barrier has emptied L1, so they come from L2; at 16 lanes per
+// atom that is the whole list in one round)
+template <class F>
+__device__ __forceinline__ void for_entries(const SpecDev &S, const void *rec, const LaneList &q,
+                                            F f) {
+    for (int t = 0, left = q.cnt; left > 0; left -= 12, t += 3) {
+        int4 x[12];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            if (left <= 4 * k) break;
+            const uint4 e = q.quad(t + k);
+            x[4 * k] = ld_rec<true>(S, rec, e.x);
+            if (left > 4 * k + 1) x[4 * k + 1] = ld_rec<true>(S, rec, e.y);
+            if (left > 4 * k + 2) x[4 * k + 2] = ld_rec<true>(S, rec, e.z);
+            if (left > 4 * k + 3) x[4 * k + 3] = ld_rec<true>(S, rec, e.w);
+        }
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            if (left <= k) break;
+            f(x[k]);
+        }
+    }
+}
+
+// the density weight w of atom u from its lanes' sums, stored in its record;
+// its energy
+template <int L, bool SC76>
+__device__ __forceinline__ float density_end(const SpecDev &S, const PotF &P, int u, bool first,
+                                             const int4 &ra, RhoSums s, float &w) {
+    s.sm = lane_sum<L>(s.sm);
+    s.sn = lane_sum<L>(s.sn);
+    s.sr = lane_sum<L>(s.sr);
+    const float cnt = (float)lane_sum<L>(s.cnt);
+    const float dr = fmaf(-cnt, P.rc, s.sr);  // sum of r - rc
+    const float rho = SC76 ? fmaf(P.am, s.sm, fmaf(P.Bm, dr, __fmul_rn(-cnt, P.Am))) : s.sm;
+    const float phn = fmaf(P.an, s.sn, fmaf(P.Bn, dr, __fmul_rn(-cnt, P.An)));
+    // w = m a^m B'(rho), B'(rho) = -eps c / (2 sqrt(rho))
+    const float rq = rho > 0.f ? rsqrtf(rho) : 0.f;
+    w = __fmul_rn(P.fpsc, rq);
+    if (first) ((int4 *)S.posfp)[u] = make_int4(ra.x, ra.y, ra.z, __float_as_int(w));
+    // the atom's energy 1/2 eps sum_j phi_n + B(rho), B = -eps c sqrt(rho)
+    return fmaf(-P.ec, rho > 0.f ? __fmul_rn(rho, rq) : 0.f, __fmul_rn(0.5f * P.eps, phn));
+}
+
+// sums of (eV/A^2) x quanta over an atom's lanes, in eV/A
+template <int L>
+__device__ __forceinline__ void force_end(const SpecDev &S, float f[3]) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) f[d] = __fmul_rn(lane_sum<L>(f[d]), S.f_q);
 }
 
 template <int L, bool SC76>
@@ -74,21 +113,9 @@ __device__ __forceinline__ void density_block(const SpecDev &S, int lb, int par,
         for_entries(S, S.rec[par], u, l, L,
                     [&](const int4 &x) { rho_pair<SC76>(P, q2, ra, x, s); });
     }
-    s.sm = lane_sum<L>(s.sm);
-    s.sn = lane_sum<L>(s.sn);
-    s.sr = lane_sum<L>(s.sr);
-    const float cnt = (float)lane_sum<L>(s.cnt);
-    if (valid && l == 0) {
-        const float dr = fmaf(-cnt, P.rc, s.sr);  // sum of r - rc
-        const float rho = SC76 ? fmaf(P.am, s.sm, fmaf(P.Bm, dr, -cnt * P.Am)) : s.sm;
-        const float phn = fmaf(P.an, s.sn, fmaf(P.Bn, dr, -cnt * P.An));
-        // w = m a^m B'(rho), B'(rho) = -eps c / (2 sqrt(rho))
-        const float rq = rho > 0.f ? rsqrtf(rho) : 0.f;
-        const float w = P.fpsc * rq;
-        // the atom's energy 1/2 eps sum_j phi_n + B(rho), B = -eps c sqrt(rho)
-        ((float *)S.pen)[u] = fmaf(-P.ec, rho > 0.f ? rho * rq : 0.f, 0.5f * P.eps * phn);
-        ((int4 *)S.posfp)[u] = make_int4(ra.x, ra.y, ra.z, __float_as_int(w));
-    }
+    float w;
+    const float pe = density_end<L, SC76>(S, P, u, valid && l == 0, ra, s, w);
+    if (valid && l == 0) ((float *)S.pen)[u] = pe;
 }
 
 template <int L, bool SC76>
@@ -99,30 +126,24 @@ __device__ __forceinline__ void force_block(const SpecDev &S, int lb, int par, c
     const int u = lb * UPB + threadIdx.x / L;
     const int l = threadIdx.x % L;
     const bool valid = u < S.n;
-    float fx = 0.f, fy = 0.f, fz = 0.f, wa = 0.f;
+    float f[3] = {0.f, 0.f, 0.f};
     if (valid) {
         const int4 ra = ((const int4 *)S.posfp)[u];
-        wa = __int_as_float(ra.w);
+        const float wa = __int_as_float(ra.w);
         const float q2 = S.f_q2;
         for_entries(S, S.posfp, u, l, L,
-                    [&](const int4 &x) { force_pair<SC76>(P, q2, ra, wa, x, fx, fy, fz); });
+                    [&](const int4 &x) { force_pair<SC76>(P, q2, ra, wa, x, f[0], f[1], f[2]); });
     }
-    // sums of (eV/A^2) x quanta
-    fx = lane_sum<L>(fx) * S.f_q;
-    fy = lane_sum<L>(fy) * S.f_q;
-    fz = lane_sum<L>(fz) * S.f_q;
-    double ke = 0.0, pe = 0.0, rr = 0.0;
-    float d2 = 0.f, dp2 = 0.f;
-    if (valid && l == 0)
-        atom_update_mixed(S, S.ctl, par, u, S.prune_on != 0, fx, fy, fz, mode, phase, done, nsteps,
-                          ke, pe, rr, d2, dp2);
-    ke = warp_sum(ke);
-    pe = warp_sum(pe);
-    rr = warp_sum(rr);
-    d2 = warp_max(d2);
-    dp2 = warp_max(dp2);
-    step_tail<TPB>(S, lb, S.nblk_pair, ke, pe, rr, (double)d2, (double)dp2, mode, phase, done,
-                   nsteps);
+    force_end<L>(S, f);
+    StepVals<FF> v = zero_vals<FF>();
+    if (valid && l == 0) {
+        AtomMixed A;
+        A.load(S, par, u);
+        atom_update_mixed(S, A, par, u, f, ((const float *)S.pen)[u], mode, phase, done, nsteps, v);
+        if (mode != MODE_EVAL) A.store(S, par ^ 1, u);
+    }
+    warp_reduce<L>(v);
+    step_tail<TPB>(S, lb, S.nblk_pair, v, mode, phase, par, done, nsteps);
 }
 
 template <int L, bool SC76>
@@ -146,62 +167,89 @@ __global__ void __launch_bounds__(TPB, 8) k_force_f32(const SpecDev *__restrict_
                          ctl->nsteps);
 }
 
-// Pruning (both precisions): every lane appends to the near part of its
-// column, in order, the entries of its far part within the pruning radius
-// (FP32 distances of the records against (rc + margin)^2 with slack).  Pairs
-// within rc are therefore all kept, in the order the lane sums them.
-//
-// Bound: the gathers of the far part's records (~118 of the ~252 entries of a
-// bulk atom at the default 2 A skin).
+template <int L, bool SC76>
+struct OpsF32 {
+    const PotF &P;
+    uint4 *cache;
+    int quads;
+    AtomMixed A;
+    LaneList q;
+    int4 ra;         // the atom's record (all its lanes)
+    float wa, pe;    // its density weight and energy
+    int u, l;
+    bool valid;
+    __device__ __forceinline__ void load(const SpecDev &S, int tile, int par) {
+        const int t = tile * 32 + (threadIdx.x & 31);
+        u = t / L;
+        l = t % L;
+        valid = u < S.n;
+        ra = make_int4(0, 0, 0, 0);
+        wa = pe = 0.f;
+        if (valid) {
+            q.fill(S, cache, u, l, L, quads);
+            ra = S.rec[par][u];
+            if (l == 0) A.load(S, par, u);
+        }
+    }
+    __device__ __forceinline__ void prune(const SpecDev &S, int par) {
+        if (!valid) return;
+        prune_lane<L, true>(S, u, l, par);
+        q.fill(S, cache, u, l, L, quads);
+        A.pref = ra;
+    }
+    __device__ __forceinline__ void store(const SpecDev &S, int par) const {
+        if (valid && l == 0) A.store(S, par, u);
+    }
+    __device__ __forceinline__ void density(const SpecDev &S, int par) {
+        RhoSums s;
+        if (valid) {
+            const float q2 = S.f_q2;
+            for_entries(S, S.rec[par], q,
+                        [&](const int4 &x) { rho_pair<SC76>(P, q2, ra, x, s); });
+        }
+        pe = density_end<L, SC76>(S, P, u, valid && l == 0, ra, s, wa);
+    }
+    __device__ __forceinline__ StepVals<FF> force(const SpecDev &S, int tile, int par, int phase,
+                                                  long long done, long long nsteps) {
+        float f[3] = {0.f, 0.f, 0.f};
+        if (valid) {
+            const float q2 = S.f_q2;
+            for_entries(S, S.posfp, q, [&](const int4 &x) {
+                force_pair<SC76>(P, q2, ra, wa, x, f[0], f[1], f[2]);
+            });
+        }
+        force_end<L>(S, f);
+        StepVals<FF> v = zero_vals<FF>();
+        if (valid && l == 0)
+            ra = atom_update_mixed(S, A, par, u, f, pe, MODE_STEP, phase, done, nsteps, v);
+        if (L > 1) {  // the new record to the atom's other lanes
+            const int src = (threadIdx.x & 31) & ~(L - 1);
+            ra.x = __shfl_sync(0xffffffffu, ra.x, src);
+            ra.y = __shfl_sync(0xffffffffu, ra.y, src);
+            ra.z = __shfl_sync(0xffffffffu, ra.z, src);
+        }
+        warp_reduce<L>(v);
+        if ((threadIdx.x & 31) == 0) store_part(part_warp(S, tile), v);
+        return v;
+    }
+};
+constexpr int RUN_WARPS_F32 = 16;
+template <int L, bool SC76>
+__global__ void __launch_bounds__(32 * RUN_WARPS_F32, 1)
+    k_run_f32(const SpecDev *specs, int nspec, const int *b2s, int nblk, RunCtl *rc,
+              cudaGraphConditionalHandle again, int quads, const PotF P) {
+    extern __shared__ uint4 list_cache[];
+    OpsF32<L, SC76> ops{P, list_cache, quads};
+    run_resident<L, FF>(specs, nspec, b2s, nblk, rc, again, ops);
+}
+
 template <int L>
 __global__ void __launch_bounds__(TPB, 8) k_prune(const SpecDev *__restrict__ specs,
                                                   const int *__restrict__ b2s, int force) {
     const SpecDev &S = specs[b2s[blockIdx.x]];
     if (!prune_active(S, force)) return;
-    const int par = S.ctl->parity;
-    constexpr int UPB = TPB / L;
-    const int u = (blockIdx.x - S.blk_pair0) * UPB + threadIdx.x / L;
-    const int l = threadIdx.x % L;
-    if (u >= S.n) return;
-    const int4 *rec = S.rec[par];
-    const int4 ra = rec[u];
-    const float rp2 = S.f_rp2q;
-    const int2 ab = S.nab[u];
-    const long long col = nl_col(u, l, L, S.capq);
-    const uint4 *p = S.nlist + col;
-    unsigned *dst = (unsigned *)(S.plist + col);
-    const int nl = chk_count(S, ab.y > l ? (ab.y - l + L - 1) / L : 0, S.cap_use);
-    int kept = ab.x / L + (l < ab.x % L);
-    auto test = [&](bool have, unsigned e, const int4 &x) {
-        const float dx = (float)(x.x - ra.x), dy = (float)(x.y - ra.y), dz = (float)(x.z - ra.z);
-        if (fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < rp2 && have) {
-            dst[(kept >> 2) * 128 + (kept & 3)] = e;
-            ++kept;
-        }
-    };
-    uint4 e = ld_quad(p);
-    for (int q = 0; q < nl; q += 4) {
-        p += 32;
-        const uint4 nx = ld_quad(p);
-        const int4 x0 = ld_rec(S, rec, e.x), x1 = ld_rec(S, rec, e.y);
-        const int4 x2 = ld_rec(S, rec, e.z), x3 = ld_rec(S, rec, e.w);
-        test(true, e.x, x0);
-        test(q + 1 < nl, e.y, x1);
-        test(q + 2 < nl, e.z, x2);
-        test(q + 3 < nl, e.w, x3);
-        e = nx;
-    }
-    S.pnn[u * L + l] = kept;
-    if (l == 0) {
-        if (S.prec == PTA_PREC_FP64) {
-            const double4_32a x = ((const double4_32a *)S.pos[par])[u];
-            S.pref[u] = make_float4((float)x.x, (float)x.y, (float)x.z, 0.f);
-        } else {
-            const float4 hi = ((const float4 *)S.pos[par])[u];
-            const float4 lo = S.lo[par][u];
-            S.pref[u] = make_float4(hi.x + lo.x, hi.y + lo.y, hi.z + lo.z, 0.f);
-        }
-    }
+    const int u = (blockIdx.x - S.blk_pair0) * (TPB / L) + threadIdx.x / L;
+    if (u < S.n) prune_lane<L, false>(S, u, threadIdx.x % L, S.ctl->parity);
 }
 
 // after the pruning: clear the flag (a separate kernel, so that every block
@@ -269,6 +317,50 @@ void launch_force(const Tab &t, int arg, cudaStream_t st) {
         else
             PTA_L_SWITCH(k_force_f32, false)
     }
+}
+
+// resident runs
+cudaError_t launch_run_f64(const Tab &t, const Group &g, RunCtl *rc,
+                           cudaGraphConditionalHandle again, cudaStream_t st);
+bool run_possible_f64(const Group &g);
+
+#define PTA_RUN_SWITCH(SC, DO)     \
+    switch (g.L) {                 \
+        case 1: DO(1, SC); break;  \
+        case 2: DO(2, SC); break;  \
+        case 4: DO(4, SC); break;  \
+        case 8: DO(8, SC); break;  \
+        default: DO(16, SC);       \
+    }
+
+bool run_possible(const Group &g) {
+    if (g.prec == PTA_PREC_FP64) return run_possible_f64(g);
+    const RunShape r = run_shape(g.nblk, g.L, RUN_WARPS_F32);
+    bool ok = false;
+#define DO(L, SC) ok = run_fits(k_run_f32<L, SC>, r)
+    if (g.sc76)
+        PTA_RUN_SWITCH(true, DO)
+    else
+        PTA_RUN_SWITCH(false, DO)
+#undef DO
+    return ok;
+}
+
+cudaError_t launch_run(const Tab &t, RunCtl *rc, cudaGraphConditionalHandle again,
+                       cudaStream_t st) {
+    const Group &g = t.grp[0];
+    if (g.prec == PTA_PREC_FP64) return launch_run_f64(t, g, rc, again, st);
+    const RunShape r = run_shape(g.nblk, g.L, RUN_WARPS_F32);
+    cudaError_t e = cudaSuccess;
+#define DO(L, SC)                                                                              \
+    e = launch_cooperative(k_run_f32<L, SC>, r, st, t.specs, t.nspec, g.b2s, g.nblk, rc, again, \
+                           r.quads, g.pf)
+    if (g.sc76)
+        PTA_RUN_SWITCH(true, DO)
+    else
+        PTA_RUN_SWITCH(false, DO)
+#undef DO
+    return e;
 }
 
 }  // namespace pta

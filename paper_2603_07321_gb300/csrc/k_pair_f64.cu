@@ -73,6 +73,14 @@ __device__ __forceinline__ double force_pair64(const PotDev &P, double r2, doubl
     return fma(y, c, -v);
 }
 
+template <bool RES>
+__device__ __forceinline__ double4_32a ld_pos64(const SpecDev &S, const double4_32a *pos, unsigned e) {
+    const double4_32a *p = pos + nl_j(nl_off(S, e));
+    if (RES) return *p;
+    // the read-only path, two 16-byte loads
+    const double2 a = __ldg((const double2 *)p), b = __ldg((const double2 *)p + 1);
+    return make_double4_32a(a.x, a.y, b.x, b.y);
+}
 // f(position) for the entries lane l of atom a reads, in list order (list
 // entries are byte offsets of 16-byte records, half of a double4's)
 template <class F>
@@ -80,12 +88,12 @@ __device__ __forceinline__ void for_entries64(const SpecDev &S, const double4_32
                                               int l, int L, F f) {
     const uint4 *p = S.plist + nl_col(a, l, L, S.capq);
     const int cnt = chk_count(S, S.pnn[a * L + l], 4 * (S.capq - 1));
-    uint4 e = __ldg(p);
+    uint4 e = ld_quad<false>(p);
     for (int t = cnt >> 2; t > 0; --t) {
         p += 32;
-        const uint4 nx = __ldg(p);
-        const double4_32a x0 = pos[nl_j(nl_off(S, e.x))], x1 = pos[nl_j(nl_off(S, e.y))];
-        const double4_32a x2 = pos[nl_j(nl_off(S, e.z))], x3 = pos[nl_j(nl_off(S, e.w))];
+        const uint4 nx = ld_quad<false>(p);
+        const double4_32a x0 = ld_pos64<false>(S, pos, e.x), x1 = ld_pos64<false>(S, pos, e.y);
+        const double4_32a x2 = ld_pos64<false>(S, pos, e.z), x3 = ld_pos64<false>(S, pos, e.w);
         f(x0);
         f(x1);
         f(x2);
@@ -93,161 +101,287 @@ __device__ __forceinline__ void for_entries64(const SpecDev &S, const double4_32
         e = nx;
     }
     const int left = cnt & 3;
-    if (left > 0) f(pos[nl_j(nl_off(S, e.x))]);
-    if (left > 1) f(pos[nl_j(nl_off(S, e.y))]);
-    if (left > 2) f(pos[nl_j(nl_off(S, e.z))]);
+    if (left > 0) f(ld_pos64<false>(S, pos, e.x));
+    if (left > 1) f(ld_pos64<false>(S, pos, e.y));
+    if (left > 2) f(ld_pos64<false>(S, pos, e.z));
+}
+
+// the same in a resident run, from the list in shared memory
+template <class F>
+__device__ __forceinline__ void for_entries64(const SpecDev &S, const double4_32a *pos,
+                                              const LaneList &q, F f) {
+    int t = 0, left = q.cnt;
+    for (; left >= 4; left -= 4, ++t) {
+        const uint4 e = q.quad(t);
+        const double4_32a x0 = ld_pos64<true>(S, pos, e.x), x1 = ld_pos64<true>(S, pos, e.y);
+        const double4_32a x2 = ld_pos64<true>(S, pos, e.z), x3 = ld_pos64<true>(S, pos, e.w);
+        f(x0);
+        f(x1);
+        f(x2);
+        f(x3);
+    }
+    if (left > 0) {
+        const uint4 e = q.quad(t);
+        f(ld_pos64<true>(S, pos, e.x));
+        if (left > 1) f(ld_pos64<true>(S, pos, e.y));
+        if (left > 2) f(ld_pos64<true>(S, pos, e.z));
+    }
+}
+
+// An atom's state outside the neighbour records.
+struct Atom64 {
+    double x[3], v[3];
+    int4 ref, pref;
+    int flag;
+    __device__ __forceinline__ void load(const SpecDev &S, int par, int a) {
+        const double4_32a q = ((const double4_32a *)S.pos[par])[a];
+        const double4_32a w = ((const double4_32a *)S.vel)[a];
+        x[0] = q.x; x[1] = q.y; x[2] = q.z;
+        v[0] = w.x; v[1] = w.y; v[2] = w.z;
+        ref = S.ref[a];
+        pref = S.prune_on ? S.pref[a] : ref;
+        flag = S.flags[a];
+    }
+    // the position goes to buffer par with every step (neighbours read it)
+    __device__ __forceinline__ void store_pos(const SpecDev &S, int par, int a) const {
+        ((double4_32a *)S.pos[par])[a] = make_double4_32a(x[0], x[1], x[2], 0.0);
+    }
+    __device__ __forceinline__ void store_vel(const SpecDev &S, int a) const {
+        ((double4_32a *)S.vel)[a] = make_double4_32a(v[0], v[1], v[2], 0.0);
+    }
+};
+
+// After the force pass of atom a (force f, energy pe): as atom_update_mixed,
+// in FP64; the new position and record go to the other buffers.
+__device__ __forceinline__ void atom_update64(const SpecDev &S, Atom64 &A, int par, int a,
+                                              const double f[3], double pe, int mode, int phase,
+                                              long long done, long long nsteps,
+                                              StepVals<double> &out) {
+    chk_force(S, f[0], f[1], f[2]);
+    const SpecCtl *ctl = S.ctl;
+    out.s[1] = pe;
+    if (A.flag == FLAG_RIGHT) out.s[2] = -(S.axis == 0 ? f[0] : (S.axis == 1 ? f[1] : f[2]));
+    auto kinetic = [&] {
+        out.s[0] = __dmul_rn(
+            S.ke_fac, fma(A.v[2], A.v[2], fma(A.v[1], A.v[1], __dmul_rn(A.v[0], A.v[0]))));
+    };
+    if (mode == MODE_EVAL) {
+        kinetic();
+        ((double4_32a *)S.eval_out)[S.orig[a]] = make_double4_32a(f[0], f[1], f[2], pe);
+        return;
+    }
+    const double kh = S.acc_half;
+    // thermal relaxation: the right grip moves along the load axis only
+    const bool rfree = A.flag == FLAG_RIGHT && ctl->relax;
+    auto kick = [&] {
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            if (A.flag == FLAG_MOBILE || (rfree && S.axis == d)) A.v[d] = fma(f[d], kh, A.v[d]);
+    };
+    if (phase == PH_RUN) {
+        kick();
+        kinetic();
+        if (S.rsum) {
+            // Eq. (mean_pos): the sampled state's position
+            double *rs = S.rsum + 4LL * S.orig[a];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) rs[d] = rs[d] + A.x[d];
+        }
+    }
+    const bool start = (phase == PH_REFRESH) || (done + 1 < nsteps);
+    if (start && (A.flag == FLAG_MOBILE || rfree)) {
+        kick();
+#pragma unroll
+        for (int d = 0; d < 3; ++d) A.x[d] = fma(A.v[d], S.dt, A.x[d]);
+    } else if (start && A.flag == FLAG_RIGHT && ctl->grip_du != 0.0) {
+        // continuous loading (fine-dynamics verification)
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            A.x[d] = __dadd_rn(A.x[d], S.axis == d ? ctl->grip_du : 0.0);
+    }
+    A.store_pos(S, par ^ 1, a);
+    const int4 r = rec_fp64(S, A.x[0], A.x[1], A.x[2]);
+    S.rec[par ^ 1][a] = r;
+    out.d2 = moved2(r, A.ref);
+    out.dp2 = moved2(r, A.pref);
+}
+
+template <int L>
+__device__ __forceinline__ double density_end64(const SpecDev &S, int a, bool first,
+                                                const double4_32a &pa, RhoSums64 s, double &w) {
+    const PotDev &P = S.pot;
+    s.sm = lane_sum<L>(s.sm);
+    s.sn = lane_sum<L>(s.sn);
+    s.sr = lane_sum<L>(s.sr);
+    const double cnt = (double)lane_sum<L>(s.cnt);
+    const double dr = fma(-cnt, P.rc, s.sr);  // sum of r - rc
+    const double rho = fma(P.am, s.sm, fma(P.Bm, dr, __dmul_rn(-cnt, P.Am)));
+    const double phn = fma(P.an, s.sn, fma(P.Bn, dr, __dmul_rn(-cnt, P.An)));
+    // w = m a^m B'(rho), B'(rho) = -eps c / (2 sqrt(rho))
+    const double sq = rho > 0.0 ? sqrt(rho) : 0.0;
+    w = rho > 0.0 ? P.fpsc / sq : 0.0;
+    if (first) ((double4_32a *)S.posfp)[a] = make_double4_32a(pa.x, pa.y, pa.z, w);
+    // the atom's energy 1/2 eps sum_j phi_n + B(rho), B = -eps c sqrt(rho)
+    return fma(-P.ec, sq, __dmul_rn(0.5 * P.eps, phn));
+}
+
+template <bool SC76>
+__device__ __forceinline__ void force_entry64(const PotDev &P, const double4_32a &pa,
+                                              const double4_32a &pj, double f[3]) {
+    double dx, dy, dz;
+    const double r2 = pair_r2(pa, pj, dx, dy, dz);
+    if (within(r2, P.rc2)) {
+        const double g = force_pair64<SC76>(P, r2, __dadd_rn(pa.w, pj.w));
+        f[0] = fma(g, dx, f[0]);
+        f[1] = fma(g, dy, f[1]);
+        f[2] = fma(g, dz, f[2]);
+    }
+}
+template <bool SC76>
+__device__ __forceinline__ void rho_entry64(const PotDev &P, const double4_32a &pa,
+                                            const double4_32a &pj, RhoSums64 &s) {
+    double dx, dy, dz;
+    const double r2 = pair_r2(pa, pj, dx, dy, dz);
+    if (within(r2, P.rc2)) rho_pair64<SC76>(P, r2, s);
+}
+
+template <int L, bool SC76>
+__device__ __forceinline__ void density_block64(const SpecDev &S, int lb, int par) {
+    const int a = lb * (TPB / L) + threadIdx.x / L;
+    const int l = threadIdx.x % L;
+    const bool valid = a < S.n;
+    const double4_32a *pos = (const double4_32a *)S.pos[par];
+    RhoSums64 s;
+    double4_32a pa = make_double4_32a(0, 0, 0, 0);
+    if (valid) {
+        pa = pos[a];
+        for_entries64(S, pos, a, l, L,
+                      [&](const double4_32a &pj) { rho_entry64<SC76>(S.pot, pa, pj, s); });
+    }
+    double w;
+    const double pe = density_end64<L>(S, a, valid && l == 0, pa, s, w);
+    if (valid && l == 0) ((double *)S.pen)[a] = pe;
+}
+
+template <int L, bool SC76>
+__device__ __forceinline__ void force_block64(const SpecDev &S, int lb, int par, int mode, int phase,
+                                              long long done, long long nsteps) {
+    const int a = lb * (TPB / L) + threadIdx.x / L;
+    const int l = threadIdx.x % L;
+    const bool valid = a < S.n;
+    double f[3] = {0, 0, 0};
+    if (valid) {
+        const double4_32a *pf = (const double4_32a *)S.posfp;
+        const double4_32a pa = pf[a];
+        for_entries64(S, pf, a, l, L,
+                      [&](const double4_32a &pj) { force_entry64<SC76>(S.pot, pa, pj, f); });
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) f[d] = lane_sum<L>(f[d]);
+    StepVals<double> v = zero_vals<double>();
+    if (valid && l == 0) {
+        Atom64 A;
+        A.load(S, par, a);
+        atom_update64(S, A, par, a, f, ((const double *)S.pen)[a], mode, phase, done, nsteps, v);
+        if (mode != MODE_EVAL) A.store_vel(S, a);
+    }
+    warp_reduce<L>(v);
+    step_tail<TPB>(S, lb, S.nblk_pair, v, mode, phase, par, done, nsteps);
 }
 
 template <int L, bool SC76>
 __global__ void __launch_bounds__(TPB) k_density_f64(const SpecDev *__restrict__ specs,
                                                      const int *__restrict__ b2s, int force) {
     const SpecDev &S = specs[b2s[blockIdx.x]];
-    const SpecCtl *ctl = S.ctl;
-    if (!force && ctl->phase == PH_IDLE) return;
-    const int par = ctl->parity;
-    constexpr int APB = TPB / L;
-    const int a = (blockIdx.x - S.blk_pair0) * APB + threadIdx.x / L;
-    const int l = threadIdx.x % L;
-    const bool valid = a < S.n;
-    const double4_32a *__restrict__ pos = (const double4_32a *)S.pos[par];
-    const PotDev &P = S.pot;
-    RhoSums64 s;
-    double4_32a pa = make_double4_32a(0, 0, 0, 0);
-    if (valid) {
-        pa = pos[a];
-        for_entries64(S, pos, a, l, L, [&](const double4_32a &pj) {
-            double dx, dy, dz;
-            const double r2 = pair_r2(pa, pj, dx, dy, dz);
-            if (within(r2, P.rc2)) rho_pair64<SC76>(P, r2, s);
-        });
-    }
-    s.sm = lane_sum<L>(s.sm);
-    s.sn = lane_sum<L>(s.sn);
-    s.sr = lane_sum<L>(s.sr);
-    const double cnt = (double)lane_sum<L>(s.cnt);
-    if (valid && l == 0) {
-        const double dr = fma(-cnt, P.rc, s.sr);  // sum of r - rc
-        const double rho = fma(P.am, s.sm, fma(P.Bm, dr, __dmul_rn(-cnt, P.Am)));
-        const double phn = fma(P.an, s.sn, fma(P.Bn, dr, __dmul_rn(-cnt, P.An)));
-        // w = m a^m B'(rho), B'(rho) = -eps c / (2 sqrt(rho))
-        const double sq = rho > 0.0 ? sqrt(rho) : 0.0;
-        const double w = rho > 0.0 ? P.fpsc / sq : 0.0;
-        // the atom's energy 1/2 eps sum_j phi_n + B(rho), B = -eps c sqrt(rho)
-        ((double *)S.pen)[a] = fma(-P.ec, sq, __dmul_rn(0.5 * P.eps, phn));
-        ((double4_32a *)S.posfp)[a] = make_double4_32a(pa.x, pa.y, pa.z, w);
-    }
+    if (!force && S.ctl->phase == PH_IDLE) return;
+    density_block64<L, SC76>(S, blockIdx.x - S.blk_pair0, S.ctl->parity);
 }
 
 template <int L, bool SC76>
 __global__ void __launch_bounds__(TPB) k_force_f64(const SpecDev *__restrict__ specs,
                                                    const int *__restrict__ b2s, int mode) {
     const SpecDev &S = specs[b2s[blockIdx.x]];
-    SpecCtl *ctl = S.ctl;
+    const SpecCtl *ctl = S.ctl;
     const int phase = ctl->phase;
     if (mode == MODE_STEP && phase == PH_IDLE) return;
-    const int par = ctl->parity;
-    const long long done = ctl->done, nsteps = ctl->nsteps;
-    constexpr int APB = TPB / L;
-    const int lb = blockIdx.x - S.blk_pair0;
-    const int a = lb * APB + threadIdx.x / L;
-    const int l = threadIdx.x % L;
-    const bool valid = a < S.n;
-    const double4_32a *__restrict__ pf = (const double4_32a *)S.posfp;
-    const PotDev &P = S.pot;
-    double fx = 0, fy = 0, fz = 0;
-    double4_32a pa = make_double4_32a(0, 0, 0, 0);
-    if (valid) {
-        pa = pf[a];
-        for_entries64(S, pf, a, l, L, [&](const double4_32a &pj) {
-            double dx, dy, dz;
-            const double r2 = pair_r2(pa, pj, dx, dy, dz);
-            if (within(r2, P.rc2)) {
-                const double g = force_pair64<SC76>(P, r2, __dadd_rn(pa.w, pj.w));
-                fx = fma(g, dx, fx);
-                fy = fma(g, dy, fy);
-                fz = fma(g, dz, fz);
-            }
-        });
-    }
-    fx = lane_sum<L>(fx);
-    fy = lane_sum<L>(fy);
-    fz = lane_sum<L>(fz);
-    double ke = 0, pe = 0, rr = 0, d2 = 0, dp2 = 0;
-    if (valid && l == 0) {
-        chk_force(S, fx, fy, fz);
-        pe = ((const double *)S.pen)[a];
-        const uint8_t flag = S.flags[a];
-        if (flag == FLAG_RIGHT) rr = -(S.axis == 0 ? fx : (S.axis == 1 ? fy : fz));
-        double4_32a v = ((const double4_32a *)S.vel)[a];
-        if (mode == MODE_EVAL) {
-            ke = __dmul_rn(S.ke_fac, fma(v.z, v.z, fma(v.y, v.y, __dmul_rn(v.x, v.x))));
-            ((double4_32a *)S.eval_out)[S.orig[a]] = make_double4_32a(fx, fy, fz, pe);
-        } else {
-            const double kh = S.acc_half;
-            // thermal relaxation: the right grip moves along the load axis only
-            const bool rfree = flag == FLAG_RIGHT && S.ctl->relax;
-            if (phase == PH_RUN) {
-                if (flag == FLAG_MOBILE) {
-                    v.x = fma(fx, kh, v.x);
-                    v.y = fma(fy, kh, v.y);
-                    v.z = fma(fz, kh, v.z);
-                } else if (rfree) {
-                    if (S.axis == 0) v.x = fma(fx, kh, v.x);
-                    else if (S.axis == 1) v.y = fma(fy, kh, v.y);
-                    else v.z = fma(fz, kh, v.z);
-                }
-                ke = __dmul_rn(S.ke_fac, fma(v.z, v.z, fma(v.y, v.y, __dmul_rn(v.x, v.x))));
-                if (S.rsum) {
-                    // Eq. (mean_pos): the sampled state's position
-                    double *rs = S.rsum + 4LL * S.orig[a];
-                    rs[0] = rs[0] + pa.x;
-                    rs[1] = rs[1] + pa.y;
-                    rs[2] = rs[2] + pa.z;
-                }
-            }
-            double x = pa.x, y = pa.y, z = pa.z;
-            const bool start = (phase == PH_REFRESH) || (done + 1 < nsteps);
-            if (start && (flag == FLAG_MOBILE || rfree)) {
-                if (flag == FLAG_MOBILE) {
-                    v.x = fma(fx, kh, v.x);
-                    v.y = fma(fy, kh, v.y);
-                    v.z = fma(fz, kh, v.z);
-                } else if (S.axis == 0) {
-                    v.x = fma(fx, kh, v.x);
-                } else if (S.axis == 1) {
-                    v.y = fma(fy, kh, v.y);
-                } else {
-                    v.z = fma(fz, kh, v.z);
-                }
-                x = fma(v.x, S.dt, x);
-                y = fma(v.y, S.dt, y);
-                z = fma(v.z, S.dt, z);
-            } else if (start && flag == FLAG_RIGHT && !rfree && S.ctl->grip_du != 0.0) {
-                // continuous loading (fine-dynamics verification)
-                const double du = S.ctl->grip_du;
-                if (S.axis == 0) x = x + du;
-                else if (S.axis == 1) y = y + du;
-                else z = z + du;
-            }
-            ((double4_32a *)S.pos[par ^ 1])[a] = make_double4_32a(x, y, z, 0.0);
-            S.rec[par ^ 1][a] = rec_fp64(S, x, y, z);
-            ((double4_32a *)S.vel)[a] = v;
-            const float4 rf = S.ref[a];
-            const double ex = x - rf.x, ey = y - rf.y, ez = z - rf.z;
-            d2 = fma(ez, ez, fma(ey, ey, __dmul_rn(ex, ex)));
-            if (S.prune_on) {
-                const float4 pr = S.pref[a];
-                const double qx = x - pr.x, qy = y - pr.y, qz = z - pr.z;
-                dp2 = fma(qz, qz, fma(qy, qy, __dmul_rn(qx, qx)));
-            }
+    force_block64<L, SC76>(S, blockIdx.x - S.blk_pair0, ctl->parity, mode, phase, ctl->done,
+                                  ctl->nsteps);
+}
+
+template <int L, bool SC76>
+struct OpsF64 {
+    uint4 *cache;
+    int quads;
+    Atom64 A;
+    LaneList q;
+    double4_32a pa;  // the atom's position and density weight (all its lanes)
+    double pe;
+    int a, l;
+    bool valid;
+    __device__ __forceinline__ void load(const SpecDev &S, int tile, int par) {
+        const int t = tile * 32 + (threadIdx.x & 31);
+        a = t / L;
+        l = t % L;
+        valid = a < S.n;
+        pa = make_double4_32a(0, 0, 0, 0);
+        pe = 0.0;
+        if (valid) {
+            q.fill(S, cache, a, l, L, quads);
+            pa = ((const double4_32a *)S.pos[par])[a];
+            if (l == 0) A.load(S, par, a);
         }
     }
-    ke = warp_sum(ke);
-    pe = warp_sum(pe);
-    rr = warp_sum(rr);
-    d2 = (double)warp_max((float)d2);
-    dp2 = (double)warp_max((float)dp2);
-    step_tail<TPB>(S, lb, S.nblk_pair, ke, pe, rr, d2, dp2, mode, phase, done, nsteps);
+    __device__ __forceinline__ void prune(const SpecDev &S, int par) {
+        if (!valid) return;
+        prune_lane<L, true>(S, a, l, par);
+        q.fill(S, cache, a, l, L, quads);
+        A.pref = S.rec[par][a];
+    }
+    __device__ __forceinline__ void store(const SpecDev &S, int par) const {
+        if (valid && l == 0) A.store_vel(S, a);
+    }
+    __device__ __forceinline__ void density(const SpecDev &S, int par) {
+        const double4_32a *pos = (const double4_32a *)S.pos[par];
+        RhoSums64 s;
+        if (valid)
+            for_entries64(S, pos, q,
+                          [&](const double4_32a &pj) { rho_entry64<SC76>(S.pot, pa, pj, s); });
+        pe = density_end64<L>(S, a, valid && l == 0, pa, s, pa.w);
+    }
+    __device__ __forceinline__ StepVals<double> force(const SpecDev &S, int tile, int par, int phase,
+                                                  long long done, long long nsteps) {
+        double f[3] = {0, 0, 0};
+        if (valid)
+            for_entries64(S, (const double4_32a *)S.posfp, q,
+                          [&](const double4_32a &pj) { force_entry64<SC76>(S.pot, pa, pj, f); });
+#pragma unroll
+        for (int d = 0; d < 3; ++d) f[d] = lane_sum<L>(f[d]);
+        StepVals<double> v = zero_vals<double>();
+        if (valid && l == 0) {
+            atom_update64(S, A, par, a, f, pe, MODE_STEP, phase, done, nsteps, v);
+            pa.x = A.x[0];
+            pa.y = A.x[1];
+            pa.z = A.x[2];
+        }
+        if (L > 1) {  // the new position to the atom's other lanes
+            const int src = (threadIdx.x & 31) & ~(L - 1);
+            pa.x = __shfl_sync(0xffffffffu, pa.x, src);
+            pa.y = __shfl_sync(0xffffffffu, pa.y, src);
+            pa.z = __shfl_sync(0xffffffffu, pa.z, src);
+        }
+        warp_reduce<L>(v);
+        if ((threadIdx.x & 31) == 0) store_part(part_warp(S, tile), v);
+        return v;
+    }
+};
+constexpr int RUN_WARPS_F64 = 16;
+template <int L, bool SC76>
+__global__ void __launch_bounds__(32 * RUN_WARPS_F64, 1)
+    k_run_f64(const SpecDev *specs, int nspec, const int *b2s, int nblk, RunCtl *rc,
+              cudaGraphConditionalHandle again, int quads) {
+    extern __shared__ uint4 list_cache[];
+    OpsF64<L, SC76> ops{list_cache, quads};
+    run_resident<L, double>(specs, nspec, b2s, nblk, rc, again, ops);
 }
 
 #define PTA_F64_SWITCH(KER, SC, ARG)                                                   \
@@ -271,6 +405,42 @@ void launch_force_f64(const Tab &t, const Group &g, int mode, cudaStream_t st) {
         PTA_F64_SWITCH(k_force_f64, true, mode)
     else
         PTA_F64_SWITCH(k_force_f64, false, mode)
+}
+
+#define PTA_RUN64_SWITCH(SC, DO)   \
+    switch (g.L) {                 \
+        case 1: DO(1, SC); break;  \
+        case 2: DO(2, SC); break;  \
+        case 4: DO(4, SC); break;  \
+        case 8: DO(8, SC); break;  \
+        default: DO(16, SC);       \
+    }
+
+bool run_possible_f64(const Group &g) {
+    const RunShape r = run_shape(g.nblk, g.L, RUN_WARPS_F64);
+    bool ok = false;
+#define DO(L, SC) ok = run_fits(k_run_f64<L, SC>, r)
+    if (g.sc76)
+        PTA_RUN64_SWITCH(true, DO)
+    else
+        PTA_RUN64_SWITCH(false, DO)
+#undef DO
+    return ok;
+}
+
+cudaError_t launch_run_f64(const Tab &t, const Group &g, RunCtl *rc,
+                           cudaGraphConditionalHandle again, cudaStream_t st) {
+    const RunShape r = run_shape(g.nblk, g.L, RUN_WARPS_F64);
+    cudaError_t e = cudaSuccess;
+#define DO(L, SC)                                                                              \
+    e = launch_cooperative(k_run_f64<L, SC>, r, st, t.specs, t.nspec, g.b2s, g.nblk, rc, again, \
+                           r.quads)
+    if (g.sc76)
+        PTA_RUN64_SWITCH(true, DO)
+    else
+        PTA_RUN64_SWITCH(false, DO)
+#undef DO
+    return e;
 }
 
 }  // namespace pta

@@ -121,6 +121,11 @@ struct Runner {
     pta_coarse_result *h_cres = nullptr;
     Tab tab{};
     cudaGraphExec_t g_chunk = nullptr, g_one = nullptr;
+    // resident runs (the table's pair blocks fit the GPU at once): one graph
+    // runs a whole burst, list builds included
+    cudaGraphExec_t g_burst = nullptr;
+    RunCtl *d_run = nullptr;
+    int *h_stuck = nullptr;
     // timing: graphs with event-record nodes around each iteration's parts
     bool timing = false;
     cudaGraphExec_t t_chunk = nullptr, t_one = nullptr;
@@ -368,6 +373,14 @@ static int compute_sizes(const pta_specimen &s, const pta_potential &p, const pt
     return PTA_OK;
 }
 
+// partials of 32 bytes: per warp of the pair blocks in resident runs, else per
+// block and per group of 32 blocks; behind them the groups' counters
+static size_t part_bytes(const Sizes &z) {
+    const size_t nb = (size_t)std::max(z.nblk_pair, z.nblk_atom);
+    return 32 * (TPB / 32) * nb + 4 * (nb / 32 + 1);
+}
+static size_t gpart_bytes(const Sizes &z) { return 32 * ((size_t)z.nblk_pair / 32 + 1); }
+
 static size_t footprint(const Sizes &z, int prec) {
     const size_t n = (size_t)z.n;
     const size_t p = (prec == PTA_PREC_FP64) ? 32 : 16;
@@ -401,8 +414,8 @@ static size_t footprint(const Sizes &z, int prec) {
         add(16 * n);                 // pref
     }
     {
-        const size_t nb = (size_t)std::max(z.nblk_pair, z.nblk_atom);
-        add(64 * (nb + 2 * (nb / 32 + 1)));  // part: block and group partials, group counters
+        add(part_bytes(z));  // part
+        add(gpart_bytes(z)); // gpart
     }
     add(24 * (size_t)z.series_cap);  // series
     add(32 * n);                     // eval_out
@@ -454,6 +467,7 @@ static void runner_free(Runner *r) {
     if (!r) return;
     if (r->g_chunk) cudaGraphExecDestroy(r->g_chunk);
     if (r->g_one) cudaGraphExecDestroy(r->g_one);
+    if (r->g_burst) cudaGraphExecDestroy(r->g_burst);
     if (r->t_chunk) cudaGraphExecDestroy(r->t_chunk);
     if (r->t_one) cudaGraphExecDestroy(r->t_one);
     for (auto e : r->ev) cudaEventDestroy(e);
@@ -551,6 +565,75 @@ static int capture_iters(Runner *r, int iters, cudaGraphExec_t *out, bool timed 
     e = cudaGraphInstantiate(out, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) {
+        cudaGetLastError();
+        return PTA_ECUDA;
+    }
+    return PTA_OK;
+}
+
+// Body graph of a conditional node added to the stream capture in `cap`.
+static int add_conditional(cudaStream_t cap, cudaGraphConditionalHandle h,
+                           cudaGraphConditionalNodeType type, cudaGraph_t *body) {
+    cudaStreamCaptureStatus cs;
+    cudaGraph_t cg = nullptr;
+    const cudaGraphNode_t *deps = nullptr;
+    const cudaGraphEdgeData *edata = nullptr;
+    size_t ndeps = 0;
+    CK(cudaStreamGetCaptureInfo(cap, &cs, nullptr, &cg, &deps, &edata, &ndeps));
+    cudaGraphNodeParams np = {};
+    np.type = cudaGraphNodeTypeConditional;
+    np.conditional.handle = h;
+    np.conditional.type = type;
+    np.conditional.size = 1;
+    cudaGraphNode_t node;
+    CK(cudaGraphAddNode(&node, cg, deps, edata, ndeps, &np));
+    *body = np.conditional.phGraph_out[0];
+    CK(cudaStreamUpdateCaptureDependencies(cap, &node, nullptr, 1, cudaStreamSetCaptureDependencies));
+    return PTA_OK;
+}
+
+// Graph of a whole burst as a resident run:
+//   WHILE (a specimen is still in its burst) {
+//       [does any need a list build?] -> IF { build kernels }
+//       [resident kernel: steps until the next build or the end] }
+// so neither the host nor a kernel boundary sits between two steps.
+static int capture_burst(Runner *r, cudaGraphExec_t *out) {
+    cudaGraph_t g = nullptr, wb = nullptr, bb = nullptr, tmp = nullptr;
+    CK(cudaGraphCreate(&g, 0));
+    cudaGraphConditionalHandle again, build;
+    bool ok = cudaGraphConditionalHandleCreate(&again, g, 1, cudaGraphCondAssignDefault) ==
+              cudaSuccess;
+    if (ok) {
+        cudaGraphNodeParams np = {};
+        np.type = cudaGraphNodeTypeConditional;
+        np.conditional.handle = again;
+        np.conditional.type = cudaGraphCondTypeWhile;
+        np.conditional.size = 1;
+        cudaGraphNode_t node;
+        ok = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &np) == cudaSuccess;
+        if (ok) wb = np.conditional.phGraph_out[0];
+    }
+    ok = ok && cudaGraphConditionalHandleCreate(&build, wb, 0, cudaGraphCondAssignDefault) ==
+                   cudaSuccess;
+    if (ok && cudaStreamBeginCaptureToGraph(r->cap, wb, nullptr, nullptr, 0,
+                                            cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+        launch_decide_build(r->tab, r->d_run, build, r->cap);
+        ok = add_conditional(r->cap, build, cudaGraphCondTypeIf, &bb) == PTA_OK;
+        if (ok && cudaStreamBeginCaptureToGraph(r->cap2, bb, nullptr, nullptr, 0,
+                                                cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+            launch_rebuild(r->tab, 0, r->cap2);
+            ok = cudaStreamEndCapture(r->cap2, &tmp) == cudaSuccess;
+        } else {
+            ok = false;
+        }
+        ok = ok && launch_run(r->tab, r->d_run, again, r->cap) == cudaSuccess;
+        ok = (cudaStreamEndCapture(r->cap, &tmp) == cudaSuccess) && ok;
+    } else {
+        ok = false;
+    }
+    ok = ok && cudaGraphInstantiate(out, g, 0) == cudaSuccess;
+    cudaGraphDestroy(g);
+    if (!ok) {
         cudaGetLastError();
         return PTA_ECUDA;
     }
@@ -664,7 +747,8 @@ static int runner_upload(Runner *r) {
     const size_t bytes = round_up(sizeof(SpecDev) * k, 256) + round_up(4 * words, 256) +
                          round_up(8 * k, 256) * 2 + round_up(4 * k, 256) +
                          round_up(sizeof(pta_averages) * k, 256) +
-                         round_up(sizeof(pta_coarse_result) * k, 256);
+                         round_up(sizeof(pta_coarse_result) * k, 256) +
+                         round_up(sizeof(RunCtl), 256);
     CKR(dev_alloc(r, bytes, &p));
     char *c = (char *)p;
     r->d_specs = (SpecDev *)c;
@@ -680,6 +764,8 @@ static int runner_upload(Runner *r) {
     r->d_avg = (pta_averages *)c;
     c += round_up(sizeof(pta_averages) * k, 256);
     r->d_cres = (pta_coarse_result *)c;
+    c += round_up(sizeof(pta_coarse_result) * k, 256);
+    r->d_run = (RunCtl *)c;
     std::vector<int> all;
     all.insert(all.end(), b2s_atom.begin(), b2s_atom.end());
     all.insert(all.end(), b2s_cell.begin(), b2s_cell.end());
@@ -716,6 +802,7 @@ static int runner_upload(Runner *r) {
     r->tab = t;
     // pinned host mirrors
     const size_t hb = 8 * k * 2 + 4 * k + sizeof(pta_averages) * k + sizeof(pta_coarse_result) * k + 64;
+    static_assert(sizeof(pta_coarse_result) % 8 == 0, "h_stuck follows the results");
     CK(cudaHostAlloc(&r->h_pin, hb, cudaHostAllocDefault));
     char *h = (char *)r->h_pin;
     r->h_nsteps = (long long *)h;
@@ -727,6 +814,8 @@ static int runner_upload(Runner *r) {
     r->h_avg = (pta_averages *)h;
     h += sizeof(pta_averages) * k;
     r->h_cres = (pta_coarse_result *)h;
+    h += sizeof(pta_coarse_result) * k;
+    r->h_stuck = (int *)h;
     return PTA_OK;
 }
 
@@ -742,8 +831,18 @@ static int runner_create(pta_ctx *const *members, int k, Runner **out) {
         cudaStreamCreateWithFlags(&r->cap2, cudaStreamNonBlocking) != cudaSuccess)
         rc = PTA_ECUDA;
     if (rc == PTA_OK) rc = runner_upload(r);
-    if (rc == PTA_OK) rc = capture_iters(r, CHUNK, &r->g_chunk);
-    if (rc == PTA_OK) rc = capture_iters(r, 1, &r->g_one);
+    const char *flat = std::getenv("PTA_GRAPH_FLAT");
+    // an adaptive burst length decides after every step whether it is the last,
+    // which a resident run learns one step late
+    bool adaptive = false;
+    for (int i = 0; i < k; ++i) adaptive |= members[i]->par.conv_lag > 0;
+    if (rc == PTA_OK && !adaptive && r->tab.ngroups == 1 && !(flat && flat[0] == '1') &&
+        run_possible(r->tab.grp[0])) {
+        rc = capture_burst(r, &r->g_burst);
+    } else {
+        if (rc == PTA_OK) rc = capture_iters(r, CHUNK, &r->g_chunk);
+        if (rc == PTA_OK) rc = capture_iters(r, 1, &r->g_one);
+    }
     if (rc != PTA_OK) {
         runner_free(r);
         return rc;
@@ -856,6 +955,8 @@ static int run_burst(Runner *r, const int64_t *nsteps, pta_averages *out, int sl
             CK(cudaGraphLaunch(r->t_one, r->stream));
             CKR(collect_times(r, 1));
         }
+    } else if (r->g_burst) {
+        if (iters > 0) CK(cudaGraphLaunch(r->g_burst, r->stream));
     } else {
         for (long long q = 0; q < iters / CHUNK && run; ++q) {
             CK(cudaGraphLaunch(r->g_chunk, r->stream));
@@ -867,7 +968,12 @@ static int run_burst(Runner *r, const int64_t *nsteps, pta_averages *out, int sl
     CKR(launch_check());
     CK(cudaMemcpyAsync(r->h_avg, r->d_avg, sizeof(pta_averages) * k, cudaMemcpyDeviceToHost,
                        r->stream));
+    *r->h_stuck = 0;
+    if (r->g_burst)
+        CK(cudaMemcpyAsync(r->h_stuck, &r->d_run->stuck, sizeof(int), cudaMemcpyDeviceToHost,
+                           r->stream));
     CK(cudaStreamSynchronize(r->stream));
+    if (*r->h_stuck) return PTA_ECUDA;
     int rc = PTA_OK;
     for (int i = 0; i < k; ++i) {
         if (out) out[i] = r->h_avg[i];
@@ -1066,7 +1172,7 @@ static int ctx_alloc_all(pta_ctx *c, const Sizes &z) {
     AL(posfp, p * n, void *);
     AL(vel, 32 * n, void *);
     AL(flags, n, uint8_t *);
-    AL(ref, 16 * n, float4 *);
+    AL(ref, 16 * n, int4 *);
     AL(atom_cell, 4 * n, int *);
     AL(cell_cnt, 4 * (size_t)z.ncell, int *);
     AL(cell_start, 4 * ((size_t)z.ncell + 1), int *);
@@ -1079,13 +1185,11 @@ static int ctx_alloc_all(pta_ctx *c, const Sizes &z) {
     AL(nab, 8 * n, int2 *);
     if (z.prune_on) {
         AL(nlist, 16 * z.list_quads, uint4 *);
-        AL(pref, 16 * n, float4 *);
+        AL(pref, 16 * n, int4 *);
     }
     {
-        // block partials (8 doubles per block), then per group of 32 blocks
-        // its partial (8 doubles) and its counter
-        const size_t nb = (size_t)std::max(z.nblk_pair, z.nblk_atom);
-        AL(part, 64 * (nb + 2 * (nb / 32 + 1)), double *);
+        AL(part, part_bytes(z), double *);
+        AL(gpart, gpart_bytes(z), double *);
     }
     AL(series, 24 * (size_t)z.series_cap, double *);
     AL(eval_out, 32 * n, double *);
@@ -1173,14 +1277,13 @@ int pta_create(const pta_specimen *spec, const pta_potential *pot, double T0, ui
     s.f_ra2q = (float)(rnear * rnear * (1.0 + band) * rq * rq);
     s.f_reach_slack = (float)(1e-3 + 1e-6 * extent);
     s.f_reach2 = (float)(s.rl2 * (1.0 + band) + 1e-3);
-    s.half_skin2 = (float)(0.25 * c->par.skin * c->par.skin);
+    s.half_skin2q = (float)(0.25 * c->par.skin * c->par.skin * (1.0 - 1e-6) * rq * rq);
     s.prune_on = z.prune_on;
     s.prune_first = z.prune_on && z.prune_margin > NEAR_MARGIN;
     {
-        // slack for the FP32 rounding of the reference positions
-        const double rp = c->pot.rc + z.prune_margin + 2e-7 * extent;
+        const double rp = c->pot.rc + z.prune_margin;
         s.f_rp2q = (float)(rp * rp * (1.0 + band) * rq * rq);
-        s.half_prune2 = (float)(0.25 * z.prune_margin * z.prune_margin);
+        s.half_prune2q = (float)(0.25 * z.prune_margin * z.prune_margin * (1.0 - 1e-6) * rq * rq);
     }
     s.pot = make_pot(c->pot);
     s.mass = c->par.mass_amu;

@@ -95,6 +95,7 @@ struct SpecCtl {
     int max_nn;                // largest neighbour count at the last build
     int prune;                 // 1: prune the inner list before the next pair pass
     int prunes;                // prunings in the current burst
+    int prune_at;              // resident runs: pass after which a pruning was asked for
     double sum[3];             // running sums of K, U, T over the burst (in step order)
     double sum_chk[3];         // adaptive length: running sums at the last check
     double conv_val[3];        // adaptive length: running average at convergence
@@ -128,15 +129,16 @@ struct SpecDev {
     double hcell, inv_h;
     int nc[3];
     int ncell;
-    // list radius (rc + skin)^2, half skin squared
+    // list radius (rc + skin)^2
     double rl2;
-    float half_skin2, f_h;
+    float f_h;
     // fixed-point records: quanta per A, A per quantum and its square, shift
     // from the 2^-12 A grid of hi to quanta; grid origin
     float f_rq, f_q, f_q2, f_org[3];
     int rec_shift;
     // squared radii in quanta: bracket of the list radius, near part, pruning
     float f_rl2q_lo, f_rl2q_hi, f_ra2q, f_rp2q;
+    float half_skin2q, half_prune2q;  // squared displacements that ask for a build, a pruning
     float f_reach2, f_reach_slack;  // list radius squared (A^2, with slack) and slack (A)
     PotDev pot;
     // integration constants
@@ -157,7 +159,7 @@ struct SpecDev {
     void *pen;      // energy of each atom, 1/2 eps sum_j phi_n + B(rho) (double; MIXED: float)
     void *vel;      // FP64: double4; MIXED: VelHL
     uint8_t *flags;
-    float4 *ref;    // positions at the last list build (skin test)
+    int4 *ref;      // records at the last list build (skin test)
     int *atom_cell, *cell_cnt, *cell_start, *cell_tmp, *cell_atoms;
     int *orig;        // original index (creation order) of the atom stored at each slot
     void *perm_tmp;   // scratch of the permutation that sorts atoms by cell
@@ -165,11 +167,11 @@ struct SpecDev {
     uint4 *nlist;     // far part of the Verlet list (null without pruning)
     int2 *nab;        // per atom: entries of the near and of the far part
     int *pnn;         // per atom and lane: entries of plist
-    float4 *pref;     // positions at the last pruning
+    int4 *pref;       // records at the last pruning
     int prune_on;
     int prune_first;  // 1: a fresh list is pruned before its first use
-    float half_prune2;
-    double *part;       // per pair block: K, U, R, max displacement^2
+    double *part;       // partials of K, U, R and displacements, per block (or warp)
+    double *gpart;      // per group of 32 blocks (resident runs)
     double *series;     // series_cap x 3 samples of the current burst
     long long series_cap;
     double *eval_out;   // n x 4: F, pe (MODE_EVAL)
@@ -185,6 +187,16 @@ struct Group {
     const int *b2s;
     int nblk;
 };
+
+// Control words of a resident run (k_run_*), each on a line of its own: the
+// arrivals at its grid barriers (reset before every launch); stuck: a
+// barrier's wait ran out.
+struct RunCtl {
+    unsigned long long arrive, pad0[15];
+    int stuck, pad1[31];
+};
+// what a step asks for, or what became of the run
+enum RunState : int { RUN_STOP = 1, RUN_BUILD = 2, RUN_PRUNE = 4, RUN_STUCK = 8 };
 
 // one launch table: the specimens and, per kernel kind, block->specimen maps
 struct Tab {
@@ -430,5 +442,11 @@ __device__ __forceinline__ bool prune_active(const SpecDev &S, int force) {
 }
 void launch_density(const Tab &t, int force, cudaStream_t st);
 void launch_force(const Tab &t, int mode, cudaStream_t st);
+// resident runs of a table of one group (see k_pair_common.cuh): does the
+// group fit, and the cooperative launch
+bool run_possible(const Group &g);
+cudaError_t launch_run(const Tab &t, RunCtl *rc, cudaGraphConditionalHandle again,
+                       cudaStream_t st);
+void launch_decide_build(const Tab &t, RunCtl *rc, cudaGraphConditionalHandle h, cudaStream_t st);
 
 }  // namespace pta
