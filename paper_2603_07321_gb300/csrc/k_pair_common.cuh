@@ -10,10 +10,11 @@
 namespace pta {
 
 // sum over the L lanes that share one atom (lanes are contiguous in the warp)
-template <int L, typename T>
-__device__ __forceinline__ T lane_sum(T v) {
+template <typename T>
+__device__ __forceinline__ T lane_sum(T v, int L) {
 #pragma unroll
-    for (int o = L / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int o = 8; o > 0; o >>= 1)
+        if (o < L) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 
@@ -49,6 +50,8 @@ __device__ __forceinline__ double shfl_xor(double v, int o) {
 }
 __device__ __forceinline__ double to_double(FF v) { return (double)v.h + (double)v.l; }
 __device__ __forceinline__ double to_double(double v) { return v; }
+__device__ __forceinline__ bool is_zero(FF v) { return v.h == 0.f; }
+__device__ __forceinline__ bool is_zero(double v) { return v == 0.0; }
 __device__ __forceinline__ void set(FF &v, float x) { v = {x, 0.f}; }
 __device__ __forceinline__ void set(double &v, double x) { v = x; }
 // non-negative floats order as their bits
@@ -61,15 +64,33 @@ struct StepVals {
     T s[3];         // K, U, R
     float d2, dp2;  // displacements
 };
-// sums over the lanes whose values count (every MINO-th), down to offset MINO
-template <int MINO, class T>
-__device__ __forceinline__ void warp_reduce(StepVals<T> &v) {
+// sums over the lanes whose values count (every mino-th), down to offset mino
+template <class T>
+__device__ __forceinline__ void warp_reduce(StepVals<T> &v, int mino) {
+    // most warps hold no right-grip atom and no reaction
+    const bool reaction = __any_sync(0xffffffffu, !is_zero(v.s[2]));
 #pragma unroll
-    for (int o = 16; o >= MINO; o >>= 1)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) v.s[q] = add(v.s[q], shfl_xor(v.s[q], o));
+    for (int o = 16; o >= mino; o >>= 1) {
+        v.s[0] = add(v.s[0], shfl_xor(v.s[0], o));
+        v.s[1] = add(v.s[1], shfl_xor(v.s[1], o));
+        if (reaction) v.s[2] = add(v.s[2], shfl_xor(v.s[2], o));
+    }
     v.d2 = warp_max(v.d2);
     v.dp2 = warp_max(v.dp2);
+}
+// the same sums with the atoms of a tile in 32 / L adjacent lanes
+template <class T>
+__device__ __forceinline__ void tile_reduce(StepVals<T> &v, int L) {
+    const bool reaction = __any_sync(0xffffffffu, !is_zero(v.s[2]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        if (o * L >= 32) continue;
+        v.s[0] = add(v.s[0], shfl_xor(v.s[0], o));
+        v.s[1] = add(v.s[1], shfl_xor(v.s[1], o));
+        if (reaction) v.s[2] = add(v.s[2], shfl_xor(v.s[2], o));
+        v.d2 = fmaxf(v.d2, __shfl_xor_sync(0xffffffffu, v.d2, o));
+        v.dp2 = fmaxf(v.dp2, __shfl_xor_sync(0xffffffffu, v.dp2, o));
+    }
 }
 // a partial in memory: three sums and the two maxima, 32 bytes
 __device__ __forceinline__ void load_part(const double *p, StepVals<FF> &v) {
@@ -123,33 +144,27 @@ __device__ __forceinline__ float moved2(const int4 &a, const int4 &b) {
 constexpr int PART = 4;           // doubles per partial
 constexpr int PART_GROUP = 32;    // blocks per group of partials
 
-// the block's partial (warp values valid in lane 0), stored by its first
-// warp; complete for a thread-0 release that follows
+// The block's partial from its atoms' values, atom t of the block in thread t
+// < NT / L: the atoms of each warp tile (32 / L of them) summed as a resident
+// run's warp does, then the block's tiles in order.  Stored by the first warp;
+// complete for a thread-0 release that follows.
 template <int NT, class T>
-__device__ __forceinline__ void block_partial(const SpecDev &S, int lb, const StepVals<T> &v) {
+__device__ __forceinline__ void block_partial(const SpecDev &S, int lb, StepVals<T> v, int L) {
     constexpr int NW = NT / 32;
-    __shared__ T sh[3][NW];
-    __shared__ float shm[2][NW];
+    __shared__ StepVals<T> sh[NW];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) {
-#pragma unroll
-        for (int q = 0; q < 3; ++q) sh[q][w] = v.s[q];
-        shm[0][w] = v.d2;
-        shm[1][w] = v.dp2;
+    if (w * 32 < NT / L) {
+        tile_reduce(v, L);
+        if ((lane & (32 / L - 1)) == 0 && threadIdx.x < NT / L) sh[threadIdx.x / (32 / L)] = v;
     }
     __syncthreads();
     if (w == 0) {
         double *P = S.part + (long long)PART * lb;
-        if (lane < 3) {
-            T a = sh[lane][0];
+        if (lane == 0) {
+            StepVals<T> a = sh[0];
 #pragma unroll
-            for (int k = 1; k < NW; ++k) a = add(a, sh[lane][k]);
-            *(T *)(P + lane) = a;
-        } else if (lane < 5) {
-            float m = shm[lane - 3][0];
-#pragma unroll
-            for (int k = 1; k < NW; ++k) m = fmaxf(m, shm[lane - 3][k]);
-            ((float *)(P + 3))[lane - 3] = m;
+            for (int k = 1; k < NW; ++k) merge(a, sh[k]);
+            store_part(P, a);
         }
         __syncwarp();
     }
@@ -169,7 +184,7 @@ __device__ __forceinline__ StepVals<T> total_of_groups(int ngroups, F group) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // a single warp holds everything of up to 32 groups: adding the other
     // warps' zeros changes nothing
-    if (w * 32 < ngroups) warp_reduce<1>(v);
+    if (w * 32 < ngroups) warp_reduce(v, 1);
     if (ngroups <= 32) return v;
     if (lane == 0) {
 #pragma unroll
@@ -266,15 +281,16 @@ __device__ inline void advance_ctl(const SpecDev &S, double K, double U, double 
 // per-warp ones of resident runs), start at 0 and are reset by their group's
 // last block.
 template <int NT, class T>
-__device__ inline void step_tail(const SpecDev &S, int lb, int nblk, const StepVals<T> &v, int mode,
-                                 int phase, int par, long long done, long long nsteps) {
+__device__ inline void step_tail(const SpecDev &S, int lb, int nblk, const StepVals<T> &v, int L,
+                                 int mode, int phase, int par, long long done,
+                                 long long nsteps) {
     __shared__ int role;  // 0: done; 1: last block of its group; 2: last group
     const int ngroups = (nblk + PART_GROUP - 1) / PART_GROUP;
     const int g = lb / PART_GROUP;
     const int gsize = min(PART_GROUP, nblk - g * PART_GROUP);
     double *groups = S.part + (long long)PART * nblk;
     unsigned *gcnt = (unsigned *)(S.part + (long long)PART * (TPB / 32) * nblk) + g;
-    block_partial<NT>(S, lb, v);
+    block_partial<NT>(S, lb, v, L);
     if (threadIdx.x == 0) {
         __threadfence();
         role = atomicAdd(gcnt, 1u) == (unsigned)(gsize - 1);
@@ -286,7 +302,7 @@ __device__ inline void step_tail(const SpecDev &S, int lb, int nblk, const StepV
     StepVals<T> a = zero_vals<T>();
     if (threadIdx.x < 32) {
         if (lane < gsize) load_part(S.part + (long long)PART * (g * PART_GROUP + lane), a);
-        warp_reduce<1>(a);
+        warp_reduce(a, 1);
         if (lane == 0) {
             *gcnt = 0u;  // every block of the group has counted: ready for the next launch
             if (ngroups > 1) {
@@ -336,7 +352,7 @@ __device__ inline void reduce_group(const SpecDev &S, int g) {
 #pragma unroll
         for (int k = 1; k < NW; ++k) merge(a, b[k]);
     }
-    warp_reduce<1>(a);
+    warp_reduce(a, 1);
     if (lane == 0) store_part(part_group(S, g), a);
 }
 template <class T>
@@ -351,7 +367,7 @@ __device__ inline StepVals<T> reduce_groups(const SpecDev &S) {
     for (int b = 0; b < ngroups; b += 32) {
         StepVals<T> u = zero_vals<T>();
         if (b + lane < ngroups) load_part(part_group(S, b + lane), u);
-        warp_reduce<1>(u);
+        warp_reduce(u, 1);
         if (b == 0) t = u;
         else merge(t, u);
     }
@@ -365,8 +381,14 @@ __device__ inline StepVals<T> reduce_groups(const SpecDev &S) {
 // read with ordinary (coherent after a barrier) loads.
 template <bool RES>
 __device__ __forceinline__ uint4 ld_quad(const uint4 *p) {
-    if (RES) return __ldcg(p);
     uint4 v;
+    if (RES) {
+        asm volatile("ld.global.L1::no_allocate.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                     : "l"(p)
+                     : "memory");
+        return v;
+    }
     asm("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];"
         : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
         : "l"(p));
@@ -385,8 +407,8 @@ __device__ __forceinline__ int4 ld_rec(const SpecDev &S, const void *rec, unsign
 //
 // Bound: the gathers of the far part's records (~118 of the ~252 entries of a
 // bulk atom at the default 2 A skin).
-template <int L, bool RES>
-__device__ __forceinline__ void prune_lane(const SpecDev &S, int u, int l, int par) {
+template <bool RES>
+__device__ __forceinline__ void prune_lane(const SpecDev &S, int u, int l, int L, int par) {
     const int4 *rec = S.rec[par];
     const int4 ra = rec[u];
     const float rp2 = S.f_rp2q;
@@ -515,86 +537,85 @@ struct GridBarrier {
     }
 };
 
-// A block of a resident run: contiguous warp tiles of the table (tile 4 b + k:
-// warp k of pair block b), one per warp, and the service warp behind them.
-// OPS (one precision and lane count): a warp's part of the passes.  Its atoms'
-// positions and velocities stay in registers from the launch to its end.
-constexpr int RESIDENT_SPECS = 4;  // descriptors kept in shared memory
-template <int L, class T, class OPS>
-__device__ __forceinline__ void run_resident(const SpecDev *specs, int nspec, const int *b2s,
-                                             int nblk, RunCtl *rc,
-                                             cudaGraphConditionalHandle again, OPS &ops) {
-    constexpr int NW = TPB / 32, GT = NW * PART_GROUP;  // tiles per group
-    __shared__ SpecDev sh[RESIDENT_SPECS];
-    __shared__ int requests;
-    const int ntile = nblk * NW, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int t0 = (int)((long long)ntile * blockIdx.x / gridDim.x);
-    const int t1 = (int)((long long)ntile * (blockIdx.x + 1) / gridDim.x);
-    const int s0 = b2s[t0 / NW];  // tiles run through the specimens in order
-    for (int k = 0; k < RESIDENT_SPECS && s0 + k < nspec; ++k) {
-        const int *src = (const int *)(specs + s0 + k);
-        for (int i = threadIdx.x; i < (int)(sizeof(SpecDev) / 4); i += blockDim.x)
-            ((int *)&sh[k])[i] = src[i];
-    }
-    if (threadIdx.x == 0) requests = 0;
-    __syncthreads();
-    auto spec = [&](int s) -> const SpecDev & {
-        return s - s0 < RESIDENT_SPECS ? sh[s - s0] : specs[s];
-    };
-    const int tile = t0 + w;
-    const bool has = tile < t1;
-    const bool service = w == (int)(blockDim.x >> 5) - 1;
-    const SpecDev &S = spec(has ? b2s[tile / NW] : s0);
-    const int local = tile - S.blk_pair0 * NW;  // tile of the specimen
-    SpecCtl *c = S.ctl;
-    // the burst as every warp follows it for its own specimen
-    int phase = has ? __ldcg(&c->phase) : (int)PH_IDLE, par = __ldcg(&c->parity);
-    bool prune = phase != PH_IDLE && S.prune_on && __ldcg(&c->prune);
-    long long done = __ldcg(&c->done);
-    const long long nsteps = __ldcg(&c->nsteps);
-    const bool mine = phase != PH_IDLE;
-    if (mine) ops.load(S, local, par);
-    // passes until the last specimen's burst is over
+constexpr int RESIDENT_SPECS = 8;  // specimens whose tiles one block may hold
+
+__device__ __forceinline__ void load_specs(SpecDev *sh, const SpecDev *specs, int ns) {
+    for (int i = threadIdx.x; i < ns * (int)(sizeof(SpecDev) / 4); i += blockDim.x)
+        ((int *)sh)[i] = ((const int *)specs)[i];
+}
+// passes until the last specimen's burst is over (every warp for itself)
+__device__ __forceinline__ int run_passes(const SpecDev *specs, int nspec) {
     long long passes = 0;
-    for (int s = lane; s < nspec; s += 32) {
+    for (int s = threadIdx.x & 31; s < nspec; s += 32) {
         const SpecCtl *q = specs[s].ctl;
         const int ph = __ldcg(&q->phase);
         if (ph != PH_IDLE)
             passes = max(passes, __ldcg(&q->nsteps) - __ldcg(&q->done) + (ph == PH_REFRESH));
     }
-    const int limit =
-        (int)__reduce_max_sync(0xffffffffu, (unsigned)min(passes, (long long)RUN_STEPS));
-    // service: the groups that begin in this block's tiles, and of those the
-    // ones that begin a specimen, whose sums this block finishes
-    unsigned starts = 0;
-    if (service) {
-        bool first = false;
-        if (t0 + lane < t1)
-            first = (t0 + lane - specs[b2s[(t0 + lane) / NW]].blk_pair0 * NW) % GT == 0;
-        starts = __ballot_sync(0xffffffffu, first);
+    return (int)__reduce_max_sync(0xffffffffu, (unsigned)min(passes, (long long)RUN_STEPS));
+}
+// one warp, at the end of a launch: does any specimen go on?
+__device__ __forceinline__ void run_again(const SpecDev *specs, int nspec, int state,
+                                          cudaGraphConditionalHandle again) {
+    const int lane = threadIdx.x & 31;
+    int active = 0;
+    for (int s = lane; s < nspec; s += 32) active |= __ldcg(&specs[s].ctl->phase) != PH_IDLE;
+    active = __any_sync(0xffffffffu, active);
+    if (lane == 0) cudaGraphSetConditional(again, active && !(state & RUN_STUCK) ? 1u : 0u);
+}
+// one lane: what a warp's displacements after pass `it` ask for
+template <class T>
+__device__ __forceinline__ void step_requests(const SpecDev &S, const StepVals<T> &v, int it,
+                                              int *requests) {
+    int r = 0;
+    if (v.d2 > S.half_skin2q) {
+        r = RUN_BUILD;
+        S.ctl->rebuild = 1;
     }
-    auto each_start = [&](auto f) {  // f(specimen, its group)
-        for (unsigned m = starts; m; m &= m - 1) {
-            const int t = t0 + __ffs(m) - 1, s = b2s[t / NW];
-            f(s, (t - spec(s).blk_pair0 * NW) / GT);
+    if (S.prune_on && v.dp2 > S.half_prune2q) {
+        r |= RUN_PRUNE;
+        S.ctl->prune_at = it;
+    }
+    if (r) atomicOr(requests, r);
+}
+
+// The service warp of a block: the sums of the groups that begin in its tiles,
+// and the control blocks of the specimens that do.  The phase and step count
+// there are those of the sums, one step behind the atoms.
+template <class T>
+struct Service {
+    const SpecDev *sh;  // the block's specimens
+    int ns, t0, t1;
+    int *requests;
+    template <class F>
+    __device__ __forceinline__ void each(F f) const {  // f(specimen, group)
+        constexpr int NW = TPB / 32, GT = NW * PART_GROUP;
+        for (int k = 0; k < ns; ++k) {
+            const int base = sh[k].blk_run0 * NW, end = base + sh[k].nblk_pair * NW;
+            const int a = max(t0, base) - base, b = min(t1, end) - base;
+            for (int g = (a + GT - 1) / GT; g * GT < b; ++g) f(sh[k], g);
         }
-    };
-    // The phase and step count in a specimen's control block are those of the
-    // sums, one step behind the atoms; the service warp that finishes them
-    // keeps them.
-    auto reduce = [&] {
-        each_start([&](int s, int g) {
-            if (__ldcg(&spec(s).ctl->phase) != PH_IDLE) reduce_group<T>(spec(s), g);
+    }
+    __device__ __forceinline__ void start() const {
+        each([&](const SpecDev &D, int g) {
+            if (g == 0 && (threadIdx.x & 31) == 0) {
+                D.ctl->rebuild = 0;  // asked for the build before this launch
+                D.ctl->prune_at = -1;
+            }
         });
-    };
-    auto finish = [&] {
-        each_start([&](int s, int g) {
-            const SpecDev &D = spec(s);
+    }
+    __device__ __forceinline__ void reduce() const {
+        each([&](const SpecDev &D, int g) {
+            if (__ldcg(&D.ctl->phase) != PH_IDLE) reduce_group<T>(D, g);
+        });
+    }
+    __device__ __forceinline__ void finish() const {
+        each([&](const SpecDev &D, int g) {
             SpecCtl *q = D.ctl;
             const int ph = __ldcg(&q->phase);
             if (g != 0 || ph == PH_IDLE) return;
             const StepVals<T> t = reduce_groups<T>(D);
-            if (lane != 0) return;
+            if ((threadIdx.x & 31) != 0) return;
             if (ph == PH_REFRESH) {
                 q->phase = PH_RUN;
                 return;
@@ -610,23 +631,52 @@ __device__ __forceinline__ void run_resident(const SpecDev *specs, int nspec, co
                 q->done = i + 1;
                 if (i + 1 >= __ldcg(&q->nsteps)) q->phase = PH_IDLE;
             } else {
-                q->err |= ERR_NAN;
+                atomicOr(&q->err, ERR_NAN);
                 q->phase = PH_IDLE;
-                atomicOr(&requests, RUN_STOP);
+                atomicOr(requests, RUN_STOP);
             }
         });
         __syncwarp();
-    };
-    if (service)
-        each_start([&](int s, int g) {
-            if (g == 0 && lane == 0) {
-                spec(s).ctl->rebuild = 0;  // asked for the build before this launch
-                spec(s).ctl->prune_at = -1;
-            }
-        });
+    }
+};
+
+// A block of a resident run: contiguous warp tiles of the table (tile 4 b + k:
+// warp k of pair block b), one per warp, and the service warp behind them.
+// OPS (one precision and lane count): a warp's part of the passes.  Its atoms'
+// positions and velocities stay in registers from the launch to its end.
+template <class T, class OPS>
+__device__ __forceinline__ void run_resident(const SpecDev *specs, int nspec, const int *b2s,
+                                             int nblk, RunCtl *rc,
+                                             cudaGraphConditionalHandle again, OPS &ops) {
+    constexpr int NW = TPB / 32;
+    __shared__ SpecDev sh[RESIDENT_SPECS];
+    __shared__ int requests;
+    const int ntile = nblk * NW, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int t0 = (int)((long long)ntile * blockIdx.x / gridDim.x);
+    const int t1 = (int)((long long)ntile * (blockIdx.x + 1) / gridDim.x);
+    const int s0 = b2s[t0 / NW];  // tiles run through the specimens in order
+    const int ns = b2s[(t1 - 1) / NW] - s0 + 1;
+    load_specs(sh, specs + s0, ns);
+    if (threadIdx.x == 0) requests = 0;
+    __syncthreads();
+    const int tile = t0 + w;
+    const bool has = tile < t1;
+    const bool service = w == (int)(blockDim.x >> 5) - 1;
+    const SpecDev &S = sh[(has ? b2s[tile / NW] : s0) - s0];
+    const int local = tile - S.blk_run0 * NW;  // tile of the specimen
+    SpecCtl *c = S.ctl;
+    // the burst as every warp follows it for its own specimen
+    int phase = has ? __ldcg(&c->phase) : (int)PH_IDLE, par = __ldcg(&c->parity);
+    bool prune = phase != PH_IDLE && S.prune_on && __ldcg(&c->prune);
+    long long done = __ldcg(&c->done);
+    const long long nsteps = __ldcg(&c->nsteps);
+    const bool mine = phase != PH_IDLE;
+    if (mine) ops.load(S, local, par);
+    const int limit = run_passes(specs, nspec);
+    const Service<T> sums{sh, ns, t0, t1, &requests};
+    if (service) sums.start();
     GridBarrier bar{rc, &requests};
     int state = 0, it = 0;
-    bool sums = false;  // a step's partials are waiting
     for (; it < limit && !(state & (RUN_BUILD | RUN_STUCK)); ++it) {
         const bool run = phase != PH_IDLE;
         if (run && prune) {
@@ -637,29 +687,17 @@ __device__ __forceinline__ void run_resident(const SpecDev *specs, int nspec, co
             }
         }
         if (run) ops.density(S, par);
-        if (service && sums) reduce();
+        if (service && it > 0) sums.reduce();
         state = bar.sync(false);
         if (state & RUN_STUCK) break;
         if (run) {
             const StepVals<T> v = ops.force(S, local, par, phase, done, nsteps);
-            if (lane == 0) {
-                int r = 0;
-                if (v.d2 > S.half_skin2q) {
-                    r = RUN_BUILD;
-                    c->rebuild = 1;
-                }
-                if (S.prune_on && v.dp2 > S.half_prune2q) {
-                    r |= RUN_PRUNE;
-                    c->prune_at = it;
-                }
-                if (r) atomicOr(&requests, r);
-            }
+            if (lane == 0) step_requests(S, v, it, &requests);
             par ^= 1;
             done += phase == PH_RUN;
             phase = done < nsteps ? PH_RUN : PH_IDLE;
         }
-        if (service && sums) finish();
-        sums = true;
+        if (service && it > 0) sums.finish();
         state = bar.sync(true);
         // of several specimens, which one asked?
         prune = (state & RUN_PRUNE) && S.prune_on && (nspec == 1 || __ldcg(&c->prune_at) == it);
@@ -670,9 +708,9 @@ __device__ __forceinline__ void run_resident(const SpecDev *specs, int nspec, co
     }
     // the last step's sums
     if (!(state & RUN_STUCK) && it > 0) {
-        if (service) reduce();
+        if (service) sums.reduce();
         state |= bar.sync(false) & RUN_STUCK;
-        if (service) finish();
+        if (service) sums.finish();
     }
     if (mine) {
         ops.store(S, par);
@@ -682,12 +720,111 @@ __device__ __forceinline__ void run_resident(const SpecDev *specs, int nspec, co
         }
     }
     state |= bar.sync(false) & RUN_STUCK;
-    if (blockIdx.x == 0 && w == 0) {
-        int active = 0;
-        for (int s = lane; s < nspec; s += 32) active |= __ldcg(&specs[s].ctl->phase) != PH_IDLE;
-        active = __any_sync(0xffffffffu, active);
-        if (lane == 0) cudaGraphSetConditional(again, active && !(state & RUN_STUCK) ? 1u : 0u);
+    if (blockIdx.x == 0 && w == 0) run_again(specs, nspec, state, again);
+}
+
+// A block of a run over a larger table: contiguous tiles again, but several
+// per warp, handed out one at a time; the atoms' state and the lists stay in
+// memory.  Against launched passes it has no launches and no conditional node
+// per step (~25 us of it on a specimen of 108,000 atoms) and no last wave:
+// the cube of 470,596 atoms fills 3.02 waves of eight blocks per SM, and the
+// blocks of the fourth ran alone for ~10% of a pass.
+struct SpecRun {
+    int phase, par, prune;
+    long long done, nsteps;
+};
+template <class T, class OPS>
+__device__ __forceinline__ void run_sweep(const SpecDev *specs, int nspec, const int *b2s, int nblk,
+                                          RunCtl *rc, cudaGraphConditionalHandle again,
+                                          const OPS &ops) {
+    constexpr int NW = TPB / 32;
+    __shared__ SpecDev sh[RESIDENT_SPECS];
+    __shared__ SpecRun run[RESIDENT_SPECS];
+    __shared__ int requests, next[2];
+    const int ntile = nblk * NW, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int t0 = (int)((long long)ntile * blockIdx.x / gridDim.x);
+    const int t1 = (int)((long long)ntile * (blockIdx.x + 1) / gridDim.x);
+    const int s0 = b2s[t0 / NW], ns = b2s[(t1 - 1) / NW] - s0 + 1;
+    load_specs(sh, specs + s0, ns);
+    if (threadIdx.x == 0) requests = next[0] = next[1] = 0;
+    __syncthreads();
+    // the burst of each specimen of this block, kept by a thread of its own
+    const int k = threadIdx.x;
+    const bool keeper = k < ns;
+    const bool owner = keeper && sh[k].blk_run0 * NW >= t0;  // holds its first tile
+    if (keeper) {
+        const SpecCtl *c = sh[k].ctl;
+        run[k].phase = __ldcg(&c->phase);
+        run[k].par = __ldcg(&c->parity);
+        run[k].prune = run[k].phase != PH_IDLE && sh[k].prune_on && __ldcg(&c->prune);
+        run[k].done = __ldcg(&c->done);
+        run[k].nsteps = __ldcg(&c->nsteps);
     }
+    const bool active0 = keeper && run[k].phase != PH_IDLE;
+    const int limit = run_passes(specs, nspec);
+    const Service<T> sums{sh, ns, t0, t1, &requests};
+    const bool service = w == 0;
+    if (service) sums.start();
+    __syncthreads();
+    auto each_tile = [&](int *ticket, auto f) {  // f(specimen of the block, its tile)
+        for (;;) {
+            int i = 0;
+            if (lane == 0) i = atomicAdd(ticket, 1);
+            i = __shfl_sync(0xffffffffu, i, 0) + t0;
+            if (i >= t1) break;
+            const int s = ns == 1 ? 0 : b2s[i / NW] - s0;
+            if (run[s].phase != PH_IDLE) f(s, i - sh[s].blk_run0 * NW);
+            __syncwarp();
+        }
+    };
+    GridBarrier bar{rc, &requests};
+    int state = 0, it = 0;
+    for (; it < limit && !(state & (RUN_BUILD | RUN_STUCK)); ++it) {
+        if (service && it > 0) sums.reduce();
+        each_tile(&next[0], [&](int s, int tile) {
+            if (run[s].prune) ops.prune(sh[s], tile, run[s].par);
+            ops.density(sh[s], tile, run[s].par);
+        });
+        state = bar.sync(false);
+        if (state & RUN_STUCK) break;
+        if (threadIdx.x == 0) next[0] = 0;
+        if (service && it > 0) sums.finish();
+        each_tile(&next[1], [&](int s, int tile) {
+            const SpecDev &S = sh[s];
+            const StepVals<T> v = ops.force(S, tile, run[s].par, run[s].phase, run[s].done,
+                                            run[s].nsteps);
+            if (lane == 0) step_requests(S, v, it, &requests);
+        });
+        state = bar.sync(true);
+        if (threadIdx.x == 0) next[1] = 0;
+        if (keeper && run[k].phase != PH_IDLE) {
+            SpecCtl *c = sh[k].ctl;
+            if (run[k].prune && owner) {
+                c->prunes = __ldcg(&c->prunes) + 1;
+                c->prune = 0;
+            }
+            run[k].par ^= 1;
+            run[k].done += run[k].phase == PH_RUN;
+            run[k].phase = run[k].done < run[k].nsteps ? PH_RUN : PH_IDLE;
+            run[k].prune = (state & RUN_PRUNE) && sh[k].prune_on &&
+                           (nspec == 1 || __ldcg(&c->prune_at) == it);
+            if ((state & RUN_STOP) && __ldcg(&c->phase) == PH_IDLE) run[k].phase = PH_IDLE;
+        }
+        __syncthreads();
+        if ((state & RUN_STOP) && nspec == 1) break;
+    }
+    // the last step's sums
+    if (!(state & RUN_STUCK) && it > 0) {
+        if (service) sums.reduce();
+        state |= bar.sync(false) & RUN_STUCK;
+        if (service) sums.finish();
+    }
+    if (owner && active0) {
+        sh[k].ctl->parity = run[k].par;
+        if (run[k].prune) sh[k].ctl->prune = 1;
+    }
+    state |= bar.sync(false) & RUN_STUCK;
+    if (blockIdx.x == 0 && w == 0) run_again(specs, nspec, state, again);
 }
 
 // f(entry) for the entries of a lane's column whose first `cached` quads lie
@@ -710,14 +847,22 @@ struct LaneList {
     }
 };
 
-// The launch shape of a resident run of nblk pair blocks: one block per SM, a
-// warp per tile, as many quads of the lists in shared memory as it holds (up
-// to the ~150 entries of a bulk atom).
+// The launch shape of a run over nblk pair blocks, one block per SM.  A warp
+// per tile, and a service warp, if that is at most RUN_WARPS warps; as many
+// quads of the lists in shared memory as it holds (up to the ~150 entries of a
+// bulk atom).  Else, up to SWEEP_TILES tiles per SM, a sweep of at most
+// sweep_warps warps: of those counts the one whose last round of tiles is
+// fullest.  Larger tables fill the GPU for several waves, and launched passes,
+// with 32 warps per SM and the read-only path, are faster: per step 66 us
+// (launched 74) at 23 tiles per SM (108,000 atoms), 138 (143) at 53, 253 (225)
+// at 97.
+constexpr int RUN_WARPS = 16, SWEEP_TILES = 56;
 struct RunShape {
     int blocks = 0, threads = 0, quads = 0;
     size_t smem = 0;
+    bool sweep = false;
 };
-inline RunShape run_shape(int nblk, int L, int max_warps) {
+inline RunShape run_shape(int nblk, int min_lanes, int sweep_warps) {
     RunShape r;
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -726,13 +871,23 @@ inline RunShape run_shape(int nblk, int L, int max_warps) {
         return r;
     }
     nsm = std::min(nsm, RUN_BLOCKS);
+    if (nsm < 1) return r;
     const int tiles = nblk * (TPB / 32);
-    const int warps = (tiles + nsm - 1) / std::max(nsm, 1) + 1;  // and the service warp
-    if (nsm < 1 || warps > max_warps) return r;
     r.blocks = std::min(nsm, tiles);
-    r.threads = 32 * warps;
-    r.quads = std::min(40 / L + 2, 160 * 1024 / (r.threads * 16));
-    r.smem = (size_t)r.quads * r.threads * 16;
+    const int per = (tiles + r.blocks - 1) / r.blocks;
+    if (per + 1 <= RUN_WARPS) {
+        r.threads = 32 * (per + 1);
+        r.quads = std::min(40 / min_lanes + 2, 160 * 1024 / (r.threads * 16));
+        r.smem = (size_t)r.quads * r.threads * 16;
+        return r;
+    }
+    if (per > SWEEP_TILES) return RunShape();
+    r.sweep = true;
+    int best = sweep_warps;
+    auto slots = [&](int w) { return (per + w - 1) / w * w; };
+    for (int w = sweep_warps; w >= sweep_warps * 3 / 4; --w)
+        if (slots(w) < slots(best)) best = w;
+    r.threads = 32 * best;
     return r;
 }
 template <class K>

@@ -19,17 +19,17 @@ namespace pta {
 // f(record) for the entries lane l of atom u reads, in list order: a quad per
 // iteration (four gathers in flight), the next quad read ahead, then what is
 // left of the last one
-template <class F>
+template <bool RES, class F>
 __device__ __forceinline__ void for_entries(const SpecDev &S, const void *rec, int u, int l, int L,
                                             F f) {
     const uint4 *p = S.plist + nl_col(u, l, L, S.capq);
     const int cnt = chk_count(S, S.pnn[u * L + l], 4 * (S.capq - 1));
-    uint4 e = ld_quad<false>(p);
+    uint4 e = ld_quad<RES>(p);
     for (int t = cnt >> 2; t > 0; --t) {
         p += 32;
-        const uint4 nx = ld_quad<false>(p);
-        const int4 x0 = ld_rec<false>(S, rec, e.x), x1 = ld_rec<false>(S, rec, e.y);
-        const int4 x2 = ld_rec<false>(S, rec, e.z), x3 = ld_rec<false>(S, rec, e.w);
+        const uint4 nx = ld_quad<RES>(p);
+        const int4 x0 = ld_rec<RES>(S, rec, e.x), x1 = ld_rec<RES>(S, rec, e.y);
+        const int4 x2 = ld_rec<RES>(S, rec, e.z), x3 = ld_rec<RES>(S, rec, e.w);
         f(x0);
         f(x1);
         f(x2);
@@ -38,9 +38,9 @@ __device__ __forceinline__ void for_entries(const SpecDev &S, const void *rec, i
     }
     const int left = cnt & 3;
     if (left) {
-        int4 x0 = ld_rec<false>(S, rec, e.x), x1 = x0, x2 = x0;
-        if (left > 1) x1 = ld_rec<false>(S, rec, e.y);
-        if (left > 2) x2 = ld_rec<false>(S, rec, e.z);
+        int4 x0 = ld_rec<RES>(S, rec, e.x), x1 = x0, x2 = x0;
+        if (left > 1) x1 = ld_rec<RES>(S, rec, e.y);
+        if (left > 2) x2 = ld_rec<RES>(S, rec, e.z);
         f(x0);
         if (left > 1) f(x1);
         if (left > 2) f(x2);
@@ -74,13 +74,13 @@ __device__ __forceinline__ void for_entries(const SpecDev &S, const void *rec, c
 
 // the density weight w of atom u from its lanes' sums, stored in its record;
 // its energy
-template <int L, bool SC76>
-__device__ __forceinline__ float density_end(const SpecDev &S, const PotF &P, int u, bool first,
-                                             const int4 &ra, RhoSums s, float &w) {
-    s.sm = lane_sum<L>(s.sm);
-    s.sn = lane_sum<L>(s.sn);
-    s.sr = lane_sum<L>(s.sr);
-    const float cnt = (float)lane_sum<L>(s.cnt);
+template <bool SC76>
+__device__ __forceinline__ float density_end(const SpecDev &S, const PotF &P, int L, int u,
+                                             bool first, const int4 &ra, RhoSums s, float &w) {
+    s.sm = lane_sum(s.sm, L);
+    s.sn = lane_sum(s.sn, L);
+    s.sr = lane_sum(s.sr, L);
+    const float cnt = (float)lane_sum(s.cnt, L);
     const float dr = fmaf(-cnt, P.rc, s.sr);  // sum of r - rc
     const float rho = SC76 ? fmaf(P.am, s.sm, fmaf(P.Bm, dr, __fmul_rn(-cnt, P.Am))) : s.sm;
     const float phn = fmaf(P.an, s.sn, fmaf(P.Bn, dr, __fmul_rn(-cnt, P.An)));
@@ -93,57 +93,52 @@ __device__ __forceinline__ float density_end(const SpecDev &S, const PotF &P, in
 }
 
 // sums of (eV/A^2) x quanta over an atom's lanes, in eV/A
-template <int L>
-__device__ __forceinline__ void force_end(const SpecDev &S, float f[3]) {
+__device__ __forceinline__ void force_end(const SpecDev &S, int L, float f[3]) {
 #pragma unroll
-    for (int d = 0; d < 3; ++d) f[d] = __fmul_rn(lane_sum<L>(f[d]), S.f_q);
+    for (int d = 0; d < 3; ++d) f[d] = __fmul_rn(lane_sum(f[d], L), S.f_q);
 }
 
-template <int L, bool SC76>
-__device__ __forceinline__ void density_block(const SpecDev &S, int lb, int par, const PotF &P) {
-    constexpr int UPB = TPB / L;
-    const int u = lb * UPB + threadIdx.x / L;
-    const int l = threadIdx.x % L;
+// the passes of one thread (lane l of atom u) with everything in memory
+template <bool SC76, bool RES>
+__device__ __forceinline__ void density_lane(const SpecDev &S, const PotF &P, int L, int u, int l,
+                                             int par) {
     const bool valid = u < S.n;
     RhoSums s;
     int4 ra = make_int4(0, 0, 0, 0);
     if (valid) {
         ra = S.rec[par][u];
         const float q2 = S.f_q2;
-        for_entries(S, S.rec[par], u, l, L,
-                    [&](const int4 &x) { rho_pair<SC76>(P, q2, ra, x, s); });
+        for_entries<RES>(S, S.rec[par], u, l, L,
+                         [&](const int4 &x) { rho_pair<SC76>(P, q2, ra, x, s); });
     }
     float w;
-    const float pe = density_end<L, SC76>(S, P, u, valid && l == 0, ra, s, w);
+    const float pe = density_end<SC76>(S, P, L, u, valid && l == 0, ra, s, w);
     if (valid && l == 0) ((float *)S.pen)[u] = pe;
 }
 
-template <int L, bool SC76>
-__device__ __forceinline__ void force_block(const SpecDev &S, int lb, int par, const PotF &P,
-                                            int mode, int phase, long long done,
-                                            long long nsteps) {
-    constexpr int UPB = TPB / L;
-    const int u = lb * UPB + threadIdx.x / L;
-    const int l = threadIdx.x % L;
-    const bool valid = u < S.n;
-    float f[3] = {0.f, 0.f, 0.f};
-    if (valid) {
+// the force on atom u, in all its lanes
+template <bool SC76, bool RES>
+__device__ __forceinline__ void force_lane(const SpecDev &S, const PotF &P, int L, int u, int l,
+                                           float f[3]) {
+    f[0] = f[1] = f[2] = 0.f;
+    if (u < S.n) {
         const int4 ra = ((const int4 *)S.posfp)[u];
         const float wa = __int_as_float(ra.w);
         const float q2 = S.f_q2;
-        for_entries(S, S.posfp, u, l, L,
-                    [&](const int4 &x) { force_pair<SC76>(P, q2, ra, wa, x, f[0], f[1], f[2]); });
+        for_entries<RES>(S, S.posfp, u, l, L, [&](const int4 &x) {
+            force_pair<SC76>(P, q2, ra, wa, x, f[0], f[1], f[2]);
+        });
     }
-    force_end<L>(S, f);
-    StepVals<FF> v = zero_vals<FF>();
-    if (valid && l == 0) {
-        AtomMixed A;
-        A.load(S, par, u);
-        atom_update_mixed(S, A, par, u, f, ((const float *)S.pen)[u], mode, phase, done, nsteps, v);
-        if (mode != MODE_EVAL) A.store(S, par ^ 1, u);
-    }
-    warp_reduce<L>(v);
-    step_tail<TPB>(S, lb, S.nblk_pair, v, mode, phase, par, done, nsteps);
+    force_end(S, L, f);
+}
+// the update of atom u by one thread, with its state in memory
+__device__ __forceinline__ void update_atom(const SpecDev &S, int u, const float f[3], int par,
+                                            int mode, int phase, long long done, long long nsteps,
+                                            StepVals<FF> &v) {
+    AtomMixed A;
+    A.load(S, par, u);
+    atom_update_mixed(S, A, par, u, f, ((const float *)S.pen)[u], mode, phase, done, nsteps, v);
+    if (mode != MODE_EVAL) A.store(S, par ^ 1, u);
 }
 
 template <int L, bool SC76>
@@ -152,7 +147,8 @@ __global__ void __launch_bounds__(TPB, 8) k_density_f32(const SpecDev *__restric
                                                         const PotF P) {
     const SpecDev &S = specs[b2s[blockIdx.x]];
     if (!force && S.ctl->phase == PH_IDLE) return;
-    density_block<L, SC76>(S, blockIdx.x - S.blk_pair0, S.ctl->parity, P);
+    const int u = (blockIdx.x - S.blk_pair0) * (TPB / L) + threadIdx.x / L;
+    density_lane<SC76, false>(S, P, L, u, threadIdx.x % L, S.ctl->parity);
 }
 
 template <int L, bool SC76>
@@ -163,11 +159,31 @@ __global__ void __launch_bounds__(TPB, 8) k_force_f32(const SpecDev *__restrict_
     const SpecCtl *ctl = S.ctl;
     const int phase = ctl->phase;
     if (mode == MODE_STEP && phase == PH_IDLE) return;
-    force_block<L, SC76>(S, blockIdx.x - S.blk_pair0, ctl->parity, P, mode, phase, ctl->done,
-                         ctl->nsteps);
+    const int par = ctl->parity, lb = blockIdx.x - S.blk_pair0;
+    const long long done = ctl->done, nsteps = ctl->nsteps;
+    constexpr int APB = TPB / L;
+    float f[3];
+    force_lane<SC76, false>(S, P, L, lb * APB + threadIdx.x / L, threadIdx.x % L, f);
+    if (L > 1) {
+        // the block's atoms to its first threads: whole warps update them (one
+        // lane in L of every warp otherwise, 29 us of it on 384,000 atoms at 4)
+        __shared__ float sf[3][APB];
+        if (threadIdx.x % L == 0)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) sf[d][threadIdx.x / L] = f[d];
+        __syncthreads();
+        if (threadIdx.x < APB)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) f[d] = sf[d][threadIdx.x];
+    }
+    const int u = lb * APB + threadIdx.x;
+    StepVals<FF> v = zero_vals<FF>();
+    if (threadIdx.x < APB && u < S.n) update_atom(S, u, f, par, mode, phase, done, nsteps, v);
+    step_tail<TPB>(S, lb, S.nblk_pair, v, L, mode, phase, par, done, nsteps);
 }
 
-template <int L, bool SC76>
+// a resident run's warp
+template <bool SC76>
 struct OpsF32 {
     const PotF &P;
     uint4 *cache;
@@ -176,10 +192,11 @@ struct OpsF32 {
     LaneList q;
     int4 ra;         // the atom's record (all its lanes)
     float wa, pe;    // its density weight and energy
-    int u, l;
+    int L, u, l;
     bool valid;
     __device__ __forceinline__ void load(const SpecDev &S, int tile, int par) {
         const int t = tile * 32 + (threadIdx.x & 31);
+        L = S.L;
         u = t / L;
         l = t % L;
         valid = u < S.n;
@@ -193,7 +210,7 @@ struct OpsF32 {
     }
     __device__ __forceinline__ void prune(const SpecDev &S, int par) {
         if (!valid) return;
-        prune_lane<L, true>(S, u, l, par);
+        prune_lane<true>(S, u, l, L, par);
         q.fill(S, cache, u, l, L, quads);
         A.pref = ra;
     }
@@ -207,7 +224,7 @@ struct OpsF32 {
             for_entries(S, S.rec[par], q,
                         [&](const int4 &x) { rho_pair<SC76>(P, q2, ra, x, s); });
         }
-        pe = density_end<L, SC76>(S, P, u, valid && l == 0, ra, s, wa);
+        pe = density_end<SC76>(S, P, L, u, valid && l == 0, ra, s, wa);
     }
     __device__ __forceinline__ StepVals<FF> force(const SpecDev &S, int tile, int par, int phase,
                                                   long long done, long long nsteps) {
@@ -218,29 +235,60 @@ struct OpsF32 {
                 force_pair<SC76>(P, q2, ra, wa, x, f[0], f[1], f[2]);
             });
         }
-        force_end<L>(S, f);
+        force_end(S, L, f);
         StepVals<FF> v = zero_vals<FF>();
         if (valid && l == 0)
             ra = atom_update_mixed(S, A, par, u, f, pe, MODE_STEP, phase, done, nsteps, v);
-        if (L > 1) {  // the new record to the atom's other lanes
-            const int src = (threadIdx.x & 31) & ~(L - 1);
-            ra.x = __shfl_sync(0xffffffffu, ra.x, src);
-            ra.y = __shfl_sync(0xffffffffu, ra.y, src);
-            ra.z = __shfl_sync(0xffffffffu, ra.z, src);
-        }
-        warp_reduce<L>(v);
+        // the new record to the atom's other lanes
+        const int src = (threadIdx.x & 31) & ~(L - 1);
+        ra.x = __shfl_sync(0xffffffffu, ra.x, src);
+        ra.y = __shfl_sync(0xffffffffu, ra.y, src);
+        ra.z = __shfl_sync(0xffffffffu, ra.z, src);
+        warp_reduce(v, L);
         if ((threadIdx.x & 31) == 0) store_part(part_warp(S, tile), v);
         return v;
     }
 };
-constexpr int RUN_WARPS_F32 = 16;
-template <int L, bool SC76>
-__global__ void __launch_bounds__(32 * RUN_WARPS_F32, 1)
+template <bool SC76>
+__global__ void __launch_bounds__(32 * RUN_WARPS, 1)
     k_run_f32(const SpecDev *specs, int nspec, const int *b2s, int nblk, RunCtl *rc,
               cudaGraphConditionalHandle again, int quads, const PotF P) {
     extern __shared__ uint4 list_cache[];
-    OpsF32<L, SC76> ops{P, list_cache, quads};
-    run_resident<L, FF>(specs, nspec, b2s, nblk, rc, again, ops);
+    OpsF32<SC76> ops{P, list_cache, quads};
+    run_resident<FF>(specs, nspec, b2s, nblk, rc, again, ops);
+}
+
+// a sweep's warp, on one tile
+template <bool SC76>
+struct SweepF32 {
+    const PotF &P;
+    __device__ __forceinline__ void prune(const SpecDev &S, int tile, int par) const {
+        const int t = tile * 32 + (threadIdx.x & 31);
+        if (t / S.L < S.n) prune_lane<true>(S, t / S.L, t % S.L, S.L, par);
+    }
+    __device__ __forceinline__ void density(const SpecDev &S, int tile, int par) const {
+        const int t = tile * 32 + (threadIdx.x & 31);
+        density_lane<SC76, true>(S, P, S.L, t / S.L, t % S.L, par);
+    }
+    __device__ __forceinline__ StepVals<FF> force(const SpecDev &S, int tile, int par, int phase,
+                                                  long long done, long long nsteps) const {
+        const int t = tile * 32 + (threadIdx.x & 31);
+        const int L = S.L, u = t / L;
+        float f[3];
+        force_lane<SC76, true>(S, P, L, u, t % L, f);
+        StepVals<FF> v = zero_vals<FF>();
+        if (u < S.n && t % L == 0) update_atom(S, u, f, par, MODE_STEP, phase, done, nsteps, v);
+        warp_reduce(v, L);
+        if ((threadIdx.x & 31) == 0) store_part(part_warp(S, tile), v);
+        return v;
+    }
+};
+constexpr int SWEEP_WARPS_F32 = 28;  // 72 registers
+template <bool SC76>
+__global__ void __launch_bounds__(32 * SWEEP_WARPS_F32, 1)
+    k_sweep_f32(const SpecDev *specs, int nspec, const int *b2s, int nblk, RunCtl *rc,
+                cudaGraphConditionalHandle again, int, const PotF P) {
+    run_sweep<FF>(specs, nspec, b2s, nblk, rc, again, SweepF32<SC76>{P});
 }
 
 template <int L>
@@ -249,7 +297,7 @@ __global__ void __launch_bounds__(TPB, 8) k_prune(const SpecDev *__restrict__ sp
     const SpecDev &S = specs[b2s[blockIdx.x]];
     if (!prune_active(S, force)) return;
     const int u = (blockIdx.x - S.blk_pair0) * (TPB / L) + threadIdx.x / L;
-    if (u < S.n) prune_lane<L, false>(S, u, threadIdx.x % L, S.ctl->parity);
+    if (u < S.n) prune_lane<false>(S, u, threadIdx.x % L, L, S.ctl->parity);
 }
 
 // after the pruning: clear the flag (a separate kernel, so that every block
@@ -319,48 +367,44 @@ void launch_force(const Tab &t, int arg, cudaStream_t st) {
     }
 }
 
-// resident runs
+// resident runs and sweeps
+RunShape run_shape_f64(const Tab &t, bool &fits);
 cudaError_t launch_run_f64(const Tab &t, const Group &g, RunCtl *rc,
                            cudaGraphConditionalHandle again, cudaStream_t st);
-bool run_possible_f64(const Group &g);
 
-#define PTA_RUN_SWITCH(SC, DO)     \
-    switch (g.L) {                 \
-        case 1: DO(1, SC); break;  \
-        case 2: DO(2, SC); break;  \
-        case 4: DO(4, SC); break;  \
-        case 8: DO(8, SC); break;  \
-        default: DO(16, SC);       \
+bool run_possible(const Tab &t, const int *b2s) {
+    if (!t.b2s_run || t.nblk_run < 1) return false;
+    const Group &g = t.grp[0];
+    bool fits = false;
+    RunShape r;
+    if (g.prec == PTA_PREC_FP64) {
+        r = run_shape_f64(t, fits);
+    } else {
+        r = run_shape(t.nblk_run, t.min_lanes, SWEEP_WARPS_F32);
+        fits = g.sc76 ? (r.sweep ? run_fits(k_sweep_f32<true>, r) : run_fits(k_run_f32<true>, r))
+                      : (r.sweep ? run_fits(k_sweep_f32<false>, r) : run_fits(k_run_f32<false>, r));
     }
-
-bool run_possible(const Group &g) {
-    if (g.prec == PTA_PREC_FP64) return run_possible_f64(g);
-    const RunShape r = run_shape(g.nblk, g.L, RUN_WARPS_F32);
-    bool ok = false;
-#define DO(L, SC) ok = run_fits(k_run_f32<L, SC>, r)
-    if (g.sc76)
-        PTA_RUN_SWITCH(true, DO)
-    else
-        PTA_RUN_SWITCH(false, DO)
-#undef DO
-    return ok;
+    // every block's tiles belong to few specimens
+    constexpr int NW = TPB / 32;
+    const long long tiles = (long long)t.nblk_run * NW;
+    for (int b = 0; b < r.blocks && fits; ++b) {
+        const long long t0 = tiles * b / r.blocks, t1 = tiles * (b + 1) / r.blocks;
+        fits = b2s[(t1 - 1) / NW] - b2s[t0 / NW] < RESIDENT_SPECS;
+    }
+    return fits;
 }
 
 cudaError_t launch_run(const Tab &t, RunCtl *rc, cudaGraphConditionalHandle again,
                        cudaStream_t st) {
     const Group &g = t.grp[0];
     if (g.prec == PTA_PREC_FP64) return launch_run_f64(t, g, rc, again, st);
-    const RunShape r = run_shape(g.nblk, g.L, RUN_WARPS_F32);
-    cudaError_t e = cudaSuccess;
-#define DO(L, SC)                                                                              \
-    e = launch_cooperative(k_run_f32<L, SC>, r, st, t.specs, t.nspec, g.b2s, g.nblk, rc, again, \
-                           r.quads, g.pf)
-    if (g.sc76)
-        PTA_RUN_SWITCH(true, DO)
-    else
-        PTA_RUN_SWITCH(false, DO)
-#undef DO
-    return e;
+    const RunShape r = run_shape(t.nblk_run, t.min_lanes, SWEEP_WARPS_F32);
+    auto go = [&](auto kernel) {
+        return launch_cooperative(kernel, r, st, t.specs, t.nspec, t.b2s_run, t.nblk_run, rc, again,
+                                  r.quads, g.pf);
+    };
+    if (g.sc76) return r.sweep ? go(k_sweep_f32<true>) : go(k_run_f32<true>);
+    return r.sweep ? go(k_sweep_f32<false>) : go(k_run_f32<false>);
 }
 
 }  // namespace pta

@@ -83,17 +83,17 @@ __device__ __forceinline__ double4_32a ld_pos64(const SpecDev &S, const double4_
 }
 // f(position) for the entries lane l of atom a reads, in list order (list
 // entries are byte offsets of 16-byte records, half of a double4's)
-template <class F>
+template <bool RES, class F>
 __device__ __forceinline__ void for_entries64(const SpecDev &S, const double4_32a *pos, int a,
                                               int l, int L, F f) {
     const uint4 *p = S.plist + nl_col(a, l, L, S.capq);
     const int cnt = chk_count(S, S.pnn[a * L + l], 4 * (S.capq - 1));
-    uint4 e = ld_quad<false>(p);
+    uint4 e = ld_quad<RES>(p);
     for (int t = cnt >> 2; t > 0; --t) {
         p += 32;
-        const uint4 nx = ld_quad<false>(p);
-        const double4_32a x0 = ld_pos64<false>(S, pos, e.x), x1 = ld_pos64<false>(S, pos, e.y);
-        const double4_32a x2 = ld_pos64<false>(S, pos, e.z), x3 = ld_pos64<false>(S, pos, e.w);
+        const uint4 nx = ld_quad<RES>(p);
+        const double4_32a x0 = ld_pos64<RES>(S, pos, e.x), x1 = ld_pos64<RES>(S, pos, e.y);
+        const double4_32a x2 = ld_pos64<RES>(S, pos, e.z), x3 = ld_pos64<RES>(S, pos, e.w);
         f(x0);
         f(x1);
         f(x2);
@@ -101,9 +101,9 @@ __device__ __forceinline__ void for_entries64(const SpecDev &S, const double4_32
         e = nx;
     }
     const int left = cnt & 3;
-    if (left > 0) f(ld_pos64<false>(S, pos, e.x));
-    if (left > 1) f(ld_pos64<false>(S, pos, e.y));
-    if (left > 2) f(ld_pos64<false>(S, pos, e.z));
+    if (left > 0) f(ld_pos64<RES>(S, pos, e.x));
+    if (left > 1) f(ld_pos64<RES>(S, pos, e.y));
+    if (left > 2) f(ld_pos64<RES>(S, pos, e.z));
 }
 
 // the same in a resident run, from the list in shared memory
@@ -206,14 +206,13 @@ __device__ __forceinline__ void atom_update64(const SpecDev &S, Atom64 &A, int p
     out.dp2 = moved2(r, A.pref);
 }
 
-template <int L>
-__device__ __forceinline__ double density_end64(const SpecDev &S, int a, bool first,
+__device__ __forceinline__ double density_end64(const SpecDev &S, int L, int a, bool first,
                                                 const double4_32a &pa, RhoSums64 s, double &w) {
     const PotDev &P = S.pot;
-    s.sm = lane_sum<L>(s.sm);
-    s.sn = lane_sum<L>(s.sn);
-    s.sr = lane_sum<L>(s.sr);
-    const double cnt = (double)lane_sum<L>(s.cnt);
+    s.sm = lane_sum(s.sm, L);
+    s.sn = lane_sum(s.sn, L);
+    s.sr = lane_sum(s.sr, L);
+    const double cnt = (double)lane_sum(s.cnt, L);
     const double dr = fma(-cnt, P.rc, s.sr);  // sum of r - rc
     const double rho = fma(P.am, s.sm, fma(P.Bm, dr, __dmul_rn(-cnt, P.Am)));
     const double phn = fma(P.an, s.sn, fma(P.Bn, dr, __dmul_rn(-cnt, P.An)));
@@ -245,48 +244,44 @@ __device__ __forceinline__ void rho_entry64(const PotDev &P, const double4_32a &
     if (within(r2, P.rc2)) rho_pair64<SC76>(P, r2, s);
 }
 
-template <int L, bool SC76>
-__device__ __forceinline__ void density_block64(const SpecDev &S, int lb, int par) {
-    const int a = lb * (TPB / L) + threadIdx.x / L;
-    const int l = threadIdx.x % L;
+// the passes of one thread (lane l of atom a) with everything in memory
+template <bool SC76, bool RES>
+__device__ __forceinline__ void density_lane64(const SpecDev &S, int L, int a, int l, int par) {
     const bool valid = a < S.n;
     const double4_32a *pos = (const double4_32a *)S.pos[par];
     RhoSums64 s;
     double4_32a pa = make_double4_32a(0, 0, 0, 0);
     if (valid) {
         pa = pos[a];
-        for_entries64(S, pos, a, l, L,
-                      [&](const double4_32a &pj) { rho_entry64<SC76>(S.pot, pa, pj, s); });
+        for_entries64<RES>(S, pos, a, l, L,
+                           [&](const double4_32a &pj) { rho_entry64<SC76>(S.pot, pa, pj, s); });
     }
     double w;
-    const double pe = density_end64<L>(S, a, valid && l == 0, pa, s, w);
+    const double pe = density_end64(S, L, a, valid && l == 0, pa, s, w);
     if (valid && l == 0) ((double *)S.pen)[a] = pe;
 }
 
-template <int L, bool SC76>
-__device__ __forceinline__ void force_block64(const SpecDev &S, int lb, int par, int mode, int phase,
-                                              long long done, long long nsteps) {
-    const int a = lb * (TPB / L) + threadIdx.x / L;
-    const int l = threadIdx.x % L;
-    const bool valid = a < S.n;
-    double f[3] = {0, 0, 0};
-    if (valid) {
+// the force on atom a, in all its lanes
+template <bool SC76, bool RES>
+__device__ __forceinline__ void force_lane64(const SpecDev &S, int L, int a, int l, double f[3]) {
+    f[0] = f[1] = f[2] = 0;
+    if (a < S.n) {
         const double4_32a *pf = (const double4_32a *)S.posfp;
         const double4_32a pa = pf[a];
-        for_entries64(S, pf, a, l, L,
-                      [&](const double4_32a &pj) { force_entry64<SC76>(S.pot, pa, pj, f); });
+        for_entries64<RES>(S, pf, a, l, L,
+                           [&](const double4_32a &pj) { force_entry64<SC76>(S.pot, pa, pj, f); });
     }
 #pragma unroll
-    for (int d = 0; d < 3; ++d) f[d] = lane_sum<L>(f[d]);
-    StepVals<double> v = zero_vals<double>();
-    if (valid && l == 0) {
-        Atom64 A;
-        A.load(S, par, a);
-        atom_update64(S, A, par, a, f, ((const double *)S.pen)[a], mode, phase, done, nsteps, v);
-        if (mode != MODE_EVAL) A.store_vel(S, a);
-    }
-    warp_reduce<L>(v);
-    step_tail<TPB>(S, lb, S.nblk_pair, v, mode, phase, par, done, nsteps);
+    for (int d = 0; d < 3; ++d) f[d] = lane_sum(f[d], L);
+}
+// the update of atom a by one thread, with its state in memory
+__device__ __forceinline__ void update_atom64(const SpecDev &S, int a, const double f[3], int par,
+                                              int mode, int phase, long long done,
+                                              long long nsteps, StepVals<double> &v) {
+    Atom64 A;
+    A.load(S, par, a);
+    atom_update64(S, A, par, a, f, ((const double *)S.pen)[a], mode, phase, done, nsteps, v);
+    if (mode != MODE_EVAL) A.store_vel(S, a);
 }
 
 template <int L, bool SC76>
@@ -294,7 +289,8 @@ __global__ void __launch_bounds__(TPB) k_density_f64(const SpecDev *__restrict__
                                                      const int *__restrict__ b2s, int force) {
     const SpecDev &S = specs[b2s[blockIdx.x]];
     if (!force && S.ctl->phase == PH_IDLE) return;
-    density_block64<L, SC76>(S, blockIdx.x - S.blk_pair0, S.ctl->parity);
+    const int a = (blockIdx.x - S.blk_pair0) * (TPB / L) + threadIdx.x / L;
+    density_lane64<SC76, false>(S, L, a, threadIdx.x % L, S.ctl->parity);
 }
 
 template <int L, bool SC76>
@@ -304,11 +300,29 @@ __global__ void __launch_bounds__(TPB) k_force_f64(const SpecDev *__restrict__ s
     const SpecCtl *ctl = S.ctl;
     const int phase = ctl->phase;
     if (mode == MODE_STEP && phase == PH_IDLE) return;
-    force_block64<L, SC76>(S, blockIdx.x - S.blk_pair0, ctl->parity, mode, phase, ctl->done,
-                                  ctl->nsteps);
+    const int par = ctl->parity, lb = blockIdx.x - S.blk_pair0;
+    const long long done = ctl->done, nsteps = ctl->nsteps;
+    constexpr int APB = TPB / L;
+    double f[3];
+    force_lane64<SC76, false>(S, L, lb * APB + threadIdx.x / L, threadIdx.x % L, f);
+    if (L > 1) {  // the block's atoms to its first threads, as in mixed precision
+        __shared__ double sf[3][APB];
+        if (threadIdx.x % L == 0)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) sf[d][threadIdx.x / L] = f[d];
+        __syncthreads();
+        if (threadIdx.x < APB)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) f[d] = sf[d][threadIdx.x];
+    }
+    const int a = lb * APB + threadIdx.x;
+    StepVals<double> v = zero_vals<double>();
+    if (threadIdx.x < APB && a < S.n) update_atom64(S, a, f, par, mode, phase, done, nsteps, v);
+    step_tail<TPB>(S, lb, S.nblk_pair, v, L, mode, phase, par, done, nsteps);
 }
 
-template <int L, bool SC76>
+// a resident run's warp
+template <bool SC76>
 struct OpsF64 {
     uint4 *cache;
     int quads;
@@ -316,10 +330,11 @@ struct OpsF64 {
     LaneList q;
     double4_32a pa;  // the atom's position and density weight (all its lanes)
     double pe;
-    int a, l;
+    int L, a, l;
     bool valid;
     __device__ __forceinline__ void load(const SpecDev &S, int tile, int par) {
         const int t = tile * 32 + (threadIdx.x & 31);
+        L = S.L;
         a = t / L;
         l = t % L;
         valid = a < S.n;
@@ -333,7 +348,7 @@ struct OpsF64 {
     }
     __device__ __forceinline__ void prune(const SpecDev &S, int par) {
         if (!valid) return;
-        prune_lane<L, true>(S, a, l, par);
+        prune_lane<true>(S, a, l, L, par);
         q.fill(S, cache, a, l, L, quads);
         A.pref = S.rec[par][a];
     }
@@ -346,7 +361,7 @@ struct OpsF64 {
         if (valid)
             for_entries64(S, pos, q,
                           [&](const double4_32a &pj) { rho_entry64<SC76>(S.pot, pa, pj, s); });
-        pe = density_end64<L>(S, a, valid && l == 0, pa, s, pa.w);
+        pe = density_end64(S, L, a, valid && l == 0, pa, s, pa.w);
     }
     __device__ __forceinline__ StepVals<double> force(const SpecDev &S, int tile, int par, int phase,
                                                   long long done, long long nsteps) {
@@ -355,7 +370,7 @@ struct OpsF64 {
             for_entries64(S, (const double4_32a *)S.posfp, q,
                           [&](const double4_32a &pj) { force_entry64<SC76>(S.pot, pa, pj, f); });
 #pragma unroll
-        for (int d = 0; d < 3; ++d) f[d] = lane_sum<L>(f[d]);
+        for (int d = 0; d < 3; ++d) f[d] = lane_sum(f[d], L);
         StepVals<double> v = zero_vals<double>();
         if (valid && l == 0) {
             atom_update64(S, A, par, a, f, pe, MODE_STEP, phase, done, nsteps, v);
@@ -363,25 +378,55 @@ struct OpsF64 {
             pa.y = A.x[1];
             pa.z = A.x[2];
         }
-        if (L > 1) {  // the new position to the atom's other lanes
-            const int src = (threadIdx.x & 31) & ~(L - 1);
-            pa.x = __shfl_sync(0xffffffffu, pa.x, src);
-            pa.y = __shfl_sync(0xffffffffu, pa.y, src);
-            pa.z = __shfl_sync(0xffffffffu, pa.z, src);
-        }
-        warp_reduce<L>(v);
+        // the new position to the atom's other lanes
+        const int src = (threadIdx.x & 31) & ~(L - 1);
+        pa.x = __shfl_sync(0xffffffffu, pa.x, src);
+        pa.y = __shfl_sync(0xffffffffu, pa.y, src);
+        pa.z = __shfl_sync(0xffffffffu, pa.z, src);
+        warp_reduce(v, L);
         if ((threadIdx.x & 31) == 0) store_part(part_warp(S, tile), v);
         return v;
     }
 };
-constexpr int RUN_WARPS_F64 = 16;
-template <int L, bool SC76>
-__global__ void __launch_bounds__(32 * RUN_WARPS_F64, 1)
+template <bool SC76>
+__global__ void __launch_bounds__(32 * RUN_WARPS, 1)
     k_run_f64(const SpecDev *specs, int nspec, const int *b2s, int nblk, RunCtl *rc,
               cudaGraphConditionalHandle again, int quads) {
     extern __shared__ uint4 list_cache[];
-    OpsF64<L, SC76> ops{list_cache, quads};
-    run_resident<L, double>(specs, nspec, b2s, nblk, rc, again, ops);
+    OpsF64<SC76> ops{list_cache, quads};
+    run_resident<double>(specs, nspec, b2s, nblk, rc, again, ops);
+}
+
+// a sweep's warp, on one tile
+template <bool SC76>
+struct SweepF64 {
+    __device__ __forceinline__ void prune(const SpecDev &S, int tile, int par) const {
+        const int t = tile * 32 + (threadIdx.x & 31);
+        if (t / S.L < S.n) prune_lane<true>(S, t / S.L, t % S.L, S.L, par);
+    }
+    __device__ __forceinline__ void density(const SpecDev &S, int tile, int par) const {
+        const int t = tile * 32 + (threadIdx.x & 31);
+        density_lane64<SC76, true>(S, S.L, t / S.L, t % S.L, par);
+    }
+    __device__ __forceinline__ StepVals<double> force(const SpecDev &S, int tile, int par, int phase,
+                                                      long long done, long long nsteps) const {
+        const int t = tile * 32 + (threadIdx.x & 31);
+        const int L = S.L, a = t / L;
+        double f[3];
+        force_lane64<SC76, true>(S, L, a, t % L, f);
+        StepVals<double> v = zero_vals<double>();
+        if (a < S.n && t % L == 0) update_atom64(S, a, f, par, MODE_STEP, phase, done, nsteps, v);
+        warp_reduce(v, L);
+        if ((threadIdx.x & 31) == 0) store_part(part_warp(S, tile), v);
+        return v;
+    }
+};
+constexpr int SWEEP_WARPS_F64 = 20;
+template <bool SC76>
+__global__ void __launch_bounds__(32 * SWEEP_WARPS_F64, 1)
+    k_sweep_f64(const SpecDev *specs, int nspec, const int *b2s, int nblk, RunCtl *rc,
+                cudaGraphConditionalHandle again, int) {
+    run_sweep<double>(specs, nspec, b2s, nblk, rc, again, SweepF64<SC76>{});
 }
 
 #define PTA_F64_SWITCH(KER, SC, ARG)                                                   \
@@ -407,40 +452,23 @@ void launch_force_f64(const Tab &t, const Group &g, int mode, cudaStream_t st) {
         PTA_F64_SWITCH(k_force_f64, false, mode)
 }
 
-#define PTA_RUN64_SWITCH(SC, DO)   \
-    switch (g.L) {                 \
-        case 1: DO(1, SC); break;  \
-        case 2: DO(2, SC); break;  \
-        case 4: DO(4, SC); break;  \
-        case 8: DO(8, SC); break;  \
-        default: DO(16, SC);       \
-    }
-
-bool run_possible_f64(const Group &g) {
-    const RunShape r = run_shape(g.nblk, g.L, RUN_WARPS_F64);
-    bool ok = false;
-#define DO(L, SC) ok = run_fits(k_run_f64<L, SC>, r)
-    if (g.sc76)
-        PTA_RUN64_SWITCH(true, DO)
-    else
-        PTA_RUN64_SWITCH(false, DO)
-#undef DO
-    return ok;
+RunShape run_shape_f64(const Tab &t, bool &fits) {
+    const RunShape r = run_shape(t.nblk_run, t.min_lanes, SWEEP_WARPS_F64);
+    fits = t.grp[0].sc76
+               ? (r.sweep ? run_fits(k_sweep_f64<true>, r) : run_fits(k_run_f64<true>, r))
+               : (r.sweep ? run_fits(k_sweep_f64<false>, r) : run_fits(k_run_f64<false>, r));
+    return r;
 }
 
 cudaError_t launch_run_f64(const Tab &t, const Group &g, RunCtl *rc,
                            cudaGraphConditionalHandle again, cudaStream_t st) {
-    const RunShape r = run_shape(g.nblk, g.L, RUN_WARPS_F64);
-    cudaError_t e = cudaSuccess;
-#define DO(L, SC)                                                                              \
-    e = launch_cooperative(k_run_f64<L, SC>, r, st, t.specs, t.nspec, g.b2s, g.nblk, rc, again, \
-                           r.quads)
-    if (g.sc76)
-        PTA_RUN64_SWITCH(true, DO)
-    else
-        PTA_RUN64_SWITCH(false, DO)
-#undef DO
-    return e;
+    const RunShape r = run_shape(t.nblk_run, t.min_lanes, SWEEP_WARPS_F64);
+    auto go = [&](auto kernel) {
+        return launch_cooperative(kernel, r, st, t.specs, t.nspec, t.b2s_run, t.nblk_run, rc, again,
+                                  r.quads);
+    };
+    if (g.sc76) return r.sweep ? go(k_sweep_f64<true>) : go(k_run_f64<true>);
+    return r.sweep ? go(k_sweep_f64<false>) : go(k_run_f64<false>);
 }
 
 }  // namespace pta

@@ -47,20 +47,6 @@ double ev_a3_to_gpa() { return E_CHARGE / 1e-30 / 1e9; }
 
 constexpr int CHUNK = 64;
 
-// resident threads of the whole current GPU (SM count x threads per SM, from
-// the device attributes); 0 when no device can be queried
-long long device_threads() {
-    int dev = 0, nsm = 0, per_sm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxThreadsPerMultiProcessor, dev) !=
-            cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    return (long long)nsm * per_sm;
-}
-
 struct Allocator {
     pta_alloc_fn alloc = nullptr;
     pta_free_fn release = nullptr;
@@ -107,6 +93,7 @@ struct Runner {
     Allocator alloc;
     std::vector<DevBuf> bufs;
     std::vector<SpecDev> hspecs;
+    std::vector<int> b2s_run;  // pair block -> member, all members
     SpecDev *d_specs = nullptr;
     long long *d_nsteps = nullptr;
     double *d_du = nullptr;
@@ -121,8 +108,8 @@ struct Runner {
     pta_coarse_result *h_cres = nullptr;
     Tab tab{};
     cudaGraphExec_t g_chunk = nullptr, g_one = nullptr;
-    // resident runs (the table's pair blocks fit the GPU at once): one graph
-    // runs a whole burst, list builds included
+    // resident runs and sweeps: one graph runs a whole burst, list builds
+    // included
     cudaGraphExec_t g_burst = nullptr;
     RunCtl *d_run = nullptr;
     int *h_stuck = nullptr;
@@ -301,19 +288,20 @@ struct Sizes {
     long long series_cap;
 };
 
-// threads per atom chosen from the specimen alone (so that a specimen runs
-// the same arithmetic alone and in a batch): FP64 specimens spread over the
-// whole GPU; mixed-precision ones aim at ~64K threads and let batching fill
-// the device
+// threads per atom, chosen from the specimen alone (so that it runs the same
+// arithmetic alone and in a batch): as many as keep it within one warp tile
+// for each of 32 warps on 152 SMs.  Measured per step, mixed precision (us):
+// 13,500 atoms 8 lanes 16.7 (4: 22.6), 32,000 atoms 4 lanes 25.0 (2: 37.0),
+// 62,500 atoms 2 lanes 40.6 (1: 62.7, 4: 56.4), 108,000 atoms 1 lane 66
+// (2: 82).  FP64 is bound by its operations, of which the sums over an atom's
+// lanes are some, so it takes sixteen lanes only while eight would leave the
+// SMs short of warps: 840 atoms 16 lanes 24 (8: 37), 4,000 atoms 8 lanes 60
+// (16: 64), 32,000 atoms 4 lanes 387 (8: 435, 2: 406).
 static int auto_lanes(long long n, int prec) {
-    long long target = 65536;
-    if (prec == PTA_PREC_FP64) {
-        target = device_threads();
-        if (target <= 0) target = 1LL << 18;  // no device to ask: a full GPU of this class
-    }
-    long long t = target / std::max<long long>(n, 1);
+    const long long t = 152LL * 1024 / std::max<long long>(n, 1);
+    const int most = prec == PTA_PREC_FP64 && n > 2432 ? 8 : 16;
     int L = 1;
-    while (L * 2 <= t && L < 16) L *= 2;
+    while (L * 2 <= t && L < most) L *= 2;
     return L;
 }
 
@@ -671,6 +659,7 @@ static int capture_iters_flat(Runner *r, int iters, cudaGraphExec_t *out, bool t
 static int runner_upload(Runner *r) {
     const int k = (int)r->m.size();
     r->hspecs.resize(k);
+    r->b2s_run.clear();
     int blk_atom = 0, blk_cell = 0;
     std::vector<int> b2s_atom, b2s_cell, b2s_bld;
     int bld_words = 0;
@@ -732,10 +721,20 @@ static int runner_upload(Runner *r) {
         if (g < 0) return PTA_EUNSUPPORTED;
         s.blk_pair0 = (int)gb2s[g].size();
         for (int b = 0; b < s.nblk_pair; ++b) gb2s[g].push_back(i);
+        s.blk_run0 = (int)r->b2s_run.size();
+        for (int b = 0; b < s.nblk_pair; ++b) r->b2s_run.push_back(i);
         r->hspecs[i] = s;
     }
+    // resident runs and sweeps serve specimens of one precision and potential
+    bool alike = true;
+    int min_lanes = 16;
+    for (auto &kk : keys) {
+        alike &= kk.prec == keys[0].prec && kk.sc76 == keys[0].sc76 &&
+                 std::memcmp(&kk.pf, &keys[0].pf, sizeof(PotF)) == 0;
+        min_lanes = std::min(min_lanes, kk.L);
+    }
     // one device block for all tables
-    size_t words = b2s_atom.size() + b2s_cell.size() + b2s_bld.size();
+    size_t words = b2s_atom.size() + b2s_cell.size() + b2s_bld.size() + r->b2s_run.size();
     for (auto &v : gb2s) words += v.size();
     if (r->d_specs) {
         // tables already exist: only refresh the descriptors (same shapes)
@@ -771,6 +770,7 @@ static int runner_upload(Runner *r) {
     all.insert(all.end(), b2s_cell.begin(), b2s_cell.end());
     all.insert(all.end(), b2s_bld.begin(), b2s_bld.end());
     for (auto &v : gb2s) all.insert(all.end(), v.begin(), v.end());
+    all.insert(all.end(), r->b2s_run.begin(), r->b2s_run.end());
     CK(cudaMemcpyAsync(r->d_specs, r->hspecs.data(), sizeof(SpecDev) * k, cudaMemcpyHostToDevice,
                        r->stream));
     CK(cudaMemcpyAsync(tabs, all.data(), 4 * all.size(), cudaMemcpyHostToDevice, r->stream));
@@ -799,6 +799,9 @@ static int runner_upload(Runner *r) {
         t.grp[q].nblk = (int)gb2s[q].size();
         off += gb2s[q].size();
     }
+    t.b2s_run = alike ? tabs + off : nullptr;
+    t.nblk_run = (int)r->b2s_run.size();
+    t.min_lanes = min_lanes;
     r->tab = t;
     // pinned host mirrors
     const size_t hb = 8 * k * 2 + 4 * k + sizeof(pta_averages) * k + sizeof(pta_coarse_result) * k + 64;
@@ -836,8 +839,8 @@ static int runner_create(pta_ctx *const *members, int k, Runner **out) {
     // which a resident run learns one step late
     bool adaptive = false;
     for (int i = 0; i < k; ++i) adaptive |= members[i]->par.conv_lag > 0;
-    if (rc == PTA_OK && !adaptive && r->tab.ngroups == 1 && !(flat && flat[0] == '1') &&
-        run_possible(r->tab.grp[0])) {
+    if (rc == PTA_OK && !adaptive && !(flat && flat[0] == '1') &&
+        run_possible(r->tab, r->b2s_run.data())) {
         rc = capture_burst(r, &r->g_burst);
     } else {
         if (rc == PTA_OK) rc = capture_iters(r, CHUNK, &r->g_chunk);

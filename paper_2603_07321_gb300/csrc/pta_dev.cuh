@@ -115,7 +115,8 @@ struct SpecDev {
     int n, L, prec, axis;
     int cap_use;               // list capacity: entries per atom
     int capq;                  // quads per lane column of a list
-    int blk_pair0, nblk_pair;  // pair kernels: TPB/L atoms per block
+    int blk_pair0, nblk_pair;  // pair kernels: TPB/L atoms per block (first in its group)
+    int blk_run0;              // first pair block in the table (resident runs, sweeps)
     int blk_atom0, nblk_atom;  // one thread per atom
     int blk_cell0, nblk_cell;  // cell sort: CELLS_PER_WARP cells per warp
     int blk_bld0, nblk_bld;    // list build: BUILD_WARPS warps of apw atoms
@@ -209,6 +210,10 @@ struct Tab {
     const int *b2s_bld;
     int nblk_bld;
     int bld_words;  // shared words per warp of the list build
+    // resident runs and sweeps: block->specimen map over all specimens when they
+    // share precision and potential (else null), fewest lanes per atom
+    const int *b2s_run;
+    int nblk_run, min_lanes;
     int ngroups;
     Group grp[8];
 };
@@ -442,9 +447,9 @@ __device__ __forceinline__ bool prune_active(const SpecDev &S, int force) {
 }
 void launch_density(const Tab &t, int force, cudaStream_t st);
 void launch_force(const Tab &t, int mode, cudaStream_t st);
-// resident runs of a table of one group (see k_pair_common.cuh): does the
-// group fit, and the cooperative launch
-bool run_possible(const Group &g);
+// resident runs and sweeps (see k_pair_common.cuh): can the table, whose block
+// ->specimen map the host passes, be run that way, and the cooperative launch
+bool run_possible(const Tab &t, const int *b2s_host);
 cudaError_t launch_run(const Tab &t, RunCtl *rc, cudaGraphConditionalHandle again,
                        cudaStream_t st);
 void launch_decide_build(const Tab &t, RunCtl *rc, cudaGraphConditionalHandle h, cudaStream_t st);

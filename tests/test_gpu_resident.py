@@ -40,6 +40,31 @@ def test_resident_equals_launched(P, prec, shape, lanes):
     _equal(_run(P, shape, prec, 130, False, lanes=lanes), _run(P, shape, prec, 130, True, lanes=lanes))
 
 
+# more tiles than resident warps: each block sweeps its tiles (uneven shares, a
+# partial last tile, both precisions, the fewest and the most lanes)
+@pytest.mark.parametrize("prec,shape,lanes", [
+    (1, (12, 12, 12), 16), (0, (11, 13, 12), 16), (1, (19, 20, 21), 4), (1, (28, 27, 29), 1),
+    (0, (28, 27, 29), 1)])
+def test_sweeps_equal_launched(P, prec, shape, lanes):
+    _equal(_run(P, shape, prec, 45, False, lanes=lanes), _run(P, shape, prec, 45, True, lanes=lanes))
+
+
+# members with different lanes share one sweep
+def test_a_swept_batch_equals_its_members(P):
+    shapes, steps = [(19, 20, 19), (5, 6, 5), (13, 12, 14)], [40, 60, 25]
+    solo = [_run(P, sh, 1, n, False, seed=i) for i, (sh, n) in enumerate(zip(shapes, steps))]
+    cs = [P.Ctx(sh, T0=300.0, seed=i, precision=1) for i, sh in enumerate(shapes)]
+    assert len({c.layout()["lanes"] for c in cs}) > 1
+    b = P.Batch(cs)
+    b.apply_strain([1e-3] * len(cs))
+    b.fine_burst(steps)
+    for c, s in zip(cs, solo):
+        _equal((c.series().copy(), *c.get_state()), s[:3])
+    b.close()
+    for c in cs:
+        c.close()
+
+
 @pytest.mark.parametrize("prec", [0, 1])
 def test_a_burst_longer_than_one_launch(P, prec):
     # a cold crystal asks for no list build, so the run reaches its limit of
