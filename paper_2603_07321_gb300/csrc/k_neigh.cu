@@ -22,13 +22,6 @@
 
 namespace pta {
 
-__device__ __forceinline__ bool build_active(const SpecDev &S, int force) {
-    const SpecCtl *c = S.ctl;
-    if (force) return true;
-    if (c->phase == PH_IDLE) return false;
-    return c->rebuild != 0 || c->list_L != S.L;
-}
-
 __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
 
 // position of atom a in FP64 (exact value of the stored representation)
@@ -85,6 +78,7 @@ __global__ void k_bin(const SpecDev *__restrict__ specs, const int *__restrict__
 __global__ void k_scan(const SpecDev *__restrict__ specs, int force) {
     const SpecDev &S = specs[blockIdx.x];
     if (!build_active(S, force)) return;
+    if (threadIdx.x == 0) S.ctl->max_nn = 0;  // the build takes the maximum
     scan_cells(S);
 }
 
@@ -361,16 +355,10 @@ __global__ void k_build_done(const SpecDev *__restrict__ specs, int force) {
     }
 }
 
-__global__ void k_reset_maxnn(const SpecDev *__restrict__ specs, int force) {
-    const SpecDev &S = specs[blockIdx.x];
-    if (!build_active(S, force)) return;
-    if (threadIdx.x == 0) S.ctl->max_nn = 0;
-}
-
 // one block: does any specimen of the table need a list build, or only a
 // pruning of its inner list, before its next pair pass?  Sets the condition
 // of the graph node that holds that work (LIST_BUILD, LIST_PRUNE, LIST_NONE).
-__global__ void k_decide_rebuild(const SpecDev *__restrict__ specs, int nspec,
+__global__ void k_decide_rebuild(const SpecDev *__restrict__ specs, int nspec, RunCtl *rc,
                                  cudaGraphConditionalHandle handle) {
     int build = 0, prune = 0;
     for (int s = threadIdx.x; s < nspec; s += blockDim.x) {
@@ -379,8 +367,10 @@ __global__ void k_decide_rebuild(const SpecDev *__restrict__ specs, int nspec,
     }
     build = __syncthreads_or(build);
     prune = __syncthreads_or(prune);
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0) {
+        rc->finished = 0;
         cudaGraphSetConditional(handle, build ? LIST_BUILD : (prune ? LIST_PRUNE : LIST_NONE));
+    }
 }
 
 // the same for resident runs, which prune by themselves: 1 when any specimen
@@ -400,8 +390,9 @@ void launch_decide_build(const Tab &t, RunCtl *rc, cudaGraphConditionalHandle h,
     k_decide_build<<<1, 128, 0, st>>>(t.specs, t.nspec, rc, h);
 }
 
-void launch_decide_rebuild(const Tab &t, cudaGraphConditionalHandle h, cudaStream_t st) {
-    k_decide_rebuild<<<1, 128, 0, st>>>(t.specs, t.nspec, h);
+void launch_decide_rebuild(const Tab &t, RunCtl *rc, cudaGraphConditionalHandle h,
+                           cudaStream_t st) {
+    k_decide_rebuild<<<1, 128, 0, st>>>(t.specs, t.nspec, rc, h);
 }
 
 int build_smem_limit(int bytes) {
@@ -410,7 +401,6 @@ int build_smem_limit(int bytes) {
 }
 
 void launch_rebuild(const Tab &t, int force, cudaStream_t st) {
-    k_reset_maxnn<<<t.nspec, 32, 0, st>>>(t.specs, force);
     k_bin<<<t.nblk_atom, TPB, 0, st>>>(t.specs, t.b2s_atom, force);
     k_scan<<<t.nspec, SCAN_THREADS, 0, st>>>(t.specs, force);
     k_scatter<<<t.nblk_atom, TPB, 0, st>>>(t.specs, t.b2s_atom, force);

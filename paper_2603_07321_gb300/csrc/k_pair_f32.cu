@@ -165,8 +165,8 @@ __global__ void __launch_bounds__(TPB, 8) k_force_f32(const SpecDev *__restrict_
     float f[3];
     force_lane<SC76, false>(S, P, L, lb * APB + threadIdx.x / L, threadIdx.x % L, f);
     if (L > 1) {
-        // the block's atoms to its first threads: whole warps update them (one
-        // lane in L of every warp otherwise, 29 us of it on 384,000 atoms at 4)
+        // the block's atoms to its first threads, so that whole warps update
+        // them and not one lane in L of every warp
         __shared__ float sf[3][APB];
         if (threadIdx.x % L == 0)
 #pragma unroll
@@ -179,11 +179,13 @@ __global__ void __launch_bounds__(TPB, 8) k_force_f32(const SpecDev *__restrict_
     const int u = lb * APB + threadIdx.x;
     StepVals<FF> v = zero_vals<FF>();
     if (threadIdx.x < APB && u < S.n) update_atom(S, u, f, par, mode, phase, done, nsteps, v);
-    step_tail<TPB>(S, lb, S.nblk_pair, v, L, mode, phase, par, done, nsteps);
+    block_partial<TPB>(S, lb, v, L);
 }
 
-// a resident run's warp
-template <bool SC76>
+// a resident run's warp; LT: the lanes per atom of every specimen, or 0.  Known,
+// they leave the sums over lanes without loops: 10.0
+// us (loops 10.7) per step of a specimen of 4,000 atoms at 16 lanes
+template <bool SC76, int LT>
 struct OpsF32 {
     const PotF &P;
     uint4 *cache;
@@ -192,11 +194,12 @@ struct OpsF32 {
     LaneList q;
     int4 ra;         // the atom's record (all its lanes)
     float wa, pe;    // its density weight and energy
-    int L, u, l;
+    int lanes, u, l;
     bool valid;
     __device__ __forceinline__ void load(const SpecDev &S, int tile, int par) {
         const int t = tile * 32 + (threadIdx.x & 31);
-        L = S.L;
+        lanes = S.L;
+        const int L = LT ? LT : lanes;
         u = t / L;
         l = t % L;
         valid = u < S.n;
@@ -210,6 +213,7 @@ struct OpsF32 {
     }
     __device__ __forceinline__ void prune(const SpecDev &S, int par) {
         if (!valid) return;
+        const int L = LT ? LT : lanes;
         prune_lane<true>(S, u, l, L, par);
         q.fill(S, cache, u, l, L, quads);
         A.pref = ra;
@@ -218,6 +222,7 @@ struct OpsF32 {
         if (valid && l == 0) A.store(S, par, u);
     }
     __device__ __forceinline__ void density(const SpecDev &S, int par) {
+        const int L = LT ? LT : lanes;
         RhoSums s;
         if (valid) {
             const float q2 = S.f_q2;
@@ -228,6 +233,7 @@ struct OpsF32 {
     }
     __device__ __forceinline__ StepVals<FF> force(const SpecDev &S, int tile, int par, int phase,
                                                   long long done, long long nsteps) {
+        const int L = LT ? LT : lanes;
         float f[3] = {0.f, 0.f, 0.f};
         if (valid) {
             const float q2 = S.f_q2;
@@ -249,12 +255,12 @@ struct OpsF32 {
         return v;
     }
 };
-template <bool SC76>
+template <bool SC76, int LT>
 __global__ void __launch_bounds__(32 * RUN_WARPS, 1)
     k_run_f32(const SpecDev *specs, int nspec, const int *b2s, int nblk, RunCtl *rc,
               cudaGraphConditionalHandle again, int quads, const PotF P) {
     extern __shared__ uint4 list_cache[];
-    OpsF32<SC76> ops{P, list_cache, quads};
+    OpsF32<SC76, LT> ops{P, list_cache, quads};
     run_resident<FF>(specs, nspec, b2s, nblk, rc, again, ops);
 }
 
@@ -300,17 +306,6 @@ __global__ void __launch_bounds__(TPB, 8) k_prune(const SpecDev *__restrict__ sp
     if (u < S.n) prune_lane<false>(S, u, threadIdx.x % L, L, S.ctl->parity);
 }
 
-// after the pruning: clear the flag (a separate kernel, so that every block
-// of the pruning kernel reads the same flag)
-__global__ void k_prune_done(const SpecDev *__restrict__ specs, int force) {
-    const SpecDev &S = specs[blockIdx.x];
-    if (!prune_active(S, force)) return;
-    if (threadIdx.x == 0) {
-        S.ctl->prune = 0;
-        S.ctl->prunes += 1;
-    }
-}
-
 void launch_prune(const Tab &t, int force, cudaStream_t st) {
     for (int i = 0; i < t.ngroups; ++i) {
         const Group &g = t.grp[i];
@@ -323,7 +318,49 @@ void launch_prune(const Tab &t, int force, cudaStream_t st) {
             default: k_prune<16><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, force); break;
         }
     }
-    k_prune_done<<<t.nspec, 32, 0, st>>>(t.specs, force);
+}
+
+// After the force pass: a block per specimen adds up its partials and advances
+// its control block; with `decide`, the last block also sets what list
+// maintenance the next step needs (counters of the specimens done and of those
+// that prune or build, in one word).
+__global__ void __launch_bounds__(32 * FINISH_WARPS)
+    k_finish(const SpecDev *__restrict__ specs, int nspec, int mode, RunCtl *rc, int decide,
+             cudaGraphConditionalHandle next) {
+    const SpecDev &S = specs[blockIdx.x];
+    SpecCtl *ctl = S.ctl;
+    const int phase = ctl->phase;
+    if (mode == MODE_EVAL || phase != PH_IDLE) {
+        const int par = ctl->parity;
+        const long long done = ctl->done, nsteps = ctl->nsteps;
+        if (S.prec == PTA_PREC_FP64) {
+            const StepVals<double> t = finish_sums<double>(S);
+            if (threadIdx.x == 0)
+                advance_ctl(S, t.s[0], t.s[1], t.s[2], t.d2, t.dp2, mode, phase, par, done, nsteps);
+        } else {
+            const StepVals<FF> t = finish_sums<FF>(S);
+            if (threadIdx.x == 0)
+                advance_ctl(S, to_double(t.s[0]), to_double(t.s[1]), to_double(t.s[2]), t.d2, t.dp2,
+                            mode, phase, par, done, nsteps);
+        }
+    }
+    if (!decide || threadIdx.x != 0) return;
+    constexpr int BITS = 21;
+    constexpr unsigned long long MASK = (1ull << BITS) - 1;
+    unsigned long long v = 1ull | (unsigned long long)prune_active(S, 0) << BITS |
+                           (unsigned long long)build_active(S, 0) << (2 * BITS);
+    v += atomicAdd(&rc->finished, v);
+    if ((v & MASK) != (unsigned long long)nspec) return;
+    rc->finished = 0;
+    cudaGraphSetConditional(next, v >> (2 * BITS)       ? LIST_BUILD
+                                  : (v >> BITS) & MASK ? LIST_PRUNE
+                                                       : LIST_NONE);
+}
+
+void launch_finish(const Tab &t, int mode, RunCtl *rc, const cudaGraphConditionalHandle *next,
+                   cudaStream_t st) {
+    k_finish<<<t.nspec, 32 * FINISH_WARPS, 0, st>>>(t.specs, t.nspec, mode, rc, next != nullptr,
+                                                    next ? *next : cudaGraphConditionalHandle());
 }
 
 // ---------------------------------------------------------------------------
@@ -381,8 +418,8 @@ bool run_possible(const Tab &t, const int *b2s) {
         r = run_shape_f64(t, fits);
     } else {
         r = run_shape(t.nblk_run, t.min_lanes, SWEEP_WARPS_F32);
-        fits = g.sc76 ? (r.sweep ? run_fits(k_sweep_f32<true>, r) : run_fits(k_run_f32<true>, r))
-                      : (r.sweep ? run_fits(k_sweep_f32<false>, r) : run_fits(k_run_f32<false>, r));
+        fits = g.sc76 ? (r.sweep ? run_fits(k_sweep_f32<true>, r) : run_fits(k_run_f32<true, 0>, r) && run_fits(k_run_f32<true, 16>, r))
+                      : (r.sweep ? run_fits(k_sweep_f32<false>, r) : run_fits(k_run_f32<false, 0>, r));
     }
     // every block's tiles belong to few specimens
     constexpr int NW = TPB / 32;
@@ -403,8 +440,9 @@ cudaError_t launch_run(const Tab &t, RunCtl *rc, cudaGraphConditionalHandle agai
         return launch_cooperative(kernel, r, st, t.specs, t.nspec, t.b2s_run, t.nblk_run, rc, again,
                                   r.quads, g.pf);
     };
-    if (g.sc76) return r.sweep ? go(k_sweep_f32<true>) : go(k_run_f32<true>);
-    return r.sweep ? go(k_sweep_f32<false>) : go(k_run_f32<false>);
+    if (r.sweep) return g.sc76 ? go(k_sweep_f32<true>) : go(k_sweep_f32<false>);
+    if (!g.sc76) return go(k_run_f32<false, 0>);
+    return t.ngroups == 1 && g.L == 16 ? go(k_run_f32<true, 16>) : go(k_run_f32<true, 0>);
 }
 
 }  // namespace pta

@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(TPB) k_force_f64(const SpecDev *__restrict__ s
     const int a = lb * APB + threadIdx.x;
     StepVals<double> v = zero_vals<double>();
     if (threadIdx.x < APB && a < S.n) update_atom64(S, a, f, par, mode, phase, done, nsteps, v);
-    step_tail<TPB>(S, lb, S.nblk_pair, v, L, mode, phase, par, done, nsteps);
+    block_partial<TPB>(S, lb, v, L);
 }
 
 // a resident run's warp

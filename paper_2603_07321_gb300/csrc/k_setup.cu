@@ -371,7 +371,6 @@ __global__ void k_burst_begin(const SpecDev *__restrict__ specs, const long long
     c->conv_mask = 0;
     c->rebuilds = 0;
     c->prunes = 0;
-    c->blocks_done = 0;
     // a burst always starts from a fresh neighbour list, so its result does
     // not depend on when earlier lists were built (checkpoints, batching)
     if (n > 0) c->rebuild = 1;

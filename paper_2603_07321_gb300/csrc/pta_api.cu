@@ -365,7 +365,7 @@ static int compute_sizes(const pta_specimen &s, const pta_potential &p, const pt
 // block and per group of 32 blocks; behind them the groups' counters
 static size_t part_bytes(const Sizes &z) {
     const size_t nb = (size_t)std::max(z.nblk_pair, z.nblk_atom);
-    return 32 * (TPB / 32) * nb + 4 * (nb / 32 + 1);
+    return 32 * (TPB / 32) * nb;
 }
 static size_t gpart_bytes(const Sizes &z) { return 32 * ((size_t)z.nblk_pair / 32 + 1); }
 
@@ -468,10 +468,10 @@ static void runner_free(Runner *r) {
 }
 
 // Graph of `iters` fine-step iterations.  Each iteration is
-//   [decide] -> SWITCH { 0: build + prune kernels, 1: prune kernels } -> density -> force
-// where the decide kernel sets the switch value on the device (2 when no
-// specimen needs either), so list maintenance costs no launch on the steps
-// that need none.  With `timed`, event-record nodes bracket the parts of each
+//   SWITCH { 0: build + prune kernels, 1: prune kernels } -> density -> force -> finish
+// where the finish kernel of the iteration before (a decide kernel ahead of
+// the first) sets the switch value on the device (2 when no specimen needs
+// either), so list maintenance costs no launch on the steps that need none.  With `timed`, event-record nodes bracket the parts of each
 // iteration (events cannot sit inside a conditional body, so the build
 // time is measured around the whole conditional).
 static int capture_iters_flat(Runner *r, int iters, cudaGraphExec_t *out, bool timed);
@@ -498,7 +498,7 @@ static int capture_iters(Runner *r, int iters, cudaGraphExec_t *out, bool timed 
     int rc = (e == cudaSuccess) ? PTA_OK : PTA_ECUDA;
     for (int i = 0; i < iters && rc == PTA_OK; ++i) {
         if (timed) cudaEventRecordWithFlags(r->ev[4 * i + 0], r->cap, cudaEventRecordExternal);
-        launch_decide_rebuild(r->tab, handles[i], r->cap);
+        if (i == 0) launch_decide_rebuild(r->tab, r->d_run, handles[0], r->cap);
         cudaStreamCaptureStatus cs;
         cudaGraph_t cg = nullptr;
         const cudaGraphNode_t *deps = nullptr;
@@ -541,6 +541,8 @@ static int capture_iters(Runner *r, int iters, cudaGraphExec_t *out, bool timed 
         launch_density(r->tab, 0, r->cap);
         if (timed) cudaEventRecordWithFlags(r->ev[4 * i + 2], r->cap, cudaEventRecordExternal);
         launch_force(r->tab, MODE_STEP, r->cap);
+        launch_finish(r->tab, MODE_STEP, r->d_run, i + 1 < iters ? &handles[i + 1] : nullptr,
+                      r->cap);
         if (timed) cudaEventRecordWithFlags(r->ev[4 * i + 3], r->cap, cudaEventRecordExternal);
     }
     cudaGraph_t gout = nullptr;
@@ -639,6 +641,7 @@ static int capture_iters_flat(Runner *r, int iters, cudaGraphExec_t *out, bool t
         launch_density(r->tab, 0, r->cap);
         if (timed) cudaEventRecordWithFlags(r->ev[4 * i + 2], r->cap, cudaEventRecordExternal);
         launch_force(r->tab, MODE_STEP, r->cap);
+        launch_finish(r->tab, MODE_STEP, r->d_run, nullptr, r->cap);
         if (timed) cudaEventRecordWithFlags(r->ev[4 * i + 3], r->cap, cudaEventRecordExternal);
     }
     cudaError_t e = cudaStreamEndCapture(r->cap, &g);
@@ -1582,6 +1585,7 @@ int pta_forces(pta_ctx *c, double *f, double *pe, int64_t n, double obs[3]) {
     if (c->hd.prune_first) launch_prune(r->tab, 1, c->stream);
     launch_density(r->tab, 1, c->stream);
     launch_force(r->tab, MODE_EVAL, c->stream);
+    launch_finish(r->tab, MODE_EVAL, nullptr, nullptr, c->stream);
     CKR(launch_check());
     std::vector<double> buf;
     if (f || pe) {
@@ -1742,7 +1746,6 @@ int pta_load_state(pta_ctx *c, const void *buf, size_t len) {
     o += sizeof(PtaDev);
     ctl.rebuild = 1;
     ctl.phase = PH_IDLE;
-    ctl.blocks_done = 0;
     const size_t n = (size_t)c->hd.n;
     const size_t p = (c->hd.prec == PTA_PREC_FP64) ? 32 : 16;
     const PermLayout Lo = perm_layout(n, c->hd.prec);

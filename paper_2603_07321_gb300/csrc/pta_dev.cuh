@@ -89,7 +89,6 @@ struct SpecCtl {
     int rebuild;     // 1: build the neighbour list before the next pair pass
     int err;         // sticky ErrBit mask
     long long nsteps, done;
-    unsigned int blocks_done;  // last-block counter of the force kernel
     int list_L;                // lanes the current list layout was built for
     int rebuilds;              // list builds in the current burst
     int max_nn;                // largest neighbour count at the last build
@@ -194,6 +193,7 @@ struct Group {
 // barrier's wait ran out.
 struct RunCtl {
     unsigned long long arrive, pad0[15];
+    unsigned long long finished, pad2[15];  // launched steps: see k_finish
     int stuck, pad1[31];
 };
 // what a step asks for, or what became of the run
@@ -436,10 +436,16 @@ void launch_force_rebuild_flag(const Tab &t, cudaStream_t st);
 void launch_rebuild(const Tab &t, int force, cudaStream_t st);
 int build_smem_limit(int bytes);  // allow k_build this much dynamic shared memory; 0 on failure
 void launch_prune(const Tab &t, int force, cudaStream_t st);
-void launch_decide_rebuild(const Tab &t, cudaGraphConditionalHandle h, cudaStream_t st);
+void launch_decide_rebuild(const Tab &t, RunCtl *rc, cudaGraphConditionalHandle h, cudaStream_t st);
 // list maintenance decided on the device: 0 build + prune, 1 prune, 2 nothing
 constexpr unsigned LIST_BUILD = 0, LIST_PRUNE = 1, LIST_NONE = 2;
 
+__device__ __forceinline__ bool build_active(const SpecDev &S, int force) {
+    const SpecCtl *c = S.ctl;
+    if (force) return true;
+    if (c->phase == PH_IDLE) return false;
+    return c->rebuild != 0 || c->list_L != S.L;
+}
 __device__ __forceinline__ bool prune_active(const SpecDev &S, int force) {
     if (!S.prune_on) return false;
     if (force) return true;
@@ -447,6 +453,9 @@ __device__ __forceinline__ bool prune_active(const SpecDev &S, int force) {
 }
 void launch_density(const Tab &t, int force, cudaStream_t st);
 void launch_force(const Tab &t, int mode, cudaStream_t st);
+// the step's end; next: handle of the next step's list maintenance, or null
+void launch_finish(const Tab &t, int mode, RunCtl *rc, const cudaGraphConditionalHandle *next,
+                   cudaStream_t st);
 // resident runs and sweeps (see k_pair_common.cuh): can the table, whose block
 // ->specimen map the host passes, be run that way, and the cooperative launch
 bool run_possible(const Tab &t, const int *b2s_host);

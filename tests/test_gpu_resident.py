@@ -65,6 +65,20 @@ def test_a_swept_batch_equals_its_members(P):
         c.close()
 
 
+# the sums of a launched pass: one group of blocks, several, a partial last one,
+# and more than one round of the finishing kernel (beyond 128 groups).  Each
+# atom's energy is one FP32 (FP64) number and the tree's error per level is
+# below 2^-44 (2^-53) of the sum of their sizes.
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("shape,lanes", [((2, 2, 3), 1), ((11, 9, 10), 1), ((20, 20, 21), 1),
+                                         ((21, 20, 20), 16)])
+def test_sums_of_a_launched_pass(P, prec, shape, lanes):
+    c = P.Ctx(shape, T0=300.0, seed=4, precision=prec, lanes=lanes)
+    f, pe, obs = c.forces()
+    assert abs(obs[1] - pe.sum(dtype=np.longdouble)) <= 24 * 2.0**-44 * np.abs(pe).sum()
+    c.close()
+
+
 @pytest.mark.parametrize("prec", [0, 1])
 def test_a_burst_longer_than_one_launch(P, prec):
     # a cold crystal asks for no list build, so the run reaches its limit of
