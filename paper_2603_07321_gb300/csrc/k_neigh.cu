@@ -7,7 +7,8 @@
 // of edge >= rc + skin; atoms outside the grid are clamped onto its border
 // cells, which keeps every pair within reach (clamping is non-expansive), and
 // are reported (PTA_ERANGE): the grid's margin is a quarter of the specimen's
-// extent, which no atom of a deforming specimen reaches.
+// extent, which no atom of a deforming specimen reaches.  Along x each cell is
+// cut in CELL_SPLIT, to fit a row's candidates to the radius.
 // After binning, the atoms themselves are permuted into cell order (cells in
 // rank order, atoms of a cell in creation order), so that
 // the 32 atoms of a warp share a cell and read overlapping neighbours, and a
@@ -52,6 +53,11 @@ __device__ __forceinline__ float3 load_pos32(const SpecDev &S, int par, int a) {
     return make_float3(h.x + l.x, h.y + l.y, h.z + l.z);
 }
 
+// an atom's place among its cell's atoms as they were counted, in the scratch
+__device__ __forceinline__ int *place_in_cell(const SpecDev &S) {
+    return (int *)((char *)S.perm_tmp + perm_layout(S.n, S.prec).cell);
+}
+
 __global__ void k_bin(const SpecDev *__restrict__ specs, const int *__restrict__ b2s, int force) {
     const SpecDev &S = specs[b2s[blockIdx.x]];
     if (!build_active(S, force)) return;
@@ -63,18 +69,17 @@ __global__ void k_bin(const SpecDev *__restrict__ specs, const int *__restrict__
     int ci[3];
     bool out = false;
     for (int d = 0; d < 3; ++d) {
-        const double q = floor((x[d] - S.org[d]) * S.inv_h);
+        const double q = floor((x[d] - S.org[d]) * (d == 0 ? S.inv_hx : S.inv_h));
         out |= !(q >= 0.0 && q < (double)S.nc[d]);
         ci[d] = clampi((int)fmax(fmin(q, 1e9), -1e9), 0, S.nc[d] - 1);
     }
     if (out) atomicOr(&S.ctl->err, ERR_GRID);
     const int c = cell_rank(S.nc, ci[0], ci[1], ci[2]);
     S.atom_cell[a] = c;
-    atomicAdd(&S.cell_cnt[c], 1);
+    place_in_cell(S)[a] = atomicAdd(&S.cell_cnt[c], 1);
 }
 
-// one block per specimen: exclusive scan of the cell counts; counts reset to
-// 0 for use as fill counters by the scatter
+// one block per specimen: exclusive scan of the cell counts
 __global__ void k_scan(const SpecDev *__restrict__ specs, int force) {
     const SpecDev &S = specs[blockIdx.x];
     if (!build_active(S, force)) return;
@@ -88,59 +93,46 @@ __global__ void k_scatter(const SpecDev *__restrict__ specs, const int *__restri
     if (!build_active(S, force)) return;
     const int a = (blockIdx.x - S.blk_atom0) * TPB + threadIdx.x;
     if (a >= S.n) return;
-    const int c = S.atom_cell[a];
-    const int slot = chk_index(S, S.cell_start[c] + atomicAdd(&S.cell_cnt[c], 1), S.n);
-    S.cell_tmp[slot] = a;
+    const int slot = chk_index(S, S.cell_start[S.atom_cell[a]] + place_in_cell(S)[a], S.n);
+    S.cell_tmp[slot] = make_int2(a, S.orig[a]);
 }
 
-// each warp orders CELLS_PER_WARP cells in turn (most cells of the grid's
-// margin are empty): a cell's atoms by creation index (rank = number of
-// smaller ones), so that the order within a cell, and with it every list
-// order, does not depend on how cells are numbered; then the cell's counter
-// is cleared for the next build
-__global__ void k_cell_sort(const SpecDev *__restrict__ specs, const int *__restrict__ b2s,
-                            int force) {
-    const SpecDev &S = specs[b2s[blockIdx.x]];
-    if (!build_active(S, force)) return;
-    const int lane = threadIdx.x & 31;
-    const int c0 = (blockIdx.x - S.blk_cell0) * CELL_WARPS * CELLS_PER_WARP + (threadIdx.x >> 5);
-    for (int i = 0; i < CELLS_PER_WARP; ++i) {
-        const int c = c0 + i * CELL_WARPS;
-        if (c >= S.ncell) return;
-        const int s = S.cell_start[c], e = S.cell_start[c + 1];
-        for (int p = s + lane; p < e; p += 32) {
-            const int v = chk_index(S, S.cell_tmp[chk_index(S, p, S.n)], S.n);
-            const int ov = S.orig[v];
-            int r = 0;
-            for (int q = s; q < e; ++q) r += (S.orig[chk_index(S, S.cell_tmp[chk_index(S, q, S.n)], S.n)] < ov);
-            S.cell_atoms[chk_index(S, s + r, S.n)] = v;
-        }
-        if (lane == 0) S.cell_cnt[c] = 0;
-    }
-}
-
-// sort the per-atom state into cell order: gather into scratch, then copy back
-__global__ void k_permute_gather(const SpecDev *__restrict__ specs, const int *__restrict__ b2s,
-                                 int force) {
+// orders every cell's atoms by creation index (rank = number of smaller ones),
+// so that the order within a cell, and with it every list order, does not
+// depend on how cells are numbered or counted; the per-atom state goes to its
+// place in the scratch, copied back by the next kernel.
+//
+// Bound: latency, and from ~100,000 atoms the state's bytes.  A thread per atom
+// reads the ~15 indices of its cell: 9 us for 52,700 atoms, 17 for 470,596.  A
+// warp per cell of four times the size, eight in turn, whose atoms' state a
+// further kernel moved, took 49 and 63 us.
+__global__ void k_order(const SpecDev *__restrict__ specs, const int *__restrict__ b2s, int force) {
     const SpecDev &S = specs[b2s[blockIdx.x]];
     if (!build_active(S, force)) return;
     const int p = (blockIdx.x - S.blk_atom0) * TPB + threadIdx.x;
     if (p >= S.n) return;
-    const int src = chk_index(S, S.cell_atoms[p], S.n);
     const int par = S.ctl->parity;
     const PermLayout Lo = perm_layout(S.n, S.prec);
     char *t = (char *)S.perm_tmp;
+    const int2 own = S.cell_tmp[p];
+    const int v = chk_index(S, own.x, S.n);
+    const int c = S.atom_cell[v];
+    const int s = S.cell_start[c], e = S.cell_start[c + 1];
+    int r = s;
+#pragma unroll 4
+    for (int q = s; q < e; ++q) r += S.cell_tmp[chk_index(S, q, S.n)].y < own.y;
+    r = chk_index(S, r, S.n);
     // velocities: 32-byte records in both precisions (double4 or VelHL)
-    ((double4_32a *)(t + Lo.vel))[p] = ((const double4_32a *)S.vel)[src];
+    ((double4_32a *)(t + Lo.vel))[r] = ((const double4_32a *)S.vel)[v];
     if (S.prec == PTA_PREC_FP64) {
-        ((double4_32a *)(t + Lo.pos))[p] = ((const double4_32a *)S.pos[par])[src];
+        ((double4_32a *)(t + Lo.pos))[r] = ((const double4_32a *)S.pos[par])[v];
     } else {
-        ((float4 *)(t + Lo.pos))[p] = ((const float4 *)S.pos[par])[src];
-        ((float4 *)(t + Lo.lo))[p] = S.lo[par][src];
+        ((float4 *)(t + Lo.pos))[r] = ((const float4 *)S.pos[par])[v];
+        ((float4 *)(t + Lo.lo))[r] = S.lo[par][v];
     }
-    ((uint8_t *)(t + Lo.flags))[p] = S.flags[src];
-    ((int *)(t + Lo.orig))[p] = S.orig[src];
-    ((int *)(t + Lo.cell))[p] = S.atom_cell[src];
+    ((uint8_t *)(t + Lo.flags))[r] = S.flags[v];
+    ((int *)(t + Lo.orig))[r] = own.y;
+    ((int *)(t + Lo.cell))[r] = c;
 }
 
 __global__ void k_permute_scatter(const SpecDev *__restrict__ specs, const int *__restrict__ b2s,
@@ -183,14 +175,14 @@ __device__ __noinline__ bool in_list_exact(const SpecDev &S, int par, int a, int
 // consecutive slots of a row of cells at a time (coalesced record reads) and
 // compact the hits in slot order through ballots into shared memory, near
 // entries from the front, far ones from the back.  Rows and cells that the
-// list radius cannot reach from the atom's place in its cell are skipped
-// (about a quarter of the 27 cells' candidates).  The near entries are then
+// list radius cannot reach from the atom's place in its cell are skipped.  The near entries are then
 // arranged by slot % 8 (see the list format) and both parts written as quads.
 //
-// Bound: instruction issue (candidate tests).  One thread per atom over the
-// same 27 cells, which this replaces, ran 1,674 tests in sequence: ~1.33 ms
-// for 470,596 atoms and a latency of ~0.1 ms for small specimens.
-__global__ void __launch_bounds__(BUILD_WARPS * 32) k_build(const SpecDev *__restrict__ specs,
+// Bound: instruction issue (80% of the slots; 2,700 instructions per atom, over
+// half of them candidate tests).  470,596 atoms: 1.28 ms (1.69 with undivided
+// cells, divisions by the lane count and 72 registers; at 64 registers eight
+// blocks share an SM), 52,700 atoms 145 us (187).
+__global__ void __launch_bounds__(BUILD_WARPS * 32, 8) k_build(const SpecDev *__restrict__ specs,
                                                            const int *__restrict__ b2s,
                                                            int force, int words) {
     extern __shared__ uint4 bsh4[];
@@ -199,15 +191,17 @@ __global__ void __launch_bounds__(BUILD_WARPS * 32) k_build(const SpecDev *__res
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const int cap = S.cap_use, L = S.L, n = S.n, par = S.ctl->parity;
+    const int sL = 31 - __clz(L);  // L is a power of two
     unsigned *buf = (unsigned *)bsh4 + (size_t)w * words;  // cap entries
     unsigned *out = buf + cap;                             // near part in list order
     int *cls = (int *)(out + cap + 128);                   // 8 counters
     const int4 *__restrict__ rec = S.rec[par];
-    const float h = S.f_h, lo2 = S.f_rl2q_lo, hi2 = S.f_rl2q_hi, ra2 = S.f_ra2q;
+    const float h = S.f_h, hi2 = S.f_rl2q_hi, ra2 = S.f_ra2q;
+    float lo2 = S.f_rl2q_lo;
     constexpr unsigned EMPTY = 0xffffffffu;
     // an atom beyond the cell grid may be farther from a candidate than the
     // records' period allows: then every hit is confirmed in FP64
-    const bool sure = !(S.ctl->err & ERR_GRID);
+    if (S.ctl->err & ERR_GRID) lo2 = 0.f;
     int most = 0;
     for (int i = 0; i < S.apw; ++i) {
         const int a = ((blockIdx.x - S.blk_bld0) * BUILD_WARPS + w) * S.apw + i;
@@ -222,7 +216,7 @@ __global__ void __launch_bounds__(BUILD_WARPS * 32) k_build(const SpecDev *__res
             const int yy = cy + dy, zz = cz + dz;
             const float sl = S.f_reach_slack;
             const float3 x = load_pos32(S, par, a);
-            const float px = x.x - S.f_org[0] - (float)cx * h;
+            const float px = x.x - S.f_org[0] - (float)cx * S.f_hx;
             const float py = x.y - S.f_org[1] - (float)cy * h;
             const float pz = x.z - S.f_org[2] - (float)cz * h;
             const float ey = dy == 0 ? 0.f : fmaxf((dy < 0 ? py : h - py) - sl, 0.f);
@@ -230,47 +224,50 @@ __global__ void __launch_bounds__(BUILD_WARPS * 32) k_build(const SpecDev *__res
             const float rem = S.f_reach2 - ey * ey - ez * ez;
             if (rem > 0.f && yy >= 0 && zz >= 0 && yy < S.nc[1] && zz < S.nc[2]) {
                 const float reach = sqrtf(rem) + sl;
-                const int x0 = (cx > 0 && px < reach) ? cx - 1 : cx;
-                const int x1 = (cx + 1 < S.nc[0] && h - px < reach) ? cx + 1 : cx;
+                // (the atom's own cell in any case: one beyond the grid is
+                // counted in the cell at its edge)
+                const int x0 = min(max(cx + (int)floorf((px - reach) * S.f_inv_hx), 0), cx);
+                const int x1 = max(min(cx + (int)floorf((px + reach) * S.f_inv_hx), S.nc[0] - 1), cx);
                 const int r0 = cell_rank(S.nc, x0, yy, zz), r1 = cell_rank(S.nc, x1, yy, zz);
                 rs = chk_count(S, S.cell_start[min(r0, r1)], n);
                 re = chk_count(S, S.cell_start[max(r0, r1) + 1], n);
             }
         }
-        int na = 0, nb = 0, tot = 0;  // stored near and far entries; all found
+        int na = 0, stored = 0, tot = 0;  // near and all entries stored; all found
         for (int r = 0; r < 9; ++r) {
             const int s = __shfl_sync(0xffffffffu, rs, r), e = __shfl_sync(0xffffffffu, re, r);
             if (s >= e) continue;
-            int4 nx = rec[min(s + lane, e - 1)];
-            for (int b = s; b < e; b += 32) {
+            int j = s + lane;
+            int4 nx = rec[min(j, e - 1)];
+            for (int b = s; b < e; b += 32, j += 32) {
                 const int4 rj = nx;
-                const int j = b + lane;
                 if (b + 32 < e) nx = rec[min(j + 32, e - 1)];
                 const float fx = (float)(rj.x - ra.x), fy = (float)(rj.y - ra.y),
                             fz = (float)(rj.z - ra.z);
                 const float r2 = fmaf(fz, fz, fmaf(fy, fy, fx * fx));
                 bool in = r2 < hi2 && j < e && j != a;
-                if (in && (r2 >= lo2 || !sure)) in = in_list_exact(S, par, a, j);
+                if (in && r2 >= lo2) in = in_list_exact(S, par, a, j);
                 const unsigned ml = __ballot_sync(0xffffffffu, in);
                 if (!ml) continue;
-                const unsigned ma = __ballot_sync(0xffffffffu, in && r2 < ra2);
-                const int k = __popc(ml);
-                tot += k;
-                if (na + nb + k > cap) continue;  // reported below
-                if (in) {
-                    if (r2 < ra2) buf[na + __popc(ma & lt)] = nl_entry(j);
-                    else buf[cap - 1 - nb - __popc(ml & ~ma & lt)] = nl_entry(j);
-                }
+                const bool near = r2 < ra2;
+                const unsigned ma = __ballot_sync(0xffffffffu, in && near);
+                const int nb = stored - na;
+                tot += __popc(ml);
+                if (tot > cap) continue;  // reported below
+                stored = tot;
+                const int k = __popc((near ? ma : ml ^ ma) & lt);
+                if (in) buf[near ? na + k : cap - 1 - nb - k] = nl_entry(j);
                 na += __popc(ma);
-                nb += k - __popc(ma);
             }
         }
+        const int nb = stored - na;
         most = max(most, tot);
         // near part: lane l gets rows [0, na / L + (l < na % L))
-        const int rows = na / L, rest = na % L;
+        const int rows = na >> sL, rest = na & (L - 1);
         const int lane0 = (int)(((long long)a * L) & 31);
         const int cells = ((rows + 4) >> 2) * 4 * L;
-        for (int m = lane; m < cells; m += 32) out[m] = EMPTY;
+        for (int m = lane; m < cells / 4; m += 32)
+            ((uint4 *)out)[m] = make_uint4(EMPTY, EMPTY, EMPTY, EMPTY);
         if (lane < 8) cls[lane] = 0;
         __syncwarp();
         int nov = 0;  // entries whose class has no row left
@@ -285,7 +282,7 @@ __global__ void __launch_bounds__(BUILD_WARPS * 32) k_build(const SpecDev *__res
             __syncwarp();
             if (act && rank == 0) cls[c] = base + __popc(peers);
             const int t = base + rank, li = t & (L - 1);
-            const int row = 8 * (t / L) + ((c - lane0 - li) & 7);
+            const int row = 8 * (t >> sL) + ((c - lane0 - li) & 7);
             const bool ok = act && row < rows + (li < rest);
             if (ok) out[((row >> 2) * L + li) * 4 + (row & 3)] = e;
             const unsigned mo = __ballot_sync(0xffffffffu, act && !ok);
@@ -296,7 +293,7 @@ __global__ void __launch_bounds__(BUILD_WARPS * 32) k_build(const SpecDev *__res
         // the rows left empty take them, in order
         for (int m0 = 0, got = 0; got < nov && m0 < cells; m0 += 32) {
             const int m = m0 + lane;
-            const int li = (m >> 2) & (L - 1), row = (m / (4 * L)) * 4 + (m & 3);
+            const int li = (m >> 2) & (L - 1), row = (m >> (sL + 2)) * 4 + (m & 3);
             const bool hole = m < cells && row < rows + (li < rest) && out[m] == EMPTY;
             const unsigned mh = __ballot_sync(0xffffffffu, hole);
             const int q = got + __popc(mh & lt);
@@ -305,29 +302,29 @@ __global__ void __launch_bounds__(BUILD_WARPS * 32) k_build(const SpecDev *__res
         }
         __syncwarp();
         uint4 *dst = S.plist + nl_col(a, 0, L, S.capq);
-        for (int m = lane; m < cells / 4; m += 32) dst[(m / L) * 32 + (m & (L - 1))] = ((uint4 *)out)[m];
+        for (int m = lane; m < cells / 4; m += 32) dst[(m >> sL) * 32 + (m & (L - 1))] = ((uint4 *)out)[m];
         // far part, entry k in lane k % L
         if (S.prune_on) {
             uint4 *far = S.nlist + nl_col(a, 0, L, S.capq);
-            const int qb = ((nb + L - 1) / L + 3) >> 2;
+            const int qb = (((nb + L - 1) >> sL) + 3) >> 2;
             for (int m = lane; m < qb * L; m += 32) {
                 unsigned v[4];
 #pragma unroll
                 for (int s = 0; s < 4; ++s) {
-                    const int k = ((m / L) * 4 + s) * L + (m & (L - 1));
+                    const int k = (((m >> sL) * 4 + s) << sL) + (m & (L - 1));
                     v[s] = k < nb ? buf[cap - 1 - k] : 0u;  // slot 0 where there is none
                 }
-                far[(m / L) * 32 + (m & (L - 1))] = make_uint4(v[0], v[1], v[2], v[3]);
+                far[(m >> sL) * 32 + (m & (L - 1))] = make_uint4(v[0], v[1], v[2], v[3]);
             }
             if (lane < L) S.pnn[a * L + lane] = rows + (lane < rest);
         } else {
             __syncwarp();
             for (int k = lane; k < nb; k += 32) {
-                const int l = k & (L - 1), row = rows + (l < rest) + k / L;
+                const int l = k & (L - 1), row = rows + (l < rest) + (k >> sL);
                 ((unsigned *)(dst + (row >> 2) * 32 + l))[row & 3] = buf[cap - 1 - k];
             }
             if (lane < L)
-                S.pnn[a * L + lane] = rows + (lane < rest) + (nb > lane ? (nb - lane + L - 1) / L : 0);
+                S.pnn[a * L + lane] = rows + (lane < rest) + (nb > lane ? (nb - lane + L - 1) >> sL : 0);
         }
         if (lane == 0) {
             S.nab[a] = make_int2(na, nb);
@@ -404,8 +401,7 @@ void launch_rebuild(const Tab &t, int force, cudaStream_t st) {
     k_bin<<<t.nblk_atom, TPB, 0, st>>>(t.specs, t.b2s_atom, force);
     k_scan<<<t.nspec, SCAN_THREADS, 0, st>>>(t.specs, force);
     k_scatter<<<t.nblk_atom, TPB, 0, st>>>(t.specs, t.b2s_atom, force);
-    k_cell_sort<<<t.nblk_cell, CELL_WARPS * 32, 0, st>>>(t.specs, t.b2s_cell, force);
-    k_permute_gather<<<t.nblk_atom, TPB, 0, st>>>(t.specs, t.b2s_atom, force);
+    k_order<<<t.nblk_atom, TPB, 0, st>>>(t.specs, t.b2s_atom, force);
     k_permute_scatter<<<t.nblk_atom, TPB, 0, st>>>(t.specs, t.b2s_atom, force);
     k_build<<<t.nblk_bld, BUILD_WARPS * 32, BUILD_WARPS * t.bld_words * 4, st>>>(
         t.specs, t.b2s_bld, force, t.bld_words);

@@ -279,7 +279,7 @@ static PotDev make_pot(const pta_potential &p) {
 // ---------------------------------------------------------------------------
 struct Sizes {
     long long n;
-    int L, capq, cap_use, nblk_pair, nblk_atom, nblk_cell, nblk_bld, apw, ncell, nc[3];
+    int L, capq, cap_use, nblk_pair, nblk_atom, nblk_bld, apw, split, ncell, nc[3];
     int prune_on, mean_pos;
     double prune_margin;
     double h, org[3];
@@ -349,8 +349,12 @@ static int compute_sizes(const pta_specimen &s, const pta_potential &p, const pt
         ncell *= z->nc[d];
     }
     if (ncell > (1LL << 30)) return PTA_EINVAL;
-    z->ncell = (int)ncell;
-    z->nblk_cell = (z->ncell + CELL_WARPS * CELLS_PER_WARP - 1) / (CELL_WARPS * CELLS_PER_WARP);
+    // cells are shorter along x, the direction in which the list build walks
+    // them, and so fits its walk to the list radius: a row takes on average
+    // 2 reach + h / split of the rows' atoms instead of 2 reach + h
+    z->split = ncell * CELL_SPLIT <= (1LL << 30) ? CELL_SPLIT : 1;
+    z->nc[0] *= z->split;
+    z->ncell = (int)(ncell * z->split);
     const long long W = 32 / z->L;
     z->list_quads = (size_t)((z->n + W - 1) / W) * 32 * z->capq;
     // records: the finest quantum whose half period, 2^31 quanta, exceeds the
@@ -390,8 +394,7 @@ static size_t footprint(const Sizes &z, int prec) {
     add(4 * n);                      // atom_cell
     add(4 * (size_t)z.ncell);        // cell_cnt
     add(4 * ((size_t)z.ncell + 1));  // cell_start
-    add(4 * n);                      // cell_tmp
-    add(4 * n);                      // cell_atoms
+    add(8 * n);                      // cell_tmp
     add(4 * n);                      // orig
     add(perm_layout(n, prec).total); // permutation scratch
     add(16 * z.list_quads);          // plist
@@ -663,8 +666,8 @@ static int runner_upload(Runner *r) {
     const int k = (int)r->m.size();
     r->hspecs.resize(k);
     r->b2s_run.clear();
-    int blk_atom = 0, blk_cell = 0;
-    std::vector<int> b2s_atom, b2s_cell, b2s_bld;
+    int blk_atom = 0;
+    std::vector<int> b2s_atom, b2s_bld;
     int bld_words = 0;
     // launch groups by (precision, lanes, potential); the potential's FP32
     // constants are kernel parameters of the group's launches
@@ -690,9 +693,6 @@ static int runner_upload(Runner *r) {
         s.blk_atom0 = blk_atom;
         blk_atom += s.nblk_atom;
         for (int b = 0; b < s.nblk_atom; ++b) b2s_atom.push_back(i);
-        s.blk_cell0 = blk_cell;
-        blk_cell += s.nblk_cell;
-        for (int b = 0; b < s.nblk_cell; ++b) b2s_cell.push_back(i);
         s.blk_bld0 = (int)b2s_bld.size();
         for (int b = 0; b < s.nblk_bld; ++b) b2s_bld.push_back(i);
         // candidates, near part in list order, class counters
@@ -737,7 +737,7 @@ static int runner_upload(Runner *r) {
         min_lanes = std::min(min_lanes, kk.L);
     }
     // one device block for all tables
-    size_t words = b2s_atom.size() + b2s_cell.size() + b2s_bld.size() + r->b2s_run.size();
+    size_t words = b2s_atom.size() + b2s_bld.size() + r->b2s_run.size();
     for (auto &v : gb2s) words += v.size();
     if (r->d_specs) {
         // tables already exist: only refresh the descriptors (same shapes)
@@ -770,7 +770,6 @@ static int runner_upload(Runner *r) {
     r->d_run = (RunCtl *)c;
     std::vector<int> all;
     all.insert(all.end(), b2s_atom.begin(), b2s_atom.end());
-    all.insert(all.end(), b2s_cell.begin(), b2s_cell.end());
     all.insert(all.end(), b2s_bld.begin(), b2s_bld.end());
     for (auto &v : gb2s) all.insert(all.end(), v.begin(), v.end());
     all.insert(all.end(), r->b2s_run.begin(), r->b2s_run.end());
@@ -782,16 +781,14 @@ static int runner_upload(Runner *r) {
     t.nspec = k;
     t.b2s_atom = tabs;
     t.nblk_atom = (int)b2s_atom.size();
-    t.b2s_cell = tabs + b2s_atom.size();
-    t.nblk_cell = (int)b2s_cell.size();
-    t.b2s_bld = tabs + b2s_atom.size() + b2s_cell.size();
+    t.b2s_bld = tabs + b2s_atom.size();
     t.nblk_bld = (int)b2s_bld.size();
     t.bld_words = bld_words;
     if (!build_smem_limit(BUILD_WARPS * bld_words * 4)) {
         cudaGetLastError();
         return PTA_ECUDA;
     }
-    size_t off = b2s_atom.size() + b2s_cell.size() + b2s_bld.size();
+    size_t off = b2s_atom.size() + b2s_bld.size();
     t.ngroups = (int)keys.size();
     for (size_t q = 0; q < keys.size(); ++q) {
         t.grp[q].prec = keys[q].prec;
@@ -1182,8 +1179,7 @@ static int ctx_alloc_all(pta_ctx *c, const Sizes &z) {
     AL(atom_cell, 4 * n, int *);
     AL(cell_cnt, 4 * (size_t)z.ncell, int *);
     AL(cell_start, 4 * ((size_t)z.ncell + 1), int *);
-    AL(cell_tmp, 4 * n, int *);
-    AL(cell_atoms, 4 * n, int *);
+    AL(cell_tmp, 8 * n, int2 *);
     AL(orig, 4 * n, int *);
     AL(perm_tmp, perm_layout(n, c->par.precision).total, void *);
     AL(plist, 16 * z.list_quads, uint4 *);
@@ -1249,7 +1245,6 @@ int pta_create(const pta_specimen *spec, const pta_potential *pot, double T0, ui
     s.apw = z.apw;
     s.nblk_pair = z.nblk_pair;
     s.nblk_atom = z.nblk_atom;
-    s.nblk_cell = z.nblk_cell;
     for (int d = 0; d < 3; ++d) {
         s.ncl[d] = c->spec.n_cells[d];
         s.org[d] = z.org[d];
@@ -1257,9 +1252,12 @@ int pta_create(const pta_specimen *spec, const pta_potential *pot, double T0, ui
     }
     s.a0 = c->spec.a0;
     s.grip_width = c->spec.grip_width;
-    s.hcell = z.h;
+    const double hx = z.h / z.split;
     s.inv_h = 1.0 / z.h;
+    s.inv_hx = 1.0 / hx;
     s.f_h = (float)z.h;
+    s.f_hx = (float)hx;
+    s.f_inv_hx = (float)(1.0 / hx);
     const double rq = std::ldexp(1.0, z.rec_bits);
     s.f_rq = (float)rq;
     s.f_q = (float)(1.0 / rq);
@@ -1268,7 +1266,7 @@ int pta_create(const pta_specimen *spec, const pta_potential *pot, double T0, ui
     double extent = 0;  // largest coordinate of the cell grid
     for (int d = 0; d < 3; ++d) {
         s.f_org[d] = (float)z.org[d];
-        extent = std::max(extent, std::fabs(z.org[d]) + z.nc[d] * z.h);
+        extent = std::max(extent, std::fabs(z.org[d]) + z.nc[d] * (d == 0 ? hx : z.h));
     }
     s.ncell = z.ncell;
     const double rl = c->pot.rc + c->par.skin;

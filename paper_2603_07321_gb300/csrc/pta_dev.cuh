@@ -16,8 +16,7 @@
 namespace pta {
 
 constexpr int TPB = 128;        // threads per block of the atom and pair kernels
-constexpr int CELL_WARPS = 8;   // warps per block of the cell-sort kernel
-constexpr int CELLS_PER_WARP = 8;  // cells one warp of the cell-sort kernel orders in turn
+constexpr int CELL_SPLIT = 4;   // cells along x per cell edge along y and z
 constexpr int SCAN_THREADS = 1024;
 constexpr int BUILD_WARPS = 4;  // warps per block of the list build
 
@@ -117,7 +116,6 @@ struct SpecDev {
     int blk_pair0, nblk_pair;  // pair kernels: TPB/L atoms per block (first in its group)
     int blk_run0;              // first pair block in the table (resident runs, sweeps)
     int blk_atom0, nblk_atom;  // one thread per atom
-    int blk_cell0, nblk_cell;  // cell sort: CELLS_PER_WARP cells per warp
     int blk_bld0, nblk_bld;    // list build: BUILD_WARPS warps of apw atoms
     int apw;
     int spec_index;            // index of this specimen in the launch table
@@ -126,12 +124,12 @@ struct SpecDev {
     double a0, grip_width;
     // cell grid
     double org[3];
-    double hcell, inv_h;
+    double inv_h, inv_hx;      // cell edges along y and z, along x
     int nc[3];
     int ncell;
     // list radius (rc + skin)^2
     double rl2;
-    float f_h;
+    float f_h, f_hx, f_inv_hx;
     // fixed-point records: quanta per A, A per quantum and its square, shift
     // from the 2^-12 A grid of hi to quanta; grid origin
     float f_rq, f_q, f_q2, f_org[3];
@@ -160,7 +158,8 @@ struct SpecDev {
     void *vel;      // FP64: double4; MIXED: VelHL
     uint8_t *flags;
     int4 *ref;      // records at the last list build (skin test)
-    int *atom_cell, *cell_cnt, *cell_start, *cell_tmp, *cell_atoms;
+    int *atom_cell, *cell_cnt, *cell_start;
+    int2 *cell_tmp;    // atoms by cell, {slot, creation index}
     int *orig;        // original index (creation order) of the atom stored at each slot
     void *perm_tmp;   // scratch of the permutation that sorts atoms by cell
     uint4 *plist;     // what the pair passes read: near part, then the pruned far part
@@ -205,8 +204,6 @@ struct Tab {
     int nspec;
     const int *b2s_atom;
     int nblk_atom;
-    const int *b2s_cell;
-    int nblk_cell;
     const int *b2s_bld;
     int nblk_bld;
     int bld_words;  // shared words per warp of the list build
@@ -369,49 +366,62 @@ __host__ __device__ inline PermLayout perm_layout(size_t n, int prec) {
 
 // one block of SCAN_THREADS threads per specimen: exclusive scan of the cell
 // counts into cell_start (cell_start[ncell] = total); the counts are reset to
-// 0 for use as fill counters by a scatter; the specimen's build count + 1
+// 0 for the next build; the specimen's build count + 1.  Each warp scans a
+// contiguous part, four cells per lane (cells along each axis are even in
+// number), behind a first reading of the parts' sums.
 __device__ __forceinline__ void scan_cells(const SpecDev &S) {
-    __shared__ int wsum[SCAN_THREADS / 32];
-    __shared__ int carry;
-    if (threadIdx.x == 0) carry = 0;
+    constexpr int NW = SCAN_THREADS / 32;
+    __shared__ int wsum[NW];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, n = S.ncell / 4;
+    int4 *cnt = (int4 *)S.cell_cnt, *start = (int4 *)S.cell_start;
+    const int part = ((n + NW - 1) / NW + 31) & ~31;
+    const int c0 = min(w * part, n), c1 = min(c0 + part, n);
+    int sum = 0;
+#pragma unroll 8
+    for (int c = c0 + lane; c < c1; c += 32) {
+        const int4 v = cnt[c];
+        sum += (v.x + v.y) + (v.z + v.w);
+    }
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if (lane == 0) wsum[w] = sum;
     __syncthreads();
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int base = 0; base < S.ncell; base += SCAN_THREADS) {
-        const int c = base + threadIdx.x;
-        const int v = (c < S.ncell) ? S.cell_cnt[c] : 0;
-        int x = v;
+    if (w == 0) {
+        const int v = wsum[lane];
+        int s = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += y;
+        }
+        wsum[lane] = s - v;
+        if (lane == 31) {
+            S.cell_start[S.ncell] = s;
+            S.ctl->rebuilds += 1;
+#if PTA_CHECK
+            if (s != S.n) atomicOr(&S.ctl->err, ERR_CHECK);  // every atom in one cell
+#endif
+        }
+    }
+    __syncthreads();
+    int carry = wsum[w];
+    const int4 zero = make_int4(0, 0, 0, 0);
+    int4 nx = c0 + lane < c1 ? cnt[c0 + lane] : zero;
+    for (int c = c0 + lane; c - lane < c1; c += 32) {
+        const int4 v = nx;
+        nx = c + 32 < c1 ? cnt[c + 32] : zero;
+        const int own = (v.x + v.y) + (v.z + v.w);
+        int x = own;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
         }
-        if (lane == 31) wsum[w] = x;
-        __syncthreads();
-        if (w == 0) {
-            int s = wsum[lane];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, s, o);
-                if (lane >= o) s += y;
-            }
-            wsum[lane] = s;  // inclusive over warps
+        if (c < c1) {
+            const int b = carry + x - own;
+            start[c] = make_int4(b, b + v.x, b + v.x + v.y, b + v.x + v.y + v.z);
+            cnt[c] = zero;
         }
-        __syncthreads();
-        const int excl = carry + (w ? wsum[w - 1] : 0) + x - v;
-        if (c < S.ncell) {
-            S.cell_start[c] = excl;
-            S.cell_cnt[c] = 0;
-        }
-        __syncthreads();
-        if (threadIdx.x == SCAN_THREADS - 1) carry = excl + v;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        S.cell_start[S.ncell] = carry;
-        S.ctl->rebuilds += 1;
-#if PTA_CHECK
-        if (carry != S.n) atomicOr(&S.ctl->err, ERR_CHECK);  // every atom in one cell
-#endif
+        carry += __shfl_sync(0xffffffffu, x, 31);
     }
 }
 

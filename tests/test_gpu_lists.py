@@ -86,3 +86,29 @@ def test_an_atom_one_record_period_away_is_no_neighbour(P, oracle, prec):
     assert np.array_equal(c_gpu, c_ref)
     assert sorted_rows(c_gpu, l_gpu) == sorted_rows(c_ref, l_ref)
     ctx.close()
+
+
+@pytest.mark.parametrize("prec,shape,lanes", [(0, (7, 4, 5), 1), (1, (4, 9, 3), 4), (1, (1, 1, 40), 2),
+                                              (0, (40, 1, 3), 16)])
+def test_lists_of_crowded_and_far_flung_atoms(P, oracle, prec, shape, lanes):
+    # more atoms in a place than a warp holds, atoms spread over the grid's
+    # margin and beyond every face of it (counted in the cells at its edge), and
+    # atoms one grid step on either side of a cell's edge
+    rng = np.random.default_rng(lanes)
+    ctx = P.Ctx(shape, T0=0.0, precision=prec, lanes=lanes)
+    pos = on_grid(PI.jittered_fcc(shape, 0.2, seed=lanes))
+    n = len(pos)
+    pick = rng.permutation(n)
+    size = 3.615 * np.array(shape)
+    crowd, far = pick[:min(48, n // 4)], pick[-min(60, n // 4):]
+    pos[crowd] = 0.5 * size + rng.uniform(-0.7, 0.7, (len(crowd), 3))
+    pos[far] = rng.uniform(-1.5 * size - 40.0, 2.5 * size + 40.0, (len(far), 3))
+    edge = pick[len(crowd):len(crowd) + 8]
+    pos[edge, 0] = np.round(pos[edge, 0] / 2.8) * 2.8 + 2.0**-12 * np.tile([-1, 1], 4)
+    pos = on_grid(pos)
+    ctx.set_state(pos, np.zeros_like(pos))
+    c_gpu, l_gpu = ctx.neighbours(cap=512)
+    c_ref, l_ref = oracle.pairs(pos, ctx.potential.rc + ctx.params.skin, cap=512, method="brute")
+    assert np.array_equal(c_gpu, c_ref)
+    assert sorted_rows(c_gpu, l_gpu) == sorted_rows(c_ref, l_ref)
+    ctx.close()
