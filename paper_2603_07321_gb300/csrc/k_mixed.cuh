@@ -182,7 +182,7 @@ __device__ __forceinline__ int4 atom_update_mixed(const SpecDev &S, AtomMixed &A
     };
     if (mode == MODE_EVAL) {
         kinetic();
-        ((double4_32a *)S.eval_out)[S.orig[a]] = make_double4_32a(f[0], f[1], f[2], pe);
+        eval_store(S, a, f[0], f[1], f[2], pe);
         return make_int4(0, 0, 0, 0);
     }
     // thermal relaxation: the right grip moves along the load axis only (its

@@ -169,11 +169,23 @@ __device__ __forceinline__ void block_partial(const SpecDev &S, int lb, StepVals
     }
 }
 
+// MODE_EVAL: force and energy of atom a in the arrays of pta_forces
+__device__ __forceinline__ void eval_store(const SpecDev &S, int a, double fx, double fy, double fz,
+                                           double pe) {
+    const int o = S.orig[a];
+    double *f = S.eval_out + 3LL * o;
+    f[0] = fx;
+    f[1] = fy;
+    f[2] = fz;
+    S.eval_out[3LL * S.n + o] = pe;
+}
+
 // One thread: the specimen's control block after a step with these totals.
 //   MODE_STEP, phase RUN:     sample (K, U, T) into the series, step count + 1,
 //                             burst over after nsteps samples
 //   MODE_STEP, phase REFRESH: forces refreshed and the first step started
-//   MODE_EVAL:                K, U, T stored in eval_obs
+//   MODE_EVAL:                K, U, T and the error bits stored behind the
+//                             atoms' forces and energies
 // and in MODE_STEP the position buffers swap, the skin test sets the
 // rebuild flag and the pruning margin test the prune flag.
 __device__ inline void advance_ctl(const SpecDev &S, double K, double U, double R, float md2,
@@ -186,9 +198,11 @@ __device__ inline void advance_ctl(const SpecDev &S, double K, double U, double 
         c->prunes += 1;
     }
     if (mode == MODE_EVAL) {
-        c->eval_obs[0] = K;
-        c->eval_obs[1] = U;
-        c->eval_obs[2] = T;
+        double *o = S.eval_out + 4LL * S.n;
+        o[0] = K;
+        o[1] = U;
+        o[2] = T;
+        o[3] = c->err;
         c->rebuild = 0;
         return;
     }

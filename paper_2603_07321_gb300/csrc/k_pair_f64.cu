@@ -167,7 +167,7 @@ __device__ __forceinline__ void atom_update64(const SpecDev &S, Atom64 &A, int p
     };
     if (mode == MODE_EVAL) {
         kinetic();
-        ((double4_32a *)S.eval_out)[S.orig[a]] = make_double4_32a(f[0], f[1], f[2], pe);
+        eval_store(S, a, f[0], f[1], f[2], pe);
         return;
     }
     const double kh = S.acc_half;

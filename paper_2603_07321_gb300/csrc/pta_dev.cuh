@@ -102,7 +102,6 @@ struct SpecCtl {
     int relax;                 // 1: thermal relaxation, right grip free along the load axis
     double grip_du;            // continuous loading: the right grip moves this far (A) along
                                // the load axis with every step (0: held fixed)
-    double eval_obs[3];        // K, U, T of the last MODE_EVAL pass
     double mb[8];              // scratch of the Maxwell-Boltzmann set-up
     pta_averages last;         // averages of the last finished burst
     PtaDev pta;
@@ -173,7 +172,7 @@ struct SpecDev {
     double *gpart;      // per group of 32 blocks (resident runs)
     double *series;     // series_cap x 3 samples of the current burst
     long long series_cap;
-    double *eval_out;   // n x 4: F, pe (MODE_EVAL)
+    double *eval_out;   // MODE_EVAL, creation order: n x 3 F, n pe, then K, U, T, error bits
     double *rsum;       // n x 4, creation order: sums of the sampled positions of the
                         // burst (Eq. (mean_pos)); null unless asked for
     double *stage;      // n x 6 doubles: import/export staging
