@@ -7,7 +7,7 @@
 // positions are an exact FP32 pair x = hi + lo (hi on a 2^-12 A grid, |lo| <=
 // 2^-13 A); velocities an exact FP32 pair v = vh + vl (|vl| <= ulp(vh) / 2) updated by
 // error-free addition, so that half-kicks lose nothing to rounding over long
-// bursts; K, U and R are converted to FP64 per atom and reduced in FP64.
+// bursts; K, U and R are summed in error-free pairs of floats.
 #pragma once
 
 #include "k_pair_common.cuh"

@@ -141,17 +141,20 @@ __device__ __forceinline__ void update_atom(const SpecDev &S, int u, const float
     if (mode != MODE_EVAL) A.store(S, par ^ 1, u);
 }
 
-template <int L, bool SC76>
+// the launched passes; LT: the lanes per atom of every specimen of the launch,
+// or 0
+template <int LT, bool SC76>
 __global__ void __launch_bounds__(TPB, 8) k_density_f32(const SpecDev *__restrict__ specs,
                                                         const int *__restrict__ b2s, int force,
                                                         const PotF P) {
     const SpecDev &S = specs[b2s[blockIdx.x]];
     if (!force && S.ctl->phase == PH_IDLE) return;
+    const int L = LT ? LT : S.L;
     const int u = (blockIdx.x - S.blk_pair0) * (TPB / L) + threadIdx.x / L;
     density_lane<SC76, false>(S, P, L, u, threadIdx.x % L, S.ctl->parity);
 }
 
-template <int L, bool SC76>
+template <int LT, bool SC76>
 __global__ void __launch_bounds__(TPB, 8) k_force_f32(const SpecDev *__restrict__ specs,
                                                       const int *__restrict__ b2s, int mode,
                                                       const PotF P) {
@@ -161,13 +164,13 @@ __global__ void __launch_bounds__(TPB, 8) k_force_f32(const SpecDev *__restrict_
     if (mode == MODE_STEP && phase == PH_IDLE) return;
     const int par = ctl->parity, lb = blockIdx.x - S.blk_pair0;
     const long long done = ctl->done, nsteps = ctl->nsteps;
-    constexpr int APB = TPB / L;
+    const int L = LT ? LT : S.L, APB = TPB / L;
     float f[3];
     force_lane<SC76, false>(S, P, L, lb * APB + threadIdx.x / L, threadIdx.x % L, f);
     if (L > 1) {
         // the block's atoms to its first threads, so that whole warps update
         // them and not one lane in L of every warp
-        __shared__ float sf[3][APB];
+        __shared__ float sf[3][TPB / (LT ? LT : 2)];
         if (threadIdx.x % L == 0)
 #pragma unroll
             for (int d = 0; d < 3; ++d) sf[d][threadIdx.x / L] = f[d];
@@ -297,11 +300,12 @@ __global__ void __launch_bounds__(32 * SWEEP_WARPS_F32, 1)
     run_sweep<FF>(specs, nspec, b2s, nblk, rc, again, SweepF32<SC76>{P});
 }
 
-template <int L>
+template <int LT>
 __global__ void __launch_bounds__(TPB, 8) k_prune(const SpecDev *__restrict__ specs,
                                                   const int *__restrict__ b2s, int force) {
     const SpecDev &S = specs[b2s[blockIdx.x]];
     if (!prune_active(S, force)) return;
+    const int L = LT ? LT : S.L;
     const int u = (blockIdx.x - S.blk_pair0) * (TPB / L) + threadIdx.x / L;
     if (u < S.n) prune_lane<false>(S, u, threadIdx.x % L, L, S.ctl->parity);
 }
@@ -311,6 +315,7 @@ void launch_prune(const Tab &t, int force, cudaStream_t st) {
         const Group &g = t.grp[i];
         if (g.nblk <= 0) continue;
         switch (g.L) {
+            case 0: k_prune<0><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, force); break;
             case 1: k_prune<1><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, force); break;
             case 2: k_prune<2><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, force); break;
             case 4: k_prune<4><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, force); break;
@@ -371,6 +376,7 @@ void launch_force_f64(const Tab &t, const Group &g, int mode, cudaStream_t st);
 
 #define PTA_L_SWITCH(KER, SC)                                                            \
     switch (g.L) {                                                                       \
+        case 0: KER<0, SC><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, arg, g.pf); break;    \
         case 1: KER<1, SC><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, arg, g.pf); break;    \
         case 2: KER<2, SC><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, arg, g.pf); break;    \
         case 4: KER<4, SC><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, arg, g.pf); break;    \

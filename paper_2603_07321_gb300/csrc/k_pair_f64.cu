@@ -284,16 +284,17 @@ __device__ __forceinline__ void update_atom64(const SpecDev &S, int a, const dou
     if (mode != MODE_EVAL) A.store_vel(S, a);
 }
 
-template <int L, bool SC76>
+template <int LT, bool SC76>
 __global__ void __launch_bounds__(TPB) k_density_f64(const SpecDev *__restrict__ specs,
                                                      const int *__restrict__ b2s, int force) {
     const SpecDev &S = specs[b2s[blockIdx.x]];
     if (!force && S.ctl->phase == PH_IDLE) return;
+    const int L = LT ? LT : S.L;
     const int a = (blockIdx.x - S.blk_pair0) * (TPB / L) + threadIdx.x / L;
     density_lane64<SC76, false>(S, L, a, threadIdx.x % L, S.ctl->parity);
 }
 
-template <int L, bool SC76>
+template <int LT, bool SC76>
 __global__ void __launch_bounds__(TPB) k_force_f64(const SpecDev *__restrict__ specs,
                                                    const int *__restrict__ b2s, int mode) {
     const SpecDev &S = specs[b2s[blockIdx.x]];
@@ -302,11 +303,11 @@ __global__ void __launch_bounds__(TPB) k_force_f64(const SpecDev *__restrict__ s
     if (mode == MODE_STEP && phase == PH_IDLE) return;
     const int par = ctl->parity, lb = blockIdx.x - S.blk_pair0;
     const long long done = ctl->done, nsteps = ctl->nsteps;
-    constexpr int APB = TPB / L;
+    const int L = LT ? LT : S.L, APB = TPB / L;
     double f[3];
     force_lane64<SC76, false>(S, L, lb * APB + threadIdx.x / L, threadIdx.x % L, f);
     if (L > 1) {  // the block's atoms to its first threads, as in mixed precision
-        __shared__ double sf[3][APB];
+        __shared__ double sf[3][TPB / (LT ? LT : 2)];
         if (threadIdx.x % L == 0)
 #pragma unroll
             for (int d = 0; d < 3; ++d) sf[d][threadIdx.x / L] = f[d];
@@ -431,6 +432,7 @@ __global__ void __launch_bounds__(32 * SWEEP_WARPS_F64, 1)
 
 #define PTA_F64_SWITCH(KER, SC, ARG)                                                   \
     switch (g.L) {                                                                     \
+        case 0: KER<0, SC><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, ARG); break;        \
         case 1: KER<1, SC><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, ARG); break;        \
         case 2: KER<2, SC><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, ARG); break;        \
         case 4: KER<4, SC><<<g.nblk, TPB, 0, st>>>(t.specs, g.b2s, ARG); break;        \

@@ -559,11 +559,4 @@ void launch_pta_update(const Tab &t, const int *ops, pta_coarse_result *out, cud
     k_pta_update<<<t.nspec, 32, 0, st>>>(t.specs, ops, out);
 }
 
-__global__ void k_force_rebuild(const SpecDev *__restrict__ specs) {
-    if (threadIdx.x == 0) specs[blockIdx.x].ctl->rebuild = 1;
-}
-void launch_force_rebuild_flag(const Tab &t, cudaStream_t st) {
-    k_force_rebuild<<<t.nspec, 32, 0, st>>>(t.specs);
-}
-
 }  // namespace pta

@@ -2,13 +2,15 @@
 // launch tables, CUDA-graph replay of the fine-step loop, batches.
 //
 // The fine-step loop of one iteration is
-//     [neighbour-list build, skipped on the device unless needed]
-//     [density pass] [force pass + fused velocity Verlet + step reduction]
+//     [neighbour-list build or pruning, skipped on the device unless needed]
+//     [density pass] [force pass + fused velocity Verlet] [step reduction]
 // for every specimen of a launch table at once.  Its kernels read each
 // specimen's phase and step counter from device memory, so the same
 // captured graph serves every burst length: a burst of n steps is n + 1
 // iterations (one force refresh, then n steps), replayed as chunks of a
-// graph of CHUNK iterations plus single iterations.
+// graph of CHUNK iterations plus single iterations; or, for tables small
+// enough (run_possible), run as a loop inside one cooperative kernel from
+// one list build to the next.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -669,22 +671,35 @@ static int runner_upload(Runner *r) {
     int blk_atom = 0;
     std::vector<int> b2s_atom, b2s_bld;
     int bld_words = 0;
-    // launch groups by (precision, lanes, potential); the potential's FP32
-    // constants are kernel parameters of the group's launches
+    // launch groups by (precision, potential); the potential's FP32 constants
+    // are kernel parameters of the group's launches.  A group whose specimens
+    // differ in lanes per atom has L = 0 and runs kernels that read them: a
+    // launch per lane count left the GPU to a few blocks at a time (a step of
+    // seven specimens of 4,000 to 256,000 atoms: 288 us, now 228).
     struct Key {
         int prec, L, sc76;
         PotF pf;
     };
-    std::vector<Key> keys;
-    std::vector<std::vector<int>> gb2s;
+    std::vector<Key> keys, kinds;  // kinds: distinct in lanes too
+    std::vector<std::vector<int>> gb2s, members;
+    auto same = [](const Key &a, const Key &b) {
+        return a.prec == b.prec && a.sc76 == b.sc76 && std::memcmp(&a.pf, &b.pf, sizeof(PotF)) == 0;
+    };
     auto group_of = [&](const Key &kk) -> int {
+        bool known = false;
+        for (const Key &q : kinds) known |= same(q, kk) && q.L == kk.L;
+        if (!known) {
+            if (kinds.size() >= 8) return -1;
+            kinds.push_back(kk);
+        }
         for (size_t q = 0; q < keys.size(); ++q)
-            if (keys[q].prec == kk.prec && keys[q].L == kk.L && keys[q].sc76 == kk.sc76 &&
-                std::memcmp(&keys[q].pf, &kk.pf, sizeof(PotF)) == 0)
+            if (same(keys[q], kk)) {
+                if (keys[q].L != kk.L) keys[q].L = 0;
                 return (int)q;
-        if (keys.size() >= 8) return -1;
+            }
         keys.push_back(kk);
         gb2s.emplace_back();
+        members.emplace_back();
         return (int)keys.size() - 1;
     };
     for (int i = 0; i < k; ++i) {
@@ -722,20 +737,25 @@ static int runner_upload(Runner *r) {
         pf.m = s.pot.m;
         const int g = group_of({s.prec, s.L, s.pot.sc76, pf});
         if (g < 0) return PTA_EUNSUPPORTED;
-        s.blk_pair0 = (int)gb2s[g].size();
-        for (int b = 0; b < s.nblk_pair; ++b) gb2s[g].push_back(i);
+        members[g].push_back(i);
         s.blk_run0 = (int)r->b2s_run.size();
         for (int b = 0; b < s.nblk_pair; ++b) r->b2s_run.push_back(i);
         r->hspecs[i] = s;
     }
-    // resident runs and sweeps serve specimens of one precision and potential
-    bool alike = true;
-    int min_lanes = 16;
-    for (auto &kk : keys) {
-        alike &= kk.prec == keys[0].prec && kk.sc76 == keys[0].sc76 &&
-                 std::memcmp(&kk.pf, &keys[0].pf, sizeof(PotF)) == 0;
-        min_lanes = std::min(min_lanes, kk.L);
+    // the longest blocks (fewest lanes) of a group start first
+    for (size_t g = 0; g < members.size(); ++g) {
+        std::stable_sort(members[g].begin(), members[g].end(),
+                         [&](int a, int b) { return r->hspecs[a].L < r->hspecs[b].L; });
+        for (int i : members[g]) {
+            SpecDev &s = r->hspecs[i];
+            s.blk_pair0 = (int)gb2s[g].size();
+            gb2s[g].insert(gb2s[g].end(), s.nblk_pair, i);
+        }
     }
+    // resident runs and sweeps serve specimens of one precision and potential
+    const bool alike = keys.size() == 1;
+    int min_lanes = 16;
+    for (const Key &q : kinds) min_lanes = std::min(min_lanes, q.L);
     // one device block for all tables
     size_t words = b2s_atom.size() + b2s_bld.size() + r->b2s_run.size();
     for (auto &v : gb2s) words += v.size();

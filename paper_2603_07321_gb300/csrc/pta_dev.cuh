@@ -180,7 +180,7 @@ struct SpecDev {
 };
 
 struct Group {
-    int prec, L, sc76;
+    int prec, L, sc76;  // L: lanes per atom, 0 where the group's specimens differ
     PotF pf;  // the group's potential (specimens of one group share it)
     const int *b2s;
     int nblk;
@@ -441,7 +441,6 @@ void launch_burst_begin(const Tab &t, const long long *nsteps, cudaStream_t st);
 void launch_burst_end(const Tab &t, int slot, pta_averages *out, cudaStream_t st);
 void launch_any_running(const Tab &t, int *flag, cudaStream_t st);
 void launch_pta_update(const Tab &t, const int *ops, pta_coarse_result *out, cudaStream_t st);
-void launch_force_rebuild_flag(const Tab &t, cudaStream_t st);
 void launch_rebuild(const Tab &t, int force, cudaStream_t st);
 int build_smem_limit(int bytes);  // allow k_build this much dynamic shared memory; 0 on failure
 void launch_prune(const Tab &t, int force, cudaStream_t st);

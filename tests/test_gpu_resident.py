@@ -65,6 +65,24 @@ def test_a_swept_batch_equals_its_members(P):
         c.close()
 
 
+# and one launch of each pass, with the members in any order
+@pytest.mark.parametrize("prec,order", [(1, (0, 1, 2)), (1, (2, 0, 1)), (0, (1, 2, 0))])
+def test_a_launched_batch_of_uneven_lanes_equals_its_members(P, prec, order):
+    shapes, steps = [(9, 20, 19), (5, 6, 5), (13, 12, 14)], [40, 60, 25]
+    solo = [_run(P, sh, prec, n, False, seed=i) for i, (sh, n) in enumerate(zip(shapes, steps))]
+    cs = [P.Ctx(shapes[i], T0=300.0, seed=i, precision=prec) for i in order]
+    assert len({c.layout()["lanes"] for c in cs}) > 1
+    b = P.Batch(cs)
+    b.set_timing(True)
+    b.apply_strain([1e-3] * len(cs))
+    b.fine_burst([steps[i] for i in order])
+    for c, i in zip(cs, order):
+        _equal((c.series().copy(), *c.get_state()), solo[i][:3])
+    b.close()
+    for c in cs:
+        c.close()
+
+
 # the sums of a launched pass: one group of blocks, several, a partial last one,
 # and more than one round of the finishing kernel (beyond 128 groups).  Each
 # atom's energy is one FP32 (FP64) number and the tree's error per level is
