@@ -619,17 +619,23 @@ def run_pta(args, wl):
     dominant = ("force", ach_force, force_ms) if force_ms >= dens_ms else ("density", ach_dens,
                                                                            dens_ms)
 
-    # launches of this library's kernels in the timed region: per fine-step
-    # iteration the decide kernel and, per (precision, lanes) group, the
-    # density and force passes; per list build 12 kernels; per pruning one
-    # kernel per group and one bookkeeping kernel; per burst the grip
-    # increment, burst start and burst end; per coarse step the update
-    groups = len({(c.params.precision, c.layout()["lanes"]) for c in ctxs})
-    builds = sum(b.rebuilds for step in results for r in step for b in r.burst)
-    prunes = sum(b.prunes for step in results for r in step for b in r.burst)
+    # launches of this library's kernels in the timed region, at least.  Tables
+    # of one precision with at most 56 warp tiles per SM advance by one kernel
+    # per list build, behind one that decides; else every fine step launches,
+    # per precision, the density and force passes, and one kernel that ends it.
+    # Per list build 7 kernels; per pruning of launched steps one per
+    # precision; per burst the grip increment, burst start and burst end; per
+    # coarse step the update
+    groups = len({c.params.precision for c in ctxs})
+    builds = sum(max(sum(b.rebuilds for b in r.burst) for r in step) for step in results)
+    prunes = sum(max(sum(b.prunes for b in r.burst) for r in step) for step in results)
     bursts = 3 * args.steps
-    launches = int(kt.iterations * (1 + 2 * groups) + builds * 12 + prunes * (groups + 1)
-                   + bursts * 3 + args.steps)
+    tiles = sum(-(-c.n * c.layout()["lanes"] // 128) * 4 for c in ctxs)
+    if groups == 1 and tiles <= 56 * n_sm and not any(c.params.conv_lag for c in ctxs):
+        launches = builds * (2 + 7)
+    else:
+        launches = kt.iterations * args.steps * (1 + 2 * groups) + builds * 7 + prunes * groups
+    launches = int(launches + bursts * 3 + args.steps)
 
     # end to end through the public API with host buffers: per step the state
     # goes host -> device from pinned memory, the coarse step runs, and the
