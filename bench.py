@@ -620,8 +620,9 @@ def run_pta(args, wl):
                                                                            dens_ms)
 
     # launches of this library's kernels in the timed region, at least.  Tables
-    # of one precision with at most 56 warp tiles per SM advance by one kernel
-    # per list build, behind one that decides; else every fine step launches,
+    # of one precision with at most 56 warp tiles per SM can advance by one kernel
+    # per list build, behind one that decides, and are counted so, whichever way
+    # they ran (fewer launches than they may have had); else every fine step launches,
     # per precision, the density and force passes, and one kernel that ends it.
     # Per list build 7 kernels; per pruning of launched steps one per
     # precision; per burst the grip increment, burst start and burst end; per

@@ -820,16 +820,19 @@ struct LaneList {
 // bulk atom).  Else, up to SWEEP_TILES tiles per SM, a sweep of at most
 // sweep_warps warps: of those counts the one whose last round of tiles is
 // fullest.  Larger tables fill the GPU for several waves, and launched passes,
-// with 32 warps per SM and the read-only path, are faster: per step 66 us
-// (launched 74) at 23 tiles per SM (108,000 atoms), 138 (143) at 53, 253 (225)
-// at 97.
+// with 32 warps per SM and the read-only path, are faster; in mixed precision
+// so are they where the last of several rounds would leave more than a tenth
+// of the warps idle (`full` = 0.9).  Per step, mixed: 27 tiles per SM 71 us
+// (launched 82), 30 tiles 106 (90), 36 tiles 112 (101), 39 tiles 114 (116), 53
+// tiles 132 (134), 97 tiles 253 (225).  FP64 passes keep the FP64 units busy
+// with fewer warps: 36 tiles 1,885 us (1,992), 53 tiles 2,778 (2,886).
 constexpr int RUN_WARPS = 16, SWEEP_TILES = 56;
 struct RunShape {
     int blocks = 0, threads = 0, quads = 0;
     size_t smem = 0;
     bool sweep = false;
 };
-inline RunShape run_shape(int nblk, int min_lanes, int sweep_warps) {
+inline RunShape run_shape(int nblk, int min_lanes, int sweep_warps, double full) {
     RunShape r;
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -854,6 +857,7 @@ inline RunShape run_shape(int nblk, int min_lanes, int sweep_warps) {
     auto slots = [&](int w) { return (per + w - 1) / w * w; };
     for (int w = sweep_warps; w >= sweep_warps * 3 / 4; --w)
         if (slots(w) < slots(best)) best = w;
+    if (per > sweep_warps && per < full * slots(best)) return RunShape();
     r.threads = 32 * best;
     return r;
 }

@@ -423,7 +423,7 @@ bool run_possible(const Tab &t, const int *b2s) {
     if (g.prec == PTA_PREC_FP64) {
         r = run_shape_f64(t, fits);
     } else {
-        r = run_shape(t.nblk_run, t.min_lanes, SWEEP_WARPS_F32);
+        r = run_shape(t.nblk_run, t.min_lanes, SWEEP_WARPS_F32, 0.9);
         fits = g.sc76 ? (r.sweep ? run_fits(k_sweep_f32<true>, r) : run_fits(k_run_f32<true, 0>, r) && run_fits(k_run_f32<true, 16>, r))
                       : (r.sweep ? run_fits(k_sweep_f32<false>, r) : run_fits(k_run_f32<false, 0>, r));
     }
@@ -441,7 +441,7 @@ cudaError_t launch_run(const Tab &t, RunCtl *rc, cudaGraphConditionalHandle agai
                        cudaStream_t st) {
     const Group &g = t.grp[0];
     if (g.prec == PTA_PREC_FP64) return launch_run_f64(t, g, rc, again, st);
-    const RunShape r = run_shape(t.nblk_run, t.min_lanes, SWEEP_WARPS_F32);
+    const RunShape r = run_shape(t.nblk_run, t.min_lanes, SWEEP_WARPS_F32, 0.9);
     auto go = [&](auto kernel) {
         return launch_cooperative(kernel, r, st, t.specs, t.nspec, t.b2s_run, t.nblk_run, rc, again,
                                   r.quads, g.pf);

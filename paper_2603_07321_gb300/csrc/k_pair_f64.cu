@@ -455,7 +455,7 @@ void launch_force_f64(const Tab &t, const Group &g, int mode, cudaStream_t st) {
 }
 
 RunShape run_shape_f64(const Tab &t, bool &fits) {
-    const RunShape r = run_shape(t.nblk_run, t.min_lanes, SWEEP_WARPS_F64);
+    const RunShape r = run_shape(t.nblk_run, t.min_lanes, SWEEP_WARPS_F64, 0.0);
     fits = t.grp[0].sc76
                ? (r.sweep ? run_fits(k_sweep_f64<true>, r) : run_fits(k_run_f64<true>, r))
                : (r.sweep ? run_fits(k_sweep_f64<false>, r) : run_fits(k_run_f64<false>, r));
@@ -464,7 +464,7 @@ RunShape run_shape_f64(const Tab &t, bool &fits) {
 
 cudaError_t launch_run_f64(const Tab &t, const Group &g, RunCtl *rc,
                            cudaGraphConditionalHandle again, cudaStream_t st) {
-    const RunShape r = run_shape(t.nblk_run, t.min_lanes, SWEEP_WARPS_F64);
+    const RunShape r = run_shape(t.nblk_run, t.min_lanes, SWEEP_WARPS_F64, 0.0);
     auto go = [&](auto kernel) {
         return launch_cooperative(kernel, r, st, t.specs, t.nspec, t.b2s_run, t.nblk_run, rc, again,
                                   r.quads);

@@ -44,7 +44,7 @@ def test_resident_equals_launched(P, prec, shape, lanes):
 # partial last tile, both precisions, the fewest and the most lanes)
 @pytest.mark.parametrize("prec,shape,lanes", [
     (1, (12, 12, 12), 16), (0, (11, 13, 12), 16), (1, (19, 20, 21), 4), (1, (28, 27, 29), 1),
-    (0, (28, 27, 29), 1)])
+    (0, (28, 27, 29), 1), (1, (19, 20, 18), 8)])
 def test_sweeps_equal_launched(P, prec, shape, lanes):
     _equal(_run(P, shape, prec, 45, False, lanes=lanes), _run(P, shape, prec, 45, True, lanes=lanes))
 
