@@ -645,18 +645,18 @@ __device__ __forceinline__ void run_resident(const SpecDev *specs, int nspec, co
     GridBarrier bar{rc, &requests};
     int state = 0, it = 0;
     for (; it < limit && !(state & (RUN_BUILD | RUN_STUCK)); ++it) {
-        const bool run = phase != PH_IDLE;
-        if (run && prune) {
-            ops.prune(S, par);
-            if (local == 0 && lane == 0) {
-                c->prunes = __ldcg(&c->prunes) + 1;
-                c->prune = 0;
-            }
-        }
+        const bool run = phase != PH_IDLE, pruned = run && prune;
+        if (pruned) ops.prune(S, par);
         if (run) ops.density(S, par);
         if (service && it > 0) sums.reduce();
         state = bar.sync(false);
         if (state & RUN_STUCK) break;
+        // cleared behind the barrier: by then every block has begun, and each
+        // warp has read the flag that it began with
+        if (pruned && local == 0 && lane == 0) {
+            c->prunes = __ldcg(&c->prunes) + 1;
+            c->prune = 0;
+        }
         if (run) {
             const StepVals<T> v = ops.force(S, local, par, phase, done, nsteps);
             if (lane == 0) step_requests(S, v, it, &requests);
