@@ -182,17 +182,22 @@ __device__ __noinline__ bool in_list_exact(const SpecDev &S, int par, int a, int
 // half of them candidate tests).  470,596 atoms: 1.28 ms (1.69 with undivided
 // cells, divisions by the lane count and 72 registers; at 64 registers eight
 // blocks share an SM), 52,700 atoms 145 us (187).
+//
+// MEM: for specimens whose capacity is too large for shared memory.
+template <bool MEM>
 __global__ void __launch_bounds__(BUILD_WARPS * 32, 8) k_build(const SpecDev *__restrict__ specs,
                                                            const int *__restrict__ b2s,
                                                            int force, int words) {
     extern __shared__ uint4 bsh4[];
     const SpecDev &S = specs[b2s[blockIdx.x]];
-    if (!build_active(S, force)) return;
+    if ((S.bld_scratch != nullptr) != MEM || !build_active(S, force)) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const int cap = S.cap_use, L = S.L, n = S.n, par = S.ctl->parity;
     const int sL = 31 - __clz(L);  // L is a power of two
     unsigned *buf = (unsigned *)bsh4 + (size_t)w * words;  // cap entries
+    if constexpr (MEM)
+        buf = S.bld_scratch + (size_t)((blockIdx.x - S.blk_bld0) * BUILD_WARPS + w) * build_words(cap);
     unsigned *out = buf + cap;                             // near part in list order
     int *cls = (int *)(out + cap + 128);                   // 8 counters
     const int4 *__restrict__ rec = S.rec[par];
@@ -393,8 +398,8 @@ void launch_decide_rebuild(const Tab &t, RunCtl *rc, cudaGraphConditionalHandle 
 }
 
 int build_smem_limit(int bytes) {
-    return cudaFuncSetAttribute(k_build, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) ==
-           cudaSuccess;
+    return cudaFuncSetAttribute(k_build<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                bytes) == cudaSuccess;
 }
 
 void launch_rebuild(const Tab &t, int force, cudaStream_t st) {
@@ -403,8 +408,10 @@ void launch_rebuild(const Tab &t, int force, cudaStream_t st) {
     k_scatter<<<t.nblk_atom, TPB, 0, st>>>(t.specs, t.b2s_atom, force);
     k_order<<<t.nblk_atom, TPB, 0, st>>>(t.specs, t.b2s_atom, force);
     k_permute_scatter<<<t.nblk_atom, TPB, 0, st>>>(t.specs, t.b2s_atom, force);
-    k_build<<<t.nblk_bld, BUILD_WARPS * 32, BUILD_WARPS * t.bld_words * 4, st>>>(
+    k_build<false><<<t.nblk_bld, BUILD_WARPS * 32, BUILD_WARPS * t.bld_words * 4, st>>>(
         t.specs, t.b2s_bld, force, t.bld_words);
+    if (t.bld_scratch)
+        k_build<true><<<t.nblk_bld, BUILD_WARPS * 32, 0, st>>>(t.specs, t.b2s_bld, force, 0);
     k_build_done<<<t.nspec, 32, 0, st>>>(t.specs, force);
 }
 

@@ -285,7 +285,7 @@ struct Sizes {
     int prune_on, mean_pos;
     double prune_margin;
     double h, org[3];
-    size_t list_quads;
+    size_t list_quads, bld_scratch;  // words of the build's scratch in memory
     int rec_bits;  // quanta of 2^-rec_bits A
     long long series_cap;
 };
@@ -332,7 +332,11 @@ static int compute_sizes(const pta_specimen &s, const pta_potential &p, const pt
     // list build: a warp per atom while that fills the GPU (152 SMs x ~48
     // warps), then several atoms in turn, which saves block starts
     z->apw = z->n >= 65536 ? 8 : (z->n >= 16384 ? 2 : 1);
+    const bool mem = z->cap_use > NEIGH_CAP_MOST;
+    const long long most = (long long)BUILD_WARPS * BUILD_SCRATCH_BLOCKS;
+    if (mem) z->apw = std::max(z->apw, (int)((z->n + most - 1) / most));
     z->nblk_bld = (int)((z->n + BUILD_WARPS * z->apw - 1) / (BUILD_WARPS * z->apw));
+    z->bld_scratch = mem ? (size_t)z->nblk_bld * BUILD_WARPS * build_words(z->cap_use) : 0;
     // cell edge a multiple of 2^-11 A and grid origin on the 2^-12 A grid, so
     // that cell centres and centre differences are exact in FP32
     z->h = std::ceil(rl * (1.0 + 1e-4) * 2048.0) / 2048.0;
@@ -402,6 +406,7 @@ static size_t footprint(const Sizes &z, int prec) {
     add(16 * z.list_quads);          // plist
     add(4 * n * (size_t)z.L);        // pnn
     add(8 * n);                      // nab
+    if (z.bld_scratch) add(4 * z.bld_scratch);
     if (z.prune_on) {
         add(16 * z.list_quads);      // nlist
         add(16 * n);                 // pref
@@ -436,7 +441,7 @@ static int validate(const pta_specimen *s, const pta_potential *p, const pta_par
     if (par->lanes != 0 && !valid_lanes(par->lanes)) return PTA_EINVAL;
     if (par->atoms_per_thread < 0 || par->atoms_per_thread > 2) return PTA_EINVAL;
     if (par->atoms_per_thread == 2) return PTA_EUNSUPPORTED;
-    if (par->neigh_cap < 0 || par->neigh_cap > 4096) return PTA_EINVAL;
+    if (par->neigh_cap < 0 || par->neigh_cap > NEIGH_CAP_MOST) return PTA_EINVAL;
     if (par->cell_tiles < -1 || par->cell_tiles > 1) return PTA_EINVAL;
     if (par->cell_tiles == 1) return PTA_EUNSUPPORTED;
     if (!std::isfinite(par->prune_margin)) return PTA_EINVAL;
@@ -671,6 +676,7 @@ static int runner_upload(Runner *r) {
     int blk_atom = 0;
     std::vector<int> b2s_atom, b2s_bld;
     int bld_words = 0;
+    bool bld_scratch = false;
     // launch groups by (precision, potential); the potential's FP32 constants
     // are kernel parameters of the group's launches.  A group whose specimens
     // differ in lanes per atom has L = 0 and runs kernels that read them: a
@@ -710,8 +716,10 @@ static int runner_upload(Runner *r) {
         for (int b = 0; b < s.nblk_atom; ++b) b2s_atom.push_back(i);
         s.blk_bld0 = (int)b2s_bld.size();
         for (int b = 0; b < s.nblk_bld; ++b) b2s_bld.push_back(i);
-        // candidates, near part in list order, class counters
-        bld_words = std::max(bld_words, 2 * s.cap_use + 128 + 16);
+        if (s.bld_scratch)
+            bld_scratch = true;
+        else
+            bld_words = std::max(bld_words, build_words(s.cap_use));
         PotF pf;
         std::memset(&pf, 0, sizeof(pf));
         pf.a = s.pot.f_a;
@@ -804,6 +812,7 @@ static int runner_upload(Runner *r) {
     t.b2s_bld = tabs + b2s_atom.size();
     t.nblk_bld = (int)b2s_bld.size();
     t.bld_words = bld_words;
+    t.bld_scratch = bld_scratch;
     if (!build_smem_limit(BUILD_WARPS * bld_words * 4)) {
         cudaGetLastError();
         return PTA_ECUDA;
@@ -1205,6 +1214,9 @@ static int ctx_alloc_all(pta_ctx *c, const Sizes &z) {
     AL(plist, 16 * z.list_quads, uint4 *);
     AL(pnn, 4 * n * (size_t)z.L, int *);
     AL(nab, 8 * n, int2 *);
+    if (z.bld_scratch) {
+        AL(bld_scratch, 4 * z.bld_scratch, unsigned *);
+    }
     if (z.prune_on) {
         AL(nlist, 16 * z.list_quads, uint4 *);
         AL(pref, 16 * n, int4 *);

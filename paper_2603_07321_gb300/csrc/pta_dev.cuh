@@ -19,6 +19,13 @@ constexpr int TPB = 128;        // threads per block of the atom and pair kernel
 constexpr int CELL_SPLIT = 4;   // cells along x per cell edge along y and z
 constexpr int SCAN_THREADS = 1024;
 constexpr int BUILD_WARPS = 4;  // warps per block of the list build
+constexpr int NEIGH_CAP_MOST = 4096;  // largest capacity that can be asked for
+// The list build's words per warp: candidates, near part in list order, class
+// counters.  Up to NEIGH_CAP_MOST entries they lie in shared memory; automatic
+// capacities can be larger (a list radius beyond ~22 A in aluminium), and then
+// they lie in memory, for at most BUILD_SCRATCH_BLOCKS blocks.
+__host__ __device__ constexpr int build_words(int cap) { return 2 * cap + 128 + 16; }
+constexpr int BUILD_SCRATCH_BLOCKS = 608;
 
 // grid quantum of the mixed-precision position split x = hi + lo:
 // hi is a multiple of 2^-12 A (exact in FP32 for |x| < 512 A), |lo| <= 2^-13 A
@@ -117,6 +124,7 @@ struct SpecDev {
     int blk_atom0, nblk_atom;  // one thread per atom
     int blk_bld0, nblk_bld;    // list build: BUILD_WARPS warps of apw atoms
     int apw;
+    unsigned *bld_scratch;     // build_words(cap_use) words per warp, or null: in shared memory
     int spec_index;            // index of this specimen in the launch table
     // lattice (creation only)
     int ncl[3];
@@ -206,6 +214,7 @@ struct Tab {
     const int *b2s_bld;
     int nblk_bld;
     int bld_words;  // shared words per warp of the list build
+    bool bld_scratch;  // a specimen's list build works in memory
     // resident runs and sweeps: block->specimen map over all specimens when they
     // share precision and potential (else null), fewest lanes per atom
     const int *b2s_run;
