@@ -397,9 +397,11 @@ void launch_decide_rebuild(const Tab &t, RunCtl *rc, cudaGraphConditionalHandle 
     k_decide_rebuild<<<1, 128, 0, st>>>(t.specs, t.nspec, rc, h);
 }
 
-int build_smem_limit(int bytes) {
+// the limit belongs to the function and so to every context of the process:
+// always the same value, that of the largest capacity
+int build_smem_limit() {
     return cudaFuncSetAttribute(k_build<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                bytes) == cudaSuccess;
+                                BUILD_SMEM_MOST) == cudaSuccess;
 }
 
 void launch_rebuild(const Tab &t, int force, cudaStream_t st) {

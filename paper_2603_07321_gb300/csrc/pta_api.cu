@@ -543,6 +543,7 @@ static int capture_iters(Runner *r, int iters, cudaGraphExec_t *out, bool timed 
             }
             if (b == (int)LIST_BUILD) launch_rebuild(r->tab, 0, r->cap2);
             launch_prune(r->tab, 0, r->cap2);
+            rc = launch_check();
             cudaGraph_t bout = nullptr;
             if (cudaStreamEndCapture(r->cap2, &bout) != cudaSuccess) rc = PTA_ECUDA;
         }
@@ -554,6 +555,8 @@ static int capture_iters(Runner *r, int iters, cudaGraphExec_t *out, bool timed 
         launch_finish(r->tab, MODE_STEP, r->d_run, i + 1 < iters ? &handles[i + 1] : nullptr,
                       r->cap);
         if (timed) cudaEventRecordWithFlags(r->ev[4 * i + 3], r->cap, cudaEventRecordExternal);
+        // a launch that was refused would be missing from the graph
+        if (launch_check() != PTA_OK) rc = PTA_ECUDA;
     }
     cudaGraph_t gout = nullptr;
     e = cudaStreamEndCapture(r->cap, &gout);
@@ -618,11 +621,13 @@ static int capture_burst(Runner *r, cudaGraphExec_t *out) {
     if (ok && cudaStreamBeginCaptureToGraph(r->cap, wb, nullptr, nullptr, 0,
                                             cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
         launch_decide_build(r->tab, r->d_run, build, r->cap);
-        ok = add_conditional(r->cap, build, cudaGraphCondTypeIf, &bb) == PTA_OK;
+        ok = launch_check() == PTA_OK;
+        ok = ok && add_conditional(r->cap, build, cudaGraphCondTypeIf, &bb) == PTA_OK;
         if (ok && cudaStreamBeginCaptureToGraph(r->cap2, bb, nullptr, nullptr, 0,
                                                 cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
             launch_rebuild(r->tab, 0, r->cap2);
-            ok = cudaStreamEndCapture(r->cap2, &tmp) == cudaSuccess;
+            ok = launch_check() == PTA_OK;
+            ok = (cudaStreamEndCapture(r->cap2, &tmp) == cudaSuccess) && ok;
         } else {
             ok = false;
         }
@@ -654,9 +659,11 @@ static int capture_iters_flat(Runner *r, int iters, cudaGraphExec_t *out, bool t
         launch_finish(r->tab, MODE_STEP, r->d_run, nullptr, r->cap);
         if (timed) cudaEventRecordWithFlags(r->ev[4 * i + 3], r->cap, cudaEventRecordExternal);
     }
+    const int rc = launch_check();
     cudaError_t e = cudaStreamEndCapture(r->cap, &g);
-    if (e != cudaSuccess) {
+    if (e != cudaSuccess || rc != PTA_OK) {
         cudaGetLastError();
+        if (e == cudaSuccess) cudaGraphDestroy(g);
         return PTA_ECUDA;
     }
     e = cudaGraphInstantiate(out, g, 0);
@@ -813,7 +820,7 @@ static int runner_upload(Runner *r) {
     t.nblk_bld = (int)b2s_bld.size();
     t.bld_words = bld_words;
     t.bld_scratch = bld_scratch;
-    if (!build_smem_limit(BUILD_WARPS * bld_words * 4)) {
+    if (!build_smem_limit()) {
         cudaGetLastError();
         return PTA_ECUDA;
     }

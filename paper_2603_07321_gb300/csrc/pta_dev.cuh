@@ -25,6 +25,7 @@ constexpr int NEIGH_CAP_MOST = 4096;  // largest capacity that can be asked for
 // capacities can be larger (a list radius beyond ~22 A in aluminium), and then
 // they lie in memory, for at most BUILD_SCRATCH_BLOCKS blocks.
 __host__ __device__ constexpr int build_words(int cap) { return 2 * cap + 128 + 16; }
+constexpr int BUILD_SMEM_MOST = BUILD_WARPS * 4 * build_words(NEIGH_CAP_MOST);
 constexpr int BUILD_SCRATCH_BLOCKS = 608;
 
 // grid quantum of the mixed-precision position split x = hi + lo:
@@ -451,7 +452,7 @@ void launch_burst_end(const Tab &t, int slot, pta_averages *out, cudaStream_t st
 void launch_any_running(const Tab &t, int *flag, cudaStream_t st);
 void launch_pta_update(const Tab &t, const int *ops, pta_coarse_result *out, cudaStream_t st);
 void launch_rebuild(const Tab &t, int force, cudaStream_t st);
-int build_smem_limit(int bytes);  // allow k_build this much dynamic shared memory; 0 on failure
+int build_smem_limit();  // allow k_build its dynamic shared memory; 0 on failure
 void launch_prune(const Tab &t, int force, cudaStream_t st);
 void launch_decide_rebuild(const Tab &t, RunCtl *rc, cudaGraphConditionalHandle h, cudaStream_t st);
 // list maintenance decided on the device: 0 build + prune, 1 prune, 2 nothing
