@@ -890,10 +890,10 @@ static int runner_create(pta_ctx *const *members, int k, Runner **out) {
     return PTA_OK;
 }
 
-// make sure every member can hold nsteps samples; refresh descriptors if a
-// series buffer moved
+// make sure every member can hold nsteps samples, and that this runner's
+// descriptors name the members' series: a context's own runner and its batch's
+// each have a copy, and either may have replaced the buffer
 static int ensure_series(Runner *r, const int64_t *nsteps) {
-    bool moved = false;
     for (size_t i = 0; i < r->m.size(); ++i) {
         pta_ctx *c = r->m[i];
         if (nsteps[i] <= c->hd.series_cap) continue;
@@ -904,16 +904,18 @@ static int ensure_series(Runner *r, const int64_t *nsteps) {
         c->hd.series = (double *)p;
         c->hd.series_cap = cap;
         CK(cudaMemcpyAsync(c->d_self, &c->hd, sizeof(SpecDev), cudaMemcpyHostToDevice, c->stream));
-        moved = true;
     }
-    if (moved) {
-        for (size_t i = 0; i < r->m.size(); ++i) {
-            r->hspecs[i].series = r->m[i]->hd.series;
-            r->hspecs[i].series_cap = r->m[i]->hd.series_cap;
-        }
+    bool moved = false;
+    for (size_t i = 0; i < r->m.size(); ++i) {
+        SpecDev &s = r->hspecs[i];
+        const SpecDev &h = r->m[i]->hd;
+        moved |= s.series != h.series || s.series_cap != h.series_cap;
+        s.series = h.series;
+        s.series_cap = h.series_cap;
+    }
+    if (moved)
         CK(cudaMemcpyAsync(r->d_specs, r->hspecs.data(), sizeof(SpecDev) * r->m.size(),
                            cudaMemcpyHostToDevice, r->stream));
-    }
     return PTA_OK;
 }
 
