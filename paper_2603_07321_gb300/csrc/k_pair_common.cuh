@@ -427,11 +427,11 @@ __device__ __forceinline__ void prune_lane(const SpecDev &S, int u, int l, int L
 // know at once, whether an atom has moved far enough for a list build or a
 // pruning, is counted in the barrier's own word.
 //
-// Every wait is bounded: a barrier not reached by all blocks within
-// BARRIER_POLLS polls (seconds) marks the run as stuck and every block
-// returns; the host reports PTA_ECUDA.
+// Every wait is bounded: a barrier not reached by all blocks within `limit`
+// polls (seconds by default) marks the run as stuck and every block returns;
+// the host reports PTA_ECUDA and refuses the specimens from then on, whose
+// blocks stopped at different points of a step.
 // ---------------------------------------------------------------------------
-constexpr unsigned BARRIER_POLLS = 1u << 22;
 // fields of RunCtl::arrive: arrivals, and how many of them came with a request
 // for a list build, a stop (a specimen failed), a pruning.  At most
 // RUN_STEPS steps per launch keep every field within its bits.
@@ -457,6 +457,7 @@ __device__ __forceinline__ void fence_gpu() {
 struct GridBarrier {
     RunCtl *rc;
     int *req;                  // shared: requests of this block's warps
+    unsigned limit;            // polls before a wait is given up
     unsigned target = 0;       // thread 0
     unsigned long long seen = 0;
 
@@ -479,9 +480,9 @@ struct GridBarrier {
             unsigned long long v;
             do {
                 v = ld_relaxed(&rc->arrive);
-            } while ((unsigned)(v & ((1u << BAR_BUILD) - 1)) < target && ++polls < BARRIER_POLLS);
+            } while ((unsigned)(v & ((1u << BAR_BUILD) - 1)) < target && ++polls < limit);
             int got = 0;
-            if (polls >= BARRIER_POLLS) {
+            if (polls >= limit) {
                 atomicExch(&rc->stuck, 1);
                 got = RUN_STUCK;
             }
@@ -614,7 +615,8 @@ struct Service {
 template <class T, class OPS>
 __device__ __forceinline__ void run_resident(const SpecDev *specs, int nspec, const int *b2s,
                                              int nblk, RunCtl *rc,
-                                             cudaGraphConditionalHandle again, OPS &ops) {
+                                             cudaGraphConditionalHandle again, unsigned polls,
+                                             OPS &ops) {
     constexpr int NW = TPB / 32;
     __shared__ SpecDev sh[RESIDENT_SPECS];
     __shared__ int requests;
@@ -642,7 +644,7 @@ __device__ __forceinline__ void run_resident(const SpecDev *specs, int nspec, co
     const int limit = run_passes(specs, nspec);
     const Service<T> sums{sh, ns, t0, t1, &requests};
     if (service) sums.start();
-    GridBarrier bar{rc, &requests};
+    GridBarrier bar{rc, &requests, polls};
     int state = 0, it = 0;
     for (; it < limit && !(state & (RUN_BUILD | RUN_STUCK)); ++it) {
         const bool run = phase != PH_IDLE, pruned = run && prune;
@@ -703,7 +705,7 @@ struct SpecRun {
 template <class T, class OPS>
 __device__ __forceinline__ void run_sweep(const SpecDev *specs, int nspec, const int *b2s, int nblk,
                                           RunCtl *rc, cudaGraphConditionalHandle again,
-                                          const OPS &ops) {
+                                          unsigned polls, const OPS &ops) {
     constexpr int NW = TPB / 32;
     __shared__ SpecDev sh[RESIDENT_SPECS];
     __shared__ SpecRun run[RESIDENT_SPECS];
@@ -744,7 +746,7 @@ __device__ __forceinline__ void run_sweep(const SpecDev *specs, int nspec, const
             __syncwarp();
         }
     };
-    GridBarrier bar{rc, &requests};
+    GridBarrier bar{rc, &requests, polls};
     int state = 0, it = 0;
     for (; it < limit && !(state & (RUN_BUILD | RUN_STUCK)); ++it) {
         if (service && it > 0) sums.reduce();

@@ -261,10 +261,10 @@ struct OpsF32 {
 template <bool SC76, int LT>
 __global__ void __launch_bounds__(32 * RUN_WARPS, 1)
     k_run_f32(const SpecDev *specs, int nspec, const int *b2s, int nblk, RunCtl *rc,
-              cudaGraphConditionalHandle again, int quads, const PotF P) {
+              cudaGraphConditionalHandle again, unsigned polls, int quads, const PotF P) {
     extern __shared__ uint4 list_cache[];
     OpsF32<SC76, LT> ops{P, list_cache, quads};
-    run_resident<FF>(specs, nspec, b2s, nblk, rc, again, ops);
+    run_resident<FF>(specs, nspec, b2s, nblk, rc, again, polls, ops);
 }
 
 // a sweep's warp, on one tile
@@ -296,8 +296,8 @@ constexpr int SWEEP_WARPS_F32 = 28;  // 72 registers
 template <bool SC76>
 __global__ void __launch_bounds__(32 * SWEEP_WARPS_F32, 1)
     k_sweep_f32(const SpecDev *specs, int nspec, const int *b2s, int nblk, RunCtl *rc,
-                cudaGraphConditionalHandle again, int, const PotF P) {
-    run_sweep<FF>(specs, nspec, b2s, nblk, rc, again, SweepF32<SC76>{P});
+                cudaGraphConditionalHandle again, unsigned polls, int, const PotF P) {
+    run_sweep<FF>(specs, nspec, b2s, nblk, rc, again, polls, SweepF32<SC76>{P});
 }
 
 template <int LT>
@@ -444,7 +444,7 @@ cudaError_t launch_run(const Tab &t, RunCtl *rc, cudaGraphConditionalHandle agai
     const RunShape r = run_shape(t.nblk_run, t.min_lanes, SWEEP_WARPS_F32, 0.9);
     auto go = [&](auto kernel) {
         return launch_cooperative(kernel, r, st, t.specs, t.nspec, t.b2s_run, t.nblk_run, rc, again,
-                                  r.quads, g.pf);
+                                  t.barrier_polls, r.quads, g.pf);
     };
     if (r.sweep) return g.sc76 ? go(k_sweep_f32<true>) : go(k_sweep_f32<false>);
     if (!g.sc76) return go(k_run_f32<false, 0>);

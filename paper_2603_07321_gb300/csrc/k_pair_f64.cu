@@ -392,10 +392,10 @@ struct OpsF64 {
 template <bool SC76>
 __global__ void __launch_bounds__(32 * RUN_WARPS, 1)
     k_run_f64(const SpecDev *specs, int nspec, const int *b2s, int nblk, RunCtl *rc,
-              cudaGraphConditionalHandle again, int quads) {
+              cudaGraphConditionalHandle again, unsigned polls, int quads) {
     extern __shared__ uint4 list_cache[];
     OpsF64<SC76> ops{list_cache, quads};
-    run_resident<double>(specs, nspec, b2s, nblk, rc, again, ops);
+    run_resident<double>(specs, nspec, b2s, nblk, rc, again, polls, ops);
 }
 
 // a sweep's warp, on one tile
@@ -426,8 +426,8 @@ constexpr int SWEEP_WARPS_F64 = 20;
 template <bool SC76>
 __global__ void __launch_bounds__(32 * SWEEP_WARPS_F64, 1)
     k_sweep_f64(const SpecDev *specs, int nspec, const int *b2s, int nblk, RunCtl *rc,
-                cudaGraphConditionalHandle again, int) {
-    run_sweep<double>(specs, nspec, b2s, nblk, rc, again, SweepF64<SC76>{});
+                cudaGraphConditionalHandle again, unsigned polls, int) {
+    run_sweep<double>(specs, nspec, b2s, nblk, rc, again, polls, SweepF64<SC76>{});
 }
 
 #define PTA_F64_SWITCH(KER, SC, ARG)                                                   \
@@ -467,7 +467,7 @@ cudaError_t launch_run_f64(const Tab &t, const Group &g, RunCtl *rc,
     const RunShape r = run_shape(t.nblk_run, t.min_lanes, SWEEP_WARPS_F64, 0.0);
     auto go = [&](auto kernel) {
         return launch_cooperative(kernel, r, st, t.specs, t.nspec, t.b2s_run, t.nblk_run, rc, again,
-                                  r.quads);
+                                  t.barrier_polls, r.quads);
     };
     if (g.sc76) return r.sweep ? go(k_sweep_f64<true>) : go(k_run_f64<true>);
     return r.sweep ? go(k_sweep_f64<false>) : go(k_run_f64<false>);

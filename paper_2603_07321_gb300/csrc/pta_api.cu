@@ -49,6 +49,15 @@ double ev_a3_to_gpa() { return E_CHARGE / 1e-30 / 1e9; }
 
 constexpr int CHUNK = 64;
 
+// polls of a resident run's grid barrier before it is given up: seconds.
+// PTA_BARRIER_POLLS sets another limit (0: every wait runs out at once), to
+// try what follows from a run that stopped.
+constexpr unsigned BARRIER_POLLS = 1u << 22;
+unsigned barrier_polls() {
+    const char *e = std::getenv("PTA_BARRIER_POLLS");
+    return e ? (unsigned)std::strtoul(e, nullptr, 10) : BARRIER_POLLS;
+}
+
 struct Allocator {
     pta_alloc_fn alloc = nullptr;
     pta_free_fn release = nullptr;
@@ -838,6 +847,7 @@ static int runner_upload(Runner *r) {
     t.b2s_run = alike ? tabs + off : nullptr;
     t.nblk_run = (int)r->b2s_run.size();
     t.min_lanes = min_lanes;
+    t.barrier_polls = barrier_polls();
     r->tab = t;
     // pinned host mirrors
     const size_t hb = 8 * k * 2 + 4 * k + sizeof(pta_averages) * k + sizeof(pta_coarse_result) * k + 64;
@@ -1096,6 +1106,15 @@ static int run_tick(Runner *r, pta_coarse_result *out, int only_init) {
         }
     }
     return rc_all;
+}
+
+// After PTA_ECUDA the members' states are unknown (a resident run that gave up
+// leaves its blocks at different points of a step): every later call that
+// would use them is refused.
+static int settle(Runner *r, int rc) {
+    if (rc == PTA_ECUDA)
+        for (pta_ctx *c : r->m) c->broken = true;
+    return rc;
 }
 
 static int ctx_solo(pta_ctx *c, Runner **r) {
@@ -1426,7 +1445,7 @@ int pta_relax(pta_ctx *c, int64_t window, int64_t max_steps, double tol_gpa, pta
     pta_averages a{};
     int rc = PTA_OK;
     while (rc == PTA_OK) {
-        rc = run_burst(r, &window, &a, -1);
+        rc = settle(r, run_burst(r, &window, &a, -1));
         if (rc != PTA_OK) break;
         total += a.nsteps;
         if (std::fabs(a.mean[2]) < tol_gpa || total + window > max_steps) break;
@@ -1435,7 +1454,6 @@ int pta_relax(pta_ctx *c, int64_t window, int64_t max_steps, double tol_gpa, pta
     launch_fix_right_grip(c->hd, c->d_self, c->stream);
     CKR(launch_check());
     CK(cudaStreamSynchronize(c->stream));
-    if (rc == PTA_ECUDA) c->broken = true;
     if (out) *out = a;
     if (steps) *steps = total;
     return rc;
@@ -1489,8 +1507,7 @@ int pta_fine_burst(pta_ctx *c, int64_t nsteps, pta_averages *out) {
     Runner *r;
     CKR(ctx_solo(c, &r));
     pta_averages a;
-    int rc = run_burst(r, &nsteps, &a, -1);
-    if (rc == PTA_ECUDA) c->broken = true;
+    int rc = settle(r, run_burst(r, &nsteps, &a, -1));
     if (out) *out = a;
     return rc;
 }
@@ -1504,11 +1521,8 @@ int pta_ramp_burst(pta_ctx *c, int64_t nsteps, double d_eps_per_step, pta_averag
     CK(cudaMemcpyAsync(&c->hd.ctl->grip_du, &c->grip_du, sizeof(double), cudaMemcpyHostToDevice,
                        c->stream));
     pta_averages a{};
-    int rc = run_burst(r, &nsteps, &a, -1);
-    if (rc == PTA_ECUDA) {
-        c->broken = true;
-        return rc;
-    }
+    int rc = settle(r, run_burst(r, &nsteps, &a, -1));
+    if (rc == PTA_ECUDA) return rc;
     // the grip advanced with every drift of the burst
     c->u += (double)a.nsteps * c->grip_du;
     c->grip_du = 0.0;
@@ -1541,12 +1555,10 @@ int pta_coarse_step(pta_ctx *c, pta_coarse_result *out) {
     CKR(ctx_solo(c, &r));
     int rc = PTA_OK;
     if (!c->pta_init) {
-        rc = run_tick(r, nullptr, 1);
+        rc = settle(r, run_tick(r, nullptr, 1));
         if (rc != PTA_OK) return rc;
     }
-    rc = run_tick(r, out, 0);
-    if (rc == PTA_ECUDA) c->broken = true;
-    return rc;
+    return settle(r, run_tick(r, out, 0));
 }
 
 int pta_coarse_update(pta_ctx *c, const double means[9], pta_coarse_result *out) {
@@ -1847,6 +1859,8 @@ static int batch_ok(pta_batch *b) {
     if (!b || !b->r) return PTA_EINVAL;
     for (auto *m : b->r->m)
         if (!m) return PTA_ESTATE;
+    for (auto *m : b->r->m)
+        if (m->broken) return PTA_ECUDA;
     return PTA_OK;
 }
 
@@ -1861,20 +1875,20 @@ int pta_batch_apply_strain(pta_batch *b, const double *d_eps) {
 int pta_batch_fine_burst(pta_batch *b, const int64_t *nsteps, pta_averages *out) {
     CKR(batch_ok(b));
     if (!nsteps) return PTA_EINVAL;
-    return run_burst(b->r, nsteps, out, -1);
+    return settle(b->r, run_burst(b->r, nsteps, out, -1));
 }
 
 int pta_batch_coarse_step(pta_batch *b, pta_coarse_result *out) {
     CKR(batch_ok(b));
     bool need_init = false;
     for (auto *m : b->r->m) need_init |= !m->pta_init;
-    if (need_init) CKR(run_tick(b->r, nullptr, 1));
-    return run_tick(b->r, out, 0);
+    if (need_init) CKR(settle(b->r, run_tick(b->r, nullptr, 1)));
+    return settle(b->r, run_tick(b->r, out, 0));
 }
 
 int pta_batch_tick(pta_batch *b, pta_coarse_result *out) {
     CKR(batch_ok(b));
-    return run_tick(b->r, out, 0);
+    return settle(b->r, run_tick(b->r, out, 0));
 }
 
 int pta_set_timing(pta_ctx *c, int enable) {

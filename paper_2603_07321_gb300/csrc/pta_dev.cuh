@@ -220,6 +220,7 @@ struct Tab {
     // share precision and potential (else null), fewest lanes per atom
     const int *b2s_run;
     int nblk_run, min_lanes;
+    unsigned barrier_polls;  // polls before a grid barrier's wait is given up
     int ngroups;
     Group grp[8];
 };
