@@ -7,7 +7,8 @@
 // positions are an exact FP32 pair x = hi + lo (hi on a 2^-12 A grid, |lo| <=
 // 2^-13 A); velocities an exact FP32 pair v = vh + vl (|vl| <= ulp(vh) / 2) updated by
 // error-free addition, so that half-kicks lose nothing to rounding over long
-// bursts; K, U and R are summed in error-free pairs of floats.
+// bursts; K, U and R are converted to FP64 per atom and
+// summed in FP64.
 #pragma once
 
 #include "k_pair_common.cuh"
@@ -171,14 +172,15 @@ struct AtomMixed {
 __device__ __forceinline__ int4 atom_update_mixed(const SpecDev &S, AtomMixed &A, int par, int a,
                                                   const float f[3], float pe, int mode, int phase,
                                                   long long done, long long nsteps,
-                                                  StepVals<FF> &out) {
+                                                  StepVals &out) {
     chk_force(S, f[0], f[1], f[2]);
     SpecCtl *ctl = S.ctl;
-    set(out.s[1], pe);
-    if (A.flag == FLAG_RIGHT) set(out.s[2], -(S.axis == 0 ? f[0] : (S.axis == 1 ? f[1] : f[2])));
+    out.s[1] = (double)pe;
+    if (A.flag == FLAG_RIGHT)
+        out.s[2] = (double)-(S.axis == 0 ? f[0] : (S.axis == 1 ? f[1] : f[2]));
     auto kinetic = [&] {
         const float x = A.vh[0] + A.vl[0], y = A.vh[1] + A.vl[1], z = A.vh[2] + A.vl[2];
-        set(out.s[0], __fmul_rn(S.f_ke_fac, fmaf(z, z, fmaf(y, y, __fmul_rn(x, x)))));
+        out.s[0] = (double)__fmul_rn(S.f_ke_fac, fmaf(z, z, fmaf(y, y, __fmul_rn(x, x))));
     };
     if (mode == MODE_EVAL) {
         kinetic();

@@ -21,87 +21,69 @@ __device__ __forceinline__ T lane_sum(T v, int L) {
 // ---------------------------------------------------------------------------
 // The state functions of a step: sums over the atoms of K, U and the reaction
 // R, and the largest squared displacements since the list build and since the
-// pruning (quanta^2).
+// pruning (quanta^2).  Sums are double in both precisions.
 //
-// Sums are double in FP64 contexts and pairs of floats (an unevaluated sum,
-// 48 bits, error-free additions) in mixed precision, whose terms are floats:
-// FP64 additions run two lanes per clock and SM here, and 15 of them per warp
-// (three sums, five shuffle stages) cost the force pass of the 470,596-atom
-// cube ~12 us.
+// FP64 additions run two lanes per clock and SM here (16 cycles per warp), so
+// the butterflies below sum K and U in one: its first stage leaves the sums of
+// K in one half of the lanes and those of U in the other, five additions for
+// both instead of ten; and most warps hold no right-grip atom and skip R.
 // ---------------------------------------------------------------------------
-struct FF {
-    float h, l;
-};
-__device__ __forceinline__ FF add(FF a, FF b) {
-    const float s = __fadd_rn(a.h, b.h), t = __fsub_rn(s, a.h);
-    const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
-    const float l = __fadd_rn(__fadd_rn(a.l, b.l), e);
-    FF r;
-    r.h = __fadd_rn(s, l);
-    r.l = __fsub_rn(l, __fsub_rn(r.h, s));
-    return r;
-}
-__device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ FF shfl_xor(FF v, int o) {
-    return {__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
-}
-__device__ __forceinline__ double shfl_xor(double v, int o) {
-    return __shfl_xor_sync(0xffffffffu, v, o);
-}
-__device__ __forceinline__ double to_double(FF v) { return (double)v.h + (double)v.l; }
-__device__ __forceinline__ double to_double(double v) { return v; }
-__device__ __forceinline__ bool is_zero(FF v) { return v.h == 0.f; }
-__device__ __forceinline__ bool is_zero(double v) { return v == 0.0; }
-__device__ __forceinline__ void set(FF &v, float x) { v = {x, 0.f}; }
-__device__ __forceinline__ void set(double &v, double x) { v = x; }
 // non-negative floats order as their bits
 __device__ __forceinline__ float warp_max(float v) {
     return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
 }
 
-template <class T>
+constexpr int PART = 4;         // doubles per partial
+constexpr int PART_GROUP = 32;  // blocks per group of partials
 struct StepVals {
-    T s[3];         // K, U, R
+    double s[3];    // K, U, R
     float d2, dp2;  // displacements
 };
-// sums over the lanes whose values count (every mino-th), down to offset mino
-template <class T>
-__device__ __forceinline__ void warp_reduce(StepVals<T> &v, int mino) {
-    // most warps hold no right-grip atom and no reaction
-    const bool reaction = __any_sync(0xffffffffu, !is_zero(v.s[2]));
+__device__ __forceinline__ double add_xor(double v, int o) {
+    return __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
+}
+// sums over the lanes whose values count, at offsets `first`, first / 2, ...
+// `last`: right in lane 0 (of each 2 first lanes)
+__device__ __forceinline__ void sum_lanes(double s[3], int first, int last) {
+    const bool upper = threadIdx.x & first;
+    double r = upper ? s[1] : s[0];
+    r = __dadd_rn(r, __shfl_xor_sync(0xffffffffu, upper ? s[0] : s[1], first));
 #pragma unroll
-    for (int o = 16; o >= mino; o >>= 1) {
-        v.s[0] = add(v.s[0], shfl_xor(v.s[0], o));
-        v.s[1] = add(v.s[1], shfl_xor(v.s[1], o));
-        if (reaction) v.s[2] = add(v.s[2], shfl_xor(v.s[2], o));
+    for (int o = 8; o > 0; o >>= 1)
+        if (o < first && o >= last) r = add_xor(r, o);
+    s[0] = r;
+    s[1] = __shfl_xor_sync(0xffffffffu, r, first);
+    if (__any_sync(0xffffffffu, s[2] != 0.0)) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            if (o <= first && o >= last) s[2] = add_xor(s[2], o);
     }
+}
+// over the lanes of a warp whose values count (every mino-th), in lane 0
+__device__ __forceinline__ void warp_reduce(StepVals &v, int mino) {
+    sum_lanes(v.s, 16, mino);
     v.d2 = warp_max(v.d2);
     v.dp2 = warp_max(v.dp2);
 }
 // the same sums with the atoms of a tile in 32 / L adjacent lanes
-template <class T>
-__device__ __forceinline__ void tile_reduce(StepVals<T> &v, int L) {
-    const bool reaction = __any_sync(0xffffffffu, !is_zero(v.s[2]));
+__device__ __forceinline__ void tile_reduce(StepVals &v, int L) {
+    sum_lanes(v.s, 16 / L, 1);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         if (o * L >= 32) continue;
-        v.s[0] = add(v.s[0], shfl_xor(v.s[0], o));
-        v.s[1] = add(v.s[1], shfl_xor(v.s[1], o));
-        if (reaction) v.s[2] = add(v.s[2], shfl_xor(v.s[2], o));
         v.d2 = fmaxf(v.d2, __shfl_xor_sync(0xffffffffu, v.d2, o));
         v.dp2 = fmaxf(v.dp2, __shfl_xor_sync(0xffffffffu, v.dp2, o));
     }
 }
 // a partial in memory: three sums and the two maxima, 32 bytes
-__device__ __forceinline__ void load_part(const double *p, StepVals<FF> &v) {
-    const float4 a = __ldcg((const float4 *)p), b = __ldcg((const float4 *)p + 1);
-    v.s[0] = {a.x, a.y};
-    v.s[1] = {a.z, a.w};
-    v.s[2] = {b.x, b.y};
-    v.d2 = b.z;
-    v.dp2 = b.w;
+__device__ __forceinline__ double pack_maxima(float d2, float dp2) {
+    return __hiloint2double(__float_as_int(dp2), __float_as_int(d2));
 }
-__device__ __forceinline__ void load_part(const double *p, StepVals<double> &v) {
+__device__ __forceinline__ double max_pair(double a, double b) {
+    return __hiloint2double(max(__double2hiint(a), __double2hiint(b)),
+                            max(__double2loint(a), __double2loint(b)));
+}
+__device__ __forceinline__ void load_part(const double *p, StepVals &v) {
     const double2 a = __ldcg((const double2 *)p), b = __ldcg((const double2 *)p + 1);
     v.s[0] = a.x;
     v.s[1] = a.y;
@@ -109,30 +91,16 @@ __device__ __forceinline__ void load_part(const double *p, StepVals<double> &v) 
     v.d2 = __int_as_float(__double2loint(b.y));
     v.dp2 = __int_as_float(__double2hiint(b.y));
 }
-__device__ __forceinline__ void store_part(double *p, const StepVals<FF> &v) {
-    ((float4 *)p)[0] = make_float4(v.s[0].h, v.s[0].l, v.s[1].h, v.s[1].l);
-    ((float4 *)p)[1] = make_float4(v.s[2].h, v.s[2].l, v.d2, v.dp2);
-}
-__device__ __forceinline__ void store_part(double *p, const StepVals<double> &v) {
+__device__ __forceinline__ void store_part(double *p, const StepVals &v) {
     ((double2 *)p)[0] = make_double2(v.s[0], v.s[1]);
-    ((double2 *)p)[1] = make_double2(
-        v.s[2], __hiloint2double(__float_as_int(v.dp2), __float_as_int(v.d2)));
+    ((double2 *)p)[1] = make_double2(v.s[2], pack_maxima(v.d2, v.dp2));
 }
 // a += b
-template <class T>
-__device__ __forceinline__ void merge(StepVals<T> &a, const StepVals<T> &b) {
+__device__ __forceinline__ void merge(StepVals &a, const StepVals &b) {
 #pragma unroll
-    for (int q = 0; q < 3; ++q) a.s[q] = add(a.s[q], b.s[q]);
+    for (int q = 0; q < 3; ++q) a.s[q] = __dadd_rn(a.s[q], b.s[q]);
     a.d2 = fmaxf(a.d2, b.d2);
     a.dp2 = fmaxf(a.dp2, b.dp2);
-}
-template <class T>
-__device__ __forceinline__ StepVals<T> zero_vals() {
-    StepVals<T> v;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) set(v.s[q], 0);
-    v.d2 = v.dp2 = 0.f;
-    return v;
 }
 
 // squared displacement of a record from an earlier one, quanta^2
@@ -141,9 +109,6 @@ __device__ __forceinline__ float moved2(const int4 &a, const int4 &b) {
     return fmaf(z, z, fmaf(y, y, __fmul_rn(x, x)));
 }
 
-constexpr int PART = 4;           // doubles per partial
-constexpr int PART_GROUP = 32;    // blocks per group of partials
-
 // The block's partial from its atoms' values, atom t of the block in thread t
 // < NT / L: the atoms of each warp tile (32 / L of them) summed as a resident
 // run's warp does, then the block's tiles in order.  The kernel behind the
@@ -151,22 +116,23 @@ constexpr int PART_GROUP = 32;    // blocks per group of partials
 // last blocks of the force pass did, every block waited at its end for its
 // stores to be visible and for an atomic: a step of 12 specimens of 32,000
 // atoms took 235 us instead of 219, of 470,596 atoms 223 instead of 220.
-template <int NT, class T>
-__device__ __forceinline__ void block_partial(const SpecDev &S, int lb, StepVals<T> v, int L) {
+template <int NT>
+__device__ __forceinline__ void block_partial(const SpecDev &S, int lb, StepVals v, int L) {
     constexpr int NW = NT / 32;
-    __shared__ StepVals<T> sh[NW];
-    const int lane = threadIdx.x & 31;
+    __shared__ __align__(16) double sh[NW][PART];
+    const int lane = threadIdx.x & 31, q = threadIdx.x;
     if ((threadIdx.x & ~31) < NT / L) {
         tile_reduce(v, L);
-        if ((lane & (32 / L - 1)) == 0 && threadIdx.x < NT / L) sh[threadIdx.x / (32 / L)] = v;
+        if ((lane & (32 / L - 1)) == 0 && threadIdx.x < NT / L)
+            store_part(sh[threadIdx.x / (32 / L)], v);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        StepVals<T> a = sh[0];
+    if (q >= PART) return;
+    // a thread per sum, and one for the maxima
+    double a = sh[0][q];
 #pragma unroll
-        for (int k = 1; k < NW; ++k) merge(a, sh[k]);
-        store_part(S.part + (long long)PART * lb, a);
-    }
+    for (int k = 1; k < NW; ++k) a = q < 3 ? __dadd_rn(a, sh[k][q]) : max_pair(a, sh[k][q]);
+    S.part[(long long)PART * lb + q] = a;
 }
 
 // MODE_EVAL: force and energy of atom a in the arrays of pta_forces
@@ -260,19 +226,18 @@ __device__ inline void advance_ctl(const SpecDev &S, double K, double U, double 
 //
 // Bound: three round trips of latency; a warp's groups are loaded together.
 constexpr int FINISH_WARPS = 16, FINISH_GROUPS = 8;
-template <class T>
-__device__ __forceinline__ StepVals<T> finish_sums(const SpecDev &S) {
+__device__ __forceinline__ StepVals finish_sums(const SpecDev &S) {
     constexpr int ROUND = FINISH_WARPS * FINISH_GROUPS;
-    __shared__ StepVals<T> sg[ROUND], sc[ROUND / 32];
+    __shared__ StepVals sg[ROUND], sc[ROUND / 32];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nblk = S.nblk_pair, ngroups = (nblk + PART_GROUP - 1) / PART_GROUP;
-    StepVals<T> t = zero_vals<T>();
+    StepVals t = StepVals{};
     for (int r = 0; r < ngroups; r += ROUND) {
-        StepVals<T> a[FINISH_GROUPS];
+        StepVals a[FINISH_GROUPS];
 #pragma unroll
         for (int k = 0; k < FINISH_GROUPS; ++k) {
             const int b = (r + k * FINISH_WARPS + w) * PART_GROUP + lane;
-            a[k] = zero_vals<T>();
+            a[k] = StepVals{};
             if (b < nblk) load_part(S.part + (long long)PART * b, a[k]);
         }
 #pragma unroll
@@ -284,7 +249,7 @@ __device__ __forceinline__ StepVals<T> finish_sums(const SpecDev &S) {
         }
         __syncthreads();
         if (w * 32 < min(ROUND, ngroups - r)) {
-            StepVals<T> u = r + w * 32 + lane < ngroups ? sg[w * 32 + lane] : zero_vals<T>();
+            StepVals u = r + w * 32 + lane < ngroups ? sg[w * 32 + lane] : StepVals{};
             if (ngroups > 1) warp_reduce(u, 1);
             if (lane == 0) sc[w] = u;
         }
@@ -307,11 +272,10 @@ __device__ __forceinline__ double *part_warp(const SpecDev &S, int tile) {
 __device__ __forceinline__ double *part_group(const SpecDev &S, int g) {
     return S.gpart + (long long)PART * g;
 }
-template <class T>
 __device__ inline void reduce_group(const SpecDev &S, int g) {
     constexpr int NW = TPB / 32;
     const int lane = threadIdx.x & 31, blk = g * PART_GROUP + lane;
-    StepVals<T> a = zero_vals<T>(), b[NW];
+    StepVals a = StepVals{}, b[NW];
     if (blk < S.nblk_pair) {
 #pragma unroll
         for (int k = 0; k < NW; ++k) load_part(part_warp(S, blk * NW + k), b[k]);
@@ -322,17 +286,16 @@ __device__ inline void reduce_group(const SpecDev &S, int g) {
     warp_reduce(a, 1);
     if (lane == 0) store_part(part_group(S, g), a);
 }
-template <class T>
-__device__ inline StepVals<T> reduce_groups(const SpecDev &S) {
+__device__ inline StepVals reduce_groups(const SpecDev &S) {
     const int lane = threadIdx.x & 31;
     const int ngroups = (S.nblk_pair + PART_GROUP - 1) / PART_GROUP;
-    StepVals<T> t = zero_vals<T>();
+    StepVals t = StepVals{};
     if (ngroups == 1) {
         if (lane == 0) load_part(part_group(S, 0), t);
         return t;
     }
     for (int b = 0; b < ngroups; b += 32) {
-        StepVals<T> u = zero_vals<T>();
+        StepVals u = StepVals{};
         if (b + lane < ngroups) load_part(part_group(S, b + lane), u);
         warp_reduce(u, 1);
         if (b == 0) t = u;
@@ -532,8 +495,7 @@ __device__ __forceinline__ void run_again(const SpecDev *specs, int nspec, int s
     if (lane == 0) cudaGraphSetConditional(again, active && !(state & RUN_STUCK) ? 1u : 0u);
 }
 // one lane: what a warp's displacements after pass `it` ask for
-template <class T>
-__device__ __forceinline__ void step_requests(const SpecDev &S, const StepVals<T> &v, int it,
+__device__ __forceinline__ void step_requests(const SpecDev &S, const StepVals &v, int it,
                                               int *requests) {
     int r = 0;
     if (v.d2 > S.half_skin2q) {
@@ -550,7 +512,6 @@ __device__ __forceinline__ void step_requests(const SpecDev &S, const StepVals<T
 // The service warp of a block: the sums of the groups that begin in its tiles,
 // and the control blocks of the specimens that do.  The phase and step count
 // there are those of the sums, one step behind the atoms.
-template <class T>
 struct Service {
     const SpecDev *sh;  // the block's specimens
     int ns, t0, t1;
@@ -574,7 +535,7 @@ struct Service {
     }
     __device__ __forceinline__ void reduce() const {
         each([&](const SpecDev &D, int g) {
-            if (__ldcg(&D.ctl->phase) != PH_IDLE) reduce_group<T>(D, g);
+            if (__ldcg(&D.ctl->phase) != PH_IDLE) reduce_group(D, g);
         });
     }
     __device__ __forceinline__ void finish() const {
@@ -582,14 +543,13 @@ struct Service {
             SpecCtl *q = D.ctl;
             const int ph = __ldcg(&q->phase);
             if (g != 0 || ph == PH_IDLE) return;
-            const StepVals<T> t = reduce_groups<T>(D);
+            const StepVals t = reduce_groups(D);
             if ((threadIdx.x & 31) != 0) return;
             if (ph == PH_REFRESH) {
                 q->phase = PH_RUN;
                 return;
             }
-            const double K = to_double(t.s[0]), U = to_double(t.s[1]),
-                         X = to_double(t.s[2]) * D.t_fac;
+            const double K = t.s[0], U = t.s[1], X = t.s[2] * D.t_fac;
             const long long i = __ldcg(&q->done);
             if (isfinite(K) && isfinite(U) && isfinite(X)) {
                 double *o = D.series + 3 * i;
@@ -612,7 +572,7 @@ struct Service {
 // warp k of pair block b), one per warp, and the service warp behind them.
 // OPS (one precision and lane count): a warp's part of the passes.  Its atoms'
 // positions and velocities stay in registers from the launch to its end.
-template <class T, class OPS>
+template <class OPS>
 __device__ __forceinline__ void run_resident(const SpecDev *specs, int nspec, const int *b2s,
                                              int nblk, RunCtl *rc,
                                              cudaGraphConditionalHandle again, unsigned polls,
@@ -642,7 +602,7 @@ __device__ __forceinline__ void run_resident(const SpecDev *specs, int nspec, co
     const bool mine = phase != PH_IDLE;
     if (mine) ops.load(S, local, par);
     const int limit = run_passes(specs, nspec);
-    const Service<T> sums{sh, ns, t0, t1, &requests};
+    const Service sums{sh, ns, t0, t1, &requests};
     if (service) sums.start();
     GridBarrier bar{rc, &requests, polls};
     int state = 0, it = 0;
@@ -660,7 +620,7 @@ __device__ __forceinline__ void run_resident(const SpecDev *specs, int nspec, co
             c->prune = 0;
         }
         if (run) {
-            const StepVals<T> v = ops.force(S, local, par, phase, done, nsteps);
+            const StepVals v = ops.force(S, local, par, phase, done, nsteps);
             if (lane == 0) step_requests(S, v, it, &requests);
             par ^= 1;
             done += phase == PH_RUN;
@@ -702,7 +662,7 @@ struct SpecRun {
     int phase, par, prune;
     long long done, nsteps;
 };
-template <class T, class OPS>
+template <class OPS>
 __device__ __forceinline__ void run_sweep(const SpecDev *specs, int nspec, const int *b2s, int nblk,
                                           RunCtl *rc, cudaGraphConditionalHandle again,
                                           unsigned polls, const OPS &ops) {
@@ -731,7 +691,7 @@ __device__ __forceinline__ void run_sweep(const SpecDev *specs, int nspec, const
     }
     const bool active0 = keeper && run[k].phase != PH_IDLE;
     const int limit = run_passes(specs, nspec);
-    const Service<T> sums{sh, ns, t0, t1, &requests};
+    const Service sums{sh, ns, t0, t1, &requests};
     const bool service = w == 0;
     if (service) sums.start();
     __syncthreads();
@@ -760,7 +720,7 @@ __device__ __forceinline__ void run_sweep(const SpecDev *specs, int nspec, const
         if (service && it > 0) sums.finish();
         each_tile(&next[1], [&](int s, int tile) {
             const SpecDev &S = sh[s];
-            const StepVals<T> v = ops.force(S, tile, run[s].par, run[s].phase, run[s].done,
+            const StepVals v = ops.force(S, tile, run[s].par, run[s].phase, run[s].done,
                                             run[s].nsteps);
             if (lane == 0) step_requests(S, v, it, &requests);
         });

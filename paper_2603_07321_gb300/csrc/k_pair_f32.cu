@@ -134,7 +134,7 @@ __device__ __forceinline__ void force_lane(const SpecDev &S, const PotF &P, int 
 // the update of atom u by one thread, with its state in memory
 __device__ __forceinline__ void update_atom(const SpecDev &S, int u, const float f[3], int par,
                                             int mode, int phase, long long done, long long nsteps,
-                                            StepVals<FF> &v) {
+                                            StepVals &v) {
     AtomMixed A;
     A.load(S, par, u);
     atom_update_mixed(S, A, par, u, f, ((const float *)S.pen)[u], mode, phase, done, nsteps, v);
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(TPB, 8) k_force_f32(const SpecDev *__restrict_
             for (int d = 0; d < 3; ++d) f[d] = sf[d][threadIdx.x];
     }
     const int u = lb * APB + threadIdx.x;
-    StepVals<FF> v = zero_vals<FF>();
+    StepVals v = StepVals{};
     if (threadIdx.x < APB && u < S.n) update_atom(S, u, f, par, mode, phase, done, nsteps, v);
     block_partial<TPB>(S, lb, v, L);
 }
@@ -234,7 +234,7 @@ struct OpsF32 {
         }
         pe = density_end<SC76>(S, P, L, u, valid && l == 0, ra, s, wa);
     }
-    __device__ __forceinline__ StepVals<FF> force(const SpecDev &S, int tile, int par, int phase,
+    __device__ __forceinline__ StepVals force(const SpecDev &S, int tile, int par, int phase,
                                                   long long done, long long nsteps) {
         const int L = LT ? LT : lanes;
         float f[3] = {0.f, 0.f, 0.f};
@@ -245,7 +245,7 @@ struct OpsF32 {
             });
         }
         force_end(S, L, f);
-        StepVals<FF> v = zero_vals<FF>();
+        StepVals v = StepVals{};
         if (valid && l == 0)
             ra = atom_update_mixed(S, A, par, u, f, pe, MODE_STEP, phase, done, nsteps, v);
         // the new record to the atom's other lanes
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(32 * RUN_WARPS, 1)
               cudaGraphConditionalHandle again, unsigned polls, int quads, const PotF P) {
     extern __shared__ uint4 list_cache[];
     OpsF32<SC76, LT> ops{P, list_cache, quads};
-    run_resident<FF>(specs, nspec, b2s, nblk, rc, again, polls, ops);
+    run_resident(specs, nspec, b2s, nblk, rc, again, polls, ops);
 }
 
 // a sweep's warp, on one tile
@@ -279,13 +279,13 @@ struct SweepF32 {
         const int t = tile * 32 + (threadIdx.x & 31);
         density_lane<SC76, true>(S, P, S.L, t / S.L, t % S.L, par);
     }
-    __device__ __forceinline__ StepVals<FF> force(const SpecDev &S, int tile, int par, int phase,
+    __device__ __forceinline__ StepVals force(const SpecDev &S, int tile, int par, int phase,
                                                   long long done, long long nsteps) const {
         const int t = tile * 32 + (threadIdx.x & 31);
         const int L = S.L, u = t / L;
         float f[3];
         force_lane<SC76, true>(S, P, L, u, t % L, f);
-        StepVals<FF> v = zero_vals<FF>();
+        StepVals v = StepVals{};
         if (u < S.n && t % L == 0) update_atom(S, u, f, par, MODE_STEP, phase, done, nsteps, v);
         warp_reduce(v, L);
         if ((threadIdx.x & 31) == 0) store_part(part_warp(S, tile), v);
@@ -297,7 +297,7 @@ template <bool SC76>
 __global__ void __launch_bounds__(32 * SWEEP_WARPS_F32, 1)
     k_sweep_f32(const SpecDev *specs, int nspec, const int *b2s, int nblk, RunCtl *rc,
                 cudaGraphConditionalHandle again, unsigned polls, int, const PotF P) {
-    run_sweep<FF>(specs, nspec, b2s, nblk, rc, again, polls, SweepF32<SC76>{P});
+    run_sweep(specs, nspec, b2s, nblk, rc, again, polls, SweepF32<SC76>{P});
 }
 
 template <int LT>
@@ -338,16 +338,9 @@ __global__ void __launch_bounds__(32 * FINISH_WARPS)
     if (mode == MODE_EVAL || phase != PH_IDLE) {
         const int par = ctl->parity;
         const long long done = ctl->done, nsteps = ctl->nsteps;
-        if (S.prec == PTA_PREC_FP64) {
-            const StepVals<double> t = finish_sums<double>(S);
-            if (threadIdx.x == 0)
-                advance_ctl(S, t.s[0], t.s[1], t.s[2], t.d2, t.dp2, mode, phase, par, done, nsteps);
-        } else {
-            const StepVals<FF> t = finish_sums<FF>(S);
-            if (threadIdx.x == 0)
-                advance_ctl(S, to_double(t.s[0]), to_double(t.s[1]), to_double(t.s[2]), t.d2, t.dp2,
-                            mode, phase, par, done, nsteps);
-        }
+        const StepVals t = finish_sums(S);
+        if (threadIdx.x == 0)
+            advance_ctl(S, t.s[0], t.s[1], t.s[2], t.d2, t.dp2, mode, phase, par, done, nsteps);
     }
     if (!decide || threadIdx.x != 0) return;
     constexpr int BITS = 21;

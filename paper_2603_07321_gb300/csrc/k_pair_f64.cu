@@ -156,7 +156,7 @@ struct Atom64 {
 __device__ __forceinline__ void atom_update64(const SpecDev &S, Atom64 &A, int par, int a,
                                               const double f[3], double pe, int mode, int phase,
                                               long long done, long long nsteps,
-                                              StepVals<double> &out) {
+                                              StepVals &out) {
     chk_force(S, f[0], f[1], f[2]);
     const SpecCtl *ctl = S.ctl;
     out.s[1] = pe;
@@ -277,7 +277,7 @@ __device__ __forceinline__ void force_lane64(const SpecDev &S, int L, int a, int
 // the update of atom a by one thread, with its state in memory
 __device__ __forceinline__ void update_atom64(const SpecDev &S, int a, const double f[3], int par,
                                               int mode, int phase, long long done,
-                                              long long nsteps, StepVals<double> &v) {
+                                              long long nsteps, StepVals &v) {
     Atom64 A;
     A.load(S, par, a);
     atom_update64(S, A, par, a, f, ((const double *)S.pen)[a], mode, phase, done, nsteps, v);
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(TPB) k_force_f64(const SpecDev *__restrict__ s
             for (int d = 0; d < 3; ++d) f[d] = sf[d][threadIdx.x];
     }
     const int a = lb * APB + threadIdx.x;
-    StepVals<double> v = zero_vals<double>();
+    StepVals v = StepVals{};
     if (threadIdx.x < APB && a < S.n) update_atom64(S, a, f, par, mode, phase, done, nsteps, v);
     block_partial<TPB>(S, lb, v, L);
 }
@@ -364,7 +364,7 @@ struct OpsF64 {
                           [&](const double4_32a &pj) { rho_entry64<SC76>(S.pot, pa, pj, s); });
         pe = density_end64(S, L, a, valid && l == 0, pa, s, pa.w);
     }
-    __device__ __forceinline__ StepVals<double> force(const SpecDev &S, int tile, int par, int phase,
+    __device__ __forceinline__ StepVals force(const SpecDev &S, int tile, int par, int phase,
                                                   long long done, long long nsteps) {
         double f[3] = {0, 0, 0};
         if (valid)
@@ -372,7 +372,7 @@ struct OpsF64 {
                           [&](const double4_32a &pj) { force_entry64<SC76>(S.pot, pa, pj, f); });
 #pragma unroll
         for (int d = 0; d < 3; ++d) f[d] = lane_sum(f[d], L);
-        StepVals<double> v = zero_vals<double>();
+        StepVals v = StepVals{};
         if (valid && l == 0) {
             atom_update64(S, A, par, a, f, pe, MODE_STEP, phase, done, nsteps, v);
             pa.x = A.x[0];
@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(32 * RUN_WARPS, 1)
               cudaGraphConditionalHandle again, unsigned polls, int quads) {
     extern __shared__ uint4 list_cache[];
     OpsF64<SC76> ops{list_cache, quads};
-    run_resident<double>(specs, nspec, b2s, nblk, rc, again, polls, ops);
+    run_resident(specs, nspec, b2s, nblk, rc, again, polls, ops);
 }
 
 // a sweep's warp, on one tile
@@ -409,13 +409,13 @@ struct SweepF64 {
         const int t = tile * 32 + (threadIdx.x & 31);
         density_lane64<SC76, true>(S, S.L, t / S.L, t % S.L, par);
     }
-    __device__ __forceinline__ StepVals<double> force(const SpecDev &S, int tile, int par, int phase,
+    __device__ __forceinline__ StepVals force(const SpecDev &S, int tile, int par, int phase,
                                                       long long done, long long nsteps) const {
         const int t = tile * 32 + (threadIdx.x & 31);
         const int L = S.L, a = t / L;
         double f[3];
         force_lane64<SC76, true>(S, L, a, t % L, f);
-        StepVals<double> v = zero_vals<double>();
+        StepVals v = StepVals{};
         if (a < S.n && t % L == 0) update_atom64(S, a, f, par, MODE_STEP, phase, done, nsteps, v);
         warp_reduce(v, L);
         if ((threadIdx.x & 31) == 0) store_part(part_warp(S, tile), v);
@@ -427,7 +427,7 @@ template <bool SC76>
 __global__ void __launch_bounds__(32 * SWEEP_WARPS_F64, 1)
     k_sweep_f64(const SpecDev *specs, int nspec, const int *b2s, int nblk, RunCtl *rc,
                 cudaGraphConditionalHandle again, unsigned polls, int) {
-    run_sweep<double>(specs, nspec, b2s, nblk, rc, again, polls, SweepF64<SC76>{});
+    run_sweep(specs, nspec, b2s, nblk, rc, again, polls, SweepF64<SC76>{});
 }
 
 #define PTA_F64_SWITCH(KER, SC, ARG)                                                   \
