@@ -39,9 +39,9 @@ __device__ __forceinline__ float powi(float s, int k) {
 // displacement in quanta (q2: square of the quantum).
 __device__ __forceinline__ float pair_r2(float q2, const int4 &a, const int4 &b, float &dx,
                                          float &dy, float &dz) {
-    dx = (float)(b.x - a.x);
-    dy = (float)(b.y - a.y);
-    dz = (float)(b.z - a.z);
+    dx = (float)rec_diff(b.x, a.x);
+    dy = (float)rec_diff(b.y, a.y);
+    dz = (float)rec_diff(b.z, a.z);
     return fmaf(dz, dz, fmaf(dy, dy, dx * dx)) * q2;
 }
 

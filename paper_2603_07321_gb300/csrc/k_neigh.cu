@@ -247,8 +247,8 @@ __global__ void __launch_bounds__(BUILD_WARPS * 32, 8) k_build(const SpecDev *__
             for (int b = s; b < e; b += 32, j += 32) {
                 const int4 rj = nx;
                 if (b + 32 < e) nx = rec[min(j + 32, e - 1)];
-                const float fx = (float)(rj.x - ra.x), fy = (float)(rj.y - ra.y),
-                            fz = (float)(rj.z - ra.z);
+                const float fx = (float)rec_diff(rj.x, ra.x), fy = (float)rec_diff(rj.y, ra.y),
+                            fz = (float)rec_diff(rj.z, ra.z);
                 const float r2 = fmaf(fz, fz, fmaf(fy, fy, fx * fx));
                 bool in = r2 < hi2 && j < e && j != a;
                 if (in && r2 >= lo2) in = in_list_exact(S, par, a, j);

@@ -105,7 +105,8 @@ __device__ __forceinline__ void merge(StepVals &a, const StepVals &b) {
 
 // squared displacement of a record from an earlier one, quanta^2
 __device__ __forceinline__ float moved2(const int4 &a, const int4 &b) {
-    const float x = (float)(a.x - b.x), y = (float)(a.y - b.y), z = (float)(a.z - b.z);
+    const float x = (float)rec_diff(a.x, b.x), y = (float)rec_diff(a.y, b.y),
+                z = (float)rec_diff(a.z, b.z);
     return fmaf(z, z, fmaf(y, y, __fmul_rn(x, x)));
 }
 
@@ -349,7 +350,8 @@ __device__ __forceinline__ void prune_lane(const SpecDev &S, int u, int l, int L
     const int nl = chk_count(S, ab.y > l ? (ab.y - l + L - 1) / L : 0, S.cap_use);
     int kept = ab.x / L + (l < ab.x % L);
     auto test = [&](bool have, unsigned e, const int4 &x) {
-        const float dx = (float)(x.x - ra.x), dy = (float)(x.y - ra.y), dz = (float)(x.z - ra.z);
+        const float dx = (float)rec_diff(x.x, ra.x), dy = (float)rec_diff(x.y, ra.y),
+                    dz = (float)rec_diff(x.z, ra.z);
         if (fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < rp2 && have) {
             dst[(kept >> 2) * 128 + (kept & 3)] = e;
             ++kept;

@@ -330,13 +330,21 @@ __host__ __device__ __forceinline__ void cell_coords(const int nc[3], int r, int
     serp_coords(nc[0], nc[1], r, x, y, z);
 }
 
+// arithmetic of records, modulo 2^32 (signed arithmetic may not wrap): the
+// difference of two coordinates, and a coordinate from quanta of 2^shift and
+// of one
+__host__ __device__ __forceinline__ int rec_diff(int a, int b) {
+    return (int)((unsigned)a - (unsigned)b);
+}
+__host__ __device__ __forceinline__ int rec_join(int hi, int lo, int shift) {
+    return (int)(((unsigned)hi << shift) + (unsigned)lo);
+}
 // one coordinate of a record: hi is a multiple of 2^-12 A and enters exactly,
 // lo is rounded to the nearest quantum (a quantum above 2^-12 A, which takes a
 // cutoff of ~0.1 mm, rounds their sum)
 __device__ __forceinline__ int rec_coord(const SpecDev &S, float hi, float lo) {
     if (S.rec_shift < 0) return __float2int_rn((hi + lo) * S.f_rq);
-    return (int)((unsigned)__float2int_rn(hi * (float)HI_SCALE) << S.rec_shift) +
-           __float2int_rn(lo * S.f_rq);
+    return rec_join(__float2int_rn(hi * (float)HI_SCALE), __float2int_rn(lo * S.f_rq), S.rec_shift);
 }
 __device__ __forceinline__ int4 rec_mixed(const SpecDev &S, float hx, float hy, float hz, float lx,
                                           float ly, float lz) {
