@@ -31,7 +31,7 @@ __device__ __forceinline__ float rcp_approx(float x) {
 
 __device__ __forceinline__ float powi(float s, int k) {
     float p = 1.f;
-    for (int i = 0; i < k; ++i) p *= s;
+    for (int i = 0; i < k; ++i) p = __fmul_rn(p, s);
     return p;
 }
 
@@ -42,7 +42,7 @@ __device__ __forceinline__ float pair_r2(float q2, const int4 &a, const int4 &b,
     dx = (float)rec_diff(b.x, a.x);
     dy = (float)rec_diff(b.y, a.y);
     dz = (float)rec_diff(b.z, a.z);
-    return fmaf(dz, dz, fmaf(dy, dy, dx * dx)) * q2;
+    return __fmul_rn(fmaf(dz, dz, fmaf(dy, dy, __fmul_rn(dx, dx))), q2);
 }
 
 // A pair beyond rc gets y = 1/r = 0 (the force pass) or r^2 = infinity, whose
@@ -76,16 +76,17 @@ __device__ __forceinline__ void rho_pair(const PotF &P, float q2, const int4 &a,
     if (SC76) {
         const float rm = in ? r2 : __int_as_float(0x7f800000);
         const float u = rcp_approx(rm), y = rsq_approx(rm);
-        const float u3 = (u * u) * u;
-        s.sm += u3;
+        const float u3 = __fmul_rn(__fmul_rn(u, u), u);
+        s.sm = __fadd_rn(s.sm, u3);
         s.sn = fmaf(u3, y, s.sn);
         s.sr = fmaf(r2, y, s.sr);
     } else {
         float y = rsq_approx(r2);
         y = in ? y : 0.f;
         y = fmaf(0.5f * y, fmaf(-r2, y * y, 1.f), y);
-        s.sm += in ? powi(P.a * y, P.m) - P.Am + P.Bm * fmaf(r2, y, -P.rc) : 0.f;
-        s.sn += powi(y, P.n);
+        const float phi = __fadd_rn(powi(__fmul_rn(P.a, y), P.m), -P.Am);
+        s.sm = __fadd_rn(s.sm, in ? fmaf(P.Bm, fmaf(r2, y, -P.rc), phi) : 0.f);
+        s.sn = __fadd_rn(s.sn, powi(y, P.n));
         s.sr = fmaf(r2, y, s.sr);
     }
     s.cnt += in;
