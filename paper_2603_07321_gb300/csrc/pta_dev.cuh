@@ -62,6 +62,7 @@ enum AtomFlag : uint8_t { FLAG_MOBILE = 0, FLAG_LEFT = 1, FLAG_RIGHT = 2 };
 struct PotDev {
     double eps, c, a, rc, rc2, An, Bn, Am, Bm, ec;
     double an, am, kn, bmq, ebn, fpsc;  // as in PotF, in FP64
+    double am_lo, fpsc_rel;  // what rounding took off am; off fpsc, relative to it
     int n, m;
     float f_eps, f_a, f_rc, f_rc2, f_An, f_Bn, f_Am, f_Bm, f_ec;
     int sc76;  // 1 when (n, m) == (7, 6): the fast specialised kernels apply
