@@ -7,8 +7,9 @@
 // of edge >= rc + skin; atoms outside the grid are clamped onto its border
 // cells, which keeps every pair within reach (clamping is non-expansive), and
 // are reported (PTA_ERANGE): the grid's margin is a quarter of the specimen's
-// extent, which no atom of a deforming specimen reaches.  Along x each cell is
-// cut in CELL_SPLIT, to fit a row's candidates to the radius.
+// extent, which no atom of a deforming specimen reaches.  Where the atoms fill
+// the grid, each cell is cut in CELL_SPLIT along x, to fit a row's candidates to
+// the radius.
 // After binning, the atoms themselves are permuted into cell order (cells in
 // rank order, atoms of a cell in creation order), so that
 // the 32 atoms of a warp share a cell and read overlapping neighbours, and a

@@ -356,8 +356,8 @@ static int compute_sizes(const pta_specimen &s, const pta_potential &p, const pt
     if (mem) z->apw = std::max(z->apw, (int)((z->n + most - 1) / most));
     z->nblk_bld = (int)((z->n + BUILD_WARPS * z->apw - 1) / (BUILD_WARPS * z->apw));
     z->bld_scratch = mem ? (size_t)z->nblk_bld * BUILD_WARPS * build_words(z->cap_use) : 0;
-    // cell edge a multiple of 2^-11 A and grid origin on the 2^-12 A grid, so
-    // that cell centres and centre differences are exact in FP32
+    // cell edge on the 2^-11 A grid, grid origin on the 2^-12 A grid (exact in
+    // FP32)
     z->h = std::ceil(rl * (1.0 + 1e-4) * 2048.0) / 2048.0;
     double maxspan = 0;
     double span[3];
@@ -376,8 +376,14 @@ static int compute_sizes(const pta_specimen &s, const pta_potential &p, const pt
     if (ncell > (1LL << 30)) return PTA_EINVAL;
     // cells are shorter along x, the direction in which the list build walks
     // them, and so fits its walk to the list radius: a row takes on average
-    // 2 reach + h / split of the rows' atoms instead of 2 reach + h
-    z->split = ncell * CELL_SPLIT <= (1LL << 30) ? CELL_SPLIT : 1;
+    // 2 reach + h / split of the rows' atoms instead of 2 reach + h.  Only where
+    // the atoms fill the grid, whose margin follows the longest edge: one block
+    // scans all cells, and each takes 8 bytes.  Force evaluations, undivided ->
+    // divided, by undivided cells per atom: 0.1-0.2 (cubes) 316 -> 304 and 2,122
+    // -> 1,944 us, 0.3-0.6 (30x23x9, 50x50x3 cells) 200 -> 199 and 205 -> 202,
+    // 1.3 (100x10x10) 715 -> 730, 10 (200x6x6) 529 -> 670, 2,000 (1000x1x3) 4,967
+    // -> 19,561 and 263 -> 880 MB.
+    z->split = 2 * ncell <= z->n ? CELL_SPLIT : 1;
     z->nc[0] *= z->split;
     z->ncell = (int)(ncell * z->split);
     const long long W = 32 / z->L;
@@ -391,7 +397,7 @@ static int compute_sizes(const pta_specimen &s, const pta_potential &p, const pt
 }
 
 // partials of 32 bytes: per warp of the pair blocks in resident runs, else per
-// block and per group of 32 blocks; behind them the groups' counters
+// block
 static size_t part_bytes(const Sizes &z) {
     const size_t nb = (size_t)std::max(z.nblk_pair, z.nblk_atom);
     return 32 * (TPB / 32) * nb;

@@ -16,7 +16,7 @@
 namespace pta {
 
 constexpr int TPB = 128;        // threads per block of the atom and pair kernels
-constexpr int CELL_SPLIT = 4;   // cells along x per cell edge along y and z
+constexpr int CELL_SPLIT = 4;   // cells along x per cell edge along y and z, where divided
 constexpr int SCAN_THREADS = 1024;
 constexpr int BUILD_WARPS = 4;  // warps per block of the list build
 constexpr int NEIGH_CAP_MOST = 4096;  // largest capacity that can be asked for
