@@ -80,7 +80,7 @@ def store(natoms: int, replicas: int, precision: int, layout: dict, rate: float)
 
 
 def tune(n_cells, precision: int = 1, replicas: int = 1, T0: float = 300.0, seed: int = 1,
-         lanes=(1, 2, 4, 8), skins=(1.0, 1.5, 2.0, 2.5), margins=(0.3,), steps: int = 200,
+         lanes=(1, 2, 4, 8, 16), skins=(1.0, 1.5, 2.0, 2.5), margins=(0.3,), steps: int = 200,
          warm: int = 50, strain: float = 1e-3, save: bool = True):
     """Time every (lanes, skin, prune_margin) candidate; returns (best,
     table): best is a dict of Ctx keyword arguments, table a list of
