@@ -237,7 +237,19 @@ int pta_get_strain(const pta_ctx *ctx, double *strain);
 
 /* One fine burst of nsteps velocity-Verlet steps from the current state
  * (which the next burst continues from, Eqs. (x_guess_step1),
- * (x_guess_step3)).  Blocks until the averages are on the host.  nsteps >= 1. */
+ * (x_guess_step3)).  Blocks until the averages are on the host.  nsteps >= 1.
+ *
+ * Specimens (and batches) of up to a few ten thousand to hundred thousand atoms
+ * advance inside one cooperative kernel over every SM of the GPU from one list
+ * build to the next: bursts of contexts on different streams take turns on
+ * that scale rather than share the GPU.  Larger ones, batches of unlike
+ * precision or potential, adaptive bursts and timed ones launch each pass.
+ * Results are the same bits either way.
+ *
+ * After PTA_ENAN the state is not usable (non-finite forces have entered it,
+ * and it lies one or two steps beyond the sample that failed); set or load
+ * another.  After PTA_ECUDA every call that would use the specimen is refused
+ * (PTA_ECUDA), for all members of a batch whose call returned it. */
 int pta_fine_burst(pta_ctx *ctx, int64_t nsteps, pta_averages *out);
 /* Continuous loading (Sec. Verification with fine dynamics): a fine burst
  * of nsteps steps during which the right grip advances by d_eps_per_step *
@@ -314,13 +326,16 @@ int pta_get_neighbours(pta_ctx *ctx, int32_t *counts, int32_t *list, int64_t n, 
 int pta_save_state(pta_ctx *ctx, void *buf, size_t *len);
 int pta_load_state(pta_ctx *ctx, const void *buf, size_t len);
 
-/* Kernel timing.  While timing is on, every fine-step iteration records
- * CUDA events (on the context's stream, inside the replayed graphs) around
- * its three parts: the neighbour-list build (usually skipped on the
- * device), the density pass and the force pass.  pta_get_timing returns the
- * summed event times in milliseconds and the number of iterations since
- * timing was switched on.  Timing costs one host synchronisation per graph
- * replay of 64 iterations. */
+/* Kernel timing.  While timing is on, every fine step launches its passes and
+ * records CUDA events (on the context's stream, inside the replayed graphs)
+ * around its three parts: list work (build or pruning, usually skipped on the
+ * device), the density pass, and the force pass with the kernel that ends the
+ * step.  Specimens that otherwise advance inside one kernel (pta_fine_burst)
+ * are launched too while timed, so that their times are those of the passes
+ * and not of an untimed step, which is faster.  pta_get_timing returns the
+ * summed event times in milliseconds and the number of iterations since timing
+ * was switched on.  Timing costs one host synchronisation per graph replay of
+ * 64 iterations. */
 typedef struct {
     double rebuild_ms, density_ms, force_ms;
     int64_t iterations;

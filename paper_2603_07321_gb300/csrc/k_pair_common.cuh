@@ -383,8 +383,10 @@ __device__ __forceinline__ void prune_lane(const SpecDev &S, int u, int l, int L
 //
 // The latency of a step is that of its chain of L2 round trips (~0.5 us
 // each), so whatever can is kept on the SM: the atoms' state, own record and
-// density weight in registers, the lists and the descriptors in shared memory
-// (a barrier empties L1), the step count by every block for itself.  What
+// density weight in registers (of the 128 a thread, which do not hold all of it
+// in mixed precision: ~130 bytes are spilled to local memory), the lists and
+// the descriptors in shared memory (a barrier empties L1), the step count by
+// every block for itself.  What
 // remains is one round of gathers per pass and two barriers.  The sums of a
 // step do not hold up the next one: a service warp in every block, beside
 // those that hold atoms, sums the groups of partials during the next density
@@ -654,12 +656,11 @@ __device__ __forceinline__ void run_resident(const SpecDev *specs, int nspec, co
     if (blockIdx.x == 0 && w == 0) run_again(specs, nspec, state, again);
 }
 
-// A block of a run over a larger table: contiguous tiles again, but several
-// per warp, handed out one at a time; the atoms' state and the lists stay in
-// memory.  Against launched passes it has no launches and no conditional node
-// per step (~25 us of it on a specimen of 108,000 atoms) and no last wave:
-// the cube of 470,596 atoms fills 3.02 waves of eight blocks per SM, and the
-// blocks of the fourth ran alone for ~10% of a pass.
+// A block of a run over a larger table: contiguous tiles again, handed out one
+// at a time, as a block's warps may have more than one each; the atoms' state
+// and the lists stay in memory.  Against launched passes it has no launches and
+// no conditional node per step (~25 us of it on a specimen of 108,000 atoms).
+// Where it stops paying: run_shape.
 struct SpecRun {
     int phase, par, prune;
     long long done, nsteps;

@@ -396,8 +396,8 @@ static int compute_sizes(const pta_specimen &s, const pta_potential &p, const pt
     return PTA_OK;
 }
 
-// partials of 32 bytes: per warp of the pair blocks in resident runs, else per
-// block
+// partials of 32 bytes: per warp of the pair blocks in resident runs and sweeps,
+// else per block; and per group of 32 blocks in the former
 static size_t part_bytes(const Sizes &z) {
     const size_t nb = (size_t)std::max(z.nblk_pair, z.nblk_atom);
     return 32 * (TPB / 32) * nb;
