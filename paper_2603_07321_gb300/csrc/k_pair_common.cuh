@@ -220,33 +220,74 @@ __device__ inline void advance_ctl(const SpecDev &S, double K, double U, double 
     c->parity = par ^ 1;
 }
 
+// Sums over the lanes of a warp of N values each (N a power of two, at most 16),
+// along the butterfly of sum_lanes: every stage halves the values that a lane
+// holds, until value i is in lanes (32 / N) i and on.
+template <int N>
+__device__ __forceinline__ double sum_transposed(double *v) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16, n = N / 2; o > 0; o >>= 1, n >>= 1) {
+        if (n == 0) {
+            v[0] = add_xor(v[0], o);
+            continue;
+        }
+        const bool upper = lane & o;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const double other = __shfl_xor_sync(0xffffffffu, upper ? v[i] : v[i + n], o);
+            v[i] = __dadd_rn(upper ? v[i + n] : v[i], other);
+        }
+    }
+    return v[0];
+}
+
 // The totals of a launched step, valid in thread 0 of a block of
 // 32 * FINISH_WARPS threads, from the force pass's block partials along a
 // fixed tree: groups of 32 consecutive blocks (one per lane, butterfly
 // shuffles), 32 groups at a time likewise, then those in order.
 //
-// Bound: three round trips of latency; a warp's groups are loaded together.
+// Bound: three round trips of latency, and the FP64 additions of one SM.  A
+// warp's eight groups are loaded together and summed together, in 16 additions
+// of a warp instead of 40: 470,596 atoms 214.5 us per step instead of 217.5.
 constexpr int FINISH_WARPS = 16, FINISH_GROUPS = 8;
 __device__ __forceinline__ StepVals finish_sums(const SpecDev &S) {
-    constexpr int ROUND = FINISH_WARPS * FINISH_GROUPS;
+    constexpr int ROUND = FINISH_WARPS * FINISH_GROUPS, G = FINISH_GROUPS;
     __shared__ StepVals sg[ROUND], sc[ROUND / 32];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nblk = S.nblk_pair, ngroups = (nblk + PART_GROUP - 1) / PART_GROUP;
     StepVals t = StepVals{};
     for (int r = 0; r < ngroups; r += ROUND) {
-        StepVals a[FINISH_GROUPS];
+        StepVals a[G];
 #pragma unroll
-        for (int k = 0; k < FINISH_GROUPS; ++k) {
-            const int b = (r + k * FINISH_WARPS + w) * PART_GROUP + lane;
+        for (int k = 0; k < G; ++k) {
+            const int b = (r + w * G + k) * PART_GROUP + lane;
             a[k] = StepVals{};
             if (b < nblk) load_part(S.part + (long long)PART * b, a[k]);
         }
+        if (r + w * G < ngroups) {
+            double v[2 * G];
+            bool reaction = false;
 #pragma unroll
-        for (int k = 0; k < FINISH_GROUPS; ++k) {
-            const int g = k * FINISH_WARPS + w;
-            if (r + g >= ngroups) break;
-            warp_reduce(a[k], 1);
-            if (lane == 0) sg[g] = a[k];
+            for (int k = 0; k < G; ++k) {
+                v[2 * k] = a[k].s[0];
+                v[2 * k + 1] = a[k].s[1];
+                reaction |= a[k].s[2] != 0.0;
+                const float d2 = warp_max(a[k].d2), dp2 = warp_max(a[k].dp2);
+                if (lane == k) {
+                    sg[w * G + k].d2 = d2;
+                    sg[w * G + k].dp2 = dp2;
+                }
+            }
+            const double ku = sum_transposed<2 * G>(v);
+            if ((lane & 1) == 0) sg[w * G + (lane >> 2)].s[(lane >> 1) & 1] = ku;
+            double x = 0.0;
+            if (__any_sync(0xffffffffu, reaction)) {
+#pragma unroll
+                for (int k = 0; k < G; ++k) v[k] = a[k].s[2];
+                x = sum_transposed<G>(v);
+            }
+            if ((lane & 3) == 0) sg[w * G + (lane >> 2)].s[2] = x;
         }
         __syncthreads();
         if (w * 32 < min(ROUND, ngroups - r)) {
