@@ -55,7 +55,10 @@ constexpr int CHUNK = 64;
 constexpr unsigned BARRIER_POLLS = 1u << 22;
 unsigned barrier_polls() {
     const char *e = std::getenv("PTA_BARRIER_POLLS");
-    return e ? (unsigned)std::strtoul(e, nullptr, 10) : BARRIER_POLLS;
+    char *end = nullptr;
+    const unsigned long v = e ? std::strtoul(e, &end, 10) : 0;
+    return e && end != e && *end == 0 ? (unsigned)std::min(v, (unsigned long)BARRIER_POLLS)
+                                      : BARRIER_POLLS;
 }
 
 struct Allocator {

@@ -63,3 +63,11 @@ def test_in_a_batch(P, monkeypatch, call):
     b.close()
     for c in cs:
         c.close()
+
+
+@pytest.mark.parametrize("text", ["", "many", "12x"])
+def test_a_limit_that_is_no_number_is_none(P, monkeypatch, text):
+    monkeypatch.setenv("PTA_BARRIER_POLLS", text)
+    c = P.Ctx((4, 4, 5), T0=300.0, seed=1, precision=1)
+    assert c.fine_burst(20).nsteps == 20
+    c.close()
