@@ -239,11 +239,12 @@ int pta_get_strain(const pta_ctx *ctx, double *strain);
  * (which the next burst continues from, Eqs. (x_guess_step1),
  * (x_guess_step3)).  Blocks until the averages are on the host.  nsteps >= 1.
  *
- * Specimens (and batches) of up to a few ten thousand to hundred thousand atoms
- * advance inside one cooperative kernel over every SM of the GPU from one list
- * build to the next: bursts of contexts on different streams take turns on
- * that scale rather than share the GPU.  Larger ones, batches of unlike
- * precision or potential, adaptive bursts and timed ones launch each pass.
+ * Specimens and batches of up to ~270,000 atoms (fewer with several threads per
+ * atom; by how they fill the GPU) advance inside one cooperative kernel over
+ * every SM from one list build to the next: bursts of contexts on different
+ * streams take turns on that scale rather than share the GPU.  Larger ones,
+ * batches of unlike precision or potential, adaptive bursts and timed ones
+ * launch each pass.
  * Results are the same bits either way.
  *
  * After PTA_ENAN the state is not usable (non-finite forces have entered it,
